@@ -552,7 +552,6 @@ static fmap_status enqueue(fmap_plan_t* p, const fmap_atoms* a, float* d_2F,
   }
   if (ev[3]) FMAP_CUDA(cudaEventRecord(ev[3], s));
   FMAP_CUDA(launch_flag_and_fixup(p, a, d_2F, s));
-  FMAP_CUDA(launch_final_reduce(p, tiles, true, d_summary, s));
   FMAP_CUDA(launch_refine(p, a, d_2F, d_summary, tiles, s));
   if (ev[4]) FMAP_CUDA(cudaEventRecord(ev[4], s));
   return FMAP_OK;

@@ -133,7 +133,8 @@ static int64_t units_of(const fmap_plan_s* p, const fmap_batch_item& it, int ph,
     case BP_FLAG_COUNT:
     case BP_FLAG_WRITE: return work ? (cells * n_ant + kFlagUnit - 1) / kFlagUnit : 0;
     case BP_FLAG_SCAN: return work ? 1 : 0;
-    case BP_FIXUP: return work ? (int64_t)(kFixSlots / kFixSlotsPerUnit) * fixup_blocks_y((int32_t)T) : 0;
+    case BP_FIXUP:
+      return work ? (int64_t)kFixUnits * fixup_blocks_y((int32_t)T, it.atoms.shared_antenna != 0) : 0;
     case BP_RED_GROUPS: {
       if (!it.d_summary || T == 0) return 0;
       const int64_t used =

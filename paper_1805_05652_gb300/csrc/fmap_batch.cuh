@@ -56,10 +56,9 @@ struct BUnits {
 // coefficients in 256-entry blocks, index-table rows, fix-up slots.
 constexpr int kCoefBlocksPerUnit = 8;
 constexpr int kIdxRowsPerUnit = 8;
-constexpr int kFixSlotsPerUnit = 4;
+constexpr int kFixUnits = 32;        // fix-up units per template group (each strides over the slots)
 constexpr int kPermPerUnit = 4096;   // chunk-major copy entries per unit
 constexpr int kBitsPerUnit = 4096;   // marked-entry bitmask words cleared per unit
-static_assert(kFixSlots % kFixSlotsPerUnit == 0, "fix-up slot groups");
 
 // Phases of the batch pipeline, in launch order.
 enum BPhase {

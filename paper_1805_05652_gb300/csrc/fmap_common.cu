@@ -277,10 +277,13 @@ __device__ __forceinline__ Partial64 widen(const Partial& q) {
 }
 
 // Level 1: block (g, t) merges slots [g*kRedGroup, (g+1)*kRedGroup) of the
-// concatenation [main tiles 0..n_tiles) ++ [fix-up slots fix0..fix0+n_fix).
-__device__ __forceinline__ void reduce_groups_body(const Partial* __restrict__ parts, int64_t n_tiles, int64_t fix0, int64_t n_fix,
+// concatenation [main tiles 0..n_tiles) ++ [fix-up slots in use, from fix0] (n_flag
+// of them marked among `entries`; null: none).
+__device__ __forceinline__ void reduce_groups_body(const Partial* __restrict__ parts, int64_t n_tiles, int64_t fix0,
+                const int32_t* __restrict__ n_flag, int64_t entries,
                 int64_t stride, int64_t n_groups, Partial64* __restrict__ groups,
     const uint3 bid, const dim3 gdim) {
+  const int64_t n_fix = n_flag ? fix_slots_used(min((int64_t)*n_flag, entries)) : 0;
   const Partial* pp = parts + (int64_t)bid.y * stride;
   const int64_t n_all = n_tiles + n_fix;
   const int64_t lo = (int64_t)bid.x * kRedGroup;
@@ -293,9 +296,10 @@ __device__ __forceinline__ void reduce_groups_body(const Partial* __restrict__ p
 }
 
 __global__ void __launch_bounds__(kRedThreads)
-k_reduce_groups(const Partial* __restrict__ parts, int64_t n_tiles, int64_t fix0, int64_t n_fix,
-                int64_t stride, int64_t n_groups, Partial64* __restrict__ groups) {
-  reduce_groups_body(parts, n_tiles, fix0, n_fix, stride, n_groups, groups, blockIdx, gridDim);
+k_reduce_groups(const Partial* __restrict__ parts, int64_t n_tiles, int64_t fix0,
+                const int32_t* __restrict__ n_flag, int64_t entries, int64_t stride,
+                int64_t n_groups, Partial64* __restrict__ groups) {
+  reduce_groups_body(parts, n_tiles, fix0, n_flag, entries, stride, n_groups, groups, blockIdx, gridDim);
 }
 
 // Level 2: one block per template over its groups; writes the summary and,
@@ -318,7 +322,7 @@ __device__ __forceinline__ void reduce_final_body(const Partial64* __restrict__ 
       t.M = r.max2F;
       t.arg = r.arg;
       t.N = r.nvalid;
-      t.pad = 0;
+      t.done[0] = t.done[1] = 0;
       tstat[bid.x] = t;
     }
     fmap_summary o;
@@ -349,27 +353,30 @@ k_reduce_final(const Partial64* __restrict__ groups, int64_t n_groups, int32_t n
 
 int64_t reduce_groups_of(int64_t slots) { return std::max<int64_t>(1, (slots + kRedGroup - 1) / kRedGroup); }
 
-static cudaError_t reduce_into(const Partial* parts, int64_t n_tiles, int64_t fix0, int64_t n_fix,
-                               int64_t stride, int32_t T, int32_t n_tau, double log_prior,
+static cudaError_t reduce_into(const Partial* parts, int64_t n_tiles, int64_t fix0,
+                               const int32_t* n_flag, int64_t entries, int64_t stride, int32_t T, int32_t n_tau, double log_prior,
                                Partial64* groups, fmap_summary* d_summary, cudaStream_t s,
                                TStat* tstat = nullptr, int32_t* ref_hist = nullptr,
                                int32_t* ref_n = nullptr) {
-  const int64_t n_groups = reduce_groups_of(n_tiles + n_fix);
+  const int64_t n_groups = reduce_groups_of(n_tiles + (n_flag ? kFixSlots : 0));
   k_reduce_groups<<<dim3((unsigned)n_groups, (unsigned)T), kRedThreads, 0, s>>>(
-      parts, n_tiles, fix0, n_fix, stride, n_groups, groups);
+      parts, n_tiles, fix0, n_flag, entries, stride, n_groups, groups);
   k_reduce_final<<<T, kRedThreads, 0, s>>>(groups, n_groups, n_tau > 0 ? n_tau : 1, log_prior,
                                            d_summary, tstat, ref_hist, ref_n);
   return cudaGetLastError();
 }
 
-cudaError_t launch_final_reduce(fmap_plan_s* p, int64_t n_tiles, bool with_fix,
+cudaError_t launch_final_reduce(fmap_plan_s* p, int64_t n_tiles, const fmap_atoms* a,
                                 fmap_summary* d_summary, cudaStream_t s) {
   if (!d_summary || p->n_templates == 0) return cudaSuccess;
-  const bool fix = with_fix && (int64_t)p->grid.n_t0 * p->grid.n_tau > 0;
+  const int64_t entries = (int64_t)p->grid.n_t0 * p->grid.n_tau *
+                          (a && !a->shared_antenna ? p->n_templates : 1);
+  const bool fix = a && entries > 0;
   p->launches += 2;
-  return reduce_into(p->ws.partials, n_tiles, p->n_tiles, fix ? kFixSlots : 0, p->part_stride,
-                     p->n_templates, p->grid.n_tau, p->log_prior, (Partial64*)p->ws.groups,
-                     d_summary, s, p->ws.tstat, p->ws.ref_hist, p->ws.ref_n);
+  return reduce_into(p->ws.partials, n_tiles, p->n_tiles, fix ? p->ws.n_flag : nullptr, entries,
+                     p->part_stride, p->n_templates, p->grid.n_tau, p->log_prior,
+                     (Partial64*)p->ws.groups, d_summary, s, p->ws.tstat, p->ws.ref_hist,
+                     p->ws.ref_n);
 }
 
 // ---------------------------------------------------------------------------
@@ -420,7 +427,7 @@ cudaError_t launch_marginalise_into(const fmap_grid& g, int32_t n_templates, con
   // the group results of the first level follow the tile partials
   Partial64* groups = (Partial64*)(parts + (int64_t)n_templates * tiles);
   groups = (Partial64*)(((uintptr_t)groups + 31) & ~(uintptr_t)31);
-  return reduce_into(parts, tiles, 0, 0, tiles, n_templates, g.n_tau, log_prior, groups,
+  return reduce_into(parts, tiles, 0, nullptr, 0, tiles, n_templates, g.n_tau, log_prior, groups,
                      d_summary, s);
 }
 
@@ -436,7 +443,7 @@ cudaError_t launch_marginalise(fmap_plan_s* p, const float* d_2F, const uint8_t*
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  return launch_final_reduce(p, tiles, false, d_summary, s);
+  return launch_final_reduce(p, tiles, nullptr, d_summary, s);
 }
 
 
@@ -467,8 +474,8 @@ __global__ void __launch_bounds__(kIdxThreads) kb_index(const BItem* __restrict_
 __global__ void __launch_bounds__(kRedThreads) kb_red_groups(const BItem* __restrict__ items,
                                                              BUnits u) {
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
-    const int64_t fix = it.cells > 0 ? kFixSlots : 0;
-    reduce_groups_body(it.partials, it.tiles_used, it.n_tiles, fix, it.part_stride, it.red_groups,
+    reduce_groups_body(it.partials, it.tiles_used, it.n_tiles, it.cells > 0 ? it.n_flag : nullptr,
+                       it.flag_entries, it.part_stride, it.red_groups,
                        (Partial64*)it.red_buf,
                        make_uint3((unsigned)(k % it.red_groups), (unsigned)(k / it.red_groups), 0),
                        dim3((unsigned)it.red_groups, (unsigned)it.T));

@@ -60,21 +60,20 @@ struct __align__(16) Partial {
 // to the fix-up of fmap_fixup.cu, which decides D > 0 from float-float sums
 // and then records the outcome in valid (3 = valid, 0 = invalid).
 constexpr double kCondThreshold = 100.0;
-// Reduction slots per template written by the fix-up kernel.
+// Reduction slots per template of the fix-up kernel: the list of ill-conditioned
+// entries is spread over just enough of them for kFixPerSlot entries each (one
+// thread per entry), or over all of them when it is longer.
 constexpr int kFixSlots = 512;
-// Below this many templates the fix-up runs one thread per listed entry
-// (else one per template), and spreads the list over just enough slots for
-// about kFixPerSlot entries each (else over all kFixSlots).
-constexpr int kFixCellModeT = 8;
 constexpr int kFixPerSlot = 128;
-// Entries [lo, hi) of fix-up slot b (of G) for a list of n entries and T
-// templates; every slot past the used ones is empty.  The fix-up kernels
-// and the refinement's scan of a slot's cells share this partition.
-__host__ __device__ inline void fix_slot_range(int64_t b, int64_t n, int32_t G, int32_t T,
-                                               int64_t* lo, int64_t* hi) {
-  const int64_t per = T < kFixCellModeT ? kFixPerSlot : 1;
-  int64_t used = (n + per - 1) / per;
-  used = used < 1 ? 1 : (used > G ? G : used);
+// Slots in use for a list of n entries (the others are neither written nor
+// read); entries [lo, hi) of slot b.  The fix-up kernel, the reductions and the
+// refinement's scan of a slot's cells share this partition.
+__host__ __device__ inline int32_t fix_slots_used(int64_t n) {
+  const int64_t used = (n + kFixPerSlot - 1) / kFixPerSlot;
+  return (int32_t)(used > kFixSlots ? kFixSlots : used);
+}
+__host__ __device__ inline void fix_slot_range(int64_t b, int64_t n, int64_t* lo, int64_t* hi) {
+  const int64_t used = fix_slots_used(n);
   *lo = b < used ? b * n / used : n;
   *hi = b < used ? (b + 1) * n / used : n;
 }
@@ -105,13 +104,14 @@ struct TileGeom {
 };
 // Per-template statistics of the fast reduction, kept for the refinement:
 // S = sum over valid cells of exp((2F - M) / 2), M = max 2F, arg its lowest
-// cell, N the valid count.
+// cell, N the valid count; done counts the blocks that finished each of the
+// refinement's two passes (the last one goes on with what follows it).
 struct __align__(32) TStat {
   double S;
   float M;
   int32_t arg;
   long long N;
-  long long pad;
+  int32_t done[2];
 };
 // Window length L(tau) in seconds: tau (rect) or floor(cut8 tau / 8) (exp,
 // cut8 = 24 by default: Eq. winexp's 3 tau).  An atom belongs to the window
@@ -336,15 +336,16 @@ const void* batch_kernel_fixup(int phase);
 cudaError_t launch_rect_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 cudaError_t launch_flag_and_fixup(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
                                   cudaStream_t s);
-// Top-cell refinement of the summaries (after launch_final_reduce); d_2F is
-// the map the compute call wrote, n_tiles the main kernel's partial slots
+// Reduction and top-cell refinement of the summaries (in place of
+// launch_final_reduce); d_2F is the map the compute call wrote, n_tiles the main kernel's partial slots
 // (geometry p->tiles).
 cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
                           fmap_summary* d_summary, int64_t n_tiles, cudaStream_t s);
 // Candidates per template of a plan's refinement (0: off).
 int32_t refine_cells_of(const fmap_plan_s* p);
-// Reduces partial slots [0, n_tiles) and, when with_fix, the fix-up slots.
-cudaError_t launch_final_reduce(fmap_plan_s* p, int64_t n_tiles, bool with_fix,
+// Reduces partial slots [0, n_tiles) and, after a compute call on atoms a (else
+// null), the fix-up slots.
+cudaError_t launch_final_reduce(fmap_plan_s* p, int64_t n_tiles, const fmap_atoms* a,
                                 fmap_summary* d_summary, cudaStream_t s);
 cudaError_t launch_marginalise(fmap_plan_s* p, const float* d_2F, const uint8_t* d_valid,
                                fmap_summary* d_summary, cudaStream_t s);
@@ -372,8 +373,8 @@ inline int32_t rel_t_entries(int32_t n_sft) { return ((n_sft + 63) / 64) * 64 + 
 
 // Tile counts of each kernel family (partials per template).
 int64_t rect_tiles(const fmap_grid& g);
-// y extent of the fix-up grid (kFixSlots x this) for a template count.
-int64_t fixup_blocks_y(int32_t n_templates);
+// Template groups of the fix-up (y extent of its grid).
+int64_t fixup_blocks_y(int32_t n_templates, bool shared);
 // The rectangular cells phase: partial slots per template, blocks and
 // dynamic shared memory of its kernel.
 int64_t rect_partial_slots(const fmap_grid& g, int32_t n_templates, int32_t shared_antenna);

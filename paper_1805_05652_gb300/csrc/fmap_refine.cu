@@ -28,6 +28,12 @@
 //      fast terms replaced by their FP64 terms,
 //        S' = e^{(M - M')/2} (S - sum_k e^{(f_k - M)/2}) + sum_k e^{(v_k - M')/2},
 //      logB = M'/2 + ln S' - ln N' + c.
+// Four launches: k_ref_head reduces the template's partials and lists the tiles,
+// k_ref_scan histograms their cells, its last block of a template cutting and
+// collecting, k_ref_collect does that for the templates whose kept cells
+// overflowed, k_ref_cells recomputes, its last block of a template rebuilding the
+// summary.  (As seven launches -- two reductions, tiles, histogram, collection,
+// cells, summary -- most of a small map's call was their latencies.)
 // Every cell outside the cut had a fast 2F more than the cut's distance d
 // below M; when d exceeds twice the fast path's error bound, no such cell
 // can hold the FP64 maximum, and the summary says so (ARGMAX_EXACT).
@@ -64,24 +70,60 @@ __device__ __forceinline__ int ref_bin_of(float v, float M) {
   return d > 0.0f ? (int)d : 0;
 }
 
+// First bin whose cumulative count reaches `want` (kRefBins if none), by one
+// warp (all lanes get it); h in shared memory.
+__device__ __forceinline__ int32_t ref_first_bin(const int32_t* h, int32_t want, int lane) {
+  constexpr int P = kRefBins / 32;
+  int32_t own = 0;
+#pragma unroll
+  for (int k = 0; k < P; ++k) own += h[lane * P + k];
+  int32_t cum = own;   // inclusive over lanes
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int32_t y = __shfl_up_sync(0xffffffffu, cum, d);
+    if (lane >= d) cum += y;
+  }
+  const unsigned reach = __ballot_sync(0xffffffffu, cum >= want);
+  int32_t at = kRefBins;
+  if (reach && lane == __ffs(reach) - 1) {
+    int32_t c = cum - own;
+    at = lane * P;
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+      c += h[lane * P + k];
+      if (c < want) ++at;   // (the lane's total reaches it: at stays below the next lane's)
+    }
+  }
+  return (int32_t)__reduce_min_sync(0xffffffffu, (unsigned)at);
+}
+
 // The last histogram bin whose cumulative count stays within the cap, at
 // most bt (the last bin whose cells all lie in scanned tiles).  When the top
 // bin alone holds more than the cap (a maximum shared by many cells within
 // 1/16 of 2F, e.g. windows truncated at the data's end), the top bin as a
 // whole while it fits the candidate buffer; else -1 (no refinement).
-__device__ __forceinline__ int32_t ref_cut_of(const int32_t* __restrict__ h, int32_t cap,
-                                              int32_t bt) {
-  int32_t cum = 0, b = -1;
-  for (int k = 0; k <= bt && k < kRefBins; ++k) {
-    cum += h[k];
-    if (cum > cap) break;
-    b = k;
-  }
-  if (b < 0 && h[0] <= kRefMaxCells) b = 0;
-  return b;
+__device__ __forceinline__ int32_t ref_cut_of(const int32_t* h, int32_t cap, int32_t bt, int lane) {
+  const int32_t b = min(ref_first_bin(h, cap + 1, lane) - 1, min(bt, kRefBins - 1));
+  return b < 0 && h[0] <= kRefMaxCells ? 0 : b;
 }
 
-// Pass 1 (one block per template): which tiles to scan.  The partials give
+// Sums over a block's warps: every lane of warp 0 gets the total.
+template <int NW>
+__device__ __forceinline__ double ref_block_sum(double v, double* sh, int lane, int warp) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  if (lane == 0) sh[warp] = v;
+  __syncthreads();
+  v = lane < NW ? sh[lane] : 0.0;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+
+// Pass 1 (one block per template): the template's reduction (maximum and count,
+// then the exp-sum relative to it and the lowest index at it; the order of the
+// additions is fixed, FP64 over the tiles' FP32 sums) into its statistics, and
+// which tiles to scan.  The partials give
 // every tile's fast maximum (a main tile's over the cells the main kernel
 // summed, a fix-up slot's over its recomputed cells: disjoint sets); with bt
 // the first bin in which the count of tiles (by their maxima) reaches the
@@ -90,59 +132,116 @@ __device__ __forceinline__ int32_t ref_cut_of(const int32_t* __restrict__ h, int
 // maximum is in a bin <= bt: those tiles are listed for the cell passes,
 // and bt is kept in cut[j].
 constexpr int kTileThreads = 1024;
-constexpr int kTileCache = 8;   // slots per thread whose bins stay in registers
+constexpr int kTileCache = 8;   // slots per thread whose maxima stay in registers
 
-__global__ void __launch_bounds__(kTileThreads)
-k_ref_tiles(const Partial* __restrict__ parts, int64_t stride, int64_t n_tiles, int64_t fix0,
-            int64_t n_fix, const TStat* __restrict__ st, int32_t cap,
-            int32_t* __restrict__ ref_ntile, int32_t* __restrict__ ref_tile,
-            int32_t* __restrict__ cut, int32_t* __restrict__ ref_ncand) {
+struct HeadArgs {
+  const Partial* parts;
+  int64_t stride, n_tiles, fix0, entries;
+  const int32_t* n_flag;
+  int32_t cap;
+  TStat* st;
+  int32_t* hist;
+  int32_t* ref_n;
+  int32_t* ref_ncand;
+  int32_t* ref_ntile;
+  int32_t* ref_tile;
+  int32_t* cut;
+};
+
+__global__ void __launch_bounds__(kTileThreads) k_ref_head(const HeadArgs A) {
+  constexpr int NW = kTileThreads / 32;
   __shared__ int32_t h[kRefBins];
+  __shared__ unsigned s_mu[NW], s_cnt[NW], s_arg[NW];
+  __shared__ double s_sum[NW];
   __shared__ int32_t s_bt, s_n;
   const int32_t j = blockIdx.x;
-  const int lane = threadIdx.x & 31;
-  for (int b = threadIdx.x; b < kRefBins; b += blockDim.x) h[b] = 0;
-  if (threadIdx.x == 0) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < kRefBins) {
+    h[tid] = 0;
+    A.hist[(int64_t)j * kRefBins + tid] = 0;
+  }
+  if (tid == 0) {
     s_n = 0;
-    ref_ncand[j] = 0;   // (the histogram pass after this one counts its kept cells)
+    A.ref_n[j] = 0;
+    A.ref_ncand[j] = 0;
+  }
+  const int64_t total = A.n_tiles + fix_slots_used(min((int64_t)*A.n_flag, A.entries));
+  const Partial* pp = A.parts + (int64_t)j * A.stride;
+  auto slot = [&](int64_t k) {
+    return *reinterpret_cast<const float4*>(pp + (k < A.n_tiles ? k : A.fix0 + (k - A.n_tiles)));
+  };
+  auto top_of = [](const float4& q) { return __float_as_int(q.w) > 0 ? q.x : -1.0f; };
+  // maximum and count (2F >= 0: the bit patterns order like the values)
+  float tops[kTileCache];
+  unsigned mu = 0u, cnt = 0u;
+  auto see = [&](const float4& q) {
+    const int32_t nv = __float_as_int(q.w);
+    if (nv > 0) {
+      mu = max(mu, __float_as_uint(q.x) + 1u);
+      cnt += (unsigned)nv;
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < kTileCache; ++i) {
+    const int64_t k = tid + (int64_t)i * kTileThreads;
+    const float4 q = k < total ? slot(k) : make_float4(-1.f, 0.f, 0.f, 0.f);
+    tops[i] = top_of(q);
+    see(q);
+  }
+#pragma unroll 4
+  for (int64_t k = tid + (int64_t)kTileCache * kTileThreads; k < total; k += kTileThreads) see(slot(k));
+  mu = __reduce_max_sync(0xffffffffu, mu);
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0) {
+    s_mu[warp] = mu;
+    s_cnt[warp] = cnt;
   }
   __syncthreads();
-  const TStat s = st[j];
-  const Partial* pp = parts + (int64_t)j * stride;
-  const int64_t total = s.N > 0 ? n_tiles + n_fix : 0;
-  auto bin_of = [&](int64_t k) {
-    if (k >= total) return -1;
-    const Partial q = pp[k < n_tiles ? k : fix0 + (k - n_tiles)];
-    return q.nvalid > 0 ? ref_bin_of(q.max2F, s.M) : -1;
-  };
-  // one shared-memory atomic per distinct bin among a warp's lanes
+  mu = __reduce_max_sync(0xffffffffu, s_mu[lane]);
+  cnt = __reduce_add_sync(0xffffffffu, s_cnt[lane]);
+  const float M = mu ? __uint_as_float(mu - 1u) : -1.0f;
+  // exp-sum: rescale factor exp((max2F - M) / 2) <= 1 in FP32 (relative error
+  // ~1e-7, the order of the FP32 tile sums themselves), accumulated in FP64;
+  // factors below 2^-126 flush to 0
+  double sum = 0.0;
+  unsigned arg = (unsigned)kNoArg;
+  if (mu) {
+#pragma unroll 4
+    for (int64_t k = tid; k < total; k += kTileThreads) {
+      const float4 q = slot(k);
+      if (__float_as_int(q.w) <= 0) continue;
+      float f;
+      asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((q.x - M) * 0.72134752044448170368f));
+      sum += (double)q.z * (double)f;
+      if (q.x == M) arg = min(arg, (unsigned)__float_as_int(q.y));
+    }
+  }
+  arg = __reduce_min_sync(0xffffffffu, arg);
+  if (lane == 0) s_arg[warp] = arg;
+  sum = ref_block_sum<NW>(sum, s_sum, lane, warp);   // (a barrier: s_arg is there too)
+  if (tid < 32) {
+    arg = __reduce_min_sync(0xffffffffu, s_arg[lane]);
+    if (tid == 0) A.st[j] = TStat{sum, M, (int32_t)arg, (long long)cnt, {0, 0}};
+  }
+  // tiles by the bins of their maxima: one shared-memory atomic per distinct bin
+  // among a warp's lanes
+  auto bin_of = [&](float top) { return top >= 0.0f ? ref_bin_of(top, M) : -1; };
   auto count = [&](int b, unsigned mask) {
     const unsigned peers = __match_any_sync(mask, b);
     if (b >= 0 && lane == __ffs(peers) - 1) atomicAdd(&h[b], __popc(peers));
   };
-  int bins[kTileCache];
 #pragma unroll
-  for (int i = 0; i < kTileCache; ++i) {
-    bins[i] = bin_of(threadIdx.x + (int64_t)i * kTileThreads);
-    count(bins[i], 0xffffffffu);
-  }
-  for (int64_t k = threadIdx.x + (int64_t)kTileCache * kTileThreads; k < total; k += kTileThreads)
-    count(bin_of(k), __activemask());
+  for (int i = 0; i < kTileCache; ++i) count(bin_of(tops[i]), 0xffffffffu);
+  for (int64_t k = tid + (int64_t)kTileCache * kTileThreads; k < total; k += kTileThreads)
+    count(bin_of(top_of(slot(k))), __activemask());
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int32_t cum = 0, bt = kRefBins - 1;
-    for (int k = 0; k < kRefBins; ++k) {
-      cum += h[k];
-      if (cum >= cap) {
-        bt = k;
-        break;
-      }
-    }
-    s_bt = bt;
+  if (warp == 0) {
+    const int32_t f = ref_first_bin(h, A.cap, lane);
+    if (lane == 0) s_bt = min(f, kRefBins - 1);
   }
   __syncthreads();
   const int32_t bt = s_bt;
-  int32_t* list = ref_tile + (int64_t)j * kRefMaxTiles;
+  int32_t* list = A.ref_tile + (int64_t)j * kRefMaxTiles;
   auto put = [&](int64_t k, int b, unsigned mask) {
     const bool take = b >= 0 && b <= bt;
     const unsigned sel = __ballot_sync(mask, take);
@@ -156,14 +255,27 @@ k_ref_tiles(const Partial* __restrict__ parts, int64_t stride, int64_t n_tiles, 
   };
 #pragma unroll
   for (int i = 0; i < kTileCache; ++i)
-    put(threadIdx.x + (int64_t)i * kTileThreads, bins[i], 0xffffffffu);
-  for (int64_t k = threadIdx.x + (int64_t)kTileCache * kTileThreads; k < total; k += kTileThreads)
-    put(k, bin_of(k), __activemask());
+    put(tid + (int64_t)i * kTileThreads, bin_of(tops[i]), 0xffffffffu);
+  for (int64_t k = tid + (int64_t)kTileCache * kTileThreads; k < total; k += kTileThreads)
+    put(k, bin_of(top_of(slot(k))), __activemask());
   __syncthreads();
-  if (threadIdx.x == 0) {
-    ref_ntile[j] = s_n;   // (more than kRefMaxTiles: truncated)
-    cut[j] = bt;
+  if (tid == 0) {
+    A.ref_ntile[j] = s_n;   // (more than kRefMaxTiles: truncated)
+    A.cut[j] = bt;
   }
+}
+
+// Counts a block of a template's pass as done; true (to all its threads) for
+// the last one, which then sees what the others wrote.
+__device__ __forceinline__ bool ref_last_block(int32_t* done, int32_t n_blocks) {
+  __shared__ int32_t s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(done, 1) == n_blocks - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  return true;
 }
 
 struct ScanArgs {
@@ -178,12 +290,12 @@ struct ScanArgs {
   const int64_t* flag_list;
   const int32_t* n_flag;
   int32_t n_templates;
-  const TStat* st;
+  TStat* st;
   const int32_t* ref_ntile;
   const int32_t* ref_tile;
   int32_t* hist;
   int32_t cap;
-  const int32_t* cut;   // [T] bt of the tile pass
+  int32_t* cut;   // [T] bt of the tile pass, then the cut
   int32_t* ref_n;
   int32_t* ref_cell;
   int32_t* ref_ncand;
@@ -217,7 +329,7 @@ __device__ __forceinline__ void ref_tile_cells(const ScanArgs& A, int32_t j, int
     const int64_t n = min((int64_t)*A.n_flag, cap);
     const int64_t b = k - A.n_tiles;
     int64_t lo, hi;
-    fix_slot_range(b, n, kFixSlots, A.n_templates, &lo, &hi);
+    fix_slot_range(b, n, &lo, &hi);
     const int64_t m = hi - lo;
     for (int64_t e = lo + m * part / A.parts + lane; e < lo + m * (part + 1) / A.parts; e += 32) {
       const int64_t entry = A.flag_list[e];
@@ -228,91 +340,105 @@ __device__ __forceinline__ void ref_tile_cells(const ScanArgs& A, int32_t j, int
   }
 }
 
-// Passes 2 and 3 over the listed tiles' cells: the histogram (collect =
-// false), which also keeps the cells in bins up to the tile pass's bound
-// (cut[j]) while they fit kRefCandCap, then the cut and the collection of
-// the cells up to it (collect = true): by the blocks (x, j) from the kept
-// cells when they fit (the same set: every cell the cut takes lies in a bin
-// <= cut[j]), else by a second scan of the tiles.  Grid (x, T), one warp per
-// tile.  The histogram and the counts were cleared by the final reduction,
-// the kept-cell count by the tile pass.
-template <bool kCollect>
+// Calls f(cell, its bin or -1) for the cells of the first nt listed tiles, whose
+// shares go to `step` warps.
+template <typename F>
+__device__ __forceinline__ void ref_scan_cells(const ScanArgs& A, int32_t j, int32_t nt, float M,
+                                               int64_t first, int64_t step, int lane, F f) {
+  const float* mp = A.map + (int64_t)j * A.cells;
+  for (int64_t it = first; it < (int64_t)nt * A.parts; it += step) {
+    const int64_t k = it / A.parts;
+    ref_tile_cells(A, j, A.ref_tile[(int64_t)j * kRefMaxTiles + k], (int32_t)(it - k * A.parts),
+                   lane, [&](int64_t c, bool owned) {
+      f((int32_t)c, owned ? ref_bin_of(mp[c], M) : -1);
+    });
+  }
+}
+
+// Pass 2 over the listed tiles' cells: the histogram, which also keeps the
+// cells in bins up to the tile pass's bound (cut[j]) while they fit
+// kRefCandCap; then, in the template's last block, the cut and the collection of
+// the cells up to it from the kept cells when they fit (the same set: every
+// cell the cut takes lies in a bin <= cut[j]), else a flag (done[0] < 0) that
+// leaves the collection to a second scan of the tiles, k_ref_collect.  Grid (x, T),
+// one warp per share of a tile.  The histogram and the counts were cleared by the
+// first pass.
 __global__ void __launch_bounds__(kRefThreads) k_ref_scan(const ScanArgs A) {
   __shared__ int32_t h[kRefBins];
-  __shared__ int32_t s_last;
+  __shared__ int32_t s_cut, s_n;
   const int32_t j = blockIdx.y;
-  const int32_t n_kept = kCollect ? A.ref_ncand[j] : 0;
-  const bool from_kept = kCollect && n_kept <= kRefCandCap;
-  if (from_kept && (int64_t)blockIdx.x * kRefThreads >= n_kept) return;   // (past the list)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (kCollect) {
-    for (int b = threadIdx.x; b < kRefBins; b += blockDim.x) h[b] = A.hist[(int64_t)j * kRefBins + b];
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = ref_cut_of(h, A.cap, A.cut[j]);
-  } else {
-    for (int b = threadIdx.x; b < kRefBins; b += blockDim.x) h[b] = 0;
-  }
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NW = kRefThreads / 32;
+  static_assert(kRefThreads == kRefBins, "one bin per thread");
+  h[tid] = 0;
   __syncthreads();
   const TStat s = A.st[j];
-  const int32_t last = kCollect ? s_last : kRefBins - 1;
-  const int32_t keep = kCollect ? -1 : A.cut[j];   // bins the histogram pass keeps
-  if (from_kept) {   // the template's blocks share its kept list
-    if (s.N <= 0 || last < 0) return;
-    const float* mp = A.map + (int64_t)j * A.cells;
-    const int32_t* cand = A.ref_cand + (int64_t)j * kRefCandCap;
-    for (int32_t k = blockIdx.x * kRefThreads + threadIdx.x; k < n_kept;
-         k += gridDim.x * kRefThreads) {
-      const int32_t c = cand[k];
-      const int b = ref_bin_of(mp[c], s.M);
-      if (b >= 0 && b <= last) {
-        const int32_t slot = atomicAdd(A.ref_n + j, 1);
-        if (slot < kRefMaxCells) A.ref_cell[(int64_t)j * kRefMaxCells + slot] = c;
-      }
+  const int32_t keep = A.cut[j];   // bins the histogram pass keeps
+  const int32_t nt = s.N > 0 ? min(A.ref_ntile[j], kRefMaxTiles) : 0;
+  const float* mp = A.map + (int64_t)j * A.cells;
+  int32_t* cand = A.ref_cand + (int64_t)j * kRefCandCap;
+  ref_scan_cells(A, j, nt, s.M, blockIdx.x * NW + warp, (int64_t)gridDim.x * NW, lane, [&](int32_t c, int b) {
+    // one shared-memory atomic per distinct bin among the lanes here
+    // (noise maps put most cells of the window in a few bins)
+    const unsigned act = __activemask();
+    const unsigned peers = __match_any_sync(act, b);
+    if (b >= 0 && lane == __ffs(peers) - 1) atomicAdd(&h[b], __popc(peers));
+    // keep the cells of bins <= keep: one global atomic per warp step
+    const bool kept = b >= 0 && b <= keep;
+    const unsigned sel = __ballot_sync(act, kept);
+    if (sel) {
+      const int leader = __ffs(sel) - 1;
+      int32_t base = 0;
+      if (lane == leader) base = atomicAdd(A.ref_ncand + j, __popc(sel));
+      base = __shfl_sync(act, base, leader);
+      const int32_t at = base + __popc(sel & ((1u << lane) - 1u));
+      if (kept && at < kRefCandCap) cand[at] = c;
     }
+  });
+  __syncthreads();
+  if (h[tid]) atomicAdd(A.hist + (int64_t)j * kRefBins + tid, h[tid]);
+  if (!ref_last_block(&A.st[j].done[0], gridDim.x)) return;
+  h[tid] = __ldcg(A.hist + (int64_t)j * kRefBins + tid);
+  if (tid == 0) s_n = 0;
+  __syncthreads();
+  if (warp == 0) {
+    const int32_t b = ref_cut_of(h, A.cap, keep, lane);
+    if (lane == 0) s_cut = A.cut[j] = b;
+  }
+  __syncthreads();
+  const int32_t last = s_cut;
+  if (nt == 0 || last < 0) return;   // (ref_n stays 0)
+  const int32_t n_kept = __ldcg(A.ref_ncand + j);
+  if (n_kept > kRefCandCap) {
+    if (tid == 0) A.st[j].done[0] = -1;
     return;
   }
-  const int32_t nt = min(A.ref_ntile[j], kRefMaxTiles);
-  if (s.N > 0 && last >= 0) {
-    const float* mp = A.map + (int64_t)j * A.cells;
-    const int64_t items = (int64_t)nt * A.parts;
-    for (int64_t it = blockIdx.x * (kRefThreads / 32) + warp; it < items;
-         it += gridDim.x * (kRefThreads / 32)) {
-      const int64_t k = it / A.parts;
-      ref_tile_cells(A, j, A.ref_tile[(int64_t)j * kRefMaxTiles + k], (int32_t)(it - k * A.parts),
-                     lane, [&](int64_t c, bool owned) {
-        int b = owned ? ref_bin_of(mp[c], s.M) : -1;
-        if (b > last) b = -1;
-        if (kCollect) {
-          if (b >= 0) {
-            const int32_t slot = atomicAdd(A.ref_n + j, 1);
-            if (slot < kRefMaxCells) A.ref_cell[(int64_t)j * kRefMaxCells + slot] = (int32_t)c;
-          }
-        } else {
-          // one shared-memory atomic per distinct bin among the lanes here
-          // (noise maps put most cells of the window in a few bins)
-          const unsigned act = __activemask();
-          const unsigned peers = __match_any_sync(act, b);
-          if (b >= 0 && lane == __ffs(peers) - 1) atomicAdd(&h[b], __popc(peers));
-          // keep the cells of bins <= keep: one global atomic per warp step
-          const bool kept = b >= 0 && b <= keep;
-          const unsigned sel = __ballot_sync(act, kept);
-          if (sel) {
-            const int leader = __ffs(sel) - 1;
-            int32_t base = 0;
-            if (lane == leader) base = atomicAdd(A.ref_ncand + j, __popc(sel));
-            base = __shfl_sync(act, base, leader);
-            const int32_t at = base + __popc(sel & ((1u << lane) - 1u));
-            if (kept && at < kRefCandCap) A.ref_cand[(int64_t)j * kRefCandCap + at] = (int32_t)c;
-          }
-        }
-      });
-    }
+  for (int32_t k = tid; k < n_kept; k += kRefThreads) {
+    const int32_t c = __ldcg(cand + k);
+    const int b = ref_bin_of(mp[c], s.M);
+    if (b < 0 || b > last) continue;
+    const int32_t slot = atomicAdd(&s_n, 1);
+    if (slot < kRefMaxCells) A.ref_cell[(int64_t)j * kRefMaxCells + slot] = c;
   }
-  if (!kCollect) {
-    __syncthreads();
-    for (int b = threadIdx.x; b < kRefBins; b += blockDim.x)
-      if (h[b]) atomicAdd(A.hist + (int64_t)j * kRefBins + b, h[b]);
-  }
+  __syncthreads();
+  if (tid == 0) A.ref_n[j] = s_n;
+}
+
+// The second scan of the tiles of the templates whose kept cells overflowed
+// (a strong signal's tiles hold many cells near the maximum).  Every block of
+// the others ends at once.
+__global__ void __launch_bounds__(kRefThreads) k_ref_collect(const ScanArgs A) {
+  const int32_t j = blockIdx.y;
+  const TStat s = A.st[j];
+  if (s.done[0] >= 0) return;
+  constexpr int NW = kRefThreads / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t last = A.cut[j], nt = min(A.ref_ntile[j], kRefMaxTiles);
+  ref_scan_cells(A, j, nt, s.M, blockIdx.x * NW + warp, (int64_t)gridDim.x * NW, lane, [&](int32_t c, int b) {
+    if (b < 0 || b > last) return;
+    const int32_t slot = atomicAdd(A.ref_n + j, 1);
+    if (slot < kRefMaxCells) A.ref_cell[(int64_t)j * kRefMaxCells + slot] = c;
+  });
 }
 
 struct RefArgs {
@@ -334,70 +460,123 @@ struct RefArgs {
   const int32_t* ref_cell;
   float* ref_fast;
   double* ref_val;
+  const TauTab* tauc;      // exponential windows
+  // the summaries
+  TStat* st;
+  const int32_t* cut;
+  const int32_t* ref_ntile;
+  double log_prior, tol;
+  fmap_summary* out;
 };
 
-// Pass 3: one warp per collected cell.  The lanes split the window's atoms
-// into 32 contiguous runs and sum them in float-float arithmetic (a value is
-// an unevaluated pair h + l, ~2^-44 relative; GB300 runs FP64 at 1/64 of the
-// FP32 rate): an exponential run takes its first weight from an FP64 exp and
-// the rest as products of per-gap decays (e^{-T_sft/tau} for one-SFT gaps), a
-// table window evaluates w per atom in FP64, a rectangular one has w = 1.  The
-// seven sums meet in a fixed butterfly; lane 0 forms D and 2F in FP64 from
-// them, records the fast and refined values and writes the refined value to
-// the map.
+// Pass 3: one warp per collected cell, lane l taking the window's atoms i0 + l +
+// 32 q (coalesced loads, a step ahead), summed in float-float arithmetic (a value
+// is an unevaluated pair h + l; GB300 runs FP64 at 1/64 of the FP32 rate): products
+// with their FMA error, added by TwoSum with the errors collected in l (Ogita, Rump
+// and Oishi's cascaded form, ~n^2 2^-48 relative for a lane's n atoms).  An
+// exponential weight starts from the decay between t0 and the first atom (FP64
+// exp) and moves on by gaps of k SFTs, each the product of two float pairs held by
+// the lanes: the powers k mod 16 of the one-SFT decay (the tau's table) and 16
+// floor(k / 16) (by squaring); FP64 exp for other gaps.  A table window evaluates w
+// per atom in FP64, a rectangular one has w = 1.  The seven sums meet in a fixed
+// butterfly; D and 2F are formed from them in FP64, by one lane per cell of the
+// block's, which records the fast and refined values and writes the refined value
+// to the map.  (With one contiguous run of atoms per lane, an FP64 exp for every gap
+// other than one SFT and the FP64 end of each cell in a warp of its own, the FP64
+// pipe was 66 % busy: 1034 us for 5 x 512 cells of a year's data with 4 % missing
+// SFTs.)
+__device__ __forceinline__ void ref_acc(FF& s, FF w, float x) {
+  const float p = __fmul_rn(w.h, x);
+  const float e = fmaf(w.l, x, fmaf(w.h, x, -p));
+  const FF t = two_sum(s.h, p);
+  s.h = t.h;
+  s.l += t.l + e;
+}
 
-__device__ __forceinline__ void ref_cell_one(const RefArgs& A, int32_t j, int32_t k, int lane) {
+// The seven sums of collected cell c of template j (every lane gets them).
+__device__ __forceinline__ void ref_cell_sums(const RefArgs& A, int32_t j, int32_t c, int lane,
+                                              uint32_t inv_t, FF (&s)[7]) {
   const fmap_grid& g = A.g;
-  const int64_t slot = (int64_t)j * kRefMaxCells + k;
-  const int32_t c = A.ref_cell[slot];
   const int32_t m = c / g.n_tau, nn = c - m * g.n_tau;
   const int32_t i0 = A.i0[m], je = A.jend[c];
-  const int32_t len = max(0, je - i0);
   const int64_t t0rel = grid_t0(g, A.ax, m) - *A.t_base;
-  const int64_t tau = grid_tau(g, A.ax, nn);
-  const double inv_tau = 1.0 / (double)tau;
-  const int32_t a_lo = i0 + (int32_t)((int64_t)len * lane / 32);
-  const int32_t a_hi = i0 + (int32_t)((int64_t)len * (lane + 1) / 32);
   const int64_t n = A.n_sft;
+  const int32_t t_sft = (int32_t)g.t_sft;
   const float* ant = A.antenna + (A.shared ? 0 : (int64_t)j * 3 * n);
   const float* x = A.fafb + (int64_t)j * 4 * n;
   const bool ex = g.window == FMAP_EXP, tw = g.window == FMAP_TABLE;
-  const double su = tw ? tab_scale(A.n_tab, exp_cut8_of(g), tau) : 0.0;
-  FF s[7];
+  const double su = tw ? tab_scale(A.n_tab, exp_cut8_of(g), grid_tau(g, A.ax, nn)) : 0.0;
 #pragma unroll
   for (int q = 0; q < 7; ++q) s[q] = FF{0.0f, 0.0f};
-  if (a_lo < a_hi) {
-    FF w{1.0f, 0.0f}, rho1{1.0f, 0.0f};
+  if (je > i0) {
+    FF w{1.0f, 0.0f}, lo{1.0f, 0.0f}, hi{1.0f, 0.0f};
+    double inv_tau = 0.0;
+    int32_t t = A.rel_t[i0];
     if (ex) {
-      w = ff_of(exp(-(double)((int64_t)A.rel_t[a_lo] - t0rel) * inv_tau));
-      rho1 = ff_of(exp(-(double)g.t_sft * inv_tau));
-    }
-    for (int32_t a = a_lo; a < a_hi; ++a) {
-      if (ex && a > a_lo) {
-        const int32_t gap = A.rel_t[a] - A.rel_t[a - 1];
-        w = ff_mul(w, gap == (int32_t)g.t_sft ? rho1 : ff_of(exp(-(double)gap * inv_tau)));
+      const TauTab* tt = A.tauc + nn;
+      inv_tau = tt->inv_tau;
+      const float2 v = tt->pw[0][lane & 15];
+      lo = FF{v.x, v.y};
+      // lane h: the power 16 h, by squaring
+      const float2 v1 = tt->pw[0][1], v15 = tt->pw[0][15];
+      FF p = ff_mul(FF{v15.x, v15.y}, FF{v1.x, v1.y});
+#pragma unroll
+      for (int b = 0; b < 5; ++b) {
+        if (lane & (1 << b)) hi = ff_mul(hi, p);
+        p = ff_mul(p, p);
       }
-      if (tw) w = ff_of(tab_weight64((double)((int64_t)A.rel_t[a] - t0rel) * su, A.wtab, A.n_tab));
-      if (g.window == FMAP_RECT) {
-        s[0] = ff_add(s[0], FF{ant[a], 0.0f});
-        s[1] = ff_add(s[1], FF{ant[n + a], 0.0f});
-        s[2] = ff_add(s[2], FF{ant[2 * n + a], 0.0f});
-        s[3] = ff_add(s[3], FF{x[a], 0.0f});
-        s[4] = ff_add(s[4], FF{x[n + a], 0.0f});
-        s[5] = ff_add(s[5], FF{x[2 * n + a], 0.0f});
-        s[6] = ff_add(s[6], FF{x[3 * n + a], 0.0f});
-      } else {
-        const FF w2 = ff_mul(w, w);
-        ff_acc(s[0], w2, ant[a]);
-        ff_acc(s[1], w2, ant[n + a]);
-        ff_acc(s[2], w2, ant[2 * n + a]);
-        ff_acc(s[3], w, x[a]);
-        ff_acc(s[4], w, x[n + a]);
-        ff_acc(s[5], w, x[2 * n + a]);
-        ff_acc(s[6], w, x[3 * n + a]);
+      const int64_t d0 = (int64_t)t - t0rel;
+      if (d0 != 0) w = ff_of(exp(-(double)d0 * inv_tau));
+    }
+    float v[7];
+    int32_t tn;
+    auto load = [&](int32_t b) {   // (lanes past the window: its last atom, unused)
+      const int32_t a = min(b + lane, je - 1);
+      tn = A.rel_t[a];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) v[q] = ant[q * n + a];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[3 + q] = x[q * n + a];
+    };
+    load(i0);
+    for (int32_t b = i0; b < je; b += 32) {
+      float u[7];
+#pragma unroll
+      for (int q = 0; q < 7; ++q) u[q] = v[q];
+      const int32_t gap = tn - t;
+      t = tn;
+      const bool on = b + lane < je;
+      if (b + 32 < je) load(b + 32);
+      if (ex) {
+        const int32_t k = (int32_t)__umulhi((uint32_t)gap << 1, inv_t);
+        const int kl = k & 15, kh = (k >> 4) & 31;
+        const FF rl{__shfl_sync(0xffffffffu, lo.h, kl), __shfl_sync(0xffffffffu, lo.l, kl)};
+        const FF rh{__shfl_sync(0xffffffffu, hi.h, kh), __shfl_sync(0xffffffffu, hi.l, kh)};
+        FF r = ff_mul(rh, rl);
+        if ((uint32_t)k >= 512u || k * t_sft != gap) r = ff_of(exp(-(double)gap * inv_tau));
+        w = ff_mul(w, r);
+      }
+      if (tw) w = ff_of(tab_weight64((double)((int64_t)t - t0rel) * su, A.wtab, A.n_tab));
+      if (on) {
+        if (g.window == FMAP_RECT) {
+#pragma unroll
+          for (int q = 0; q < 7; ++q) {
+            const FF y = two_sum(s[q].h, u[q]);
+            s[q].h = y.h;
+            s[q].l += y.l;
+          }
+        } else {
+          const FF w2 = ff_mul(w, w);
+#pragma unroll
+          for (int q = 0; q < 3; ++q) ref_acc(s[q], w2, u[q]);
+#pragma unroll
+          for (int q = 3; q < 7; ++q) ref_acc(s[q], w, u[q]);
+        }
       }
     }
   }
+#pragma unroll
+  for (int q = 0; q < 7; ++q) s[q] = fast_two_sum(s[q].h, s[q].l);
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1)
 #pragma unroll
@@ -405,89 +584,88 @@ __device__ __forceinline__ void ref_cell_one(const RefArgs& A, int32_t j, int32_
       const FF o{__shfl_xor_sync(0xffffffffu, s[q].h, d), __shfl_xor_sync(0xffffffffu, s[q].l, d)};
       s[q] = ff_add(s[q], o);
     }
-  if (lane == 0) {
-    double v7[7];
+}
+
+// 2F of the cell in slot k of template j from its sums, in FP64 (one lane).
+__device__ __forceinline__ void ref_cell_end(const RefArgs& A, int32_t j, int32_t k, const FF* s) {
+  const int64_t slot = (int64_t)j * kRefMaxCells + k;
+  const int32_t c = A.ref_cell[slot];
+  const int32_t len = A.jend[c] - A.i0[c / A.g.n_tau];
+  double v7[7];
 #pragma unroll
-    for (int q = 0; q < 7; ++q) v7[q] = (double)s[q].h + (double)s[q].l;
-    const double Aa = v7[0], Bb = v7[1], Cc = v7[2];
-    const double D = Aa * Bb - Cc * Cc;
-    const bool ok = len >= 2 && D > 0.0;
-    double v = 0.0;
-    if (ok)
-      v = 2.0 * (Bb * (v7[3] * v7[3] + v7[4] * v7[4]) + Aa * (v7[5] * v7[5] + v7[6] * v7[6]) -
-                 2.0 * Cc * (v7[3] * v7[5] + v7[4] * v7[6])) / D;
-    float* mp = A.map + (int64_t)j * A.cells + c;
-    A.ref_fast[slot] = *mp;
-    A.ref_val[slot] = ok ? v : -1.0;
-    *mp = (float)v;
-  }
+  for (int q = 0; q < 7; ++q) v7[q] = (double)s[q].h + (double)s[q].l;
+  const double Aa = v7[0], Bb = v7[1], Cc = v7[2];
+  const double D = Aa * Bb - Cc * Cc;
+  const bool ok = len >= 2 && D > 0.0;
+  double v = 0.0;
+  if (ok)
+    v = 2.0 * (Bb * (v7[3] * v7[3] + v7[4] * v7[4]) + Aa * (v7[5] * v7[5] + v7[6] * v7[6]) -
+               2.0 * Cc * (v7[3] * v7[5] + v7[4] * v7[6])) / D;
+  float* mp = A.map + (int64_t)j * A.cells + c;
+  A.ref_fast[slot] = *mp;
+  A.ref_val[slot] = ok ? v : -1.0;
+  *mp = (float)v;
 }
 
-__global__ void __launch_bounds__(kRefThreads) k_ref_cells(const RefArgs A) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int32_t j = blockIdx.y;
-  const int32_t n_cand = min(A.ref_n[j], kRefMaxCells);
-  for (int32_t k = blockIdx.x * (kRefThreads / 32) + warp; k < n_cand;
-       k += gridDim.x * (kRefThreads / 32))
-    ref_cell_one(A, j, k, lane);
-}
-
-// Pass 4: one block per template rebuilds its summary from the fast
+// Pass 4: a template's last block rebuilds its summary from the fast
 // statistics and the collected cells.  Every exp-term is in (0, 1] (relative
 // to the fast or the refined maximum, both held by a collected cell) and is
 // summed as an integer in 2^-51 units, so the sums do not depend on the
 // order in which the cells were collected (<= 4096 terms <= 2^63: no overflow,
-// relative error < 1e-12).
-constexpr int kFinalThreads = 256;
-
-__global__ void __launch_bounds__(kFinalThreads)
-k_ref_final(const TStat* __restrict__ st, const int32_t* __restrict__ hist,
-            const int32_t* __restrict__ cut, int32_t cap, const int32_t* __restrict__ ref_ntile,
-            const int32_t* __restrict__ ref_n, const int32_t* __restrict__ ref_cell,
-            const float* __restrict__ ref_fast, const double* __restrict__ ref_val, int32_t n_tau,
-            double log_prior, double tol, fmap_summary* __restrict__ out) {
-  constexpr int NW = kFinalThreads / 32;
+// relative error < 1e-12).  Where no cell was collected, or none is valid, the
+// fast reduction stands (flags 0).
+__device__ __forceinline__ void ref_fast_summary(const RefArgs& A, int32_t j) {
+  const TStat s = A.st[j];
+  fmap_summary o;
+  o.flags = 0;
+  o.n_valid = s.N;
+  o.max2F = s.N > 0 ? s.M : 0.0f;
+  o.m = s.N > 0 ? s.arg / A.g.n_tau : -1;
+  o.n = s.N > 0 ? s.arg % A.g.n_tau : -1;
+  o.logB = s.N > 0 ? 0.5 * (double)s.M + log(s.S) - log((double)s.N) + A.log_prior : nan("");
+  A.out[j] = o;
+}
+__device__ __forceinline__ void ref_summary(const RefArgs& A, int32_t j, int32_t n) {
+  constexpr int NW = kRefThreads / 32;
   __shared__ double s_mx[NW];
   __shared__ unsigned long long s_sub[NW], s_add[NW];
-  __shared__ long long s_nv[NW];
-  __shared__ int32_t s_arg[NW];
-  const int32_t j = blockIdx.x;
+  __shared__ int32_t s_nv[NW], s_arg[NW];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const TStat s = st[j];
-  const int32_t n = min(ref_n[j], kRefMaxCells);
-  if (s.N <= 0 || n <= 0) return;   // the fast summary stands (flags 0)
+  const TStat s = A.st[j];
   const int64_t base = (int64_t)j * kRefMaxCells;
   double mx = -1.0;
-  for (int32_t k = threadIdx.x; k < n; k += kFinalThreads) mx = fmax(mx, ref_val[base + k]);
+  for (int32_t k = threadIdx.x; k < n; k += kRefThreads) mx = fmax(mx, __ldcg(A.ref_val + base + k));
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, d));
   if (lane == 0) s_mx[warp] = mx;
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < NW; ++w) mx = fmax(mx, s_mx[w]);
-  if (mx < 0.0) return;   // no collected cell valid in FP64: keep the fast summary
+  if (mx < 0.0) {   // no collected cell valid in FP64
+    if (threadIdx.x == 0) ref_fast_summary(A, j);
+    return;
+  }
   constexpr double kFix = 2251799813685248.0;   // 2^51
   unsigned long long sub = 0ull, add = 0ull;
-  long long nv = 0;
-  int32_t arg = 0x7fffffff;
+  int32_t nv = 0, arg = 0x7fffffff;
   const double M = (double)s.M;
-  for (int32_t k = threadIdx.x; k < n; k += kFinalThreads) {
-    const double ef = exp(0.5 * fmin((double)ref_fast[base + k] - M, 0.0));
+  for (int32_t k = threadIdx.x; k < n; k += kRefThreads) {
+    const double ef = exp(0.5 * fmin((double)__ldcg(A.ref_fast + base + k) - M, 0.0));
     sub += (unsigned long long)__double2ull_rn(ef * kFix);
-    const double v = ref_val[base + k];
+    const double v = __ldcg(A.ref_val + base + k);
     if (v >= 0.0) {
       add += (unsigned long long)__double2ull_rn(exp(0.5 * (v - mx)) * kFix);
       nv += 1;
-      if (v == mx) arg = min(arg, ref_cell[base + k]);
+      if (v == mx) arg = min(arg, A.ref_cell[base + k]);
     }
   }
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) {
     sub += __shfl_xor_sync(0xffffffffu, sub, d);
     add += __shfl_xor_sync(0xffffffffu, add, d);
-    nv += __shfl_xor_sync(0xffffffffu, nv, d);
-    arg = min(arg, __shfl_xor_sync(0xffffffffu, arg, d));
   }
+  nv = __reduce_add_sync(0xffffffffu, nv);
+  arg = __reduce_min_sync(0xffffffffu, arg);
   if (lane == 0) {
     s_sub[warp] = sub;
     s_add[warp] = add;
@@ -504,20 +682,47 @@ k_ref_final(const TStat* __restrict__ st, const int32_t* __restrict__ hist,
   }
   const double Sp = exp(0.5 * (M - mx)) * fmax(s.S - (double)sub / kFix, 0.0) + (double)add / kFix;
   const long long Np = s.N - n + nv;
-  const int32_t b = ref_cut_of(hist + (int64_t)j * kRefBins, cap, cut[j]);
+  const int32_t b = A.cut[j];
   const double depth = b + 1 >= kRefBins ? (double)kRefWindow
                                          : (double)(b + 1) * (double)kRefWindow / kRefBins;
   fmap_summary o;
   o.max2F = (float)mx;
-  o.m = arg / n_tau;
-  o.n = arg % n_tau;
-  const bool complete = ref_ntile[j] <= kRefMaxTiles;   // every candidate tile scanned
+  o.m = arg / A.g.n_tau;
+  o.n = arg % A.g.n_tau;
+  const bool complete = A.ref_ntile[j] <= kRefMaxTiles;   // every candidate tile scanned
   o.flags = (int32_t)FMAP_SUMMARY_REFINED |
-            (complete && depth > 2.0 * tol * fmax(mx, 1.0) ? (int32_t)FMAP_SUMMARY_ARGMAX_EXACT
-                                                            : 0);
-  o.logB = 0.5 * mx + log(Sp) - log((double)Np) + log_prior;
+            (complete && depth > 2.0 * A.tol * fmax(mx, 1.0) ? (int32_t)FMAP_SUMMARY_ARGMAX_EXACT
+                                                              : 0);
+  o.logB = 0.5 * mx + log(Sp) - log((double)Np) + A.log_prior;
   o.n_valid = Np;
-  out[j] = o;
+  A.out[j] = o;
+}
+
+__global__ void __launch_bounds__(kRefThreads) k_ref_cells(const RefArgs A) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t j = blockIdx.y;
+  const int32_t n_cand = min(A.ref_n[j], kRefMaxCells);
+  const uint32_t t_sft = (uint32_t)A.g.t_sft;
+  const uint32_t inv_t = (uint32_t)(((1ull << 31) + t_sft - 1) / t_sft);   // (as gap_inverse)
+  constexpr int NW = kRefThreads / 32;
+  __shared__ FF s_sum[NW][7];
+  if (n_cand <= 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ref_fast_summary(A, j);
+    return;
+  }
+  for (int32_t k0 = blockIdx.x * NW; k0 < n_cand; k0 += gridDim.x * NW) {
+    if (k0 + warp < n_cand) {
+      FF s[7];
+      ref_cell_sums(A, j, A.ref_cell[(int64_t)j * kRefMaxCells + k0 + warp], lane, inv_t, s);
+#pragma unroll
+      for (int q = 0; q < 7; ++q)
+        if (lane == q) s_sum[warp][q] = s[q];
+    }
+    __syncthreads();
+    if (warp == 0 && lane < NW && k0 + lane < n_cand) ref_cell_end(A, j, k0 + lane, s_sum[lane]);
+    __syncthreads();
+  }
+  if (ref_last_block(&A.st[j].done[1], gridDim.x)) ref_summary(A, j, n_cand);
 }
 
 cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
@@ -527,13 +732,25 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
   const int32_t T = p->n_templates;
   if (cap <= 0 || !d_2F || !d_summary || T == 0 || cells == 0 || p->n_sft == 0)
-    return cudaSuccess;
+    return launch_final_reduce(p, n_tiles, a, d_summary, s);
   Workspace& w = p->ws;
   const int32_t sh = a->shared_antenna ? 1 : 0;
-  // (the final reduction cleared the cell histogram and the candidate counts)
-  k_ref_tiles<<<T, kTileThreads, 0, s>>>(w.partials, p->part_stride, n_tiles, p->n_tiles, kFixSlots,
-                                        w.tstat, cap, w.ref_ntile, w.ref_tile, w.ref_bin,
-                                        w.ref_ncand);
+  HeadArgs H;
+  H.parts = w.partials;
+  H.stride = p->part_stride;
+  H.n_tiles = n_tiles;
+  H.fix0 = p->n_tiles;
+  H.entries = cells * (sh ? 1 : T);
+  H.n_flag = w.n_flag;
+  H.cap = cap;
+  H.st = w.tstat;
+  H.hist = w.ref_hist;
+  H.ref_n = w.ref_n;
+  H.ref_ncand = w.ref_ncand;
+  H.ref_ntile = w.ref_ntile;
+  H.ref_tile = w.ref_tile;
+  H.cut = w.ref_bin;
+  k_ref_head<<<T, kTileThreads, 0, s>>>(H);
   ScanArgs S;
   S.map = d_2F;
   S.coef = w.coef;
@@ -565,8 +782,8 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   const unsigned gx = (unsigned)std::max<int64_t>(
       (2 * (int64_t)cap * S.parts + wpb - 1) / wpb, ((int64_t)p->n_sm * 4 + T - 1) / T);
   const dim3 grid(std::min<unsigned>(gx, 4096u), (unsigned)T);
-  k_ref_scan<false><<<grid, kRefThreads, 0, s>>>(S);
-  k_ref_scan<true><<<grid, kRefThreads, 0, s>>>(S);
+  k_ref_scan<<<grid, kRefThreads, 0, s>>>(S);
+  k_ref_collect<<<grid, kRefThreads, 0, s>>>(S);
   RefArgs A;
   A.rel_t = w.rel_t;
   A.t_base = w.t_base;
@@ -586,11 +803,15 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   A.ref_cell = w.ref_cell;
   A.ref_fast = w.ref_fast;
   A.ref_val = w.ref_val;
+  A.tauc = g.window == FMAP_EXP ? w.tauc : nullptr;
+  A.st = w.tstat;
+  A.cut = w.ref_bin;
+  A.ref_ntile = w.ref_ntile;
+  A.log_prior = p->log_prior;
+  A.tol = fast_tol(p);
+  A.out = d_summary;
   k_ref_cells<<<dim3((unsigned)((cap + wpb - 1) / wpb), (unsigned)T), kRefThreads, 0, s>>>(A);
-  k_ref_final<<<T, kFinalThreads, 0, s>>>(w.tstat, w.ref_hist, w.ref_bin, cap, w.ref_ntile, w.ref_n,
-                               w.ref_cell, w.ref_fast, w.ref_val, g.n_tau, p->log_prior,
-                               fast_tol(p), d_summary);
-  p->launches += 5;
+  p->launches += 4;
   return cudaGetLastError();
 }
 
