@@ -94,14 +94,69 @@ static bool precision_supported(int window, fmap_precision prec) {
 }
 
 struct Layout {
-  size_t rel_t, t_base, dev_err, i0, jend, coef, parts, groups, flag_blocks, n_flag, flag_list, pa, px,
-      esuf, xop, perm_ant, perm_x, perm_gap, rec_cells, rec_decay, tauc, ax, wtab, flag_bits, tstat, ref_hist, ref_bin,
+  size_t rel_t, t_base, irr, dev_err, i0, jend, coef, parts, groups, flag_blocks, n_flag, flag_list, pa, px,
+      xop, perm_ant, perm_x, tauc, ax, wtab, flag_bits, tstat, ref_hist, ref_bin,
       ref_n, ref_cell, ref_fast, ref_val, own_map, ref_ntile, ref_tile, ref_ncand, ref_cand, total;
   int64_t n_tiles;
-  int32_t tau_chunk;
 };
 
-static constexpr size_t kEsufBudget = size_t(1) << 30;
+// Bytes of a plan's refinement scratch (after the marked-entry list).
+static size_t ref_scratch_bytes(int32_t T) {
+  const size_t Tn = (size_t)std::max<int32_t>(T, 1);
+  size_t b = 0;
+  for (const size_t per : {sizeof(TStat), sizeof(int32_t) * kRefBins, sizeof(int32_t),
+                           sizeof(int32_t) * kRefMaxTiles, sizeof(int32_t), sizeof(int32_t),
+                           sizeof(int32_t), sizeof(int32_t) * kRefCandCap,
+                           sizeof(int32_t) * kRefMaxCells, sizeof(float) * kRefMaxCells,
+                           sizeof(double) * kRefMaxCells})
+    b += align_up(per * Tn, 256);
+  return b;
+}
+// The sweeps' chunk maps lie where the list of ill-conditioned entries goes
+// later in the same call (8 bytes per entry), and the refinement's scratch after
+// it, and are used as far as they fit there; recurrence plans outside batches
+// have room of their own for 4 bytes per (tau, atom) and 16 per cell more.
+static int64_t sweep_room(const fmap_grid& g, int32_t n_sft, int32_t T, uint32_t flags) {
+  const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
+  const int64_t t_ant = (flags & FMAP_PLAN_PER_TEMPLATE_ANTENNA) ? std::max<int32_t>(T, 1) : 1;
+  int64_t room = 8 * cells * t_ant;
+  if (!(flags & kPlanBatch)) {
+    room += (int64_t)ref_scratch_bytes(T);
+    if ((flags & FMAP_PLAN_EXP_RECURRENCE) && T >= 2)
+      room += 4 * (int64_t)g.n_tau * n_sft + 16 * cells;
+  }
+  return room;
+}
+AntGeom plan_ant_geom(const fmap_grid& g, int32_t n_sft, int32_t T, uint32_t flags, bool shared) {
+  return ant_geom(g, n_sft, shared ? 1 : T, (flags & kPlanBatch) != 0,
+                  sweep_room(g, n_sft, T, flags));
+}
+static int64_t rec_agg_bytes(const RecGeom& q, int32_t T) {
+  return 4 * (int64_t)q.n_grp * q.n_chunks * ((int64_t)T * 256 + 64);
+}
+RecGeom plan_rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, uint32_t flags, bool shared,
+                      int32_t tpb) {
+  const AntGeom a = plan_ant_geom(g, n_sft, T, flags, shared);
+  return rec_geom(g, n_sft, T, shared, (flags & kPlanBatch) != 0, tpb,
+                  sweep_room(g, n_sft, T, flags) - 4 * ant_agg_floats(a, shared ? 1 : T));
+}
+// Calls f(ant, rec, templates' antenna sets) with every work split that a plan
+// may run: a call may share the antenna rows or not, batches choose the
+// templates per warp by timing.
+template <typename F>
+static void for_sweep_geoms(const fmap_grid& g, int32_t n_sft, int32_t T, uint32_t flags, F f) {
+  const bool batch = (flags & kPlanBatch) != 0;
+  for (const bool shared : {true, false}) {
+    if (!shared && !(flags & FMAP_PLAN_PER_TEMPLATE_ANTENNA)) continue;
+    const AntGeom a = plan_ant_geom(g, n_sft, T, flags, shared);
+    for (const int32_t tpb : {0, 1, 2, 4}) {
+      if (tpb != 0 && !batch) continue;
+      RecGeom q{};
+      if (flags & FMAP_PLAN_EXP_RECURRENCE) q = plan_rec_geom(g, n_sft, T, flags, shared, tpb);
+      f(a, q, shared ? (int64_t)1 : (int64_t)T);
+    }
+  }
+}
 
 static Layout layout_of(const fmap_grid* g, int32_t n_sft, int32_t T, fmap_precision prec,
                         uint32_t flags) {
@@ -115,7 +170,12 @@ static Layout layout_of(const fmap_grid* g, int32_t n_sft, int32_t T, fmap_preci
     tiles = std::max<int64_t>(tiles, (g->n_t0 + 127) / 128);
   } else {
     tiles = std::max<int64_t>(tiles, exp_tiles(*g));
-    if (flags & FMAP_PLAN_EXP_RECURRENCE) tiles = std::max<int64_t>(tiles, g->n_tau);
+    if (flags & FMAP_PLAN_EXP_RECURRENCE) {
+      for_sweep_geoms(*g, n_sft, T, flags, [&](const AntGeom&, const RecGeom& q, int64_t) {
+        tiles = std::max<int64_t>(tiles, (int64_t)q.ntr * q.n_grp);
+      });
+      tiles = std::max<int64_t>(tiles, g->n_tau);
+    }
   }
   L.n_tiles = tiles;
   size_t off = 0;
@@ -125,7 +185,8 @@ static Layout layout_of(const fmap_grid* g, int32_t n_sft, int32_t T, fmap_preci
     return at;
   };
   L.rel_t = take(sizeof(int32_t) * (size_t)rel_t_entries(n_sft));
-  L.t_base = take(sizeof(int64_t));
+  L.t_base = take(sizeof(int64_t) + sizeof(int32_t));
+  L.irr = L.t_base + sizeof(int64_t);
   L.dev_err = take(sizeof(uint32_t));
   L.i0 = take(sizeof(int32_t) * std::max<int32_t>(g->n_t0, 1));
   L.jend = take(sizeof(int32_t) * std::max<int64_t>(cells, 1));
@@ -138,7 +199,14 @@ static Layout layout_of(const fmap_grid* g, int32_t n_sft, int32_t T, fmap_preci
   L.flag_blocks = take(sizeof(int32_t) * ((entries + kFlagUnit - 1) / kFlagUnit));
   L.flag_bits = take(sizeof(uint32_t) * (size_t)flag_words((int64_t)entries));
   L.n_flag = take(sizeof(int32_t));
-  L.flag_list = take(sizeof(int64_t) * entries);
+  int64_t list = (int64_t)(sizeof(int64_t) * entries);
+  if (g->window == FMAP_EXP) {   // (the sweeps' chunk maps, before both are written)
+    const int64_t after = (flags & kPlanBatch) ? 0 : (int64_t)ref_scratch_bytes(T);
+    for_sweep_geoms(*g, n_sft, T, flags, [&](const AntGeom& a, const RecGeom& q, int64_t n_ant) {
+      list = std::max(list, 4 * ant_agg_floats(a, n_ant) + rec_agg_bytes(q, T) - after);
+    });
+  }
+  L.flag_list = take((size_t)list);
   if (!(flags & kPlanBatch)) {  // refinement of the summaries
     const size_t Tn = (size_t)std::max<int32_t>(T, 1);
     L.tstat = take(sizeof(TStat) * Tn);
@@ -155,31 +223,16 @@ static Layout layout_of(const fmap_grid* g, int32_t n_sft, int32_t T, fmap_preci
     L.own_map = (flags & FMAP_PLAN_MAP_BUFFER)
                     ? take(sizeof(float) * (size_t)std::max<int64_t>(cells, 1) * Tn) : 0;
   }
-  L.pa = L.px = L.esuf = L.xop = L.perm_ant = L.perm_x = L.perm_gap = L.rec_cells =
-      L.rec_decay = L.tauc = L.wtab = 0;
+  L.pa = L.px = L.xop = L.perm_ant = L.perm_x = L.tauc = L.wtab = 0;
   const size_t np1 = (size_t)n_sft + 1;
   if (g->window == FMAP_RECT) {
     L.pa = take(sizeof(float) * 8 * np1 * (size_t)t_ant);   // (a2, b2, ab, 0) float pairs
     L.px = take(2 * sizeof(float4) * np1 * (size_t)std::max<int32_t>(T, 1));
   } else {
-    const size_t per_tau = 3 * sizeof(float2) * np1;
-    int64_t chunk = (int64_t)std::max<size_t>(1, kEsufBudget / per_tau);
-    chunk = std::min<int64_t>(chunk, std::max<int32_t>(g->n_tau, 1));
-    L.tau_chunk = (int32_t)chunk;
-    // the suffix sums live in shared memory when the data set fits there
-    L.esuf = take(exp_antenna_fits(n_sft) ? 8 : per_tau * (size_t)chunk);
-    const size_t perm = sizeof(float4) * (size_t)perm_entries_max(n_sft);
-    L.perm_ant = take(perm * (size_t)t_ant);
-    if (flags & FMAP_PLAN_EXP_RECURRENCE) {
-      L.perm_x = take(perm * (size_t)std::max<int32_t>(T, 1));
-      L.perm_gap = take(sizeof(int32_t) * (size_t)perm_entries_max(n_sft));
-      // window records (and the shared antenna's coefficients) re-read by
-      // every template after the first
-      if (T >= 2 && !(flags & kPlanBatch)) {
-        L.rec_cells = take((t_ant == 1 ? 2 : 1) * sizeof(float4) * (size_t)std::max<int64_t>(cells, 1));
-        L.rec_decay = take(sizeof(float) * (size_t)perm_entries_max(n_sft) *
-                           (size_t)std::max<int32_t>(g->n_tau, 1));
-      }
+    if (g->window == FMAP_EXP) {
+      L.perm_ant = take(sizeof(float4) * (size_t)n_sft * (size_t)t_ant);
+      if (flags & FMAP_PLAN_EXP_RECURRENCE)
+        L.perm_x = take(sizeof(float4) * (size_t)n_sft * (size_t)std::max<int32_t>(T, 1));
     }
     L.tauc = take(sizeof(TauTab) * (size_t)std::max<int32_t>(g->n_tau, 1));
     if (g->window == FMAP_TABLE) L.wtab = take(sizeof(float2) * (kTabMax + 1));
@@ -281,13 +334,13 @@ fmap_status plan_init(fmap_plan_s* p, const fmap_grid* grid, int32_t n_sft, int3
   if (!base || bytes < L.total) return arg_fail("workspace smaller than the plan's footprint");
   p->n_tiles = L.n_tiles;
   p->part_stride = L.n_tiles + kFixSlots;
-  p->tau_chunk = L.tau_chunk;
   char* b = (char*)base;
   Workspace& w = p->ws;
   w.base = base;
   w.bytes = L.total;
   w.rel_t = (int32_t*)(b + L.rel_t);
   w.t_base = (int64_t*)(b + L.t_base);
+  w.irr = (int32_t*)(b + L.irr);
   w.dev_err = (uint32_t*)(b + L.dev_err);
   w.i0 = (int32_t*)(b + L.i0);
   w.jend = (int32_t*)(b + L.jend);
@@ -319,16 +372,19 @@ fmap_status plan_init(fmap_plan_s* p, const fmap_grid* grid, int32_t n_sft, int3
     w.pa = (float4*)(b + L.pa);
     w.px = (float4*)(b + L.px);
   } else {
-    w.esuf = (float2*)(b + L.esuf);
-    w.perm_ant = (float4*)(b + L.perm_ant);
+    if (L.perm_ant) w.perm_ant = (float4*)(b + L.perm_ant);
     if (L.perm_x) w.perm_x = (float4*)(b + L.perm_x);
-    if (L.perm_gap) w.perm_gap = (int32_t*)(b + L.perm_gap);
-    if (L.rec_cells) w.rec_cells = (float4*)(b + L.rec_cells);
-    if (L.rec_decay) w.rec_decay = (float*)(b + L.rec_decay);
+    if (grid->window == FMAP_EXP) {
+      w.agg = (float*)(b + L.flag_list);
+      for (int sh = 0; sh < 2; ++sh) p->ant[sh] = plan_ant_geom(*grid, n_sft, n_templates, flags, sh != 0);
+    }
     if (L.wtab) w.wtab = (float2*)(b + L.wtab);
     w.tauc = (TauTab*)(b + L.tauc);
     if (L.xop) w.xop = (void*)(b + L.xop);
   }
+  if (flags & FMAP_PLAN_EXP_RECURRENCE)
+    for (int sh = 0; sh < 2; ++sh)
+      p->rec[sh] = plan_rec_geom(*grid, n_sft, n_templates, flags, sh != 0, 0);
   p->needs_err_reset = true;
   return FMAP_OK;
 }
@@ -540,6 +596,7 @@ static fmap_status enqueue(fmap_plan_t* p, const fmap_atoms* a, float* d_2F,
       FMAP_CUDA(launch_exp_plain(p, a, d_2F, s, &tiles));
   } else {
     FMAP_CUDA(launch_exp_perm(p, a, s));
+    FMAP_CUDA(launch_exp_agg(p, a, s));
     FMAP_CUDA(launch_exp_coef(p, a, s));
     if (ev[2]) FMAP_CUDA(cudaEventRecord(ev[2], s));
     if (p->flags & FMAP_PLAN_EXP_RECURRENCE) {

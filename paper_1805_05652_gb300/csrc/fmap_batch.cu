@@ -38,30 +38,29 @@ namespace {
 constexpr int kOccCandidates[] = {1, 2, 4, 8};
 
 struct Tuning {
-  int occ[BP_COUNT];
+  int occ[BP_ALL];
   int rec_tpb;   // templates per block of the recurrence phase
 };
 
 std::mutex g_tune_mu;
 std::map<std::string, Tuning> g_tune_cache;
 
-// lanes: the scan width of the wave's exp instances (batch_scan_lanes).
-const void* phase_kernel(int ph, int lanes) {
+// max_g: the most templates per warp of the wave's recurrences.
+const void* phase_kernel(int ph, int max_g) {
   if (const void* k = batch_kernel_common(ph)) return k;
   if (const void* k = batch_kernel_rect(ph)) return k;
-  if (const void* k = batch_kernel_exp(ph, lanes)) return k;
-  if (const void* k = batch_kernel_exp_rec(ph, lanes)) return k;
+  if (const void* k = batch_kernel_exp(ph)) return k;
+  if (const void* k = batch_kernel_exp_rec(ph, max_g)) return k;
   return batch_kernel_fixup(ph);
 }
 
-int phase_threads(int ph, int lanes) {
+int phase_threads(int ph) {
   switch (ph) {
     case BP_FLAG_COUNT:
     case BP_FLAG_SCAN:
     case BP_FLAG_WRITE: return 1024;
     case BP_FIXUP: return 128;
-    case BP_EXP_ANT:
-    case BP_EXP_REC: return lanes;
+    case BP_EXP_REC: return 32 * kRecWarps;
     default: return 256;
   }
 }
@@ -70,11 +69,11 @@ int phase_threads(int ph, int lanes) {
 
 struct Wave {
   std::vector<int32_t> items;            // instance indices (heaviest first)
-  int lanes = kScanLanes;                // scan width of its exp instances
   BItem* d_items = nullptr;
-  int64_t* d_offsets = nullptr;          // [BP_COUNT][n + 1]
+  int64_t* d_offsets = nullptr;          // [BP_ALL][n + 1]
   std::vector<int64_t> totals;           // units per phase
-  size_t dyn_smem[BP_COUNT] = {};
+  size_t dyn_smem[BP_ALL] = {};
+  int max_g = 1;                         // most templates per warp of its recurrences
 };
 
 }  // namespace fmap
@@ -87,7 +86,7 @@ struct fmap_batch_s {
   std::vector<fmap::Wave> waves;
   char* ws = nullptr;                    // instance workspaces of the largest wave
   size_t ws_bytes = 0;
-  unsigned long long* d_counters = nullptr;   // [waves][BP_COUNT]
+  unsigned long long* d_counters = nullptr;   // [waves][BP_ALL]
   uint32_t* d_err = nullptr;             // shared device status word
   fmap::Tuning tune{};
   cudaStream_t cap = nullptr;
@@ -101,6 +100,20 @@ namespace fmap {
 static fmap_status batch_fail(const std::string& m, fmap_status st = FMAP_ERR_ARG) {
   set_error(m);
   return st;
+}
+
+static RecGeom batch_rec_geom(const fmap_plan_s* p, const fmap_batch_item& it, int rec_tpb) {
+  return plan_rec_geom(p->grid, p->n_sft, p->n_templates, p->flags, it.atoms.shared_antenna != 0,
+                       rec_tpb);
+}
+
+// Partial slots per template that the cells phase of instance `p` writes.
+static int64_t tiles_used_of(const fmap_plan_s* p, const fmap_batch_item& it, int rec_tpb) {
+  const fmap_grid& g = p->grid;
+  if ((int64_t)g.n_t0 * g.n_tau == 0) return 0;
+  if (g.window == FMAP_RECT) return rect_partial_slots(g, p->n_templates, it.atoms.shared_antenna);
+  const RecGeom q = batch_rec_geom(p, it, rec_tpb);
+  return (int64_t)q.ntr * q.n_grp;
 }
 
 // Work units of instance `p` in phase `ph` (0: phase not used by it).
@@ -119,15 +132,30 @@ static int64_t units_of(const fmap_plan_s* p, const fmap_batch_item& it, int ph,
     case BP_EXP_PERM: {
       if (rect || cells == 0) return 0;
       const int32_t n_x = (p->flags & FMAP_PLAN_EXP_RECURRENCE) ? (int32_t)T : 0;
-      return (exp_copy_entries(p->n_sft, p->lanes, (int32_t)n_ant, n_x, g.n_tau) + kPermPerUnit - 1) /
+      return (exp_copy_entries(p->n_sft, (int32_t)n_ant, n_x, g.n_tau) + kPermPerUnit - 1) /
              kPermPerUnit;
     }
-    case BP_RECT_ANT: return rect && cells > 0 && p->n_sft > 0 ? n_ant : 0;
-    case BP_EXP_ANT: return !rect && cells > 0 ? g.n_tau * n_ant : 0;
+    case BP_RECT_ANT:   // antenna rows, then data rows
+      return rect && cells > 0 && p->n_sft > 0 ? n_ant + (work ? T : 0) : 0;
+    case BP_EXP_AGG: {   // antenna chunk maps, then the data's
+      if (rect || cells == 0 || p->n_sft == 0) return 0;
+      const AntGeom a = p->ant[it.atoms.shared_antenna ? 1 : 0];
+      const RecGeom q = batch_rec_geom(p, it, rec_tpb);
+      return (a.n_grp * n_ant * a.n_chunks + (work ? (int64_t)q.n_grp * q.n_chunks * q.n_tgrp : 0) +
+              kSweepWarps - 1) / kSweepWarps;
+    }
+    case BP_EXP_ANT: {
+      if (rect || cells == 0) return 0;
+      const AntGeom q = p->ant[it.atoms.shared_antenna ? 1 : 0];
+      return (q.n_grp * n_ant * q.n_seg + kSweepWarps - 1) / kSweepWarps;
+    }
     case BP_RECT_COEF:
       return rect && cells > 0 ? (cells * n_ant + 256 * kCoefBlocksPerUnit - 1) / (256 * kCoefBlocksPerUnit) : 0;
-    case BP_RECT_DATA: return rect && work && p->n_sft > 0 ? T : 0;
-    case BP_EXP_REC: return !rect && work ? g.n_tau * ((T + rec_tpb - 1) / rec_tpb) : 0;
+    case BP_EXP_REC: {
+      if (rect || !work) return 0;
+      const RecGeom q = batch_rec_geom(p, it, rec_tpb);
+      return ((int64_t)q.n_grp * q.n_seg * q.n_tgrp + kRecWarps - 1) / kRecWarps;
+    }
     case BP_RECT_CELLS:
       return rect && work ? rect_cells_blocks(g, (int32_t)T, it.atoms.shared_antenna) : 0;
     case BP_FLAG_COUNT:
@@ -137,8 +165,7 @@ static int64_t units_of(const fmap_plan_s* p, const fmap_batch_item& it, int ph,
       return work ? (int64_t)kFixUnits * fixup_blocks_y((int32_t)T, it.atoms.shared_antenna != 0) : 0;
     case BP_RED_GROUPS: {
       if (!it.d_summary || T == 0) return 0;
-      const int64_t used =
-          cells > 0 ? (rect ? rect_partial_slots(g, (int32_t)T, it.atoms.shared_antenna) : g.n_tau) : 0;
+      const int64_t used = tiles_used_of(p, it, rec_tpb);
       return reduce_groups_of(used + (cells > 0 ? kFixSlots : 0)) * T;
     }
     case BP_RED_FINAL: return it.d_summary && T > 0 ? T : 0;
@@ -155,13 +182,15 @@ static BItem make_bitem(const fmap_plan_s* p, const fmap_batch_item& it, uint32_
   b.T = p->n_templates;
   b.shared = it.atoms.shared_antenna ? 1 : 0;
   b.n_ant = b.shared ? 1 : b.T;
-  b.groups = std::max(1, (b.T + rec_tpb - 1) / rec_tpb);
+  if (g.window == FMAP_EXP) {
+    b.ag = p->ant[b.shared];
+    b.rg = batch_rec_geom(p, it, rec_tpb);
+  }
   b.n_alloc = rel_t_entries(p->n_sft);
-  b.lanes = p->lanes;
   b.cells = (int64_t)g.n_t0 * g.n_tau;
   b.n_tiles = p->n_tiles;
   b.part_stride = p->part_stride;
-  b.tiles_used = b.cells > 0 ? (g.window == FMAP_RECT ? rect_partial_slots(g, b.T, b.shared) : g.n_tau) : 0;
+  b.tiles_used = tiles_used_of(p, it, rec_tpb);
   b.red_groups = reduce_groups_of(b.tiles_used + (b.cells > 0 ? kFixSlots : 0));
   b.flag_entries = b.cells * b.n_ant;
   b.log_prior = p->log_prior;
@@ -186,8 +215,8 @@ static BItem make_bitem(const fmap_plan_s* p, const fmap_batch_item& it, uint32_
   b.pa = w.pa;
   b.perm_ant = w.perm_ant;
   b.perm_x = w.perm_x;
-  b.perm_gap = w.perm_gap;
-  b.rec_cells = w.rec_cells;
+  b.agg = w.agg;
+  b.irr = w.irr;
   b.tauc = w.tauc;
   b.ax = nullptr;   // batches take uniform grids
   b.px = w.px;
@@ -198,30 +227,25 @@ static BItem make_bitem(const fmap_plan_s* p, const fmap_batch_item& it, uint32_
 static fmap_status build_wave_tables(fmap_batch_s* B, Wave& wv, const Tuning& tn) {
   const int n = (int)wv.items.size();
   std::vector<BItem> h(n);
-  std::vector<int64_t> off((size_t)BP_COUNT * (n + 1), 0);
-  wv.totals.assign(BP_COUNT, 0);
-  for (int ph = 0; ph < BP_COUNT; ++ph) wv.dyn_smem[ph] = 0;
+  std::vector<int64_t> off((size_t)BP_ALL * (n + 1), 0);
+  wv.totals.assign(BP_ALL, 0);
+  wv.max_g = 1;
+  for (int ph = 0; ph < BP_ALL; ++ph) wv.dyn_smem[ph] = 0;
   for (int k = 0; k < n; ++k) {
     const int32_t i = wv.items[k];
     const fmap_plan_s* p = B->plans[i];
     h[k] = make_bitem(p, B->items[i], B->d_err, tn.rec_tpb);
-    for (int ph = 0; ph < BP_COUNT; ++ph) {
+    wv.max_g = std::max(wv.max_g, (int)h[k].rg.G);
+    for (int ph = 0; ph < BP_ALL; ++ph) {
       const int64_t u = units_of(p, B->items[i], ph, tn.rec_tpb);
       off[(size_t)ph * (n + 1) + k + 1] = off[(size_t)ph * (n + 1) + k] + u;
       if (u > 0) {
-        if (ph == BP_EXP_ANT)
-          wv.dyn_smem[ph] = std::max(wv.dyn_smem[ph], exp_antenna_smem(p->n_sft));
-        if (ph == BP_EXP_REC)
-          wv.dyn_smem[ph] = std::max(
-              wv.dyn_smem[ph],
-              exp_rec_smem(p->n_sft, p->grid.n_t0,
-                           (h[k].T + h[k].groups - 1) / std::max(1, h[k].groups)));
         if (ph == BP_RECT_CELLS)
           wv.dyn_smem[ph] = std::max(wv.dyn_smem[ph], rect_cells_smem(p->n_templates, B->items[i].atoms.shared_antenna));
       }
     }
   }
-  for (int ph = 0; ph < BP_COUNT; ++ph) wv.totals[ph] = off[(size_t)ph * (n + 1) + n];
+  for (int ph = 0; ph < BP_ALL; ++ph) wv.totals[ph] = off[(size_t)ph * (n + 1) + n];
   if (!wv.d_items) {
     FMAP_CUDA(cudaMalloc(&wv.d_items, sizeof(BItem) * std::max(n, 1)));
     FMAP_CUDA(cudaMalloc(&wv.d_offsets, sizeof(int64_t) * off.size()));
@@ -237,10 +261,8 @@ static fmap_status enqueue_phase(fmap_batch_s* B, int w, int ph, int occ, cudaSt
   Wave& wv = B->waves[w];
   const int64_t total = wv.totals[ph];
   if (total == 0) return FMAP_OK;
-  const void* k = phase_kernel(ph, wv.lanes);
-  const int threads = phase_threads(ph, wv.lanes);
-  // narrower exp blocks: the same occupancy candidates in units of 256 threads
-  if (ph == BP_EXP_ANT || ph == BP_EXP_REC) occ *= kScanLanes / wv.lanes;
+  const void* k = phase_kernel(ph, wv.max_g);
+  const int threads = phase_threads(ph);
   const size_t smem = wv.dyn_smem[ph];
   if (smem > 0)
     FMAP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -248,7 +270,7 @@ static fmap_status enqueue_phase(fmap_batch_s* B, int w, int ph, int occ, cudaSt
   FMAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&max_occ, k, threads, smem));
   max_occ = std::max(1, max_occ);
   const int64_t grid = std::min<int64_t>(total, (int64_t)B->n_sm * std::min(occ, max_occ));
-  unsigned long long* ctr = B->d_counters + (size_t)w * BP_COUNT + ph;
+  unsigned long long* ctr = B->d_counters + (size_t)w * BP_ALL + ph;
   FMAP_CUDA(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s));
   BUnits u;
   u.offsets = wv.d_offsets + (size_t)ph * (wv.items.size() + 1);
@@ -278,7 +300,6 @@ static fmap_status place_wave(fmap_batch_s* B, int w) {
     st = plan_init(p, &it.grid, it.atoms.n_sft, it.atoms.n_templates, FMAP_FP64, flags,
                    B->ws + off, bytes);
     if (st != FMAP_OK) return st;
-    p->lanes = batch_scan_lanes(it.atoms.n_sft);   // the wave's exp kernels use this width
     off += (bytes + 255) / 256 * 256;
   }
   return FMAP_OK;
@@ -320,22 +341,28 @@ static fmap_status autotune(fmap_batch_s* B) {
   Tuning best = B->tune;
   fmap_status st = place_wave(B, 0);
   if (st == FMAP_OK) st = build_wave_tables(B, B->waves[0], best);
-  // one full pass so every phase's inputs exist
-  for (int ph = 0; st == FMAP_OK && ph < BP_COUNT; ++ph) st = enqueue_phase(B, 0, ph, best.occ[ph], s);
-  for (int ph = 0; st == FMAP_OK && ph < BP_COUNT; ++ph) {
-    if (B->waves[0].totals[ph] == 0) continue;
-    // Candidates are timed by re-running one phase on the outputs of the full
-    // pass; the compaction phases are not idempotent (the scan turns counts
-    // into offsets in place), so they keep the default occupancy.
-    if (ph == BP_FLAG_COUNT || ph == BP_FLAG_SCAN || ph == BP_FLAG_WRITE) continue;
+  // The phases in launch order, so that each one's inputs exist and stand while
+  // it is timed (phases reuse each other's scratch: the sweeps' chunk maps lie
+  // where the marked-entry list is written after them).
+  for (int ph : kBatchOrder) {
+    if (st != FMAP_OK || B->waves[0].totals[ph] == 0) continue;
+    // Candidates are timed by re-running one phase on the outputs of those
+    // before it; the compaction phases are not idempotent (the scan turns counts
+    // into offsets in place), so they run once, at the default occupancy.
+    if (ph == BP_FLAG_COUNT || ph == BP_FLAG_SCAN || ph == BP_FLAG_WRITE) {
+      st = enqueue_phase(B, 0, ph, best.occ[ph], s);
+      continue;
+    }
     const bool rec = ph == BP_EXP_REC;
-    const int tpbs[] = {1, 2, 4, 8};
+    const int tpbs[] = {1, 2, 4};
     float best_ms = 1e30f;
-    for (int ti = 0; ti < (rec ? 4 : 1) && st == FMAP_OK; ++ti) {
+    for (int ti = 0; ti < (rec ? 3 : 1) && st == FMAP_OK; ++ti) {
       Tuning tr = best;
       if (rec) {
         tr.rec_tpb = tpbs[ti];
+        cudaStreamSynchronize(s);   // (the tables are in use until then)
         st = build_wave_tables(B, B->waves[0], tr);
+        if (st == FMAP_OK) st = enqueue_phase(B, 0, BP_EXP_AGG, best.occ[BP_EXP_AGG], s);
       }
       for (int oc : kOccCandidates) {
         if (st != FMAP_OK) break;
@@ -360,7 +387,10 @@ static fmap_status autotune(fmap_batch_s* B) {
         }
       }
     }
-    if (rec && st == FMAP_OK) st = build_wave_tables(B, B->waves[0], best);
+    if (rec && st == FMAP_OK) {
+      cudaStreamSynchronize(s);
+      st = build_wave_tables(B, B->waves[0], best);
+    }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -445,53 +475,32 @@ fmap_status fmap_batch_plan(fmap_batch_t** out, const fmap_batch_item* items, in
                                                     : (double)it.grid.n_tau * it.atoms.n_sft;
     B->cost[i] = (double)it.atoms.n_sft + (cells + sums) * std::max(1, it.atoms.n_templates);
   }
-  // Shared-memory class of an instance: the exp phases launch with the
-  // largest dynamic shared memory of their wave, so instances are grouped by
-  // the number of blocks per SM that their exp kernels allow (rect instances
-  // take the first class).  Within a class, heaviest first; waves are filled
-  // greedily within the budget and never mix classes.  The class also
-  // separates the exp scan widths (batch_scan_lanes), whose kernels differ.
-  std::vector<int> cls(n_items, 0);
-  auto lane_index = [](int32_t n) {
-    return batch_scan_lanes(n) == 64 ? 0 : batch_scan_lanes(n) == 128 ? 1 : 2;
-  };
-  for (int32_t i = 0; i < n_items; ++i) {
-    const fmap_batch_item& it = items[i];
-    if (it.grid.window != FMAP_EXP) continue;
-    const size_t sm = std::max(
-        exp_rec_smem(it.atoms.n_sft, it.grid.n_t0, std::min(it.atoms.n_templates, 2)),
-        exp_antenna_smem(it.atoms.n_sft));
-    const int smem_cls = sm <= (56u << 10) ? 0 : sm <= (75u << 10) ? 1 : sm <= (113u << 10) ? 2 : 3;
-    cls[i] = 4 * smem_cls + lane_index(it.atoms.n_sft);
-  }
+  // Heaviest first; waves are filled greedily within the budget.
   std::vector<int32_t> order(n_items);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-    return cls[a] != cls[b] ? cls[a] < cls[b] : B->cost[a] > B->cost[b];
+    return B->cost[a] > B->cost[b];
   });
   const size_t budget = workspace_budget ? workspace_budget : (size_t)8 << 30;
   size_t cur = 0, peak = 0;
-  int cur_cls = -1;
   for (int32_t i : order) {
     if (foot[i] > budget) {
       batch_free(B);
       return batch_fail("instance " + std::to_string(i) + " alone exceeds the workspace budget",
                         FMAP_ERR_NOMEM);
     }
-    if (B->waves.empty() || cur + foot[i] > budget || cls[i] != cur_cls) {
+    if (B->waves.empty() || cur + foot[i] > budget) {
       B->waves.emplace_back();
       cur = 0;
-      cur_cls = cls[i];
     }
     B->waves.back().items.push_back(i);
-    if (items[i].grid.window == FMAP_EXP) B->waves.back().lanes = batch_scan_lanes(items[i].atoms.n_sft);
     cur += foot[i];
     peak = std::max(peak, cur);
   }
   cudaError_t e = cudaMalloc((void**)&B->ws, std::max<size_t>(peak, 256));
   if (e == cudaSuccess)
     e = cudaMalloc((void**)&B->d_counters,
-                   sizeof(unsigned long long) * BP_COUNT * std::max<size_t>(B->waves.size(), 1));
+                   sizeof(unsigned long long) * BP_ALL * std::max<size_t>(B->waves.size(), 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&B->d_err, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(B->d_err, 0, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking);
@@ -501,8 +510,8 @@ fmap_status fmap_batch_plan(fmap_batch_t** out, const fmap_batch_item* items, in
     return batch_fail("batch allocation failed", FMAP_ERR_NOMEM);
   }
   B->ws_bytes = peak;
-  for (int ph = 0; ph < BP_COUNT; ++ph) B->tune.occ[ph] = 4;
-  B->tune.rec_tpb = 1;
+  for (int ph = 0; ph < BP_ALL; ++ph) B->tune.occ[ph] = 4;
+  B->tune.rec_tpb = 4;
   fmap_status st = FMAP_OK;
   if ((flags & FMAP_BATCH_AUTOTUNE) && !B->waves.empty()) st = autotune(B);
   // Every wave's plans start at the workspace base: waves run one after the
@@ -519,8 +528,8 @@ fmap_status fmap_batch_plan(fmap_batch_t** out, const fmap_batch_item* items, in
   }
   if (st == FMAP_OK) {
     for (size_t w = 0; w < B->waves.size() && st == FMAP_OK; ++w)
-      for (int ph = 0; ph < BP_COUNT && st == FMAP_OK; ++ph)
-        st = enqueue_phase(B, (int)w, ph, B->tune.occ[ph], B->cap);
+      for (int ph : kBatchOrder)
+        if (st == FMAP_OK) st = enqueue_phase(B, (int)w, ph, B->tune.occ[ph], B->cap);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(B->cap, &g);
     if (st == FMAP_OK && e != cudaSuccess) st = cuda_fail(e, "cudaStreamEndCapture");
@@ -577,22 +586,23 @@ fmap_status fmap_batch_profile(fmap_batch_t* B, fmap_stream stream, float* phase
   static_assert(FMAP_BATCH_N_PHASES == BP_COUNT, "phase count");
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t launches = B->n_launches;
-  std::vector<cudaEvent_t> ev(2 * B->waves.size() * BP_COUNT, nullptr);
+  std::vector<cudaEvent_t> ev(2 * B->waves.size() * BP_ALL, nullptr);
   for (auto& e : ev) FMAP_CUDA(cudaEventCreate(&e));
   fmap_status st = FMAP_OK;
   for (size_t w = 0; w < B->waves.size() && st == FMAP_OK; ++w)
-    for (int ph = 0; ph < BP_COUNT && st == FMAP_OK; ++ph) {
-      cudaEventRecord(ev[2 * (w * BP_COUNT + ph)], s);
+    for (int ph : kBatchOrder) {
+      if (st != FMAP_OK) break;
+      cudaEventRecord(ev[2 * (w * BP_ALL + ph)], s);
       st = enqueue_phase(B, (int)w, ph, B->tune.occ[ph], s);
-      cudaEventRecord(ev[2 * (w * BP_COUNT + ph) + 1], s);
+      cudaEventRecord(ev[2 * (w * BP_ALL + ph) + 1], s);
     }
   cudaError_t e = cudaStreamSynchronize(s);
   if (st == FMAP_OK && e != cudaSuccess) st = cuda_fail(e, "fmap_batch_profile");
   for (size_t w = 0; w < B->waves.size() && st == FMAP_OK; ++w)
-    for (int ph = 0; ph < BP_COUNT; ++ph) {
+    for (int ph : kBatchOrder) {
       float ms = 0.f;
-      cudaEventElapsedTime(&ms, ev[2 * (w * BP_COUNT + ph)], ev[2 * (w * BP_COUNT + ph) + 1]);
-      phase_ms[ph] += ms;
+      cudaEventElapsedTime(&ms, ev[2 * (w * BP_ALL + ph)], ev[2 * (w * BP_ALL + ph) + 1]);
+      phase_ms[ph == BP_EXP_AGG ? (int)BP_EXP_ANT : ph] += ms;
     }
   for (auto& x : ev) cudaEventDestroy(x);
   B->n_launches = launches;

@@ -14,7 +14,9 @@ namespace fmap {
 
 struct BItem {
   fmap_grid g;
-  int32_t n_sft, T, shared, n_ant, groups, n_alloc, lanes;
+  int32_t n_sft, T, shared, n_ant, n_alloc;
+  AntGeom ag;
+  RecGeom rg;
   int64_t cells, n_tiles, part_stride, red_groups, tiles_used, flag_entries;
   double log_prior;
   const int64_t* t;
@@ -37,8 +39,8 @@ struct BItem {
   float4* pa;
   float4* perm_ant;
   float4* perm_x;
-  int32_t* perm_gap;
-  float4* rec_cells;
+  float* agg;
+  int32_t* irr;
   TauTab* tauc;
   int64_t* ax;
   float4* px;
@@ -57,7 +59,7 @@ struct BUnits {
 constexpr int kCoefBlocksPerUnit = 8;
 constexpr int kIdxRowsPerUnit = 8;
 constexpr int kFixUnits = 32;        // fix-up units per template group (each strides over the slots)
-constexpr int kPermPerUnit = 4096;   // chunk-major copy entries per unit
+constexpr int kPermPerUnit = 1024;   // exp copy entries per unit
 constexpr int kBitsPerUnit = 4096;   // marked-entry bitmask words cleared per unit
 
 // Phases of the batch pipeline, in launch order.
@@ -77,8 +79,16 @@ enum BPhase {
   BP_FIXUP,
   BP_RED_GROUPS,
   BP_RED_FINAL,
-  BP_COUNT
+  BP_COUNT,
+  // Launched before BP_EXP_ANT and reported with it.
+  BP_EXP_AGG = BP_COUNT,
+  BP_ALL
 };
+// The launches of a wave (BP_RECT_ANT also scans the data rows).
+constexpr int kBatchOrder[] = {BP_PREP, BP_INDEX, BP_EXP_PERM, BP_RECT_ANT, BP_EXP_AGG, BP_EXP_ANT,
+                               BP_RECT_COEF, BP_EXP_REC, BP_RECT_CELLS, BP_FLAG_COUNT,
+                               BP_FLAG_SCAN, BP_FLAG_WRITE, BP_FIXUP, BP_RED_GROUPS, BP_RED_FINAL};
+
 
 // A block claims units in increasing order, so the instance of its next
 // unit is at or after that of its last one: thread 0 gallops forward from

@@ -25,8 +25,9 @@ __device__ __forceinline__ void finite_check(const float* __restrict__ v, int64_
 __device__ __forceinline__ void prep_body(const int64_t* __restrict__ t, int32_t n, int32_t n_alloc,
                        int32_t* __restrict__ rel_t, int64_t* __restrict__ t_base,
                        uint32_t* __restrict__ err, const float* __restrict__ ant, int64_t n_ant_vals,
-                       const float* __restrict__ x, int64_t n_x_vals,
+                       const float* __restrict__ x, int64_t n_x_vals, int32_t* __restrict__ irr,
     const uint3 bid, const dim3 gdim) {
+  if (bid.x == 0 && threadIdx.x == 0) *irr = 0;   // (set by the exp copy step)
   {
     const int64_t g0 = bid.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t step = (int64_t)gdim.x * blockDim.x;
@@ -54,8 +55,9 @@ __device__ __forceinline__ void prep_body(const int64_t* __restrict__ t, int32_t
 __global__ void k_prep(const int64_t* __restrict__ t, int32_t n, int32_t n_alloc,
                        int32_t* __restrict__ rel_t, int64_t* __restrict__ t_base,
                        uint32_t* __restrict__ err, const float* __restrict__ ant,
-                       int64_t n_ant_vals, const float* __restrict__ x, int64_t n_x_vals) {
-  prep_body(t, n, n_alloc, rel_t, t_base, err, ant, n_ant_vals, x, n_x_vals, blockIdx, gridDim);
+                       int64_t n_ant_vals, const float* __restrict__ x, int64_t n_x_vals,
+                       int32_t* __restrict__ irr) {
+  prep_body(t, n, n_alloc, rel_t, t_base, err, ant, n_ant_vals, x, n_x_vals, irr, blockIdx, gridDim);
 }
 
 // Window index tables: i0[m] = first atom with t >= t0_m; jend[m][n] = one
@@ -163,7 +165,7 @@ cudaError_t launch_prep(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
   const int blocks = (int)std::min<int64_t>((want + threads - 1) / threads, (int64_t)p->n_sm * 16);
   k_prep<<<std::max(blocks, 1), threads, 0, s>>>(a->t, p->n_sft, rel_t_entries(p->n_sft),
                                                  p->ws.rel_t, p->ws.t_base, p->ws.dev_err,
-                                                 a->antenna, n_ant, a->fafb, n_x);
+                                                 a->antenna, n_ant, a->fafb, n_x, p->ws.irr);
   p->launches += 1;
   return cudaGetLastError();
 }
@@ -454,7 +456,7 @@ __global__ void __launch_bounds__(256) kb_prep(const BItem* __restrict__ items, 
     const int64_t ru = it.n_sft > 0 ? (it.n_alloc + 255) / 256 : 0;
     if (k < ru) {
       prep_body(it.t, it.n_sft, it.n_alloc, it.rel_t, it.t_base, it.dev_err, it.antenna,
-                (int64_t)3 * it.n_sft * it.n_ant, it.fafb, (int64_t)4 * it.n_sft * it.T,
+                (int64_t)3 * it.n_sft * it.n_ant, it.fafb, (int64_t)4 * it.n_sft * it.T, it.irr,
                 make_uint3((unsigned)k, 0, 0), dim3((unsigned)ru));
     } else {
       const int64_t w0 = (k - ru) * kBitsPerUnit;

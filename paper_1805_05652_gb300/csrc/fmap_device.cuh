@@ -153,56 +153,103 @@ __device__ __forceinline__ FF ff_fma_sum(FF s, FF r, FF e) {
   const float te = (s.h - (t - bb)) + (p - bb);
   return fast_two_sum(t, (s.l + fmaf(r.h, e.l, fmaf(r.l, e.h, pe))) + te);
 }
-// x + r e
-__device__ __forceinline__ FF ff_axpy(FF r, FF e, float x) {
-  const float p = r.h * e.h;
-  const float pe = fmaf(r.h, e.h, -p);
-  const FF s = two_sum(x, p);
-  return fast_two_sum(s.h, s.l + pe + fmaf(r.h, e.l, r.l * e.h));
-}
-__device__ __forceinline__ FF ff_shfl_down(FF v, int d) {
-  return {__shfl_down_sync(0xffffffffu, v.h, d), __shfl_down_sync(0xffffffffu, v.l, d)};
-}
 __device__ __forceinline__ FF ff_of(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
 }
 
-// Fills the per-tau constants of one tau value (one thread).  The one-SFT decay is
-// an FP64 exp split into a float pair; its powers come by binary powering in
-// float-float (~k ulp of 2^-48).
-__device__ __forceinline__ void tau_tab_fill(const fmap_grid& g, int64_t tau, TauTab* out) {
-  TauTab t;
-  t.inv_tau = 1.0 / (double)tau;
-#pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    const double inv_s = (double)(s + 1) * t.inv_tau;
-    t.c2[s] = (float)(-1.4426950408889634 * inv_s);
-    const FF rho1 = ff_of(exp(-(double)g.t_sft * inv_s));
-    for (int k = 0; k < kPowTab; ++k) {
-      FF acc{1.0f, 0.0f}, r = rho1;
-      for (int q = k; q; q >>= 1) {
-        if (q & 1) acc = ff_mul(acc, r);
-        r = ff_mul(r, r);
-      }
-      t.pw[s][k] = make_float2(acc.h, acc.l);
-    }
-  }
-  *out = t;
+// ---- packed f32x2 arithmetic (.x in the low half): two FP32 operations an
+// instruction.
+__device__ __forceinline__ uint64_t pk2(float x, float y) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(x), "f"(y));
+  return r;
 }
-// Decay over one gap between consecutive atoms: a table entry (pw of the
-// tau's TauTab) for gaps of 1..kPowTab-1 whole SFTs, FP64 exp otherwise
-// (gaps off the T_sft lattice; inv_s = s / tau).
-__device__ __forceinline__ FF gap_decay(int32_t gap, int32_t t_sft, float inv_tsft,
-                                        const float2* __restrict__ tab, double inv_s) {
-  const int32_t k = __float2int_rn((float)gap * inv_tsft);
-  if (k >= 1 && k < kPowTab && k * t_sft == gap) {
-    const float2 v = tab[k];
-    return {v.x, v.y};
-  }
-  return ff_of(exp(-(double)gap * inv_s));
+__device__ __forceinline__ void up2(uint64_t a, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(x), "=f"(y) : "l"(a));
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
+// 2F of one cell from its window sums (fa, fb as f32x2 re/im pairs);
+// nb2 = (-beta, -beta); k1 = -inf marks a cell that takes no part.
+__device__ __forceinline__ float two_f_pairs(uint64_t fa, uint64_t fb, uint64_t nb2, float k1,
+                                             float k2, uint64_t tiny2) {
+  const uint64_t e = fma2(nb2, fa, fb);
+  const uint64_t pa = fma2(fa, fa, tiny2);
+  const uint64_t pe = mul2(e, e);
+  float a0, a1, e0, e1;
+  up2(pa, a0, a1);
+  up2(pe, e0, e1);
+  return fmaf(k1, a0 + a1, k2 * (e0 + e1));
+}
+
+// r a per half as two scalar products: ptxas contracts a packed product into a
+// packed addition that follows it (.rn or not: measured), and an error-free
+// transformation of the sum would then count the product's error twice.
+__device__ __forceinline__ uint64_t mul2_apart(float r, uint64_t a) {
+  float x, y;
+  up2(a, x, y);
+  return pk2(__fmul_rn(r, x), __fmul_rn(r, y));
+}
+// Two float-float values side by side (h and l as f32x2).
+struct FF2 {
+  uint64_t h, l;
+};
+__device__ __forceinline__ FF2 fast_two_sum2(uint64_t a, uint64_t b) {
+  const uint64_t s = add2(a, b);
+  return {s, sub2(b, sub2(s, a))};
+}
+// s + r e per half, s a plain f32x2 value and r a float pair common to both
+// halves: TwoProd of the high parts, TwoSum with s, one renormalisation
+// (~2^-46 relative).
+__device__ __forceinline__ FF2 ff2_fma_sum(uint64_t s, FF r, const FF2& e) {
+  const uint64_t rh = pk2(r.h, r.h);
+  const uint64_t p = mul2_apart(r.h, e.h);
+  const uint64_t pe = fma2(rh, e.h, mul2(pk2(-r.h, -r.h), e.h));   // (the addend is -p)
+  const uint64_t t = add2(s, p);
+  const uint64_t bb = sub2(t, s);
+  const uint64_t te = add2(sub2(s, sub2(t, bb)), sub2(p, bb));
+  return fast_two_sum2(t, add2(fma2(rh, e.l, fma2(pk2(r.l, r.l), e.h, pe)), te));
+}
+
+// Fills one half (s = 0: the weight w, s = 1: w^2) of the per-tau constants of
+// one tau value (one thread).  The one-SFT decay is an FP64 exp split into a
+// float pair; its powers come by repeated multiplication in float-float (k
+// roundings of ~2^-47).  One thread per (tau, half) and 15 products: binary
+// powering of every entry by one thread per tau was a chain of ~2000
+// instructions, the longest of the copy kernel.
+__device__ __forceinline__ void tau_tab_fill(const fmap_grid& g, int64_t tau, int s, TauTab* out) {
+  const double inv_tau = 1.0 / (double)tau;
+  const double inv_s = (double)(s + 1) * inv_tau;
+  if (s == 0) out->inv_tau = inv_tau;
+  out->c2[s] = (float)(-1.4426950408889634 * inv_s);
+  const FF rho1 = ff_of(exp(-(double)g.t_sft * inv_s));
+  FF acc{1.0f, 0.0f};
+#pragma unroll
+  for (int k = 0; k < kPowTab; ++k) {
+    out->pw[s][k] = make_float2(acc.h, acc.l);
+    acc = ff_mul(acc, rho1);
+  }
+}
 // Generic window w(x) from its table (entries k = 0..n-1: (w_k, w_{k+1} -
 // w_k), then the sentinel (0, 0)): linear between samples, 0 past the last.
 // u = x (n - 1) / X is the position in sample units (u >= 0).

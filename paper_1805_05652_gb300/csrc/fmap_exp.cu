@@ -1,13 +1,13 @@
 // Exponential-window F-map (Eq. winexp, cut after 3 tau).
 //
 // Antenna part (shared by every template of a sky position): A, B, C with the
-// squared weight w^2 = e^{-2(t - t0)/tau}, in FP64, from a decayed suffix
-// sum per tau:
-//     E[i] = x_i + e^{-2(t_{i+1} - t_i)/tau} E[i+1],   E[N] = 0,
+// squared weight w^2 = e^{-2(t - t0)/tau}, from a decayed suffix sum per tau in
+// float-float arithmetic (the FP32 pipe; GB300's FP64 rate is 1/64 of it):
+//     E[i] = x_i + e^{-2(t_{i+1} - t_i)/tau} E[i+1],
 //     A(t0, tau) = e^{-2(t_{i0} - t0)/tau} (E[i0] - e^{-2(t_j - t_{i0})/tau} E[j])
 // for the window's atoms [i0, j).  The recurrence is contractive, so the
 // subtraction loses at most a factor 1/(1 - e^{-6}) of relative accuracy.
-// Then D = AB - C^2 in FP64 and the per-cell 2F coefficients.
+// Then D = AB - C^2 in float-float and the per-cell 2F coefficients.
 //
 // Data part: Fa, Fb = sum_a w(t_a) X[a, col] over the window, a contraction
 // of the weight matrix W[(t0, tau), a] with the 4T data columns.  Here the
@@ -18,23 +18,12 @@
 
 #include <type_traits>
 
+#include <algorithm>
+
 #include "fmap_batch.cuh"
-#include "fmap_device.cuh"
+#include "fmap_sweep.cuh"
 
 namespace fmap {
-
-constexpr int kSufThreads = 256;
-
-// r^k for small k >= 1 by binary powering (relative error ~k ulp).
-__device__ __forceinline__ double ipow(double r, int k) {
-  double acc = 1.0;
-  while (k) {
-    if (k & 1) acc *= r;
-    r *= r;
-    k >>= 1;
-  }
-  return acc;
-}
 
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -42,141 +31,22 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// Decayed suffix sums of the three antenna rows for one tau, by a parallel
-// backward scan of the affine maps E -> x + rho E over the block's threads,
-// in float-float arithmetic (the FP32 pipe; GB300's FP64 rate is 1/64 of
-// it): E[c * (n + 1) + i] for c = a2, b2, ab and i = 0..n (E[n] = 0), each as
-// an (h, l) pair.  E may be in global or shared memory; the block must call
-// it together.
-// NT = the plan's scan width: the threads of the block and the width of the
-// chunk-major copy.
-template <int NT>
-__device__ __forceinline__ void antenna_suffix(const float4* __restrict__ perm, int32_t n,
-                                               const fmap_grid& g,
-                                               const TauTab* __restrict__ tt, float2* E,
-                                               float (*sR)[NT / 32],
-                                               float (*sS)[2][NT / 32]) {
-  const double inv_s = 2.0 * tt->inv_tau;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int C = (int)scan_chunk(n, NT);
-  const int s0 = min(n, tid * C), e0 = min(n, s0 + C);
-  // Decay over one gap: e^{-2 gap / tau}, from the tau's table of powers of
-  // the one-SFT decay (FP64 exp off the T_sft lattice).
-  const float inv_tsft = 1.0f / (float)g.t_sft;
-  auto rho_of_gap = [&](int32_t gap) -> FF {
-    return gap_decay(gap, g.t_sft, inv_tsft, tt->pw[1], inv_s);
-  };
-  // The chunk's atoms (three antenna rows and the gap to the next atom) are
-  // read kSufChunk at a time ahead of each serial run, so the chain does not
-  // wait on memory per atom; the chunk-major copy makes each of these loads
-  // one contiguous 512-byte row per warp.
-  constexpr int kSufChunk = 8;
-  float xa[kSufChunk][3];
-  int32_t gap[kSufChunk];
-  auto load_chunk = [&](int b0) {
-#pragma unroll
-    for (int q = 0; q < kSufChunk; ++q) {
-      const int i = b0 + q;
-      const bool in = i < e0;
-      const float4 v = in ? __ldg(perm + (int64_t)(i - s0) * NT + tid)
-                          : make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-      xa[q][0] = v.x;
-      xa[q][1] = v.y;
-      xa[q][2] = v.z;
-      gap[q] = __float_as_int(v.w);
-    }
-  };
-  auto rho_q = [&](int q) -> FF { return gap[q] < 0 ? FF{0.0f, 0.0f} : rho_of_gap(gap[q]); };
-  // phase 1: compose this thread's chunk: E[s0] = S + R E[e0]
-  FF R{1.0f, 0.0f}, S[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  for (int b0 = s0 + ((e0 - s0 - 1) / kSufChunk) * kSufChunk; e0 > s0 && b0 >= s0;
-       b0 -= kSufChunk) {
-    load_chunk(b0);
-#pragma unroll
-    for (int q = kSufChunk - 1; q >= 0; --q) {
-      if (b0 + q >= e0) continue;
-      const FF r = rho_q(q);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) S[c] = ff_axpy(r, S[c], xa[q][c]);
-      R = ff_mul(r, R);
-    }
-  }
-  // phase 2: inclusive suffix composition within the warp (self o later)
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const FF Ro = ff_shfl_down(R, d);
-    FF So[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) So[c] = ff_shfl_down(S[c], d);
-    if (lane + d < 32) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) S[c] = ff_add(S[c], ff_mul(R, So[c]));
-      R = ff_mul(R, Ro);
-    }
-  }
-  // exclusive within the warp: composition of lanes lane+1 .. 31
-  FF hR = ff_shfl_down(R, 1), hS[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) hS[c] = ff_shfl_down(S[c], 1);
-  if (lane == 31) {
-    hR = {1.0f, 0.0f};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) hS[c] = {0.0f, 0.0f};
-  }
-  if (lane == 0) {
-    sR[0][warp] = R.h;
-    sR[1][warp] = R.l;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      sS[c][0][warp] = S[c].h;
-      sS[c][1][warp] = S[c].l;
-    }
-  }
-  __syncthreads();
-  // composition of the later warps, applied to E[N] = 0: only its S matters
-  FF lS[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  for (int v = NT / 32 - 1; v > warp; --v) {
-    const FF Rv{sR[0][v], sR[1][v]};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) lS[c] = ff_add(FF{sS[c][0][v], sS[c][1][v]}, ff_mul(Rv, lS[c]));
-  }
-  FF e[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) e[c] = ff_add(hS[c], ff_mul(hR, lS[c]));
-  // phase 3: recompute the chunk from its carry E[e0] and store
-  const int64_t np1 = (int64_t)n + 1;
-  for (int b0 = s0 + ((e0 - s0 - 1) / kSufChunk) * kSufChunk; e0 > s0 && b0 >= s0;
-       b0 -= kSufChunk) {
-    load_chunk(b0);
-#pragma unroll
-    for (int q = kSufChunk - 1; q >= 0; --q) {
-      const int i = b0 + q;
-      if (i >= e0) continue;
-      const FF r = rho_q(q);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        e[c] = ff_axpy(r, e[c], xa[q][c]);
-        E[c * np1 + i] = make_float2(e[c].h, e[c].l);
-      }
-    }
-  }
-  if (tid == 0) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) E[c * np1 + n] = make_float2(0.0f, 0.0f);
-  }
-}
-
-// Global-memory suffix sums for one tau of a tau chunk (long data sets).
-__global__ void __launch_bounds__(kSufThreads)
-k_exp_suffix(const float4* __restrict__ perm, const TauTab* __restrict__ tauc, int32_t n,
-             fmap_grid g, int32_t n_lo, float2* __restrict__ esuf) {
-  static_assert(kSufThreads == kScanLanes, "data sets past shared memory take the widest scan");
-  __shared__ float sR[2][kSufThreads / 32];
-  __shared__ float sS[3][2][kSufThreads / 32];
-  const int ni = blockIdx.x;
-  antenna_suffix<kSufThreads>(perm, n, g, tauc + n_lo + ni,
-                              esuf + (int64_t)ni * 3 * ((int64_t)n + 1), sR, sS);
-}
+// ---------------------------------------------------------------------------
+// Antenna sums and coefficients, in two launches of independent warps.
+//
+//   k_sweep_agg (fmap_exp_rec.cu): per (32 tau, chunk of atoms) the affine map E[first] = S + R
+//     E[next chunk's first] of the decayed suffix recurrence, in float-float.
+//   k_exp_antenna: per (32 tau, run of t0 rows) a warp composes the chunks'
+//     maps down to the chunks that hold its last row's i0 and j, steps both
+//     cursors to those atoms, and sweeps its rows (fmap_sweep.cuh).
+//
+// Bound by instruction issue: about 45 float-float operations per cell for the
+// sums and 75 for the coefficients.  The chunk maps keep a short run of rows
+// cheap to start (a window's atoms would otherwise be summed again by each run),
+// so that the rows split into enough warps to fill the GPU.
+// ---------------------------------------------------------------------------
+constexpr int kAntWarps = kSweepWarps;
+constexpr int kAntThreads = 32 * kAntWarps;
 
 // Tail factors above this size are taken from FP64 exp as float pairs: the
 // window sum E[i0] - tail E[j] then loses 1 / (1 - tail) of relative accuracy
@@ -184,167 +54,219 @@ k_exp_suffix(const float4* __restrict__ perm, const TauTab* __restrict__ tauc, i
 // further (windows cut well before 3 tau, or starting in a long gap).
 constexpr float kTailExact = 1.0f / 32.0f;
 
-// A, B, C of the cell (t0, tau) from the suffix sums E of its tau, then its
-// coefficients; c2 = -2 log2(e) / tau, inv_tau = 1 / tau.  t_i0 and t_j are
-// the relative times of atoms i0 and j (read only when the window holds
-// atoms, and t_j only when j < n).
-__device__ __forceinline__ Coef exp_cell_coef_t(int32_t t_i0, int32_t t_j, int32_t n,
-                                                int64_t t0, float c2,
-                                                double inv_tau, int32_t i0, int32_t j,
-                                                int64_t t_base, const float2* E) {
-  const int32_t count = j - i0;
-  FF S[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  if (count > 0) {
-    const int64_t t0rel = t0 - t_base;
-    const int64_t np1 = (int64_t)n + 1;
+// (out of line, as slow_decay)
+static __device__ __noinline__ float2 exact_tail(int32_t dj, double inv_s) {
+  const FF v = ff_of(exp(-(double)dj * inv_s));
+  return make_float2(v.h, v.l);
+}
+
+template <bool IRR>
+__device__ __forceinline__ void exp_antenna_unit(
+    const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base, int32_t n,
+    const fmap_grid& g, const float4* __restrict__ ant, const TauTab* __restrict__ tauc,
+    const int64_t* __restrict__ ax, const int32_t* __restrict__ i0tab,
+    const int32_t* __restrict__ jend, const AntGeom& q, const float* __restrict__ agg,
+    Coef* __restrict__ coef, uint32_t* __restrict__ bits, int64_t unit, float2* s_pw, int lane) {
+  const int32_t seg = (int32_t)(unit % q.n_seg);
+  const int64_t ag = unit / q.n_seg;
+  const int32_t grp = (int32_t)(ag % q.n_grp);
+  const int64_t ta = ag / q.n_grp;
+  const int32_t ni = grp * 32 + lane, nn = min(ni, g.n_tau - 1);
+  const int32_t m_lo = seg * q.rows, m_hi = min(g.n_t0, m_lo + q.rows);
+  const TauTab* tt = tauc + nn;
+  sweep_tab_load<2>(s_pw, tt, lane);
+  const float c2 = tt->c2[1];
+  const int64_t tb = n > 0 ? *t_base : 0;
+  const float4* x = ant + ta * n;
+  const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
+  // (each cursor's next atom is loaded one step ahead)
+  auto step = [&](AntE& e, float4& v, int32_t a) {
+    const float4 w = v;
+    v = __ldg(x + max(a - 1, 0));
+    ant_step(e, sweep_decay<2, IRR>(s_pw, __float_as_int(w.w), lane, rel_t, a, tt), w);
+  };
+  const int32_t jt = jend[(int64_t)(m_hi - 1) * g.n_tau + nn];
+  const int32_t it = i0tab[m_hi - 1];
+  AntE Ei = ant_zero(), Ej = ant_zero();
+  int32_t ic, jc;
+  if (q.n_chunks > 0) {
+    // E at the first atoms of the chunks after those holding j and i0 of the
+    // last row (E = 0 at the end of the chunk of the warp's last window end)
+    const int32_t bj = (jt + q.chunk - 1) / q.chunk, bi = (it + q.chunk - 1) / q.chunk;
+    FF E[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    const float* o = agg + ag * q.n_chunks * 256 + lane;
+    constexpr int B = 2;   // chunk maps loaded ahead
+    for (int32_t b0 = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)bj);; b0 -= B) {
+      float w[B][8];
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[u][e] = o[(int64_t)max(b0 - 1 - u, 0) * 256 + 32 * e];
+      bool done = false;
+#pragma unroll
+      for (int u = 0; u < B; ++u) {
+        if (b0 - u == bj) ant_put(Ej, E);
+        if (b0 - u <= bi) {
+          done = true;
+          break;
+        }
+        const FF R{w[u][6], w[u][7]};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) E[c] = ff_fma_sum(FF{w[u][2 * c], w[u][2 * c + 1]}, R, E[c]);
+      }
+      if (done) break;
+    }
+    ant_put(Ei, E);
+    ic = min(n, bi * q.chunk);
+    jc = min(n, bj * q.chunk);
+  } else {
+    // E starts from zero at each lane's window end of the last row
+    jc = jt;
+    ic = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)jt);
+    const int32_t j_all = (int32_t)__reduce_min_sync(0xffffffffu, (unsigned)jt);
+    while (ic > max(it, j_all)) {   // atoms past some lanes' ends
+      --ic;
+      const float4 v = __ldg(x + ic);
+      if (ic < jt)
+        ant_step(Ei, sweep_decay<2, IRR>(s_pw, __float_as_int(v.w), lane, rel_t, ic, tt), v);
+    }
+  }
+  float4 vi = n > 0 ? __ldg(x + max(ic - 1, 0)) : float4{}, vj = n > 0 ? __ldg(x + max(jc - 1, 0)) : float4{};
+  // the window ends and starts of a row are loaded one row ahead
+  int32_t i0 = it, j = jt;
+  for (int32_t m = m_hi - 1; m >= m_lo; --m) {
+    const int64_t cell = (int64_t)m * g.n_tau + nn;
+    int32_t i0n = 0, jn = 0;
+    if (m > m_lo) {
+      i0n = i0tab[m - 1];
+      jn = jend[cell - g.n_tau];
+    }
+    while (ic > i0) step(Ei, vi, --ic);
+    while (jc > j) step(Ej, vj, --jc);
+    ant_norm(Ei);
+    ant_norm(Ej);
     // The prefactor scales A, B, C alike (F changes by its relative error
     // only): FP32 exp2 is accurate enough.  The tail is FP32 exp2 while it is
     // small (~e^{-6} of the window sum for the default 3 tau cut), FP64 exp
     // otherwise.
-    const int64_t d0 = (int64_t)t_i0 - t0rel;
-    const float pre = d0 == 0 ? 1.0f : ex2_approx(c2 * (float)d0);
-    FF tail{0.0f, 0.0f};
-    if (j < n) {
-      const int32_t dj = t_j - t_i0;
-      tail.h = ex2_approx(c2 * (float)dj);
-      if (tail.h > kTailExact) tail = ff_of(exp(-2.0 * (double)dj * inv_tau));
-    }
+    FF S[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    if (j > i0) {
+      const int32_t ti = rel_t[i0];
+      const int64_t d0 = (int64_t)ti - (grid_t0(g, ax, m) - tb);
+      FF ei[3], ej[3];
+      ant_get(Ei, ei);
+      ant_get(Ej, ej);
+      FF tail{0.0f, 0.0f};
+      if (j < n) {
+        const int32_t dj = rel_t[j] - ti;
+        tail.h = ex2_approx(c2 * (float)dj);
+        if (tail.h > kTailExact) {
+          const float2 v = exact_tail(dj, 2.0 * tt->inv_tau);
+          tail = {v.x, v.y};
+        }
+      }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float2 a = E[c * np1 + i0], b = E[c * np1 + j];
-      S[c] = ff_mul_f(ff_sub(FF{a.x, a.y}, ff_mul(FF{b.x, b.y}, tail)), pre);
-    }
-  }
-  return make_coef_ff(S[0], S[1], S[2], count);
-}
-__device__ __forceinline__ Coef exp_cell_coef(const int32_t* __restrict__ rel_t, int32_t n,
-                                              int64_t t0, float c2,
-                                              double inv_tau, int32_t i0, int32_t j,
-                                              int64_t t_base, const float2* E) {
-  const bool any = j > i0;
-  return exp_cell_coef_t(any ? rel_t[i0] : 0, any && j < n ? rel_t[j] : 0, n, t0, c2, inv_tau,
-                         i0, j, t_base, E);
-}
-
-// cells a thread loads ahead in the antenna kernels (fewer for the narrowest
-// scan, whose batch variant runs at the highest occupancy)
-template <int NT>
-constexpr int cells_in_flight() { return NT >= 128 ? 4 : 2; }
-
-// Fused antenna step for data sets that fit shared memory: one block per
-// (tau_n, antenna set) keeps the suffix sums in shared memory and writes the
-// coefficients of every cell (t0_m, tau_n).  Blocks run tau-fastest, so their
-// strided coefficient stores merge in L2.
-template <int NT>
-__device__ __forceinline__ void exp_antenna_body(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base, int32_t n,
-              fmap_grid g, const float4* __restrict__ perm_ant, const TauTab* __restrict__ tauc,
-              const int64_t* __restrict__ ax, const int32_t* __restrict__ i0tab,
-              const int32_t* __restrict__ jend, Coef* __restrict__ coef,
-              uint32_t* __restrict__ bits, const uint3 bid, const dim3 gdim) {
-  extern __shared__ float2 s_E[];
-  __shared__ float sR[2][NT / 32];
-  __shared__ float sS[3][2][NT / 32];
-  const int ni = bid.x, ta = bid.y;
-  const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
-  const TauTab* tt = tauc + ni;
-  antenna_suffix<NT>(perm_ant + (int64_t)ta * perm_entries(n, NT), n, g, tt, s_E, sR, sS);
-  __syncthreads();
-  const int64_t tb = n > 0 ? *t_base : 0;
-  // U cells per thread at a time: their window indices, then the atom times
-  // those select, are all loaded before any is used, so the loads' latencies
-  // overlap.
-  constexpr int U = cells_in_flight<NT>();
-  for (int32_t m0 = threadIdx.x; m0 < g.n_t0; m0 += NT * U) {
-    int32_t i0v[U], jv[U], ti[U], tj[U];
+      for (int c = 0; c < 3; ++c) S[c] = ff_sub(ei[c], ff_mul(ej[c], tail));
+      if (d0 != 0) {
+        const float pre = ex2_approx(c2 * (float)d0);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int32_t m = m0 + u * NT;
-      const bool in = m < g.n_t0;
-      i0v[u] = in ? i0tab[m] : 0;
-      jv[u] = in ? jend[(int64_t)m * g.n_tau + ni] : 0;
+        for (int c = 0; c < 3; ++c) S[c] = ff_mul_f(S[c], pre);
+      }
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const bool any = jv[u] > i0v[u];
-      ti[u] = any ? rel_t[i0v[u]] : 0;
-      tj[u] = any && jv[u] < n ? rel_t[jv[u]] : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int32_t m = m0 + u * NT;
-      if (m < g.n_t0)
-        store_coef(coef, bits, (int64_t)ta * cells + (int64_t)m * g.n_tau + ni,
-                   exp_cell_coef_t(ti[u], tj[u], n, grid_t0(g, ax, m), tt->c2[1], tt->inv_tau,
-                                   i0v[u], jv[u], tb, s_E));
-    }
+    const Coef cf = make_coef_ff(S[0], S[1], S[2], j - i0);
+    if (ni < g.n_tau) store_coef(coef, bits, ta * cells + cell, cf);
+    i0 = i0n;
+    j = jn;
   }
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(kAntThreads, 3)
 k_exp_antenna(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base, int32_t n,
-              fmap_grid g, const float4* __restrict__ perm_ant, const TauTab* __restrict__ tauc,
+              const fmap_grid g, const float4* __restrict__ ant, const TauTab* __restrict__ tauc,
               const int64_t* __restrict__ ax, const int32_t* __restrict__ i0tab,
-              const int32_t* __restrict__ jend, Coef* __restrict__ coef,
-              uint32_t* __restrict__ bits) {
-  exp_antenna_body<NT>(rel_t, t_base, n, g, perm_ant, tauc, ax, i0tab, jend, coef, bits, blockIdx,
-                       gridDim);
+              const int32_t* __restrict__ jend, const AntGeom q, const float* __restrict__ agg,
+              Coef* __restrict__ coef, uint32_t* __restrict__ bits,
+              const int32_t* __restrict__ irr, int64_t units) {
+  __shared__ float2 s_pw[kAntWarps][kSweepTab];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t unit = (int64_t)blockIdx.x * kAntWarps + warp;
+  if (unit >= units) return;
+  if (*irr)
+    exp_antenna_unit<true>(rel_t, t_base, n, g, ant, tauc, ax, i0tab, jend, q, agg, coef, bits,
+                           unit, s_pw[warp], lane);
+  else
+    exp_antenna_unit<false>(rel_t, t_base, n, g, ant, tauc, ax, i0tab, jend, q, agg, coef, bits,
+                            unit, s_pw[warp], lane);
 }
 
-// Chunk-major copies of one instance's atoms for the scans: entry
-// q lanes + t of a set holds atom i = t C + q (zeros past the last atom; lanes
-// = the plan's scan width, C = scan_chunk(n, lanes)):
-// sets 0..n_ant-1 the antenna rows with the gap to the next atom, sets
-// n_ant.. the data rows of each template (when perm_x is given); then the
-// per-tau constants (n_tau more entries).
+// Chunks of 16 atoms for short data sets (a warp's start is then a handful
+// of steps), 128 for long ones (fewer maps to compose), larger ones where the
+// maps have no room (agg_room bytes), none where the rows make a single run per
+// 32 tau anyway; rows
+// per warp so that about 16 warps per SM run at once, at least 4 (the start
+// costs about as much as eight); in a batch, whose instances fill the GPU
+// together, 64.
+AntGeom ant_geom(const fmap_grid& g, int32_t n_sft, int64_t n_ant, bool batch, int64_t agg_room) {
+  AntGeom q{};
+  q.n_grp = std::max(1, (g.n_tau + 31) / 32);
+  const int64_t warps = q.n_grp * std::max<int64_t>(n_ant, 1);   // per run of rows
+  const int64_t want = ((int64_t)kSms * 16 + warps - 1) / warps;
+  q.rows = batch ? 64 : (int32_t)std::max<int64_t>(4, (g.n_t0 + want - 1) / want);
+  q.n_seg = std::max(1, (g.n_t0 + q.rows - 1) / q.rows);
+  q.chunk = n_sft <= 1024 ? 16 : n_sft <= 4096 ? 32 : 128;
+  q.n_chunks = (n_sft + q.chunk - 1) / q.chunk;
+  if (q.n_seg == 1 && q.n_chunks > 0 && g.n_t0 > 64) q.n_chunks = 0;
+  while (1024 * warps * q.n_chunks > agg_room && q.chunk < 1024) {
+    q.chunk *= 2;
+    q.n_chunks = (n_sft + q.chunk - 1) / q.chunk;
+  }
+  if (1024 * warps * q.n_chunks > agg_room) q.n_chunks = 0;
+  return q;
+}
+
+// Copies of one instance's atoms for the sweeps, one 16-byte entry per atom:
+// sets 0..n_ant-1 the antenna rows with the code of the gap to the next atom
+// (gap_code), sets n_ant.. the data rows of each template (recurrence plans);
+// before them the per-tau constants (two entries per tau).
 __device__ __forceinline__ void exp_perm_body(const int32_t* __restrict__ rel_t, int32_t n,
-                                              int32_t lanes,
                                               const float* __restrict__ antenna, int32_t n_ant,
                                               const float* __restrict__ fafb, int32_t n_x,
                                               float4* __restrict__ perm_ant,
                                               float4* __restrict__ perm_x,
-                                              int32_t* __restrict__ perm_gap, const fmap_grid& g,
+                                              int32_t* __restrict__ irr, const fmap_grid& g,
                                               const int64_t* __restrict__ ax,
                                               TauTab* __restrict__ tauc, int64_t e_begin,
                                               int64_t e_end, int64_t e_step) {
-  const int64_t P = perm_entries(n, lanes), C = scan_chunk(n, lanes);
-  const int64_t n_copy = P * (int64_t)(n_ant + n_x);
-  for (int64_t e = e_begin; e < e_end; e += e_step) {
-    if (e >= n_copy) {   // entries past the copies: the per-tau constants
-      tau_tab_fill(g, grid_tau(g, ax, e - n_copy), tauc + (e - n_copy));
+  const int64_t n_tau2 = 2 * (int64_t)g.n_tau;
+  for (int64_t e0 = e_begin; e0 < e_end; e0 += e_step) {
+    if (e0 < n_tau2) {   // the longest entries first
+      tau_tab_fill(g, grid_tau(g, ax, e0 >> 1), (int)(e0 & 1), tauc + (e0 >> 1));
       continue;
     }
-    const int64_t set = e / P, r = e - set * P;
-    const int64_t q = r / lanes, t = r - q * lanes;
-    const int64_t i = t * C + q;
-    const bool in = i < n;
+    const int64_t e = e0 - n_tau2;
+    const int64_t set = e / n, i = e - set * n;
     if (set < n_ant) {
       const float* a = antenna + set * 3 * (int64_t)n;
-      float4 v = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-      if (in) {
-        const int32_t gap = i + 1 < n ? rel_t[i + 1] - rel_t[i] : -1;
-        v = make_float4(a[i], a[n + i], a[2 * (int64_t)n + i], __int_as_float(gap));
-      }
-      perm_ant[e] = v;
-      if (set == 0 && perm_gap) perm_gap[r] = __float_as_int(v.w);
+      const int32_t t = rel_t[i];
+      const int32_t code = i + 1 < n ? gap_code(rel_t[i + 1] - t, (int32_t)g.t_sft) : -1;
+      perm_ant[e] = make_float4(a[i], a[n + i], a[2 * (int64_t)n + i], __int_as_float(code));
+      if (set == 0 && code == 0) *irr = 1;   // (cleared by the input checks)
     } else {
       const int64_t tq = set - n_ant;
       const float* x = fafb + tq * 4 * (int64_t)n;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (in) v = make_float4(x[i], x[n + i], x[2 * (int64_t)n + i], x[3 * (int64_t)n + i]);
-      perm_x[tq * P + r] = v;
+      perm_x[tq * n + i] = make_float4(x[i], x[n + i], x[2 * (int64_t)n + i], x[3 * (int64_t)n + i]);
     }
   }
 }
 
-__global__ void k_exp_perm(const int32_t* __restrict__ rel_t, int32_t n, int32_t lanes,
+__global__ void k_exp_perm(const int32_t* __restrict__ rel_t, int32_t n,
                            const float* __restrict__ antenna, int32_t n_ant,
                            const float* __restrict__ fafb, int32_t n_x,
                            float4* __restrict__ perm_ant, float4* __restrict__ perm_x,
-                           int32_t* __restrict__ perm_gap, fmap_grid g,
+                           int32_t* __restrict__ irr, const fmap_grid g,
                            const int64_t* __restrict__ ax, TauTab* __restrict__ tauc) {
-  const int64_t total = exp_copy_entries(n, lanes, n_ant, n_x, g.n_tau);
-  exp_perm_body(rel_t, n, lanes, antenna, n_ant, fafb, n_x, perm_ant, perm_x, perm_gap, g, ax, tauc,
+  const int64_t total = exp_copy_entries(n, n_ant, n_x, g.n_tau);
+  exp_perm_body(rel_t, n, antenna, n_ant, fafb, n_x, perm_ant, perm_x, irr, g, ax, tauc,
                 (int64_t)blockIdx.x * blockDim.x + threadIdx.x, total,
                 (int64_t)gridDim.x * blockDim.x);
 }
@@ -353,79 +275,28 @@ cudaError_t launch_exp_perm(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s)
   if ((int64_t)p->grid.n_t0 * p->grid.n_tau == 0) return cudaSuccess;
   const int32_t n_ant = a->shared_antenna ? 1 : p->n_templates;
   const int32_t n_x = p->ws.perm_x ? p->n_templates : 0;
-  const int64_t total = exp_copy_entries(p->n_sft, p->lanes, n_ant, n_x, p->grid.n_tau);
+  const int64_t total = exp_copy_entries(p->n_sft, n_ant, n_x, p->grid.n_tau);
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)p->n_sm * 16);
-  k_exp_perm<<<blocks, 256, 0, s>>>(p->ws.rel_t, p->n_sft, p->lanes, a->antenna, n_ant, a->fafb, n_x,
-                                    p->ws.perm_ant, p->ws.perm_x, p->ws.perm_gap, p->grid,
+  k_exp_perm<<<blocks, 256, 0, s>>>(p->ws.rel_t, p->n_sft, a->antenna, n_ant, a->fafb, n_x,
+                                    p->ws.perm_ant, p->ws.perm_x, p->ws.irr, p->grid,
                                     plan_axes(p), p->ws.tauc);
   p->launches += 1;
   return cudaGetLastError();
-}
-
-constexpr int kAntennaSmemMaxSft = 9000;   // 3 x (n + 1) float pairs <= 216 KB
-
-// Per-cell coefficients of the cells of one tau chunk (global suffix sums).
-__global__ void k_exp_coef(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base,
-                           int32_t n, fmap_grid g, int32_t n_lo, int32_t n_chunk,
-                           const int32_t* __restrict__ i0tab, const int32_t* __restrict__ jend,
-                           const float2* __restrict__ esuf, const TauTab* __restrict__ tauc,
-                           const int64_t* __restrict__ ax, Coef* __restrict__ coef,
-                           uint32_t* __restrict__ bits, int64_t e_base) {
-  const int64_t total = (int64_t)g.n_t0 * n_chunk;
-  const int64_t np1 = (int64_t)n + 1;
-  const int64_t tb = n > 0 ? *t_base : 0;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < total;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t m = c / n_chunk;
-    const int32_t nl = (int32_t)(c - m * n_chunk);
-    const int64_t nn = n_lo + nl;
-    const int64_t cell = m * g.n_tau + nn;
-    store_coef(coef, bits, e_base + cell,
-               exp_cell_coef(rel_t, n, grid_t0(g, ax, m), tauc[nn].c2[1], tauc[nn].inv_tau,
-                             i0tab[m], jend[cell], tb, esuf + (int64_t)nl * 3 * np1));
-  }
 }
 
 cudaError_t launch_exp_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
   const fmap_grid& g = p->grid;
   if ((int64_t)g.n_t0 * g.n_tau == 0) return cudaSuccess;
   const int n_ant = a->shared_antenna ? 1 : p->n_templates;
-  const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
-  if (p->n_sft <= kAntennaSmemMaxSft) {
-    const size_t smem = exp_antenna_smem(p->n_sft);
-    auto run = [&](auto kern, int nt) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      kern<<<dim3((unsigned)g.n_tau, (unsigned)n_ant), nt, smem, s>>>(
-          p->ws.rel_t, p->ws.t_base, p->n_sft, g, p->ws.perm_ant, p->ws.tauc, plan_axes(p),
-          p->ws.i0, p->ws.jend, p->ws.coef, p->ws.flag_bits);
-    };
-    switch (p->lanes) {
-      case 64: run(k_exp_antenna<64>, 64); break;
-      case 128: run(k_exp_antenna<128>, 128); break;
-      default: run(k_exp_antenna<256>, 256); break;
-    }
-    p->launches += 1;
-    return cudaGetLastError();
-  }
-  for (int ta = 0; ta < n_ant; ++ta) {
-    const float4* perm = p->ws.perm_ant + (int64_t)ta * perm_entries(p->n_sft, p->lanes);
-    for (int32_t lo = 0; lo < g.n_tau; lo += p->tau_chunk) {
-      const int32_t len = std::min<int32_t>(p->tau_chunk, g.n_tau - lo);
-      if (p->n_sft > 0) {
-        k_exp_suffix<<<len, kSufThreads, 0, s>>>(perm, p->ws.tauc, p->n_sft, g, lo, p->ws.esuf);
-        p->launches += 1;
-      }
-      const int64_t total = (int64_t)g.n_t0 * len;
-      const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)p->n_sm * 16);
-      k_exp_coef<<<blocks, 256, 0, s>>>(p->ws.rel_t, p->ws.t_base, p->n_sft, g, lo, len, p->ws.i0,
-                                        p->ws.jend, p->ws.esuf, p->ws.tauc, plan_axes(p),
-                                        p->ws.coef, p->ws.flag_bits, ta * cells);
-      p->launches += 1;
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
-  }
-  return cudaSuccess;
+  if (n_ant == 0) return cudaSuccess;
+  const AntGeom& q = p->ant[a->shared_antenna ? 1 : 0];
+  const int64_t ag = (int64_t)q.n_grp * n_ant;
+  const int64_t units = ag * q.n_seg;
+  k_exp_antenna<<<(unsigned)((units + kAntWarps - 1) / kAntWarps), kAntThreads, 0, s>>>(
+      p->ws.rel_t, p->ws.t_base, p->n_sft, g, p->ws.perm_ant, p->ws.tauc, plan_axes(p), p->ws.i0,
+      p->ws.jend, q, p->ws.agg, p->ws.coef, p->ws.flag_bits, p->ws.irr, units);
+  p->launches += 1;
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -568,30 +439,35 @@ cudaError_t launch_exp_plain(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, c
 __global__ void __launch_bounds__(256) kb_exp_perm(const BItem* __restrict__ items, BUnits u) {
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
     const int32_t n_x = it.perm_x ? it.T : 0;
-    const int64_t total = exp_copy_entries(it.n_sft, it.lanes, it.n_ant, n_x, it.g.n_tau);
+    const int64_t total = exp_copy_entries(it.n_sft, it.n_ant, n_x, it.g.n_tau);
     const int64_t e0 = k * kPermPerUnit;
-    exp_perm_body(it.rel_t, it.n_sft, it.lanes, it.antenna, it.n_ant, it.fafb, n_x, it.perm_ant, it.perm_x,
-                  it.perm_gap, it.g, it.ax, it.tauc, e0 + threadIdx.x, min(total, e0 + kPermPerUnit), 256);
+    exp_perm_body(it.rel_t, it.n_sft, it.antenna, it.n_ant, it.fafb, n_x, it.perm_ant, it.perm_x,
+                  it.irr, it.g, it.ax, it.tauc, e0 + threadIdx.x, min(total, e0 + kPermPerUnit), 256);
   });
 }
-// (the register budget of 3 blocks of 256 threads per SM, for any width)
-template <int NT>
-__global__ void __launch_bounds__(NT, 768 / NT) kb_exp_ant(const BItem* __restrict__ items,
-                                                        BUnits u) {
+__global__ void __launch_bounds__(kAntThreads, 2) kb_exp_ant(const BItem* __restrict__ items,
+                                                             BUnits u) {
+  __shared__ float2 s_pw[kAntWarps][kSweepTab];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
-    exp_antenna_body<NT>(it.rel_t, it.t_base, it.n_sft, it.g, it.perm_ant, it.tauc, it.ax, it.i0,
-                         it.jend, it.coef, it.flag_bits,
-                         make_uint3((unsigned)(k % it.g.n_tau), (unsigned)(k / it.g.n_tau), 0),
-                         dim3((unsigned)it.g.n_tau, (unsigned)it.n_ant));
+    const int64_t unit = k * kAntWarps + warp;
+    if (unit >= (int64_t)it.ag.n_grp * it.n_ant * it.ag.n_seg) return;
+    if (*it.irr)
+      exp_antenna_unit<true>(it.rel_t, it.t_base, it.n_sft, it.g, it.perm_ant, it.tauc, it.ax,
+                             it.i0, it.jend, it.ag, it.agg, it.coef, it.flag_bits, unit,
+                             s_pw[warp], lane);
+    else
+      exp_antenna_unit<false>(it.rel_t, it.t_base, it.n_sft, it.g, it.perm_ant, it.tauc, it.ax,
+                              it.i0, it.jend, it.ag, it.agg, it.coef, it.flag_bits, unit,
+                              s_pw[warp], lane);
   });
 }
-const void* batch_kernel_exp(int phase, int lanes) {
-  if (phase == BP_EXP_PERM) return (const void*)kb_exp_perm;
-  if (phase != BP_EXP_ANT) return nullptr;
-  return lanes == 64 ? (const void*)kb_exp_ant<64>
-                     : lanes == 128 ? (const void*)kb_exp_ant<128> : (const void*)kb_exp_ant<256>;
+const void* batch_kernel_exp(int phase) {
+  switch (phase) {
+    case BP_EXP_PERM: return (const void*)kb_exp_perm;
+    case BP_EXP_ANT: return (const void*)kb_exp_ant;
+  }
+  return nullptr;
 }
-size_t exp_antenna_smem(int32_t n_sft) { return sizeof(float2) * 3 * ((size_t)n_sft + 1); }
-bool exp_antenna_fits(int32_t n_sft) { return n_sft <= kAntennaSmemMaxSft; }
 
 }  // namespace fmap

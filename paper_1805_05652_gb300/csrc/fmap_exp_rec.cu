@@ -1,61 +1,52 @@
 // Exponential window by the decayed suffix recurrence (plan flag
-// FMAP_PLAN_EXP_RECURRENCE).
+// FMAP_PLAN_EXP_RECURRENCE): the data sums, 2F and its reductions.
 //
-// The exponential weight factorises in t0: for the atoms [i0, j) of a window,
-//   sum_a e^{-(t_a - t0)/tau} x_a = e^{-(t_{i0} - t0)/tau} (E[i0] - e^{-(t_j - t_{i0})/tau} E[j]),
-//   E[i] = x_i + e^{-(t_{i+1} - t_i)/tau} E[i+1],  E[N] = 0,
-// an exact rearrangement of the window sums of Eq. (winexp).  One recurrence
-// per (tau, data column) replaces the per-cell sums: O(N_tau N_SFT) work per
-// column instead of O(sum of window lengths).  The recurrence runs as a
-// parallel backward scan of the affine maps E -> x + rho E.  What spans the
-// data set -- the decay products and the composition of the chunks' maps,
-// whose errors would otherwise accumulate over up to N_SFT steps -- runs in
-// compensated FP32 (float pairs, ~2^-44 relative); the chunk-local sums (at
-// most C = 21..35 terms at 5000..9000 SFTs) run in plain FP32, and E is formed
-// in FP32 as E = L + Q E[chunk end].  A chunk-local error is at most ~C ulp of
-// the chunk's own partial sums, small against E where the window is long
-// (slow decay) and limited to the few undecayed terms where it is short:
-// emulated on the 5000-SFT workload (every tau class, the cells outside the
-// fix-up), the worst relative 2F error is 1.7e-6 against 1.2e-6 for
-// compensated chunk sums.
+// fmap_sweep.cuh states the rearrangement and the mapping: a warp takes 32
+// consecutive tau, a run of t0 rows from the last to the first, and G templates;
+// each lane carries E at i0 and at j of its tau and advances both atom by atom.
 //
-// One block per (tau_n, group of templates); each thread owns a chunk of
-// atoms (odd length C, read from the chunk-major copy).  Per template of the
-// group:
-//   1. the chunk-local suffix sums L[i] (E with E[chunk end] = 0) of the 4
-//      data columns, one FP32 FMA per atom and column (at most C terms; see
-//      below); on the first template also the products Q[i] of the decays
-//      from atom i to the chunk's end, in float-float (the same for every
-//      template, kept in shared memory) and the chunk's product R;
-//   2. the carries E[chunk end] by a suffix composition of the chunks'
-//      (L[s0], R) maps, in float-float, within the warp and over the warps;
-//   3. E[i] = L[i] + Q[i] E[chunk end] in place (one FMA per column, where
-//      recomputing the chunk from its carry would repeat step 1);
-//   4. the column of cells (t0_m, tau_n) for every m from E, with the
-//      window records (i0, j, prefactor, tail factor; and the coefficients
-//      when the antenna is shared) computed on the block's first template and
-//      re-read from a tau-major array on the others (the groups of one tau
-//      each write the same values there).
-// Blocks run tau-fastest, so the blocks writing neighbouring tau of the same
-// map rows run together and their stores merge in L2.
+// Arithmetic.  E at i0 is kept as L + Q K: K the value at the atom of the last
+// renormalisation in float-float, Q the (float-float) product of the decays
+// since, L the FP32 sum of the atoms since (decayed by float pairs, so that its
+// rounding error is a few ulp of its own partial sums and the decays add none);
+// every rec_run(N) atoms K <- L + Q K in float-float, so nothing accumulates over
+// the data set.  E at j enters through
+// the tail factor e^{-(t_j - t_{i0})/tau} <= e^{-3}..e^{-2} for the 3 tau cut:
+// there a plain FP32 recurrence with float-pair decays (no systematic decay
+// error; its random rounding error is scaled by the tail) is enough.  Windows
+// cut before 3 tau, whose tail is near 1, carry E at j like E at i0.
+//
+// A warp starts from zero at its last row's window ends and sums those windows
+// first (long runs of rows, many templates), or, where the rows must be split
+// into short runs to make enough warps, from the decayed sums of chunks of
+// atoms formed ahead by k_sweep_agg.
+//
+// Bound by instruction issue.  One block per tau with E in shared memory and a
+// scan over the atoms per template (two block barriers, four passes over shared
+// memory) took 73.8 ms for 1024 templates x 5000 SFTs over 2000 x 2000 cells,
+// latency-bound at 44 % issue.
 #include <math.h>
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "fmap_batch.cuh"
-#include "fmap_device.cuh"
+#include "fmap_sweep.cuh"
 
 namespace fmap {
 
-constexpr int kRecChunk = 8;        // SFTs of data prefetched per serial run of the scan
-constexpr int kRecMaxGroups = 32;   // template groups per tau (blocks per tau)
-constexpr int kRecMaxSft = 9000;    // one template's suffix sums in shared memory (180 KB)
-
-// Shared memory of the recurrence: E of one template (4 columns) and Q.
-__host__ __device__ __forceinline__ size_t rec_smem_base(int32_t n_sft) {
-  return sizeof(float) * 5 * ((size_t)n_sft + 1) + 16;
+constexpr int kRecMaxSft = 9000;    // the recurrence's declared range
+// Atoms between renormalisations: one in 256 of the data set, 3 to 21.  The
+// FP32 sums of a run are the largest rounding error of short windows (measured
+// against 64 bits, 400-630 SFTs: 1.2e-7 of the map's norm with runs of 3, 3e-7
+// with 24), while a renormalisation costs 26 instructions per template.
+__host__ __device__ __forceinline__ int32_t rec_run(int32_t n) {
+  return min(21, max(3, ((n + 255) / 256) | 1));
 }
+constexpr int kRecThreads = 32 * kRecWarps;
+constexpr int kAggThreads = 32 * kSweepWarps;
+constexpr int kRecTileRows = 32;    // t0 rows of a reduction tile (32 tau wide), at most
 
 __device__ __forceinline__ float rec_ex2(float x) {
   float y;
@@ -63,367 +54,696 @@ __device__ __forceinline__ float rec_ex2(float x) {
   return y;
 }
 
-// NT = the plan's scan width: threads of the block and width of the
-// chunk-major copy; U = cells a thread loads ahead.
-template <int NT, int U>
-__device__ __forceinline__ void exp_rec_body(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base, int32_t n,
-          fmap_grid g, const int32_t* __restrict__ i0tab, const int32_t* __restrict__ jend,
-          const Coef* __restrict__ coef, int32_t shared_antenna, const float4* __restrict__ perm_x,
-          const int32_t* __restrict__ perm_gap, float4* __restrict__ recs,
-          float* __restrict__ rdec, const TauTab* __restrict__ tauc,
-          const int64_t* __restrict__ ax, int32_t n_templates, int32_t n_groups,
-          float* __restrict__ map, Partial* __restrict__ parts, int64_t stride,
-    const uint3 bid, const dim3 gdim) {
-  constexpr int NW = NT / 32;
-  extern __shared__ __align__(16) float s_dyn[];
-  const int64_t np1 = (int64_t)n + 1;
-  // [n + 1] L, then E, of one template: the 4 data columns of an atom as one
-  // float4 (one 16-byte access where four 4-byte ones would be)
-  float4* s_e = reinterpret_cast<float4*>(s_dyn);
-  float* s_q = s_dyn + 4 * np1;    // [n] decay product from atom i to its chunk's end
-  __shared__ float sR[2][NW];      // each warp's product of its chunks' R
-  __shared__ float sS[4][2][NW];   // each warp's composed S (per template)
-  __shared__ float sK[4][2][NW];   // E at each warp's end (per template)
-  __shared__ Partial scratch[2 * NW];   // the block reductions, alternately
-  const int ni = bid.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const TauTab* tt = tauc + ni;
-  // Decay after atom i: gaps of k whole SFTs from the tau's table of
-  // float-float powers of the one-SFT decay, other gaps by FP64 exp; the gaps
-  // come from the chunk-major copy with the data.
-  const float inv_tsft = 1.0f / (float)g.t_sft;
-  const double inv_tau = tt->inv_tau;
-  const int C = (int)scan_chunk(n, NT);
-  const int s0 = min(n, tid * C), e0 = min(n, s0 + C);
-  const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
-  const float c2 = tt->c2[0];
-  const bool short_cut = exp_cut8_of(g) < 24;   // window cut before 3 tau
-  const int64_t tb = n > 0 ? *t_base : 0;
-  // 0 after the last atom
-  int32_t gq[kRecChunk];
-  auto decay = [&](int32_t gap) -> FF {
-    if (gap > 0) return gap_decay(gap, g.t_sft, inv_tsft, tt->pw[0], inv_tau);
-    return gap < 0 ? FF{0.0f, 0.0f} : FF{1.0f, 0.0f};
-  };
-  const int b_last = s0 + ((e0 - s0 - 1) / kRecChunk) * kRecChunk;   // last run's start
-  // window records of tau_n, and coefficients (shared antenna); the array is
-  // absent (null) in single-template plans
-  float4* rec_a = recs ? recs + (int64_t)ni * g.n_t0 : nullptr;
-  float4* rec_c = recs ? recs + cells + (int64_t)ni * g.n_t0 : nullptr;
-  // FP32 decays of tau_n in the chunk-major order (absent: computed from the
-  // gaps every template)
-  float* rd = rdec ? rdec + (int64_t)ni * perm_entries(n, NT) : nullptr;
-  const int32_t t_lo = (int32_t)((int64_t)bid.y * n_templates / n_groups);
-  const int32_t t_hi = (int32_t)((int64_t)(bid.y + 1) * n_templates / n_groups);
-  FF R{1.0f, 0.0f};   // the chunk's product of decays (from the first template on)
-  for (int32_t tq = t_lo; tq < t_hi; ++tq) {
-    const bool first = tq == t_lo;
-    // (the previous template's cells are done with s_e: its block reduction
-    // passed a barrier after every warp's cells)
-    const float4* x = perm_x + (int64_t)tq * perm_entries(n, NT);   // chunk-major data rows
-    // 1. chunk-local suffix sums L[i] in plain FP32 (and on the first
-    // template the decay products Q[i] in float-float); the data of each run
-    // of kRecChunk SFTs is loaded before its serial chain
-    float L[4] = {0.f, 0.f, 0.f, 0.f};
-    float Qh = 1.0f, Qc = 0.0f;
-    float xv[kRecChunk][4];
-    const bool cached = rd && !first;   // decays from the first template's pass
-    for (int b0 = b_last; e0 > s0 && b0 >= s0; b0 -= kRecChunk) {
+// One atom of G templates: (re, im) pairs of Fa and Fb.
+template <int G>
+struct Atom {
+  ulonglong2 x[G];
+  // xs: the templates' strides (the last group's missing templates repeat its
+  // last one)
+  __device__ __forceinline__ void load(const float4* __restrict__ xp, const uint2& xs, int32_t a) {
+    const uint32_t i = (uint32_t)max(a, 0);
 #pragma unroll
-      for (int q = 0; q < kRecChunk; ++q) {
-        const int i = b0 + q;
-        const int64_t o = (int64_t)(i - s0) * NT + tid;
-        const float4 v = (i < e0) ? __ldg(x + o) : make_float4(0.f, 0.f, 0.f, 0.f);
-        // gq holds the gap, or the cached decay's bits (written by this same
-        // thread: a plain load)
-        gq[q] = (i < e0) ? (cached ? __float_as_int(rd[o]) : __ldg(perm_gap + o)) : 0;
-        xv[q][0] = v.x;
-        xv[q][1] = v.y;
-        xv[q][2] = v.z;
-        xv[q][3] = v.w;
+    for (int g = 0; g < G; ++g)
+      x[g] = __ldg(reinterpret_cast<const ulonglong2*>(xp) + (i + min((uint32_t)g, xs.y) * xs.x));
+  }
+};
+
+// E = L + Q K of G templates (re/im pairs of Fa and Fb as f32x2).
+template <int G>
+struct Cursor {
+  uint64_t L[G][2], Kh[G][2], Kl[G][2];
+  float Qh, Qc;
+  int32_t run;
+  __device__ __forceinline__ void reset() {
+#pragma unroll
+    for (int g = 0; g < G; ++g) L[g][0] = L[g][1] = 0ull;
+    Qh = 1.0f;
+    Qc = 0.0f;
+    run = 0;
+  }
+  __device__ __forceinline__ void zero() {
+    reset();
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) Kh[g][c] = Kl[g][c] = 0ull;
+  }
+  // K <- L + Q K, L <- 0, Q <- 1
+  __device__ __forceinline__ void renorm() {
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const FF2 k = ff2_fma_sum(L[g][c], FF{Qh, Qc}, FF2{Kh[g][c], Kl[g][c]});
+        Kh[g][c] = k.h;
+        Kl[g][c] = k.l;
       }
+    reset();
+  }
+  // one atom earlier, r its decay
+  __device__ __forceinline__ void step(FF r, const Atom<G>& a) {
+    const uint64_t rh = pk2(r.h, r.h), rl = pk2(r.l, r.l);
 #pragma unroll
-      for (int q = kRecChunk - 1; q >= 0; --q) {
-        // (only the run at the chunk's end is partial: the same for the
-        // warp's lanes but the last thread's)
-        if (b0 + q >= e0) continue;
-        float rh;
-        if (cached) {
-          rh = __int_as_float(gq[q]);
-        } else {
-          const FF r = decay(gq[q]);
-          rh = r.h;
-          if (first) {
-            ch_mul(r, Qh, Qc);
-            s_q[b0 + q] = Qh + Qc;
-            if (rd) rd[(int64_t)(b0 + q - s0) * NT + tid] = r.h;
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) L[c] = fmaf(rh, L[c], xv[q][c]);
-        s_e[b0 + q] = make_float4(L[0], L[1], L[2], L[3]);
-      }
-      if (first) ch_norm(Qh, Qc);
+    for (int g = 0; g < G; ++g) {
+      L[g][0] = fma2(rh, L[g][0], fma2(rl, L[g][0], a.x[g].x));
+      L[g][1] = fma2(rh, L[g][1], fma2(rl, L[g][1], a.x[g].y));
     }
-    if (first) R = {Qh, Qc};
-    // 2. carries: suffix composition of the chunks' maps E[s0] = S + R E[e0],
-    // within the warp (Rw: the product over lanes lane..31), then over the
-    // warps (warp 0, lane v = warp v)
-    FF S[4] = {{L[0], 0.f}, {L[1], 0.f}, {L[2], 0.f}, {L[3], 0.f}};
-    FF Rw = R;
+    ch_mul(r, Qh, Qc);
+    ++run;
+  }
+  // E as float pairs / in FP32
+  __device__ __forceinline__ void set(int g, int c, const FF2& v) {
+    Kh[g][c] = v.h;
+    Kl[g][c] = v.l;
+  }
+  __device__ __forceinline__ uint64_t scale() const { return pk2(Qh + Qc, Qh + Qc); }
+  __device__ __forceinline__ uint64_t get(int g, int c, uint64_t q) const {
+    return fma2(q, Kh[g][c], L[g][c]);
+  }
+};
+// E of G templates by the plain recurrence with float-pair decays.
+template <int G>
+struct PlainCursor {
+  uint64_t E[G][2];
+  __device__ __forceinline__ void zero() {
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const FF Ro = ff_shfl_down(Rw, 1 << k);
+    for (int g = 0; g < G; ++g) E[g][0] = E[g][1] = 0ull;
+  }
+  __device__ __forceinline__ void step(FF r, const Atom<G>& a) {
+    const uint64_t rh = pk2(r.h, r.h), rl = pk2(r.l, r.l);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const FF So = ff_shfl_down(S[c], 1 << k);
-        if (lane + (1 << k) < 32) S[c] = ff_fma_sum(S[c], Rw, So);
-      }
-      if (lane + (1 << k) < 32) Rw = ff_mul(Rw, Ro);
+    for (int g = 0; g < G; ++g) {
+      E[g][0] = fma2(rh, E[g][0], fma2(rl, E[g][0], a.x[g].x));
+      E[g][1] = fma2(rh, E[g][1], fma2(rl, E[g][1], a.x[g].y));
     }
-    FF hR = ff_shfl_down(Rw, 1), hS[4];
-    if (lane == 31) hR = {1.0f, 0.0f};
+  }
+  __device__ __forceinline__ void set(int g, int c, const FF2& v) { E[g][c] = v.h; }
+  __device__ __forceinline__ uint64_t scale() const { return 0ull; }
+  __device__ __forceinline__ uint64_t get(int g, int c, uint64_t) const { return E[g][c]; }
+};
+
+struct RecArgs {
+  const int32_t* rel_t;
+  const int64_t* t_base;
+  const int32_t* irr;   // nonzero: some gap has code 0
+  int32_t n, T;
+  fmap_grid g;
+  RecGeom q;
+  const int32_t* i0tab;
+  const int32_t* jend;
+  const Coef* coef;
+  const float4* x;      // [T][n]
+  const TauTab* tauc;
+  const int64_t* ax;
+  float* agg;           // chunk maps: S [T][n_grp][n_chunks][8][32], then R [n_grp][n_chunks][2][32]
+  float* map;
+  Partial* parts;
+  int64_t stride;
+};
+__device__ __forceinline__ float* rec_agg_r(const RecArgs& A) {
+  return A.agg + (int64_t)A.T * A.q.n_grp * A.q.n_chunks * 256;
+}
+
+__device__ __forceinline__ uint32_t gap_inverse(int32_t t_sft) {
+  return (uint32_t)(((1ull << 31) + (uint32_t)t_sft - 1) / (uint32_t)t_sft);
+}
+// Relative time of atom a; one SFT past the last for a = n (E is zero there).
+__device__ __forceinline__ int32_t atom_time(const RecArgs& A, int32_t a) {
+  return a < A.n ? __ldg(A.rel_t + a) : __ldg(A.rel_t + A.n - 1) + (int32_t)A.g.t_sft;
+}
+
+// Chunk maps of one (template group, 32 tau, chunk): E[first] = S + R E[next].
+template <int G, bool IRR>
+__device__ __forceinline__ void rec_agg_unit(const RecArgs& A, int64_t unit, float2* s_pw,
+                                             int lane) {
+  const RecGeom& q = A.q;
+  const int32_t tg0 = (int32_t)(unit % q.n_tgrp) * G;
+  const int64_t u1 = unit / q.n_tgrp;
+  const int32_t ch = (int32_t)(u1 % q.n_chunks);
+  const int32_t grp = (int32_t)(u1 / q.n_chunks);
+  const TauTab* tt = A.tauc + min(grp * 32 + lane, A.g.n_tau - 1);
+  sweep_tab_load<1>(s_pw, tt, lane);
+  const int32_t n_t = min(G, A.T - tg0);
+  const float4* x = A.x + (int64_t)tg0 * A.n;
+  const uint2 xs = make_uint2((uint32_t)A.n, (uint32_t)(n_t - 1));
+  const int32_t lo = ch * q.chunk, hi = min(A.n, lo + q.chunk);
+  const int32_t run = rec_run(A.n);
+  Cursor<G> E;
+  E.zero();
+  FF R{1.0f, 0.0f};
+  const int32_t t_sft = (int32_t)A.g.t_sft;
+  const uint32_t inv = gap_inverse(t_sft);
+  int32_t tn = atom_time(A, hi);
+  constexpr int B = G == 4 ? 2 : 4;   // atoms loaded ahead of the serial chain
+  for (int32_t a1 = hi; a1 > lo; a1 -= B) {
+    Atom<G> at[B];
+    int32_t t[B];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      hS[c] = ff_shfl_down(S[c], 1);
-      if (lane == 31) hS[c] = {0.0f, 0.0f};
+    for (int u = 0; u < B; ++u) {
+      at[u].load(x, xs, a1 - 1 - u);
+      t[u] = __ldg(A.rel_t + max(a1 - 1 - u, 0));
     }
-    if (lane == 0) {
-      sR[0][warp] = Rw.h;
-      sR[1][warp] = Rw.l;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        sS[c][0][warp] = S[c].h;
-        sS[c][1][warp] = S[c].l;
-      }
+    for (int u = 0; u < B; ++u) {
+      if (a1 - 1 - u < lo) break;
+      E.step(sweep_gap_decay<1, IRR>(s_pw, tn - t[u], inv, t_sft, lane, tt), at[u]);
+      tn = t[u];
     }
-    __syncthreads();
-    if (warp == 0) {
-      FF Rv = lane < NW ? FF{sR[0][lane], sR[1][lane]} : FF{1.0f, 0.0f};
-      FF Sv[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        Sv[c] = lane < NW ? FF{sS[c][0][lane], sS[c][1][lane]} : FF{0.0f, 0.0f};
-#pragma unroll
-      for (int k = 0; (1 << k) < NW; ++k) {
-        const FF Ro = ff_shfl_down(Rv, 1 << k);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const FF So = ff_shfl_down(Sv[c], 1 << k);
-          if (lane + (1 << k) < NW) Sv[c] = ff_fma_sum(Sv[c], Rv, So);
-        }
-        if (lane + (1 << k) < NW) Rv = ff_mul(Rv, Ro);
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        FF K = ff_shfl_down(Sv[c], 1);   // E at the end of warp `lane`
-        if (lane >= NW - 1) K = {0.0f, 0.0f};
-        if (lane < NW) {
-          sK[c][0][lane] = K.h;
-          sK[c][1][lane] = K.l;
-        }
-      }
+    if (E.run >= run) {
+      R = ff_mul(R, FF{E.Qh, E.Qc});
+      E.renorm();
     }
-    __syncthreads();
-    // 3. E[i] = L[i] + Q[i] E[e0]
-    float Ke[4];
+  }
+  R = ff_mul(R, FF{E.Qh, E.Qc});
+  E.renorm();
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const FF e = ff_fma_sum(hS[c], hR, FF{sK[c][0][warp], sK[c][1][warp]});
-      Ke[c] = e.h + e.l;
+  for (int k = 0; k < G; ++k) {
+    if (k >= n_t) break;
+    float* o = A.agg + (((int64_t)(tg0 + k) * q.n_grp + grp) * q.n_chunks + ch) * 256 + lane;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      up2(E.Kh[k][c], o[128 * c], o[128 * c + 32]);
+      up2(E.Kl[k][c], o[128 * c + 64], o[128 * c + 96]);
     }
-    for (int i = s0; i < e0; ++i) {
-      const float qi = s_q[i];
-      float4 e = s_e[i];
-      e.x = fmaf(qi, Ke[0], e.x);
-      e.y = fmaf(qi, Ke[1], e.y);
-      e.z = fmaf(qi, Ke[2], e.z);
-      e.w = fmaf(qi, Ke[3], e.w);
-      s_e[i] = e;
-    }
-    if (tid == 0) s_e[n] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    // 4. cells (t0_m, tau_n), all m
-    const bool fresh = first || !recs;   // records computed here (no array: one template)
-    // U cells per thread at a time: their records (or, when computed here,
-    // their window indices and then the atom times those select) are all
-    // loaded before any is used, so the loads' latencies overlap
-    Partial acc = partial_empty();
-    for (int32_t mb = tid; mb < g.n_t0; mb += NT * U) {
-      float4 ra[U], rc[U];
-      if (fresh) {
-        int32_t i0v[U], jv[U], ti[U], tj[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int32_t m = mb + u * NT;
-          const bool in = m < g.n_t0;
-          i0v[u] = in ? i0tab[m] : 0;
-          jv[u] = in ? jend[(int64_t)m * g.n_tau + ni] : 0;
-          if (shared_antenna) {
-            const Coef cf = in ? coef[(int64_t)m * g.n_tau + ni] : Coef{0.f, 0.f, 0.f, 0.f};
-            rc[u] = make_float4(cf.k1, cf.beta, cf.k2, cf.valid);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const bool any = jv[u] > i0v[u];
-          ti[u] = any ? rel_t[i0v[u]] : 0;
-          tj[u] = any && jv[u] < n ? rel_t[jv[u]] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          // the window [i0, j), its prefactor and its tail factor
-          const int32_t m = mb + u * NT;
-          float pre = 0.0f, tail = 0.0f;
-          if (jv[u] > i0v[u]) {
-            const int64_t d0 = (int64_t)ti[u] - (grid_t0(g, ax, m) - tb);
-            pre = d0 == 0 ? 1.0f : rec_ex2(c2 * (float)d0);
-            if (jv[u] < n) {
-              // Approximate FP32 exp2 for the tail: ~e^{-3} of the window
-              // sum for the default 3 tau cut.  Windows cut before 3 tau make
-              // it large, where the difference E[i0] - tail E[j] loses 1 / (1
-              // - tail): there a tail above 1/2 comes from the correctly
-              // rounded-to-1-ulp exp2f.  (An FP64 exp here, even behind a
-              // branch never taken, slowed this kernel by 12 %.)
-              const float dj = (float)(tj[u] - ti[u]);
-              tail = rec_ex2(c2 * dj);
-              if (short_cut && tail > 0.5f) tail = exp2f(c2 * dj);
-            }
-          }
-          ra[u] = make_float4(__int_as_float(i0v[u]), __int_as_float(jv[u]), pre, tail);
-          if (recs && m < g.n_t0) {   // (read back by this same thread on later templates)
-            rec_a[m] = ra[u];
-            if (shared_antenna) rec_c[m] = rc[u];
-          }
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int32_t m = mb + u * NT;
-          const bool in = m < g.n_t0;
-          ra[u] = in ? rec_a[m] : make_float4(0.f, 0.f, 0.f, 0.f);
-          if (shared_antenna) rc[u] = in ? rec_c[m] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      }
-      if (!shared_antenna) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int32_t m = mb + u * NT;
-          const Coef cf = m < g.n_t0 ? coef[(int64_t)tq * cells + (int64_t)m * g.n_tau + ni]
-                                     : Coef{0.f, 0.f, 0.f, 0.f};
-          rc[u] = make_float4(cf.k1, cf.beta, cf.k2, cf.valid);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int32_t m = mb + u * NT;
-        if (m >= g.n_t0) break;
-        const int64_t cell = (int64_t)m * g.n_tau + ni;
-        const int32_t i0 = __float_as_int(ra[u].x), j = __float_as_int(ra[u].y);
-        float f[4] = {0.f, 0.f, 0.f, 0.f};
-        if (j > i0) {
-          const float4 ej = s_e[j], ei = s_e[i0];
-          f[0] = ra[u].z * fmaf(-ra[u].w, ej.x, ei.x);
-          f[1] = ra[u].z * fmaf(-ra[u].w, ej.y, ei.y);
-          f[2] = ra[u].z * fmaf(-ra[u].w, ej.z, ei.z);
-          f[3] = ra[u].z * fmaf(-ra[u].w, ej.w, ei.w);
-        }
-        const Coef cf{rc[u].x, rc[u].y, rc[u].z, rc[u].w};
-        const float v = two_f(cf, f[0], f[1], f[2], f[3]);
-        const bool ok = cf.valid == 1.0f;
-        if (map && cf.valid != 2.0f) map[(int64_t)tq * cells + cell] = ok ? v : 0.0f;
-        partial_add(acc, v, (int32_t)cell, ok);
-      }
-    }
-    acc = partial_block_reduce_alt<NW>(acc, scratch, tq - t_lo);
-    if (tid == 0) parts[(int64_t)tq * stride + ni] = acc;
+  }
+  if (tg0 == 0) {
+    float* o = rec_agg_r(A) + ((int64_t)grp * q.n_chunks + ch) * 64 + lane;
+    o[0] = R.h;
+    o[32] = R.l;
   }
 }
 
-// MB blocks of 256 threads' register budget per SM, for any width: MB = 3
-// where shared memory lets three blocks reside, else 2 (more registers, no
-// occupancy lost).
-template <int NT, int MB>
-__global__ void __launch_bounds__(NT, MB * 256 / NT)
-k_exp_rec(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base, int32_t n,
-          fmap_grid g, const int32_t* __restrict__ i0tab, const int32_t* __restrict__ jend,
-          const Coef* __restrict__ coef, int32_t shared_antenna, const float4* __restrict__ perm_x,
-          const int32_t* __restrict__ perm_gap, float4* __restrict__ recs, float* __restrict__ rdec,
-          const TauTab* __restrict__ tauc, const int64_t* __restrict__ ax, int32_t n_templates,
-          int32_t n_groups, float* __restrict__ map, Partial* __restrict__ parts, int64_t stride) {
-  exp_rec_body<NT, MB == 2 ? 4 : 2>(rel_t, t_base, n, g, i0tab, jend, coef, shared_antenna, perm_x, perm_gap, recs,
-                   rdec, tauc, ax, n_templates, n_groups, map, parts, stride, blockIdx, gridDim);
+// SHORT: windows cut before 3 tau.  SH: coefficients shared by the templates.
+// IRR: some gap is not 1..15 whole SFTs.
+template <int G, bool SHORT, bool SH, bool IRR>
+__device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, float2* s_pw,
+                                             int lane) {
+  const fmap_grid& g = A.g;
+  const RecGeom& q = A.q;
+  constexpr int NC = SH ? 1 : G;   // coefficient sets
+  // each cursor's next atom is loaded a step ahead, where registers allow
+  constexpr bool PF = G < 4;
+  static_assert(PF || !SHORT, "four templates: the 3 tau cut only");
+  // unit: template groups fastest (they share the rows' indices and
+  // coefficients), then row runs, then tau from the longest windows down
+  const int32_t tg0 = (int32_t)(unit % q.n_tgrp) * G;
+  const int64_t u1 = unit / q.n_tgrp;
+  const int32_t seg = (int32_t)(u1 % q.n_seg);
+  const int32_t grp = q.n_grp - 1 - (int32_t)(u1 / q.n_seg);
+  const int32_t n = A.n, n_tau = g.n_tau, run = rec_run(n);
+  const int32_t ni = grp * 32 + lane, nn = min(ni, n_tau - 1);
+  const bool in_grid = ni < n_tau;
+  const int32_t m_lo = seg * q.rows, m_hi = min(g.n_t0, m_lo + q.rows);
+  const int32_t n_t = min(G, A.T - tg0);        // templates present
+  const TauTab* tt = A.tauc + nn;
+  sweep_tab_load<1>(s_pw, tt, lane);
+  const float c2 = tt->c2[0];
+  const int64_t cells = (int64_t)g.n_t0 * n_tau;
+  const int64_t tb = n > 0 ? *A.t_base : 0;
+  const float4* x = A.x + (int64_t)tg0 * n;
+  const uint2 xs = make_uint2((uint32_t)n, (uint32_t)(n_t - 1));
+  const int32_t t_sft = (int32_t)g.t_sft;
+  const uint32_t inv = gap_inverse(t_sft);
+  int32_t i0 = A.i0tab[m_hi - 1], j = A.jend[(int64_t)(m_hi - 1) * n_tau + nn];
+  Cursor<G> Ei;
+  Ei.zero();
+  typename std::conditional<SHORT, Cursor<G>, PlainCursor<G>>::type Ej;
+  Ej.zero();
+  int32_t ic, jc;
+  if (q.n_chunks > 0) {
+    // E at the first atoms of the chunks after those holding j and i0
+    const int32_t bj = (j + q.chunk - 1) / q.chunk, bi = (i0 + q.chunk - 1) / q.chunk;
+    FF2 E[G][2];
+#pragma unroll
+    for (int k = 0; k < G; ++k) E[k][0] = E[k][1] = FF2{0ull, 0ull};
+    const float* ro = rec_agg_r(A) + (int64_t)grp * q.n_chunks * 64 + lane;
+    const float* so = A.agg + ((int64_t)tg0 * q.n_grp + grp) * q.n_chunks * 256 + lane;
+    const int64_t sk = (int64_t)q.n_grp * q.n_chunks * 256;
+    constexpr int B = G == 1 ? 4 : 1;   // chunk maps loaded ahead
+    for (int32_t b0 = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)bj);; b0 -= B) {
+      FF R[B];
+      float v[B][G][8];
+#pragma unroll
+      for (int u = 0; u < B; ++u) {
+        const int32_t c = max(b0 - 1 - u, 0);
+        R[u] = {ro[c * 64], ro[c * 64 + 32]};
+#pragma unroll
+        for (int k = 0; k < G; ++k)
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[u][k][e] = so[(int64_t)c * 256 + min(k, n_t - 1) * sk + 32 * e];
+      }
+      bool done = false;
+#pragma unroll
+      for (int u = 0; u < B; ++u) {
+        const int32_t b = b0 - u;
+        if (b == bj) {
+#pragma unroll
+          for (int k = 0; k < G; ++k) {
+            Ej.set(k, 0, E[k][0]);
+            Ej.set(k, 1, E[k][1]);
+          }
+        }
+        if (b <= bi) {
+          done = true;
+          break;
+        }
+#pragma unroll
+        for (int k = 0; k < G; ++k)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const float* w = &v[u][k][4 * c];
+            const FF2 p = ff2_fma_sum(pk2(w[0], w[1]), R[u], E[k][c]);
+            E[k][c] = fast_two_sum2(p.h, add2(p.l, pk2(w[2], w[3])));
+          }
+      }
+      if (done) break;
+    }
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      Ei.set(k, 0, E[k][0]);
+      Ei.set(k, 1, E[k][1]);
+    }
+    ic = min(n, bi * q.chunk);
+    jc = min(n, bj * q.chunk);
+  } else {
+    // E starts from zero at each lane's window end of the last row
+    jc = j;
+    ic = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)j);
+    const int32_t j_all = (int32_t)__reduce_min_sync(0xffffffffu, (unsigned)j);
+    int32_t tn = n > 0 ? atom_time(A, ic) : 0;
+    while (ic > max(i0, j_all)) {   // atoms past some lanes' ends
+      --ic;
+      Atom<G> at;
+      at.load(x, xs, ic);
+      const int32_t t = __ldg(A.rel_t + ic);
+      const FF r = sweep_gap_decay<1, IRR>(s_pw, tn - t, inv, t_sft, lane, tt);
+      tn = t;
+      if (ic < j) Ei.step(r, at);
+    }
+    Ei.renorm();   // (the lanes' runs differ: from here they are equal)
+  }
+  // times of the cursors' atoms, and of the next ones (loaded a step ahead)
+  int32_t ti = n > 0 ? atom_time(A, ic) : 0, tj = n > 0 ? atom_time(A, jc) : 0;
+  int32_t ei = n > 0 ? __ldg(A.rel_t + max(ic - 1, 0)) : 0;
+  int32_t ej = n > 0 ? __ldg(A.rel_t + max(jc - 1, 0)) : 0;
+  Atom<G> ai, aj;
+  if (PF) {
+    ai.load(x, xs, ic - 1);
+    aj.load(x, xs, jc - 1);
+  } else {   // to the last row's window (below, the first row's loop does it)
+    Atom<G> at;
+    at.load(x, xs, ic - 1);
+    while (ic > i0) {
+      --ic;
+      const Atom<G> cur = at;
+      const int32_t t = ei;
+      at.load(x, xs, ic - 1);
+      ei = __ldg(A.rel_t + max(ic - 1, 0));
+      Ei.step(sweep_gap_decay<1, IRR>(s_pw, ti - t, inv, t_sft, lane, tt), cur);
+      ti = t;
+      if (Ei.run >= run) Ei.renorm();
+    }
+  }
+  // per template and tile: maximum, its row, sum of e^{(v - maximum) / 2};
+  // valid cells
+  float M[G], sum[G];
+  int32_t arg[G], nv[NC];
+  auto clear = [&]() {
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      M[k] = -1.0f;
+      sum[k] = 0.0f;
+      arg[k] = 0;
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) nv[k] = 0;
+  };
+  clear();
+  constexpr float kHalfLog2e = 0.72134752044448170368f;   // log2(e) / 2
+  const uint64_t tiny2 = pk2(1e-30f, 1e-30f);
+  int32_t m_flush = ((m_hi - 1) / q.tile_rows) * q.tile_rows;   // the tile's first row
+  int64_t t0r = grid_t0(g, A.ax, m_hi - 1) - tb;
+  uint32_t cell = (uint32_t)(m_hi - 1) * (uint32_t)n_tau + (uint32_t)nn;   // (cells < 2^31)
+  const float4* cp = reinterpret_cast<const float4*>(A.coef) + (SH ? 0 : (int64_t)tg0 * cells);
+  float4 cf[NC];
+#pragma unroll
+  for (int k = 0; k < NC; ++k) cf[k] = __ldg(cp + min(k, n_t - 1) * cells + cell);
+  float* const mp = A.map ? A.map + (int64_t)tg0 * cells : nullptr;
+  const bool store = mp && in_grid;
+  for (int32_t m = m_hi - 1; m >= m_lo; --m) {
+    if (!PF) {   // the atoms this row most often steps over, before anything waits
+      ai.load(x, xs, ic - 1);
+      aj.load(x, xs, jc - 1);
+    }
+    int32_t i0n = 0, jn = 0;
+    float4 cn[NC];
+    if (m > m_lo) {
+      i0n = __ldg(A.i0tab + (m - 1));
+      jn = __ldg(A.jend + (cell - (uint32_t)n_tau));
+#pragma unroll
+      for (int k = 0; k < NC; ++k)
+        cn[k] = __ldg(cp + min(k, n_t - 1) * cells + (cell - (uint32_t)n_tau));
+    }
+    if constexpr (PF) {
+      while (ic > i0) {
+        --ic;
+        const Atom<G> cur = ai;
+        const int32_t t = ei;
+        ei = __ldg(A.rel_t + max(ic - 1, 0));
+        ai.load(x, xs, ic - 1);
+        Ei.step(sweep_gap_decay<1, IRR>(s_pw, ti - t, inv, t_sft, lane, tt), cur);
+        ti = t;
+        if (Ei.run >= run) Ei.renorm();
+      }
+      while (jc > j) {
+        --jc;
+        const Atom<G> cur = aj;
+        const int32_t t = ej;
+        ej = __ldg(A.rel_t + max(jc - 1, 0));
+        aj.load(x, xs, jc - 1);
+        Ej.step(sweep_gap_decay<1, IRR>(s_pw, tj - t, inv, t_sft, lane, tt), cur);
+        tj = t;
+        if constexpr (SHORT)
+          if (Ej.run >= run) Ej.renorm();
+      }
+    } else {
+      const FF ri = sweep_gap_decay<1, IRR>(s_pw, ti - ei, inv, t_sft, lane, tt);
+      const FF rj = sweep_gap_decay<1, IRR>(s_pw, tj - ej, inv, t_sft, lane, tt);
+      if (ic > i0) {
+        --ic;
+        Ei.step(ri, ai);
+        ti = ei;
+        while (ic > i0) {
+          --ic;
+          ei = __ldg(A.rel_t + ic);
+          ai.load(x, xs, ic);
+          Ei.step(sweep_gap_decay<1, IRR>(s_pw, ti - ei, inv, t_sft, lane, tt), ai);
+          ti = ei;
+          if (Ei.run >= run) Ei.renorm();
+        }
+        ei = __ldg(A.rel_t + max(ic - 1, 0));
+        if (Ei.run >= run) Ei.renorm();
+      }
+      if (jc > j) {
+        --jc;
+        Ej.step(rj, aj);
+        tj = ej;
+        while (jc > j) {
+          --jc;
+          ej = __ldg(A.rel_t + jc);
+          aj.load(x, xs, jc);
+          Ej.step(sweep_gap_decay<1, IRR>(s_pw, tj - ej, inv, t_sft, lane, tt), aj);
+          tj = ej;
+        }
+        ej = __ldg(A.rel_t + max(jc - 1, 0));
+      }
+    }
+    // Tail factor and squared prefactor of the window [i0, j) (an empty one is
+    // invalid).  Approximate FP32 exp2 for the tail: ~e^{-3} of the window sum
+    // for the default 3 tau cut.  Windows cut before 3 tau make it large, where
+    // the difference E[i0] - tail E[j] loses 1 / (1 - tail): there a tail
+    // above 1/2 comes from the correctly rounded-to-1-ulp exp2f.
+    const float dj = (float)(tj - ti);
+    float tail = rec_ex2(c2 * dj);
+    if (SHORT && tail > 0.5f) tail = exp2f(c2 * dj);
+    float pre2 = 1.0f;
+    const int32_t d0 = (int32_t)(ti - t0r);
+    if (d0 != 0) {
+      const float pre = rec_ex2(c2 * (float)d0);
+      pre2 = pre * pre;
+    }
+    const uint64_t qi = Ei.scale(), qj = Ej.scale(), nt = pk2(-tail, -tail);
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const float4 c = cf[SH ? 0 : k];
+      // cells that take no part (invalid, or left to the fix-up): -inf, which
+      // no maximum takes, whose exp-term is 0 and whose map entry is 0
+      const bool ok = c.w == 1.0f && in_grid;
+      const float k1 = ok ? c.x * pre2 : -INFINITY, k2 = ok ? c.z * pre2 : 0.0f;
+      if (SH ? k == 0 : true) nv[SH ? 0 : k] += ok ? 1 : 0;
+      const uint64_t f0 = fma2(nt, Ej.get(k, 0, qj), Ei.get(k, 0, qi));
+      const uint64_t f1 = fma2(nt, Ej.get(k, 1, qj), Ei.get(k, 1, qi));
+      const float v = two_f_pairs(f0, f1, pk2(-c.y, -c.y), k1, k2, tiny2);
+      if (store && k < n_t) (mp + k * cells)[cell] = fmaxf(v, 0.0f);
+      // rows come in descending order: the later one wins a tie
+      const float ex = rec_ex2(fabsf(v - M[k]) * -kHalfLog2e);
+      const bool up = v >= M[k];
+      sum[k] = up ? fmaf(sum[k], ex, 1.0f) : sum[k] + ex;
+      M[k] = fmaxf(M[k], v);
+      arg[k] = up ? m : arg[k];
+    }
+    if (m == m_flush) {   // one partial per (template, tile)
+      m_flush -= q.tile_rows;
+      const int64_t slot = (int64_t)(m / q.tile_rows) * q.n_grp + grp;
+#pragma unroll
+      for (int k = 0; k < G; ++k) {
+        const Partial r = partial_warp_reduce(
+            Partial{M[k], arg[k] * n_tau + ni, sum[k], nv[SH ? 0 : k]});
+        if (lane == 0 && k < n_t) A.parts[(int64_t)(tg0 + k) * A.stride + slot] = r;
+      }
+      clear();
+    }
+    i0 = i0n;
+    j = jn;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) cf[k] = cn[k];
+    cell -= (uint32_t)n_tau;
+    t0r = A.ax ? (m > m_lo ? A.ax[m - 1] - tb : 0) : t0r - g.dt0;
+  }
+}
+
+// (registers: the state of four templates takes about 160, of one about 100)
+template <int G, bool SHORT, bool SH>
+__global__ void __launch_bounds__(kRecThreads, G == 4 ? 3 : G == 2 ? 4 : 5)
+k_exp_rec(const RecArgs A, int64_t units) {
+  __shared__ float2 s_pw[kRecWarps][kSweepTab];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t unit = (int64_t)blockIdx.x * kRecWarps + warp;
+  if (unit >= units) return;
+  if (*A.irr) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw[warp], lane);
+  else exp_rec_unit<G, SHORT, SH, false>(A, unit, s_pw[warp], lane);
+}
+// Chunk maps of the antenna rows (units [0, ant_units)), then of the data.
+struct AntAgg {
+  const float4* ant;
+  float* agg;
+  AntGeom q;
+  int64_t units;
+};
+template <int G, bool IRR>
+__device__ __forceinline__ void sweep_agg_unit(const RecArgs& A, const AntAgg& N, int64_t unit,
+                                               float2* s_pw, int lane) {
+  if (unit < N.units)
+    exp_agg_unit<IRR>(A.rel_t, A.n, N.ant, A.tauc, A.g, N.q, N.agg, unit, s_pw, lane);
+  else
+    rec_agg_unit<G, IRR>(A, unit - N.units, s_pw, lane);
+}
+template <int G>
+__global__ void __launch_bounds__(kAggThreads)
+k_sweep_agg(const RecArgs A, const AntAgg N, int64_t units) {
+  __shared__ float2 s_pw[kSweepWarps][kSweepTab];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t unit = (int64_t)blockIdx.x * kSweepWarps + warp;
+  if (unit >= units) return;
+  if (*A.irr) sweep_agg_unit<G, true>(A, N, unit, s_pw[warp], lane);
+  else sweep_agg_unit<G, false>(A, N, unit, s_pw[warp], lane);
 }
 
 bool exp_rec_supported(int32_t n_sft, int32_t) { return n_sft <= kRecMaxSft; }
+
+// The work split, by a count of issue slots (as measured, at the issue rate
+// each form reaches: 233 instructions a row at 40 % for two templates, 352 at 36 %
+// for four).  A warp's start costs the window's atoms, or the composition of
+// half the chunk maps and the atoms of a chunk for each cursor.  A scheduler needs
+// about three warps to hide the latencies: below that, time goes with one warp's
+// work.
+RecGeom rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, bool shared, bool batch, int32_t tpb,
+                 int64_t agg_room) {
+  RecGeom best{};
+  double best_t = 0.0;
+  const int32_t n_grp = std::max(1, (g.n_tau + 31) / 32);
+  // (four templates per warp only with coefficients in common and the 3 tau cut,
+  // by registers)
+  int32_t g_max = shared && exp_cut8_of(g) >= 24 ? 4 : 2;
+  if (tpb > 0) g_max = std::min(g_max, tpb);
+  double win = 0.0;   // atoms of the windows, averaged over tau
+  for (int k = 0; k < 16; ++k) {
+    const int64_t tau = g.tau_min + (int64_t)std::max(0, g.n_tau - 1) * k / 15 * g.dtau;
+    win += std::min<double>(n_sft, (double)window_len(g, tau) / (double)g.t_sft) / 16.0;
+  }
+  const double more = std::min<double>((double)n_sft, std::max(0.0, (double)g.dt0 / (double)g.t_sft - 1.0));
+  const int32_t chunk = n_sft <= 512 ? 16 : n_sft <= 1024 ? 32 : n_sft <= 4096 ? 64 : 128;
+  const int32_t n_chunks = (n_sft + chunk - 1) / chunk;
+  const double slots = kSms * 4.0;
+  for (int G = 1; G <= g_max && (G == 1 || G <= T); G *= 2) {
+    const int32_t tgrp = std::max(1, (T + G - 1) / G);
+    if (G == 4 && (double)n_grp * tgrp < slots) break;   // (few warps per scheduler: two templates)
+    for (int maps = 0; maps < 2; ++maps) {
+      // chunk maps only where there are few warps, and room for them
+      if (maps && (n_sft == 0 || (int64_t)n_grp * T > 4096 ||
+                   4 * (int64_t)n_grp * n_chunks * ((int64_t)T * 256 + 64) > agg_room))
+        continue;
+      const double start = maps ? 0.5 * n_chunks * (30.0 + 90.0 * G) + 1.5 * chunk * (40.0 + 30.0 * G)
+                                : win * (40.0 + 30.0 * G);
+      const double ahead = maps ? chunk * (60.0 + 35.0 * G) *
+                                      std::max(3.0, (double)n_grp * tgrp * n_chunks / slots)
+                                : 0.0;
+      for (int32_t seg = 1; seg <= 256; seg = seg < 4 ? seg + 1 : seg + seg / 3) {
+        const int32_t rows = (g.n_t0 + seg - 1) / seg;
+        if (seg > 1 && rows < 4) break;
+        if (batch && seg > 1 && rows < 48) break;   // (instances run side by side)
+        const double work = start + rows * (150.0 + 210.0 * G + more * (60.0 + 50.0 * G));
+        // a batch has other instances to fill the GPU: total work counts
+        const double t = ahead + work * (batch ? (double)n_grp * tgrp * seg / slots + 0.3
+                                               : std::max(3.0, (double)n_grp * tgrp * seg / slots));
+        if (best.G == 0 || t < best_t) {
+          best_t = t;
+          best.G = G;
+          best.rows = std::max(1, rows);
+          best.chunk = maps ? chunk : 0;
+          best.n_chunks = maps ? n_chunks : 0;
+        }
+      }
+    }
+  }
+  RecGeom& q = best;
+  q.n_grp = n_grp;
+  if (q.rows > kRecTileRows) q.rows = (q.rows + kRecTileRows - 1) / kRecTileRows * kRecTileRows;
+  q.tile_rows = std::min(q.rows, kRecTileRows);
+  q.n_seg = std::max(1, (g.n_t0 + q.rows - 1) / q.rows);
+  q.ntr = std::max(1, (g.n_t0 + q.tile_rows - 1) / q.tile_rows);
+  q.n_tgrp = std::max(1, (T + q.G - 1) / q.G);
+  return q;
+}
+// (the data's chunk maps follow the antenna rows')
+static RecArgs rec_args(const fmap_plan_s* p, const RecGeom& q, const AntGeom& a, int64_t n_ant,
+                        float* d_2F) {
+  return RecArgs{p->ws.rel_t, p->ws.t_base, p->ws.irr, p->n_sft, p->n_templates, p->grid, q,
+                 p->ws.i0, p->ws.jend, p->ws.coef, p->ws.perm_x, p->ws.tauc,
+                 plan_axes(p), p->ws.agg + ant_agg_floats(a, n_ant), d_2F, p->ws.partials, p->part_stride};
+}
+
+cudaError_t launch_exp_agg(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
+  const fmap_grid& g = p->grid;
+  const int n_ant = a->shared_antenna ? 1 : p->n_templates;
+  if ((int64_t)g.n_t0 * g.n_tau == 0 || n_ant == 0 || p->n_sft == 0) return cudaSuccess;
+  AntAgg N{p->ws.perm_ant, p->ws.agg, p->ant[a->shared_antenna ? 1 : 0], 0};
+  N.units = (int64_t)N.q.n_grp * n_ant * N.q.n_chunks;
+  RecGeom q{};
+  q.G = 1;
+  if ((p->flags & FMAP_PLAN_EXP_RECURRENCE) && p->n_templates > 0)
+    q = p->rec[a->shared_antenna ? 1 : 0];
+  const int64_t units = N.units + (int64_t)q.n_grp * q.n_chunks * q.n_tgrp;
+  if (units == 0) return cudaSuccess;
+  const RecArgs A = rec_args(p, q, N.q, n_ant, nullptr);
+  auto run = [&](auto kern) {
+    kern<<<(unsigned)((units + kSweepWarps - 1) / kSweepWarps), kAggThreads, 0, s>>>(A, N, units);
+  };
+  q.G == 1 ? run(k_sweep_agg<1>) : q.G == 2 ? run(k_sweep_agg<2>) : run(k_sweep_agg<4>);
+  p->launches += 1;
+  return cudaGetLastError();
+}
 
 cudaError_t launch_exp_rec(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaStream_t s,
                            int64_t* tiles_used) {
   const fmap_grid& g = p->grid;
   *tiles_used = 0;
   if ((int64_t)g.n_t0 * g.n_tau == 0 || p->n_templates == 0) return cudaSuccess;
-  *tiles_used = g.n_tau;
-  p->tiles = TileGeom{0, g.n_t0, 1, 1, g.n_tau};   // one tau column per tile
-  const size_t smem = exp_rec_smem(p->n_sft, g.n_t0, p->n_templates);
-  const bool three = smem + 1024 <= 227 * 1024 / 3;
-  // The templates are split into G groups, one block per (tau, group), with
-  // G chosen so that the blocks fill whole waves of the resident slots: the
-  // step takes about ceil(blocks / slots) block times, and a block's time is
-  // its templates plus about 1.5 templates' worth of first-template work
-  // (decay products, window records).  Measured on GB300: 1024 templates x
-  // 2000 tau, G = 5 is 7 % faster than one block per tau; 16 x 1000, G = 2
-  // is 8 % faster.
-  const int nt = p->lanes == 64 || p->lanes == 128 ? p->lanes : 256;
-  const int64_t per_sm = std::max<int64_t>(
-      1, std::min<int64_t>({(int64_t)(three ? 3 : 2) * 256 / nt, (int64_t)2048 / nt,
-                            (int64_t)(227 * 1024) / (int64_t)(smem + 1024)}));
-  const int64_t slots = (int64_t)p->n_sm * per_sm;
-  int32_t groups = 1;
-  double best = 0.0;
-  for (int32_t G = 1; G <= std::min<int32_t>(p->n_templates, kRecMaxGroups); ++G) {
-    const double waves = std::ceil((double)g.n_tau * G / (double)slots);
-    const double cost = waves * ((double)((p->n_templates + G - 1) / G) + 1.5);
-    if (G == 1 || cost < best) {
-      best = cost;
-      groups = G;
-    }
-  }
-  dim3 grid((unsigned)g.n_tau, (unsigned)groups);
-  auto run = [&](auto kern, int nt) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<grid, nt, smem, s>>>(p->ws.rel_t, p->ws.t_base, p->n_sft, g, p->ws.i0, p->ws.jend,
-                                p->ws.coef, a->shared_antenna, p->ws.perm_x, p->ws.perm_gap,
-                                p->ws.rec_cells, p->ws.rec_decay, p->ws.tauc, plan_axes(p), p->n_templates, groups, d_2F,
-                                p->ws.partials, p->part_stride);
+  const RecGeom q = p->rec[a->shared_antenna ? 1 : 0];
+  *tiles_used = (int64_t)q.ntr * q.n_grp;
+  p->tiles = TileGeom{0, q.tile_rows, 32, q.ntr, q.n_grp};
+  const RecArgs A = rec_args(p, q, p->ant[a->shared_antenna ? 1 : 0],
+                             a->shared_antenna ? 1 : p->n_templates, d_2F);
+  auto run = [&](auto kern, int64_t units) {
+    kern<<<(unsigned)((units + kRecWarps - 1) / kRecWarps), kRecThreads, 0, s>>>(A, units);
+    p->launches += 1;
   };
-  switch (p->lanes) {
-    case 64: three ? run(k_exp_rec<64, 3>, 64) : run(k_exp_rec<64, 2>, 64); break;
-    case 128: three ? run(k_exp_rec<128, 3>, 128) : run(k_exp_rec<128, 2>, 128); break;
-    default: three ? run(k_exp_rec<256, 3>, 256) : run(k_exp_rec<256, 2>, 256); break;
-  }
-  p->launches += 1;
+  const int64_t units = (int64_t)q.n_grp * q.n_seg * q.n_tgrp;
+  const bool brief = exp_cut8_of(g) < 24;
+  auto pick = [&](auto one, auto two, auto four) {
+    q.G == 1 ? run(one, units) : q.G == 2 ? run(two, units) : run(four, units);
+  };
+  if (a->shared_antenna)
+    brief ? pick(k_exp_rec<1, true, true>, k_exp_rec<2, true, true>, k_exp_rec<2, true, true>)
+          : pick(k_exp_rec<1, false, true>, k_exp_rec<2, false, true>, k_exp_rec<4, false, true>);
+  else
+    brief ? pick(k_exp_rec<1, true, false>, k_exp_rec<2, true, false>, k_exp_rec<2, true, false>)
+          : pick(k_exp_rec<1, false, false>, k_exp_rec<2, false, false>, k_exp_rec<2, false, false>);
   return cudaGetLastError();
 }
 
 
-// ---- persistent multi-instance dispatcher (uneven batches) ----
-// (the register budget of 3 blocks of 256 threads per SM, for any width)
-template <int NT>
-__global__ void __launch_bounds__(NT, 768 / NT) kb_exp_rec(const BItem* __restrict__ items,
-                                                        BUnits u) {
+// ---- persistent multi-instance dispatchers (uneven batches) ----
+static __device__ __forceinline__ RecArgs rec_args(const BItem& it) {
+  return RecArgs{it.rel_t, it.t_base, it.irr, it.n_sft, it.T, it.g, it.rg, it.i0, it.jend, it.coef,
+                 it.perm_x, it.tauc, it.ax, it.agg + ant_agg_floats(it.ag, it.n_ant), it.map,
+                 it.partials, it.part_stride};
+}
+__global__ void __launch_bounds__(kAggThreads, 2) kb_sweep_agg(const BItem* __restrict__ items,
+                                                               BUnits u) {
+  __shared__ float2 s_pw[kSweepWarps][kSweepTab];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
-    exp_rec_body<NT, 2>(it.rel_t, it.t_base, it.n_sft, it.g, it.i0, it.jend, it.coef, it.shared,
-                     it.perm_x, it.perm_gap, it.rec_cells, nullptr, it.tauc, it.ax, it.T, it.groups, it.map, it.partials,
-                     it.part_stride,
-                     make_uint3((unsigned)(k % it.g.n_tau), (unsigned)(k / it.g.n_tau), 0),
-                     dim3((unsigned)it.g.n_tau, (unsigned)it.groups));
+    const int64_t unit = k * kSweepWarps + warp;
+    const AntAgg N{it.perm_ant, it.agg, it.ag, (int64_t)it.ag.n_grp * it.n_ant * it.ag.n_chunks};
+    if (unit >= N.units + (int64_t)it.rg.n_grp * it.rg.n_chunks * it.rg.n_tgrp) return;
+    const RecArgs A = rec_args(it);
+    if (it.rg.G == 1) {
+      if (*it.irr) sweep_agg_unit<1, true>(A, N, unit, s_pw[warp], lane);
+      else sweep_agg_unit<1, false>(A, N, unit, s_pw[warp], lane);
+    } else if (it.rg.G == 2) {
+      if (*it.irr) sweep_agg_unit<2, true>(A, N, unit, s_pw[warp], lane);
+      else sweep_agg_unit<2, false>(A, N, unit, s_pw[warp], lane);
+    } else {
+      if (*it.irr) sweep_agg_unit<4, true>(A, N, unit, s_pw[warp], lane);
+      else sweep_agg_unit<4, false>(A, N, unit, s_pw[warp], lane);
+    }
   });
 }
-const void* batch_kernel_exp_rec(int phase, int lanes) {
-  if (phase != BP_EXP_REC) return nullptr;
-  return lanes == 64 ? (const void*)kb_exp_rec<64>
-                     : lanes == 128 ? (const void*)kb_exp_rec<128> : (const void*)kb_exp_rec<256>;
+template <int G, bool SHORT, bool SH>
+static __device__ __forceinline__ void rec_batch_unit(const RecArgs& A, int64_t unit, float2* s_pw,
+                                                      int lane) {
+  if (*A.irr) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw, lane);
+  else exp_rec_unit<G, SHORT, SH, false>(A, unit, s_pw, lane);
 }
-size_t exp_rec_smem(int32_t n_sft, int32_t, int32_t) { return rec_smem_base(n_sft); }
+// MAXG: the most templates per warp of the wave's instances (registers).
+template <int MAXG>
+__global__ void __launch_bounds__(kRecThreads, MAXG == 1 ? 4 : 3)
+kb_exp_rec(const BItem* __restrict__ items, BUnits u) {
+  __shared__ float2 s_pw[kRecWarps][kSweepTab];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  batch_loop(items, u, [&](const BItem& it, int64_t k) {
+    const int64_t unit = k * kRecWarps + warp;
+    if (unit >= (int64_t)it.rg.n_grp * it.rg.n_seg * it.rg.n_tgrp) return;
+    const RecArgs A = rec_args(it);
+    const bool brief = exp_cut8_of(it.g) < 24;
+    if constexpr (MAXG >= 4)
+      if (it.rg.G == 4) return rec_batch_unit<4, false, true>(A, unit, s_pw[warp], lane);
+    if constexpr (MAXG >= 2)
+      if (it.rg.G == 2) {
+        if (it.shared) {
+          if (brief) rec_batch_unit<2, true, true>(A, unit, s_pw[warp], lane);
+          else rec_batch_unit<2, false, true>(A, unit, s_pw[warp], lane);
+        } else {
+          if (brief) rec_batch_unit<2, true, false>(A, unit, s_pw[warp], lane);
+          else rec_batch_unit<2, false, false>(A, unit, s_pw[warp], lane);
+        }
+        return;
+      }
+    if (it.shared) {
+      if (brief) rec_batch_unit<1, true, true>(A, unit, s_pw[warp], lane);
+      else rec_batch_unit<1, false, true>(A, unit, s_pw[warp], lane);
+    } else {
+      if (brief) rec_batch_unit<1, true, false>(A, unit, s_pw[warp], lane);
+      else rec_batch_unit<1, false, false>(A, unit, s_pw[warp], lane);
+    }
+  });
+}
+const void* batch_kernel_exp_rec(int phase, int max_g) {
+  if (phase == BP_EXP_AGG) return (const void*)kb_sweep_agg;
+  if (phase != BP_EXP_REC) return nullptr;
+  return max_g >= 4 ? (const void*)kb_exp_rec<4>
+                    : max_g == 2 ? (const void*)kb_exp_rec<2> : (const void*)kb_exp_rec<1>;
+}
 
 }  // namespace fmap

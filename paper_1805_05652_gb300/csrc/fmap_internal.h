@@ -79,8 +79,7 @@ __host__ __device__ inline void fix_slot_range(int64_t b, int64_t n, int64_t* lo
 }
 // Internal plan flag (not part of the C ABI) of batch instances, whose
 // workspaces are kept lean: the plan never refines its summaries (no
-// refinement arrays), and the recurrence recomputes its window records per
-// template (no record array).
+// refinement arrays).
 constexpr uint32_t kPlanBatch = 1u << 16;
 // Top-cell refinement (fmap_refine.cu): candidates per template (at most),
 // histogram bins over the window of kRefWindow (2F units) below the maximum.
@@ -131,32 +130,27 @@ constexpr int kFlagUnit = 32768;
 __host__ __device__ inline int64_t flag_words(int64_t entries) {
   return (entries + kFlagUnit - 1) / kFlagUnit * (kFlagUnit / 32);
 }
-// Threads of the exponential-window scans ("lanes", 64, 128 or 256, a plan
-// property): thread t of a scan owns the atoms [t C, t C + C), C =
-// ceil(N / lanes), and the scans read the atoms from a chunk-major copy
-// (entry q lanes + t holds atom t C + q), so the loads of a warp at one chunk
-// position are contiguous.  Single plans scan with 256 threads; batches, whose
-// many short units favour throughput over the latency of one tau, take fewer
-// for short data sets (batch_scan_lanes), so that combining the threads'
-// chunks stays cheap next to the chunks themselves.
-constexpr int kScanLanes = 256;   // the most threads of a scan
-__host__ __device__ inline int32_t batch_scan_lanes(int32_t n_sft) {
-  return n_sft <= 1024 ? 128 : 256;
+// SMs of a GB300: the sweeps' work splits (which fix the reduction tiles, and
+// so the workspace) are chosen for it.
+constexpr int kSms = 152;
+constexpr int kSweepWarps = 8;   // warps (units of work) per block of the sweeps
+constexpr int kRecWarps = 4;     // and of the recurrence
+// Work split of the exponential antenna sweep (fmap_exp.cu): groups of 32 tau,
+// chunks of atoms whose decayed sums are formed ahead, runs of t0 rows.
+struct AntGeom {
+  int32_t chunk, n_chunks, n_grp, rows, n_seg;
+};
+// Floats of the antenna rows' chunk maps.
+__host__ __device__ inline int64_t ant_agg_floats(const AntGeom& q, int64_t n_ant) {
+  return 256 * (int64_t)q.n_grp * q.n_chunks * n_ant;
 }
-// Atoms per thread: odd, so that the threads' chunk starts (stride C) fall
-// in distinct shared-memory banks across a warp.
-__host__ __device__ inline int64_t scan_chunk(int32_t n_sft, int32_t lanes) {
-  return (((int64_t)n_sft + lanes - 1) / lanes) | 1;
-}
-__host__ __device__ inline int64_t perm_entries(int32_t n_sft, int32_t lanes) {
-  return scan_chunk(n_sft, lanes) * lanes;
-}
-// The most entries of any scan width (workspaces take this).
-__host__ __device__ inline int64_t perm_entries_max(int32_t n_sft) {
-  int64_t e = perm_entries(n_sft, 64);
-  e = e > perm_entries(n_sft, 128) ? e : perm_entries(n_sft, 128);
-  return e > perm_entries(n_sft, 256) ? e : perm_entries(n_sft, 256);
-}
+// Work split of the recurrence (fmap_exp_rec.cu): groups of 32 tau, G
+// templates per warp (n_tgrp groups), runs of t0 rows; reduction tiles of
+// tile_rows rows x one tau (ntr tiles down a column).
+struct RecGeom {
+  int32_t n_grp, G, n_tgrp, rows, n_seg, tile_rows, ntr;
+  int32_t chunk, n_chunks;   // chunk maps the warps start from (0: none)
+};
 // Grid values t0_m and tau_n: Eq. Fmn's uniform grid, or the plan's explicit
 // axes ax (t0 values, then tau values) when given (non-null).
 __host__ __device__ inline int64_t grid_t0(const fmap_grid& g, const int64_t* ax, int64_t m) {
@@ -165,11 +159,11 @@ __host__ __device__ inline int64_t grid_t0(const fmap_grid& g, const int64_t* ax
 __host__ __device__ inline int64_t grid_tau(const fmap_grid& g, const int64_t* ax, int64_t n) {
   return ax ? ax[g.n_t0 + n] : g.tau_min + n * g.dtau;
 }
-// Entries of the exp copy step: the chunk-major copies, then one per tau.
+// Entries of the exp copy step: two per tau, then one per atom and set.
 // (plan_axes, after the plan struct: the axes to pass kernels, or null.)
-__host__ __device__ inline int64_t exp_copy_entries(int32_t n_sft, int32_t lanes, int32_t n_ant,
-                                                    int32_t n_x, int32_t n_tau) {
-  return perm_entries(n_sft, lanes) * (int64_t)(n_ant + n_x) + n_tau;
+__host__ __device__ inline int64_t exp_copy_entries(int32_t n_sft, int32_t n_ant, int32_t n_x,
+                                                    int32_t n_tau) {
+  return 2 * (int64_t)n_tau + (int64_t)n_sft * ((int64_t)n_ant + n_x);
 }
 // Per-tau constants of the exponential window, for the weight w (s = 1) and
 // the antenna weight w^2 (s = 2): the decays over gaps of k = 0..kPowTab-1
@@ -195,6 +189,7 @@ struct Workspace {
   size_t bytes = 0;
   int32_t* rel_t = nullptr;      // [round_up(N, 64) + 64] t - t[0], zero padded
   int64_t* t_base = nullptr;     // [1] t[0]
+  int32_t* irr = nullptr;        // [1] nonzero: a gap is not 1..kPowTab-1 whole SFTs (exp)
   uint32_t* dev_err = nullptr;   // [1] latched device error bits
   int32_t* i0 = nullptr;         // [n_t0] first atom with t >= t0_m
   int32_t* jend = nullptr;       // [n_t0][n_tau] one past the last atom of each window
@@ -208,7 +203,6 @@ struct Workspace {
   // rect
   float4* pa = nullptr;          // [T_ant][N+1][2] FP64 antenna prefix (a2, b2, ab, 0) as hi4, lo4
   float4* px = nullptr;          // [T][N+1][2] float-float data prefix (hi4, lo4)
-  // exp: chunk-major copies of the atoms (perm_entries(N, lanes) per set)
   // refinement: per-template fast statistics, histogram, chosen cut, the
   // candidates (cell, fast 2F, FP64 2F) and the plan's own map (if any)
   TStat* tstat = nullptr;        // [T]
@@ -223,23 +217,15 @@ struct Workspace {
   float* ref_fast = nullptr;     // [T][kRefMaxCells]
   double* ref_val = nullptr;     // [T][kRefMaxCells] (-1: invalid in FP64)
   float* own_map = nullptr;      // [T][cells] (FMAP_PLAN_MAP_BUFFER)
-  float4* perm_ant = nullptr;    // [T_ant][.] (a2, b2, ab, gap to the next atom as int bits; -1 last)
-  float4* perm_x = nullptr;      // [T][.] (Fa re, Fa im, Fb re, Fb im); recurrence plans
-  int32_t* perm_gap = nullptr;   // [.] gap to the next atom (-1 last); recurrence plans
-  // recurrence plans: per cell, tau-major ([n_tau][n_t0]), the window record
-  // (i0, j as int bits, prefactor, tail factor), then a copy of the
-  // coefficients (shared antenna): written by the recurrence kernel's first
-  // template, read by the rest (absent with one template)
-  float4* rec_cells = nullptr;   // [2][cells]
-  // recurrence plans with two or more templates: the FP32 decay after each
-  // atom, per tau in the chunk-major order (first template writes, the rest
-  // read)
-  float* rec_decay = nullptr;    // [n_tau][perm_entries]
+  // exp: one 16-byte entry per atom
+  float4* perm_ant = nullptr;    // [T_ant][N] (a2, b2, ab, gap code)
+  float4* perm_x = nullptr;      // [T][N] (Fa re, Fa im, Fb re, Fb im); recurrence plans
+  float* agg = nullptr;          // chunk maps: antenna [T_ant][n_grp][n_chunks][8][32], then the
+                                 // data's [T][n_grp][n_chunks][8][32] and [n_grp][n_chunks][2][32]
+                                 // decays (where the marked-entry list goes later)
   TauTab* tauc = nullptr;        // [n_tau] per-tau decay constants
   float2* wtab = nullptr;        // table windows: [kTabMax + 1] (w_k, w_{k+1} - w_k), then (0, 0)
   int64_t* ax = nullptr;         // [n_t0 + n_tau] explicit axes: t0 values, then tau values
-  // exp
-  float2* esuf = nullptr;        // [tau_chunk][3][N+1] float-float decayed suffix sums
   // tensor-core operands
   void* xop = nullptr;           // split X operands (layout per precision)
   // host-API staging
@@ -266,7 +252,6 @@ struct fmap_plan_s {
   int n_sm = 0;
   int64_t n_tiles = 0;        // partial slots per template of the main kernels
   int64_t part_stride = 0;    // n_tiles + kFixSlots
-  int32_t tau_chunk = 0;      // exp: tau values per suffix launch
   size_t xop_bytes = 0;
   bool host_staging = false;
   // explicit (t0, tau) axes set by fmap_plan_axes (in ws.ax; else the uniform
@@ -274,7 +259,8 @@ struct fmap_plan_s {
   bool explicit_axes = false;
   std::vector<int64_t> ax_host;
   int32_t n_tab = 0;             // table windows: samples set by fmap_plan_window_table
-  int32_t lanes = fmap::kScanLanes;   // exp scan width (threads per tau)
+  fmap::AntGeom ant[2] = {};     // exp plans: work splits with own [0] / shared [1] antenna rows
+  fmap::RecGeom rec[2] = {};
   // TMA descriptors (CUtensorMap, 128 bytes each) of the split X operands
   alignas(64) unsigned char tmap_hi[128] = {};
   alignas(64) unsigned char tmap_lo[128] = {};
@@ -313,6 +299,9 @@ cudaError_t launch_index(fmap_plan_s* p, const int64_t* d_t, cudaStream_t s);
 cudaError_t launch_rect(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaStream_t s,
                         int64_t* tiles_used, cudaEvent_t mark);
 cudaError_t launch_exp_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
+// Chunk maps of the antenna rows (and, in recurrence plans that start from
+// them, of the data).
+cudaError_t launch_exp_agg(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 cudaError_t launch_exp_perm(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 cudaError_t launch_table_antenna(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 cudaError_t launch_exp_plain(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaStream_t s,
@@ -322,16 +311,21 @@ cudaError_t launch_exp_tc(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cuda
 cudaError_t launch_exp_rec(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaStream_t s,
                            int64_t* tiles_used);
 bool exp_rec_supported(int32_t n_sft, int32_t n_t0);
-bool exp_antenna_fits(int32_t n_sft);
-size_t exp_antenna_smem(int32_t n_sft);
-// Dynamic shared memory of the recurrence for blocks of up to tpb templates.
-size_t exp_rec_smem(int32_t n_sft, int32_t n_t0, int32_t tpb);
+// Work splits of the sweeps (batch: instances of a batch, which fill the GPU
+// together; tpb: most templates per warp of the recurrence, 0: any; agg_room:
+// bytes that the chunk maps may take).
+AntGeom ant_geom(const fmap_grid& g, int32_t n_sft, int64_t n_ant, bool batch, int64_t agg_room);
+RecGeom rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, bool shared, bool batch,
+                 int32_t tpb, int64_t agg_room);
+// Both with the room of a plan's workspace.
+AntGeom plan_ant_geom(const fmap_grid& g, int32_t n_sft, int32_t T, uint32_t flags, bool shared);
+RecGeom plan_rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, uint32_t flags, bool shared,
+                      int32_t tpb);
 // Dispatcher kernels of the batch phases, by file (nullptr: not that file's).
 const void* batch_kernel_common(int phase);
 const void* batch_kernel_rect(int phase);
-// The exp scan phases have one dispatcher per scan width.
-const void* batch_kernel_exp(int phase, int lanes);
-const void* batch_kernel_exp_rec(int phase, int lanes);
+const void* batch_kernel_exp(int phase);
+const void* batch_kernel_exp_rec(int phase, int max_g);
 const void* batch_kernel_fixup(int phase);
 cudaError_t launch_rect_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 cudaError_t launch_flag_and_fixup(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,

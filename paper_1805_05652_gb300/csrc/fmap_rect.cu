@@ -64,12 +64,18 @@ __device__ __forceinline__ void block_exscan(const double (&v)[NC], double (&exc
   __syncthreads();
 }
 
+// Shared memory of the scans (the batch's scan kernel runs both of them).
+struct ScanSmem {
+  float tile[4][kScanTile];
+  double sh[4][kScanThreads];
+};
+
 // Prefix of the data rows of one template: px[t][i] = (hi[4], lo[4]) of
 // sum_{a < i} x_a for i = 0..N.
 __device__ __forceinline__ void rect_scan_data_body(const float* __restrict__ fafb, int32_t n, float4* __restrict__ px,
-    const uint3 bid, const dim3 gdim) {
-  __shared__ float tile[4][kScanTile];
-  __shared__ double sh[4][kScanThreads];
+    const uint3 bid, ScanSmem& sm) {
+  auto& tile = sm.tile;
+  auto& sh = sm.sh;
   const int64_t tm = bid.x;
   const float* x = fafb + tm * 4 * (int64_t)n;
   float4* out = px + tm * 2 * (int64_t)(n + 1);
@@ -119,15 +125,16 @@ __device__ __forceinline__ void rect_scan_data_body(const float* __restrict__ fa
 
 __global__ void __launch_bounds__(kScanThreads)
 k_rect_scan_data(const float* __restrict__ fafb, int32_t n, float4* __restrict__ px) {
-  rect_scan_data_body(fafb, n, px, blockIdx, gridDim);
+  __shared__ ScanSmem sm;
+  rect_scan_data_body(fafb, n, px, blockIdx, sm);
 }
 
 // FP64 prefix of the antenna rows, stored as float pairs: pa[ta][i] =
 // (sum a2, sum b2, sum ab, 0) over a < i.
 __device__ __forceinline__ void rect_scan_antenna_body(const float* __restrict__ antenna, int32_t n, P4* __restrict__ pa,
-    const uint3 bid, const dim3 gdim) {
-  __shared__ float tile[3][kScanTile];
-  __shared__ double sh[3][kScanThreads];
+    const uint3 bid, ScanSmem& sm) {
+  auto& tile = sm.tile;
+  auto& sh = sm.sh;
   const int64_t ta = bid.x;
   const float* x = antenna + ta * 3 * (int64_t)n;
   P4* out = pa + ta * (int64_t)(n + 1);
@@ -174,7 +181,8 @@ __device__ __forceinline__ void rect_scan_antenna_body(const float* __restrict__
 
 __global__ void __launch_bounds__(kScanThreads)
 k_rect_scan_antenna(const float* __restrict__ antenna, int32_t n, P4* __restrict__ pa) {
-  rect_scan_antenna_body(antenna, n, pa, blockIdx, gridDim);
+  __shared__ ScanSmem sm;
+  rect_scan_antenna_body(antenna, n, pa, blockIdx, sm);
 }
 
 // Per-cell coefficients (shared by the templates of one antenna set) from the
@@ -297,48 +305,6 @@ __device__ __forceinline__ void st_stream(float* p, float v) {
 __device__ __forceinline__ void lds_pairs(uint32_t a, uint64_t& xy, uint64_t& zw) {
   asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];\n" : "=l"(xy), "=l"(zw) : "r"(a));
 }
-__device__ __forceinline__ uint64_t pk2(float x, float y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ void up2(uint64_t a, float& x, float& y) {
-  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(x), "=f"(y) : "l"(a));
-}
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("sub.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
-// 2F of one cell from its window sums (fa, fb as f32x2 re/im pairs);
-// nb2 = (-beta, -beta); k1 = -inf marks a cell that takes no part.
-__device__ __forceinline__ float two_f_pairs(uint64_t fa, uint64_t fb, uint64_t nb2, float k1,
-                                             float k2, uint64_t tiny2) {
-  const uint64_t e = fma2(nb2, fa, fb);
-  const uint64_t pa = fma2(fa, fa, tiny2);
-  const uint64_t pe = mul2(e, e);
-  float a0, a1, e0, e1;
-  up2(pa, a0, a1);
-  up2(pe, e0, e1);
-  return fmaf(k1, a0 + a1, k2 * (e0 + e1));
-}
-
 template <bool kShared>
 __device__ __forceinline__ void rect_cells_body(const int32_t* __restrict__ i0tab,
     const int32_t* __restrict__ jend, const Coef* __restrict__ coef,
@@ -718,11 +684,14 @@ cudaError_t launch_rect(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaSt
 
 
 // ---- persistent multi-instance dispatchers (uneven batches) ----
-__global__ void __launch_bounds__(kScanThreads) kb_rect_ant(const BItem* __restrict__ items,
-                                                            BUnits u) {
+__global__ void __launch_bounds__(kScanThreads) kb_rect_scans(const BItem* __restrict__ items,
+                                                              BUnits u) {
+  __shared__ ScanSmem sm;
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
-    rect_scan_antenna_body(it.antenna, it.n_sft, (P4*)it.pa, make_uint3((unsigned)k, 0, 0),
-                           dim3((unsigned)it.n_ant));
+    if (k < it.n_ant)
+      rect_scan_antenna_body(it.antenna, it.n_sft, (P4*)it.pa, make_uint3((unsigned)k, 0, 0), sm);
+    else
+      rect_scan_data_body(it.fafb, it.n_sft, it.px, make_uint3((unsigned)(k - it.n_ant), 0, 0), sm);
   });
 }
 __global__ void __launch_bounds__(256) kb_rect_coef(const BItem* __restrict__ items, BUnits u) {
@@ -732,13 +701,6 @@ __global__ void __launch_bounds__(256) kb_rect_coef(const BItem* __restrict__ it
       rect_coef_body(it.i0, it.jend, (const P4*)it.pa, it.n_sft, it.g.n_t0, it.g.n_tau, it.n_ant,
                      it.coef, it.flag_bits, make_uint3((unsigned)(k * kCoefBlocksPerUnit + q), 0, 0),
                      dim3(nb));
-  });
-}
-__global__ void __launch_bounds__(kScanThreads) kb_rect_data(const BItem* __restrict__ items,
-                                                             BUnits u) {
-  batch_loop(items, u, [&](const BItem& it, int64_t k) {
-    rect_scan_data_body(it.fafb, it.n_sft, it.px, make_uint3((unsigned)k, 0, 0),
-                        dim3((unsigned)it.T));
   });
 }
 __global__ void __launch_bounds__(kCellThreads, 2) kb_rect_cells(const BItem* __restrict__ items,
@@ -757,9 +719,8 @@ __global__ void __launch_bounds__(kCellThreads, 2) kb_rect_cells(const BItem* __
 }
 const void* batch_kernel_rect(int phase) {
   switch (phase) {
-    case BP_RECT_ANT: return (const void*)kb_rect_ant;
+    case BP_RECT_ANT: return (const void*)kb_rect_scans;
     case BP_RECT_COEF: return (const void*)kb_rect_coef;
-    case BP_RECT_DATA: return (const void*)kb_rect_data;
     case BP_RECT_CELLS: return (const void*)kb_rect_cells;
   }
   return nullptr;
