@@ -240,6 +240,7 @@ static fmap_status build_wave_tables(fmap_batch_s* B, Wave& wv, const Tuning& tn
       const int64_t u = units_of(p, B->items[i], ph, tn.rec_tpb);
       off[(size_t)ph * (n + 1) + k + 1] = off[(size_t)ph * (n + 1) + k] + u;
       if (u > 0) {
+        if (ph == BP_RECT_ANT) wv.dyn_smem[ph] = rect_scan_smem();
         if (ph == BP_RECT_CELLS)
           wv.dyn_smem[ph] = std::max(wv.dyn_smem[ph], rect_cells_smem(p->n_templates, B->items[i].atoms.shared_antenna));
       }

@@ -572,15 +572,16 @@ RecGeom rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, bool shared, bool
     win += std::min<double>(n_sft, (double)window_len(g, tau) / (double)g.t_sft) / 16.0;
   }
   const double more = std::min<double>((double)n_sft, std::max(0.0, (double)g.dt0 / (double)g.t_sft - 1.0));
-  const int32_t chunk = n_sft <= 512 ? 16 : n_sft <= 1024 ? 32 : n_sft <= 4096 ? 64 : 128;
-  const int32_t n_chunks = (n_sft + chunk - 1) / chunk;
+  const int32_t chunk0 = n_sft <= 512 ? 16 : n_sft <= 1024 ? 32 : n_sft <= 4096 ? 64 : 128;
   const double slots = kSms * 4.0;
   for (int G = 1; G <= g_max && (G == 1 || G <= T); G *= 2) {
     const int32_t tgrp = std::max(1, (T + G - 1) / G);
     if (G == 4 && (double)n_grp * tgrp < slots) break;   // (few warps per scheduler: two templates)
-    for (int maps = 0; maps < 2; ++maps) {
+    for (int maps = 0; maps < 4; ++maps) {   // none, or chunks of chunk0, 2 chunk0, 4 chunk0
+      const int32_t chunk = chunk0 << std::max(0, maps - 1);
+      const int32_t n_chunks = (n_sft + chunk - 1) / chunk;
       // chunk maps only where there are few warps, and room for them
-      if (maps && (n_sft == 0 || (int64_t)n_grp * T > 4096 ||
+      if (maps && (n_sft == 0 || (!batch && (int64_t)n_grp * T > 4096) ||
                    4 * (int64_t)n_grp * n_chunks * ((int64_t)T * 256 + 64) > agg_room))
         continue;
       const double start = maps ? 0.5 * n_chunks * (30.0 + 90.0 * G) + 1.5 * chunk * (40.0 + 30.0 * G)

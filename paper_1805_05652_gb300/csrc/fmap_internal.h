@@ -374,6 +374,8 @@ int64_t fixup_blocks_y(int32_t n_templates, bool shared);
 int64_t rect_partial_slots(const fmap_grid& g, int32_t n_templates, int32_t shared_antenna);
 int64_t rect_cells_blocks(const fmap_grid& g, int32_t n_templates, int32_t shared_antenna);
 size_t rect_cells_smem(int32_t n_templates, int32_t shared_antenna);
+// Dynamic shared memory of the prefix scans.
+size_t rect_scan_smem();
 int64_t exp_tiles(const fmap_grid& g);
 int64_t marg_tiles(const fmap_grid& g);
 bool exp_tc_available(fmap_precision prec);

@@ -1,7 +1,8 @@
 // Rectangular-window F-map (Eq. winrect).
 //
-// FMAP_FP64: prefix sums over SFTs in FP64, then O(1) differencing per cell.
-//   Every FP64 prefix is kept as an unevaluated float pair hi + lo; a window
+// FMAP_FP64: exact prefix sums over SFTs in 64-bit fixed point, then O(1)
+//   differencing per cell.
+//   Every prefix is kept as an unevaluated float pair hi + lo; a window
 //   sum is (hi_j - hi_i) + (lo_j - lo_i), whose rounding error is relative
 //   to the window sum itself and not to the (possibly much larger) prefix.
 //   The antenna sums A, B, C are differenced in float-float (~2^-44 of the
@@ -18,7 +19,7 @@
 namespace fmap {
 
 constexpr int kScanThreads = 256;
-constexpr int kScanPer = 8;
+constexpr int kScanPer = 4;
 constexpr int kScanTile = kScanThreads * kScanPer;
 constexpr int kCellThreads = 256;
 
@@ -36,153 +37,210 @@ int64_t rect_tiles(const fmap_grid& g) {
          ((g.n_tau + kTileCols - 1) / kTileCols);
 }
 
-// Exclusive block scan of NC doubles per thread (sums of each thread's
-// chunk); returns the thread's exclusive prefix in `excl` and the block total
-// in `total`.
-template <int NC>
-__device__ __forceinline__ void block_exscan(const double (&v)[NC], double (&excl)[NC],
-                                             double (&total)[NC], double (*sh)[kScanThreads]) {
-  const int tid = threadIdx.x;
-#pragma unroll
-  for (int c = 0; c < NC; ++c) sh[c][tid] = v[c];
-  __syncthreads();
-  // Hillis-Steele inclusive scan in shared memory (log2(256) = 8 steps).
-  for (int off = 1; off < kScanThreads; off <<= 1) {
-    double add[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) add[c] = tid >= off ? sh[c][tid - off] : 0.0;
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < NC; ++c) sh[c][tid] += add[c];
-    __syncthreads();
-  }
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    excl[c] = sh[c][tid] - v[c];
-    total[c] = sh[c][kScanThreads - 1];
-  }
-  __syncthreads();
-}
-
-// Shared memory of the scans (the batch's scan kernel runs both of them).
+// Prefix sums of NC rows of n atoms by one block: out[2 i], out[2 i + 1] = hi,
+// lo of sum_{a < i} for i = 0..n (columns past NC are 0).  The sums are exact
+// 64-bit integers in units of 2^-S, S the largest with n max|x| 2^S < 2^61 per
+// row, and the pair holds the top 48 bits.  (The same scan in FP64, which GB300
+// runs at 1/64 of the FP32 rate, took eight FP64 operations per atom and row:
+// 423 us for 1024 templates of 5000 atoms, and 24 us for one block alone.)
+// The unit is fixed by the row's maximum, so rows whose level changes by more
+// than 2^35 / n from one stretch of 32 atoms to another (an outlier or a step;
+// the windows before it would lose their sums), rows below 2^-58 and blocks of
+// fewer than 64 atoms are summed in FP64.
+// A tile of kScanTile atoms at a time: each thread sums kScanPer neighbours,
+// the warps scan the threads' sums by shuffles, and the entries leave through
+// shared memory so that the block writes whole lines.
 struct ScanSmem {
   float tile[4][kScanTile];
-  double sh[4][kScanThreads];
+  float4 ent[2 * kScanTile];
+  unsigned long long wsum[4][kScanThreads / 32];
+  float wmax[4][kScanThreads / 32], wmin[4][kScanThreads / 32];
+};
+constexpr int32_t kScanFixMin = 64;   // fewest atoms of an integer scan
+
+// Exponent e of a row with maximum mx (mx < 2^e).
+__host__ __device__ inline int scan_exponent(float mx) {
+  int e = 0;
+  if (mx > 0.0f) frexpf(mx, &e);
+  return e;
+}
+// Place of entry float4 k in the staging buffer: a thread's entries are 2 kScanPer
+// float4 apart, so the low three bits take its number and a warp's stores spread
+// over the banks.
+__device__ __forceinline__ int scan_place(int k) { return k ^ ((k / (2 * kScanPer)) & 7); }
+
+// The two accumulators: integers in units of down = 1 / up (both powers of two;
+// the scaling is exact but for underflow), and FP64.
+template <typename Acc> struct ScanAcc;
+template <> struct ScanAcc<unsigned long long> {
+  static __device__ __forceinline__ unsigned long long in(float x, float up) {
+    return (unsigned long long)__float2ll_rn(x * up);
+  }
+  static __device__ __forceinline__ float2 pair(unsigned long long v, float down) {
+    const float h = __ll2float_rn((long long)v);
+    return make_float2(h * down, __ll2float_rn((long long)v - __float2ll_rn(h)) * down);
+  }
+};
+template <> struct ScanAcc<double> {
+  static __device__ __forceinline__ double in(float x, float) { return (double)x; }
+  static __device__ __forceinline__ float2 pair(double v, float) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+  }
 };
 
-// Prefix of the data rows of one template: px[t][i] = (hi[4], lo[4]) of
-// sum_{a < i} x_a for i = 0..N.
-__device__ __forceinline__ void rect_scan_data_body(const float* __restrict__ fafb, int32_t n, float4* __restrict__ px,
-    const uint3 bid, ScanSmem& sm) {
-  auto& tile = sm.tile;
-  auto& sh = sm.sh;
-  const int64_t tm = bid.x;
-  const float* x = fafb + tm * 4 * (int64_t)n;
-  float4* out = px + tm * 2 * (int64_t)(n + 1);
-  const int tid = threadIdx.x;
-  double carry[4] = {0.0, 0.0, 0.0, 0.0};
-  if (tid == 0) {
-    out[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-    out[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  for (int64_t base = 0; base < n; base += kScanTile) {
-    for (int k = tid; k < kScanTile; k += kScanThreads) {
-      const int64_t a = base + k;
+template <int NC, typename Acc>
+__device__ __forceinline__ void rect_scan_tiles(const float* __restrict__ x, int32_t n,
+                                                const float (&up)[NC], const float (&down)[NC],
+                                                float4* __restrict__ out, ScanSmem& sm) {
+  constexpr int NW = kScanThreads / 32;
+  using A = ScanAcc<Acc>;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  Acc(*wsum)[NW] = reinterpret_cast<Acc(*)[NW]>(sm.wsum);
+  Acc carry[NC];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) tile[c][k] = a < n ? x[c * (int64_t)n + a] : 0.0f;
-    }
+  for (int c = 0; c < NC; ++c) carry[c] = Acc(0);
+  for (int32_t base = 0; base < n; base += kScanTile) {
     __syncthreads();
-    double loc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = tid; k < kScanTile; k += kScanThreads)
 #pragma unroll
-    for (int e = 0; e < kScanPer; ++e)
+      for (int c = 0; c < NC; ++c) sm.tile[c][k] = base + k < n ? x[c * (int64_t)n + base + k] : 0.0f;
+    __syncthreads();
+    Acc v[NC][kScanPer], own[NC], inc[NC];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) loc[c] += (double)tile[c][tid * kScanPer + e];
-    double ex[4], tot[4];
-    block_exscan<4>(loc, ex, tot, sh);
-    double run[4];
+    for (int c = 0; c < NC; ++c) {
+      own[c] = Acc(0);
+      const float4* t4 = reinterpret_cast<const float4*>(&sm.tile[c][tid * kScanPer]);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) run[c] = carry[c] + ex[c];
+      for (int e = 0; e < kScanPer; e += 4) {
+        const float4 t = t4[e / 4];
+        v[c][e] = A::in(t.x, up[c]);
+        v[c][e + 1] = A::in(t.y, up[c]);
+        v[c][e + 2] = A::in(t.z, up[c]);
+        v[c][e + 3] = A::in(t.w, up[c]);
+        own[c] += v[c][e] + v[c][e + 1] + v[c][e + 2] + v[c][e + 3];
+      }
+      inc[c] = own[c];
+    }
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const Acc y = __shfl_up_sync(0xffffffffu, inc[c], d);
+        if (lane >= d) inc[c] += y;
+      }
+    if (lane == 31)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) wsum[c][warp] = inc[c];
+    __syncthreads();
+    Acc run[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      run[c] = carry[c];
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const Acc t = wsum[c][w];
+        if (w < warp) run[c] += t;
+        carry[c] += t;
+      }
+      const Acc before = __shfl_up_sync(0xffffffffu, inc[c], 1);
+      if (lane > 0) run[c] += before;
+    }
 #pragma unroll
     for (int e = 0; e < kScanPer; ++e) {
-      const int64_t a = base + tid * kScanPer + e;
-      float hi[4], lo[4];
+      float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        run[c] += (double)tile[c][tid * kScanPer + e];
-        hi[c] = (float)run[c];
-        lo[c] = (float)(run[c] - (double)hi[c]);
+      for (int c = 0; c < NC; ++c) {
+        run[c] += v[c][e];
+        const float2 p = A::pair(run[c], down[c]);
+        hi[c] = p.x;
+        lo[c] = p.y;
       }
-      if (a < n) {
-        out[2 * (a + 1)] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-        out[2 * (a + 1) + 1] = make_float4(lo[0], lo[1], lo[2], lo[3]);
-      }
+      const int k = 2 * (tid * kScanPer + e);
+      sm.ent[scan_place(k)] = make_float4(hi[0], hi[1], hi[2], hi[3]);
+      sm.ent[scan_place(k + 1)] = make_float4(lo[0], lo[1], lo[2], lo[3]);
     }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) carry[c] += tot[c];
     __syncthreads();
+    const int32_t m = 2 * min(kScanTile, n - base);
+    for (int32_t k = tid; k < m; k += kScanThreads) out[2 * (int64_t)(base + 1) + k] = sm.ent[scan_place(k)];
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads)
-k_rect_scan_data(const float* __restrict__ fafb, int32_t n, float4* __restrict__ px) {
-  __shared__ ScanSmem sm;
-  rect_scan_data_body(fafb, n, px, blockIdx, sm);
+// (out of line: the common path's registers and instructions stay its own)
+template <int NC>
+__device__ __noinline__ void rect_scan_fp64(const float* __restrict__ x, int32_t n,
+                                            float4* __restrict__ out, ScanSmem& sm) {
+  const float one[NC] = {};
+  rect_scan_tiles<NC, double>(x, n, one, one, out, sm);
 }
 
-// FP64 prefix of the antenna rows, stored as float pairs: pa[ta][i] =
-// (sum a2, sum b2, sum ab, 0) over a < i.
-__device__ __forceinline__ void rect_scan_antenna_body(const float* __restrict__ antenna, int32_t n, P4* __restrict__ pa,
-    const uint3 bid, ScanSmem& sm) {
-  auto& tile = sm.tile;
-  auto& sh = sm.sh;
-  const int64_t ta = bid.x;
-  const float* x = antenna + ta * 3 * (int64_t)n;
-  P4* out = pa + ta * (int64_t)(n + 1);
-  const int tid = threadIdx.x;
-  double carry[3] = {0.0, 0.0, 0.0};
-  if (tid == 0) out[0] = P4{make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-  for (int64_t base = 0; base < n; base += kScanTile) {
-    for (int k = tid; k < kScanTile; k += kScanThreads) {
-      const int64_t a = base + k;
+template <int NC>
+__device__ __forceinline__ void rect_scan_body(const float* __restrict__ x, int32_t n,
+                                               float4* __restrict__ out, ScanSmem& sm) {
+  constexpr int NW = kScanThreads / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < 2) out[tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool fix = n >= kScanFixMin;
+  float up[NC], down[NC];
+  if (fix) {
+    // each row's maximum, and the smallest maximum of its stretches of 32 atoms
+    // (all-zero stretches do not count)
+    float mx[NC], mn[NC];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) tile[c][k] = a < n ? x[c * (int64_t)n + a] : 0.0f;
-    }
-    __syncthreads();
-    double loc[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int e = 0; e < kScanPer; ++e)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) loc[c] += (double)tile[c][tid * kScanPer + e];
-    double ex[3], tot[3];
-    block_exscan<3>(loc, ex, tot, sh);
-    double run[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) run[c] = carry[c] + ex[c];
-#pragma unroll
-    for (int e = 0; e < kScanPer; ++e) {
-      const int64_t a = base + tid * kScanPer + e;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) run[c] += (double)tile[c][tid * kScanPer + e];
-      if (a < n) {
-        float hi[3], lo[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          hi[c] = (float)run[c];
-          lo[c] = (float)(run[c] - (double)hi[c]);
-        }
-        out[a + 1] = P4{make_float4(hi[0], hi[1], hi[2], 0.f), make_float4(lo[0], lo[1], lo[2], 0.f)};
+    for (int c = 0; c < NC; ++c) {
+      mx[c] = 0.0f;
+      mn[c] = 3.402823466e38f;
+#pragma unroll 4
+      for (int32_t a = tid; a < n + lane - 31; a += kScanThreads) {   // (whole stretches)
+        const float m = __uint_as_float(
+            __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(x[c * (int64_t)n + a]))));
+        mx[c] = fmaxf(mx[c], m);
+        if (m > 0.0f) mn[c] = fminf(mn[c], m);
+      }
+      const int32_t rest = n & ~31;   // the last atoms: part of the maximum only
+      if (warp == 0 && rest + lane < n) mx[c] = fmaxf(mx[c], fabsf(x[c * (int64_t)n + rest + lane]));
+      mx[c] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx[c])));
+      if (lane == 0) {
+        sm.wmax[c][warp] = mx[c];
+        sm.wmin[c][warp] = mn[c];
       }
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) carry[c] += tot[c];
     __syncthreads();
+    const int bits = 32 - __clz(n);   // n < 2^bits
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        mx[c] = fmaxf(mx[c], sm.wmax[c][w]);
+        mn[c] = fminf(mn[c], sm.wmin[c][w]);
+      }
+      const int e = scan_exponent(mx[c]), S = 61 - bits - e;
+      fix = fix && (mx[c] == 0.0f || (S <= 119 && S >= -100 && scan_exponent(mn[c]) >= e + bits - 35));
+      const int Sc = max(-100, min(119, S));
+      up[c] = __int_as_float((Sc + 127) << 23);
+      down[c] = __int_as_float((127 - Sc) << 23);
+    }
   }
+  if (fix) rect_scan_tiles<NC, unsigned long long>(x, n, up, down, out, sm);
+  else rect_scan_fp64<NC>(x, n, out, sm);
 }
 
-__global__ void __launch_bounds__(kScanThreads)
-k_rect_scan_antenna(const float* __restrict__ antenna, int32_t n, P4* __restrict__ pa) {
-  __shared__ ScanSmem sm;
-  rect_scan_antenna_body(antenna, n, pa, blockIdx, sm);
+// Scans of the antenna sets (blocks [0, n_ant)), then of the templates' data.
+__device__ __forceinline__ void rect_scan_unit(const float* antenna, const float* fafb, int32_t n,
+                                               int32_t n_ant, P4* pa, float4* px, int32_t b,
+                                               ScanSmem& sm) {
+  if (b < n_ant)
+    rect_scan_body<3>(antenna + (int64_t)b * 3 * n, n, (float4*)(pa + (int64_t)b * (n + 1)), sm);
+  else
+    rect_scan_body<4>(fafb + (int64_t)(b - n_ant) * 4 * n, n,
+                      px + (int64_t)(b - n_ant) * 2 * (n + 1), sm);
+}
+
+__global__ void __launch_bounds__(kScanThreads, 2)
+k_rect_scans(const float* __restrict__ antenna, const float* __restrict__ fafb, int32_t n,
+             int32_t n_ant, P4* __restrict__ pa, float4* __restrict__ px) {
+  extern __shared__ __align__(16) unsigned char s_scan[];
+  rect_scan_unit(antenna, fafb, n, n_ant, pa, px, blockIdx.x, *reinterpret_cast<ScanSmem*>(s_scan));
 }
 
 // Per-cell coefficients (shared by the templates of one antenna set) from the
@@ -621,10 +679,17 @@ cudaError_t launch_rect_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s
   if (cells == 0) return cudaSuccess;
   const int n_ant = a->shared_antenna ? 1 : p->n_templates;
   if (n_ant == 0) return cudaSuccess;
+  // the FP32 form takes its data sums from the atoms
+  const int n_x = p->precision == FMAP_FP32 ? 0 : p->n_templates;
   if (p->n_sft > 0) {
-    k_rect_scan_antenna<<<n_ant, kScanThreads, 0, s>>>(a->antenna, p->n_sft, (P4*)p->ws.pa);
+    cudaError_t e = cudaFuncSetAttribute(k_rect_scans, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(ScanSmem));
+    if (e != cudaSuccess) return e;
+    k_rect_scans<<<(unsigned)(n_ant + n_x), kScanThreads, sizeof(ScanSmem), s>>>(
+        a->antenna, a->fafb, p->n_sft, n_ant, (P4*)p->ws.pa, p->ws.px);
   } else {
     cudaMemsetAsync(p->ws.pa, 0, sizeof(P4) * n_ant, s);
+    cudaMemsetAsync(p->ws.px, 0, 2 * sizeof(float4) * p->n_templates, s);
   }
   const int64_t total = cells * n_ant;
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)p->n_sm * 16);
@@ -650,12 +715,6 @@ cudaError_t launch_rect(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaSt
                                                   d_2F, p->ws.partials, p->part_stride);
     p->launches += 1;
     return cudaGetLastError();
-  }
-  if (p->n_sft > 0) {
-    k_rect_scan_data<<<p->n_templates, kScanThreads, 0, s>>>(a->fafb, p->n_sft, p->ws.px);
-    p->launches += 1;
-  } else {
-    cudaMemsetAsync(p->ws.px, 0, 2 * sizeof(float4) * p->n_templates, s);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -684,16 +743,15 @@ cudaError_t launch_rect(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaSt
 
 
 // ---- persistent multi-instance dispatchers (uneven batches) ----
-__global__ void __launch_bounds__(kScanThreads) kb_rect_scans(const BItem* __restrict__ items,
+__global__ void __launch_bounds__(kScanThreads, 2) kb_rect_scans(const BItem* __restrict__ items,
                                                               BUnits u) {
-  __shared__ ScanSmem sm;
+  extern __shared__ __align__(16) unsigned char s_scan[];
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
-    if (k < it.n_ant)
-      rect_scan_antenna_body(it.antenna, it.n_sft, (P4*)it.pa, make_uint3((unsigned)k, 0, 0), sm);
-    else
-      rect_scan_data_body(it.fafb, it.n_sft, it.px, make_uint3((unsigned)(k - it.n_ant), 0, 0), sm);
+    rect_scan_unit(it.antenna, it.fafb, it.n_sft, it.n_ant, (P4*)it.pa, it.px, (int32_t)k,
+                   *reinterpret_cast<ScanSmem*>(s_scan));
   });
 }
+size_t rect_scan_smem() { return sizeof(ScanSmem); }
 __global__ void __launch_bounds__(256) kb_rect_coef(const BItem* __restrict__ items, BUnits u) {
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
     const unsigned nb = (unsigned)((it.cells * it.n_ant + 255) / 256);
