@@ -185,7 +185,7 @@ static Layout layout_of(const fmap_grid* g, int32_t n_sft, int32_t T, fmap_preci
     return at;
   };
   L.rel_t = take(sizeof(int32_t) * (size_t)rel_t_entries(n_sft));
-  L.t_base = take(sizeof(int64_t) + sizeof(int32_t));
+  L.t_base = take(sizeof(int64_t) + sizeof(int32_t) * kIrrWords);
   L.irr = L.t_base + sizeof(int64_t);
   L.dev_err = take(sizeof(uint32_t));
   L.i0 = take(sizeof(int32_t) * std::max<int32_t>(g->n_t0, 1));
@@ -574,14 +574,7 @@ static fmap_status enqueue(fmap_plan_t* p, const fmap_atoms* a, float* d_2F,
   cudaEvent_t ev[FMAP_N_PHASES + 1] = {};
   if (evp)
     for (int k = 0; k <= FMAP_N_PHASES; ++k) ev[k] = evp[k];
-  FMAP_CUDA(launch_prep(p, a, s));
-  {   // the bitmask of ill-conditioned entries, set by the coefficient kernels
-    const int64_t ent = (int64_t)p->grid.n_t0 * p->grid.n_tau *
-                        (a->shared_antenna ? 1 : std::max<int32_t>(p->n_templates, 1));
-    if (ent > 0)
-      FMAP_CUDA(cudaMemsetAsync(p->ws.flag_bits, 0, sizeof(uint32_t) * (size_t)flag_words(ent), s));
-  }
-  FMAP_CUDA(launch_index(p, a->t, s));
+  FMAP_CUDA(launch_front(p, a, s));
   if (ev[1]) FMAP_CUDA(cudaEventRecord(ev[1], s));
   int64_t tiles = 0;
   if (window == FMAP_RECT) {
@@ -595,7 +588,6 @@ static fmap_status enqueue(fmap_plan_t* p, const fmap_atoms* a, float* d_2F,
     else
       FMAP_CUDA(launch_exp_plain(p, a, d_2F, s, &tiles));
   } else {
-    FMAP_CUDA(launch_exp_perm(p, a, s));
     FMAP_CUDA(launch_exp_agg(p, a, s));
     FMAP_CUDA(launch_exp_coef(p, a, s));
     if (ev[2]) FMAP_CUDA(cudaEventRecord(ev[2], s));

@@ -1,188 +1,11 @@
-// Kernels shared by both windows: input preparation, the window index tables
-// (Eq. Fmn grid, window membership of Eq. winrect / winexp), the final
-// per-template reduction and the standalone marginalisation.
+// Kernels shared by both windows: the final per-template reduction, the standalone
+// marginalisation, and a batch's input and index phases.
 #include <math.h>
 
 #include "fmap_batch.cuh"
-#include "fmap_device.cuh"
+#include "fmap_front.cuh"
 
 namespace fmap {
-
-// Non-finite check of n values (antenna or data rows): DEV_ERR_NONFINITE
-// is latched if any is NaN or infinite (|x| <= FLT_MAX fails for both; one
-// atomic per warp at most).
-__device__ __forceinline__ void finite_check(const float* __restrict__ v, int64_t n,
-                                             int64_t i0, int64_t step, uint32_t* __restrict__ err) {
-  bool bad = false;
-  for (int64_t i = i0; i < n; i += step) bad |= !(fabsf(v[i]) <= 3.402823466e38f);
-  const unsigned who = __ballot_sync(__activemask(), bad);
-  if (bad && (int)(threadIdx.x & 31) == __ffs(who) - 1) atomicOr(err, DEV_ERR_NONFINITE);
-}
-
-// t -> t - t[0] as int32, with the data checks (strictly increasing,
-// span < 2^31 s) latched into the plan's status word, and the atoms' values
-// checked for NaN and infinities.
-__device__ __forceinline__ void prep_body(const int64_t* __restrict__ t, int32_t n, int32_t n_alloc,
-                       int32_t* __restrict__ rel_t, int64_t* __restrict__ t_base,
-                       uint32_t* __restrict__ err, const float* __restrict__ ant, int64_t n_ant_vals,
-                       const float* __restrict__ x, int64_t n_x_vals, int32_t* __restrict__ irr,
-    const uint3 bid, const dim3 gdim) {
-  if (bid.x == 0 && threadIdx.x == 0) *irr = 0;   // (set by the exp copy step)
-  {
-    const int64_t g0 = bid.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t step = (int64_t)gdim.x * blockDim.x;
-    if (ant) finite_check(ant, n_ant_vals, g0, step, err);
-    if (x) finite_check(x, n_x_vals, g0, step, err);
-  }
-  if (n <= 0) return;
-  const int64_t base = t[0];
-  for (int64_t i = n + bid.x * (int64_t)blockDim.x + threadIdx.x; i < n_alloc;
-       i += (int64_t)gdim.x * blockDim.x)
-    rel_t[i] = 0;
-  for (int64_t i = bid.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gdim.x * blockDim.x) {
-    const int64_t ti = t[i];
-    const int64_t d = ti - base;
-    uint32_t e = 0;
-    if (d < 0 || d > 0x7fffffffLL - 1) e |= DEV_ERR_SPAN;
-    if (i + 1 < n && t[i + 1] <= ti) e |= DEV_ERR_ORDER;
-    if (e) atomicOr(err, e);
-    rel_t[i] = (int32_t)(d & 0x7fffffffLL);
-    if (i == 0) *t_base = base;
-  }
-}
-
-__global__ void k_prep(const int64_t* __restrict__ t, int32_t n, int32_t n_alloc,
-                       int32_t* __restrict__ rel_t, int64_t* __restrict__ t_base,
-                       uint32_t* __restrict__ err, const float* __restrict__ ant,
-                       int64_t n_ant_vals, const float* __restrict__ x, int64_t n_x_vals,
-                       int32_t* __restrict__ irr) {
-  prep_body(t, n, n_alloc, rel_t, t_base, err, ant, n_ant_vals, x, n_x_vals, irr, blockIdx, gridDim);
-}
-
-// Window index tables: i0[m] = first atom with t >= t0_m; jend[m][n] = one
-// past the last atom whose SFT ends by t0_m + L_n (L = window_len(tau_n)),
-// clamped to >= i0[m], so the window holds atoms [i0, jend).  One block per
-// group of kIdxGroup t0 rows: each warp finds one row's atom range
-// [i0, j(n_tau - 1)) by a warp-wide search, the union of the group's ranges
-// of relative times is staged in shared memory once (coalesced), and every
-// (row, tau) searches it there; longer unions search global memory.
-constexpr int kIdxThreads = 256;
-constexpr int kIdxGroup = kIdxThreads / 32;   // t0 rows per block pass (one warp each)
-constexpr int kIdxCap = 8192;   // staged relative times (32 KB)
-
-// First index in [lo, hi) of the ascending int32 times with t > x (int64).
-__device__ __forceinline__ int32_t upper_bound_i32(const int32_t* t, int32_t lo, int32_t hi,
-                                                   int64_t x) {
-  while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    if ((int64_t)t[mid] <= x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// The same search by one whole warp: 32 probes per round narrow the range
-// 32-fold, so a data set of N atoms takes ~log32(N) dependent loads instead
-// of log2(N).  Returns the first index in [lo, hi) whose time exceeds x (hi
-// if none) to every lane.
-__device__ __forceinline__ int32_t warp_upper_bound_i32(const int32_t* t, int32_t lo, int32_t hi,
-                                                        int64_t x, int lane) {
-  while (hi - lo > 32) {
-    const int32_t step = (hi - lo + 31) / 32;
-    const int32_t p = lo + lane * step;
-    const bool le = p < hi && (int64_t)t[p] <= x;   // the probes below the answer
-    const int c = __popc(__ballot_sync(0xffffffffu, le));
-    if (c == 0) return lo;
-    const int32_t base = lo;
-    lo = base + (c - 1) * step + 1;
-    hi = min(hi, base + c * step);
-  }
-  const int32_t p = lo + lane;
-  const bool le = p < hi && (int64_t)t[p] <= x;
-  return lo + __popc(__ballot_sync(0xffffffffu, le));
-}
-
-__device__ __forceinline__ void index_body(const int32_t* __restrict__ rel_t,
-                                           const int64_t* __restrict__ t_base, int32_t n_sft,
-                                           fmap_grid g, const int64_t* __restrict__ ax,
-                                           int32_t* __restrict__ i0tab,
-                                           int32_t* __restrict__ jend, int32_t m0, int32_t R) {
-  __shared__ int32_t s_t[kIdxCap];
-  __shared__ int32_t s_lo[kIdxGroup], s_hi[kIdxGroup];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t tb = n_sft > 0 ? *t_base : 0;
-  const int64_t lmax = window_len(g, grid_tau(g, ax, g.n_tau - 1)) - g.t_sft;
-  if (warp < R) {   // warp r: row m0 + r's first atom with t >= t0 and the last any window takes
-    const int32_t m = m0 + warp;
-    const int64_t t0rel = grid_t0(g, ax, m) - tb;
-    const int32_t lo = warp_upper_bound_i32(rel_t, 0, n_sft, t0rel - 1, lane);
-    const int32_t hi = max(lo, warp_upper_bound_i32(rel_t, lo, n_sft, t0rel + lmax, lane));
-    if (lane == 0) {
-      s_lo[warp] = lo;
-      s_hi[warp] = hi;
-      i0tab[m] = lo;
-    }
-  }
-  __syncthreads();
-  // Both ends grow with t0, so the group's rows search within [lo of its
-  // first row, hi of its last), staged once when it fits.
-  const int32_t base = s_lo[0], span = s_hi[R - 1] - base;
-  const bool staged = span <= kIdxCap;
-  if (staged)
-    for (int k = tid; k < span; k += kIdxThreads) s_t[k] = rel_t[base + k];
-  __syncthreads();
-  for (int32_t r = 0; r < R; ++r) {   // no barrier between rows: their searches overlap
-    const int32_t m = m0 + r, lo = s_lo[r], hi = s_hi[r];
-    const int64_t t0rel = grid_t0(g, ax, m) - tb;
-    int32_t* row = jend + (int64_t)m * g.n_tau;
-    for (int32_t nn = tid; nn < g.n_tau; nn += kIdxThreads) {
-      const int64_t lim = t0rel + window_len(g, grid_tau(g, ax, nn)) - g.t_sft;
-      row[nn] = staged ? base + upper_bound_i32(s_t, lo - base, hi - base, lim)
-                       : upper_bound_i32(rel_t, lo, hi, lim);
-    }
-  }
-  __syncthreads();   // s_t, s_lo and s_hi are reused by the block's next group
-}
-
-__global__ void __launch_bounds__(kIdxThreads)
-k_index(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base, int32_t n_sft,
-        fmap_grid g, const int64_t* __restrict__ ax, int32_t* __restrict__ i0tab,
-        int32_t* __restrict__ jend, int32_t grp) {
-  const int32_t n_grp = (g.n_t0 + grp - 1) / grp;
-  for (int32_t q = blockIdx.x; q < n_grp; q += gridDim.x)
-    index_body(rel_t, t_base, n_sft, g, ax, i0tab, jend, q * grp, min(grp, g.n_t0 - q * grp));
-}
-
-cudaError_t launch_prep(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
-  if (p->n_sft <= 0) return cudaSuccess;
-  const int threads = 256;
-  const int64_t n = p->n_sft;
-  const int64_t n_ant = 3 * n * (a->shared_antenna ? 1 : std::max<int32_t>(p->n_templates, 1));
-  const int64_t n_x = 4 * n * (int64_t)p->n_templates;
-  // enough threads for the timestamps, and for the value checks at a few
-  // values per thread
-  const int64_t want = std::max<int64_t>(n, (n_ant + n_x) / 8);
-  const int blocks = (int)std::min<int64_t>((want + threads - 1) / threads, (int64_t)p->n_sm * 16);
-  k_prep<<<std::max(blocks, 1), threads, 0, s>>>(a->t, p->n_sft, rel_t_entries(p->n_sft),
-                                                 p->ws.rel_t, p->ws.t_base, p->ws.dev_err,
-                                                 a->antenna, n_ant, a->fafb, n_x, p->ws.irr);
-  p->launches += 1;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_index(fmap_plan_s* p, const int64_t* d_t, cudaStream_t s) {
-  (void)d_t;
-  const int64_t cells = (int64_t)p->grid.n_t0 * p->grid.n_tau;
-  if (cells == 0) return cudaSuccess;
-  // rows per group: as many as keep about four blocks per SM busy (1..8)
-  const int32_t grp = (int32_t)std::max<int64_t>(
-      1, std::min<int64_t>(kIdxGroup, p->grid.n_t0 / ((int64_t)p->n_sm * 4)));
-  const int blocks = (int)std::min<int64_t>((p->grid.n_t0 + grp - 1) / grp, (int64_t)p->n_sm * 8);
-  k_index<<<blocks, kIdxThreads, 0, s>>>(p->ws.rel_t, p->ws.t_base, p->n_sft, p->grid, plan_axes(p),
-                                         p->ws.i0, p->ws.jend, grp);
-  p->launches += 1;
-  return cudaGetLastError();
-}
 
 // ---------------------------------------------------------------------------
 // Final reduction in two levels, accumulated in FP64: level 1 merges groups of
@@ -467,10 +290,11 @@ __global__ void __launch_bounds__(256) kb_prep(const BItem* __restrict__ items, 
 }
 static_assert(kIdxRowsPerUnit == kIdxGroup, "a batch index unit is one row group");
 __global__ void __launch_bounds__(kIdxThreads) kb_index(const BItem* __restrict__ items, BUnits u) {
+  __shared__ IndexSmem sm;
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
     const int32_t m0 = (int32_t)k * kIdxRowsPerUnit;
-    index_body(it.rel_t, it.t_base, it.n_sft, it.g, it.ax, it.i0, it.jend, m0,
-               min(kIdxRowsPerUnit, it.g.n_t0 - m0));
+    index_body(RelStored{it.rel_t}, it.n_sft > 0 ? *it.t_base : 0, it.n_sft, it.g, it.ax, it.i0,
+               it.jend, m0, min(kIdxRowsPerUnit, it.g.n_t0 - m0), sm);
   });
 }
 __global__ void __launch_bounds__(kRedThreads) kb_red_groups(const BItem* __restrict__ items,

@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "fmap_batch.cuh"
+#include "fmap_front.cuh"
 #include "fmap_sweep.cuh"
 
 namespace fmap {
@@ -191,7 +192,7 @@ k_exp_antenna(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_b
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t unit = (int64_t)blockIdx.x * kAntWarps + warp;
   if (unit >= units) return;
-  if (*irr)
+  if (irregular(irr))
     exp_antenna_unit<true>(rel_t, t_base, n, g, ant, tauc, ax, i0tab, jend, q, agg, coef, bits,
                            unit, s_pw[warp], lane);
   else
@@ -222,66 +223,6 @@ AntGeom ant_geom(const fmap_grid& g, int32_t n_sft, int64_t n_ant, bool batch, i
   }
   if (1024 * warps * q.n_chunks > agg_room) q.n_chunks = 0;
   return q;
-}
-
-// Copies of one instance's atoms for the sweeps, one 16-byte entry per atom:
-// sets 0..n_ant-1 the antenna rows with the code of the gap to the next atom
-// (gap_code), sets n_ant.. the data rows of each template (recurrence plans);
-// before them the per-tau constants (two entries per tau).
-__device__ __forceinline__ void exp_perm_body(const int32_t* __restrict__ rel_t, int32_t n,
-                                              const float* __restrict__ antenna, int32_t n_ant,
-                                              const float* __restrict__ fafb, int32_t n_x,
-                                              float4* __restrict__ perm_ant,
-                                              float4* __restrict__ perm_x,
-                                              int32_t* __restrict__ irr, const fmap_grid& g,
-                                              const int64_t* __restrict__ ax,
-                                              TauTab* __restrict__ tauc, int64_t e_begin,
-                                              int64_t e_end, int64_t e_step) {
-  const int64_t n_tau2 = 2 * (int64_t)g.n_tau;
-  for (int64_t e0 = e_begin; e0 < e_end; e0 += e_step) {
-    if (e0 < n_tau2) {   // the longest entries first
-      tau_tab_fill(g, grid_tau(g, ax, e0 >> 1), (int)(e0 & 1), tauc + (e0 >> 1));
-      continue;
-    }
-    const int64_t e = e0 - n_tau2;
-    const int64_t set = e / n, i = e - set * n;
-    if (set < n_ant) {
-      const float* a = antenna + set * 3 * (int64_t)n;
-      const int32_t t = rel_t[i];
-      const int32_t code = i + 1 < n ? gap_code(rel_t[i + 1] - t, (int32_t)g.t_sft) : -1;
-      perm_ant[e] = make_float4(a[i], a[n + i], a[2 * (int64_t)n + i], __int_as_float(code));
-      if (set == 0 && code == 0) *irr = 1;   // (cleared by the input checks)
-    } else {
-      const int64_t tq = set - n_ant;
-      const float* x = fafb + tq * 4 * (int64_t)n;
-      perm_x[tq * n + i] = make_float4(x[i], x[n + i], x[2 * (int64_t)n + i], x[3 * (int64_t)n + i]);
-    }
-  }
-}
-
-__global__ void k_exp_perm(const int32_t* __restrict__ rel_t, int32_t n,
-                           const float* __restrict__ antenna, int32_t n_ant,
-                           const float* __restrict__ fafb, int32_t n_x,
-                           float4* __restrict__ perm_ant, float4* __restrict__ perm_x,
-                           int32_t* __restrict__ irr, const fmap_grid g,
-                           const int64_t* __restrict__ ax, TauTab* __restrict__ tauc) {
-  const int64_t total = exp_copy_entries(n, n_ant, n_x, g.n_tau);
-  exp_perm_body(rel_t, n, antenna, n_ant, fafb, n_x, perm_ant, perm_x, irr, g, ax, tauc,
-                (int64_t)blockIdx.x * blockDim.x + threadIdx.x, total,
-                (int64_t)gridDim.x * blockDim.x);
-}
-
-cudaError_t launch_exp_perm(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
-  if ((int64_t)p->grid.n_t0 * p->grid.n_tau == 0) return cudaSuccess;
-  const int32_t n_ant = a->shared_antenna ? 1 : p->n_templates;
-  const int32_t n_x = p->ws.perm_x ? p->n_templates : 0;
-  const int64_t total = exp_copy_entries(p->n_sft, n_ant, n_x, p->grid.n_tau);
-  const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)p->n_sm * 16);
-  k_exp_perm<<<blocks, 256, 0, s>>>(p->ws.rel_t, p->n_sft, a->antenna, n_ant, a->fafb, n_x,
-                                    p->ws.perm_ant, p->ws.perm_x, p->ws.irr, p->grid,
-                                    plan_axes(p), p->ws.tauc);
-  p->launches += 1;
-  return cudaGetLastError();
 }
 
 cudaError_t launch_exp_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
@@ -441,8 +382,8 @@ __global__ void __launch_bounds__(256) kb_exp_perm(const BItem* __restrict__ ite
     const int32_t n_x = it.perm_x ? it.T : 0;
     const int64_t total = exp_copy_entries(it.n_sft, it.n_ant, n_x, it.g.n_tau);
     const int64_t e0 = k * kPermPerUnit;
-    exp_perm_body(it.rel_t, it.n_sft, it.antenna, it.n_ant, it.fafb, n_x, it.perm_ant, it.perm_x,
-                  it.irr, it.g, it.ax, it.tauc, e0 + threadIdx.x, min(total, e0 + kPermPerUnit), 256);
+    exp_perm_body(RelStored{it.rel_t}, it.n_sft, it.antenna, it.n_ant, it.fafb, n_x, it.perm_ant, it.perm_x,
+                  it.irr, it.dev_err, it.g, it.ax, it.tauc, e0 + threadIdx.x, min(total, e0 + kPermPerUnit), 256);
   });
 }
 __global__ void __launch_bounds__(kAntThreads, 2) kb_exp_ant(const BItem* __restrict__ items,
@@ -452,7 +393,7 @@ __global__ void __launch_bounds__(kAntThreads, 2) kb_exp_ant(const BItem* __rest
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
     const int64_t unit = k * kAntWarps + warp;
     if (unit >= (int64_t)it.ag.n_grp * it.n_ant * it.ag.n_seg) return;
-    if (*it.irr)
+    if (irregular(it.irr))
       exp_antenna_unit<true>(it.rel_t, it.t_base, it.n_sft, it.g, it.perm_ant, it.tauc, it.ax,
                              it.i0, it.jend, it.ag, it.agg, it.coef, it.flag_bits, unit,
                              s_pw[warp], lane);

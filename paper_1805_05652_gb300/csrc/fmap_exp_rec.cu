@@ -145,7 +145,7 @@ struct PlainCursor {
 struct RecArgs {
   const int32_t* rel_t;
   const int64_t* t_base;
-  const int32_t* irr;   // nonzero: some gap has code 0
+  const int32_t* irr;   // any word nonzero: some gap has code 0
   int32_t n, T;
   fmap_grid g;
   RecGeom q;
@@ -520,7 +520,7 @@ k_exp_rec(const RecArgs A, int64_t units) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t unit = (int64_t)blockIdx.x * kRecWarps + warp;
   if (unit >= units) return;
-  if (*A.irr) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw[warp], lane);
+  if (irregular(A.irr)) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw[warp], lane);
   else exp_rec_unit<G, SHORT, SH, false>(A, unit, s_pw[warp], lane);
 }
 // Chunk maps of the antenna rows (units [0, ant_units)), then of the data.
@@ -545,7 +545,7 @@ k_sweep_agg(const RecArgs A, const AntAgg N, int64_t units) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t unit = (int64_t)blockIdx.x * kSweepWarps + warp;
   if (unit >= units) return;
-  if (*A.irr) sweep_agg_unit<G, true>(A, N, unit, s_pw[warp], lane);
+  if (irregular(A.irr)) sweep_agg_unit<G, true>(A, N, unit, s_pw[warp], lane);
   else sweep_agg_unit<G, false>(A, N, unit, s_pw[warp], lane);
 }
 
@@ -690,13 +690,13 @@ __global__ void __launch_bounds__(kAggThreads, 2) kb_sweep_agg(const BItem* __re
     if (unit >= N.units + (int64_t)it.rg.n_grp * it.rg.n_chunks * it.rg.n_tgrp) return;
     const RecArgs A = rec_args(it);
     if (it.rg.G == 1) {
-      if (*it.irr) sweep_agg_unit<1, true>(A, N, unit, s_pw[warp], lane);
+      if (irregular(it.irr)) sweep_agg_unit<1, true>(A, N, unit, s_pw[warp], lane);
       else sweep_agg_unit<1, false>(A, N, unit, s_pw[warp], lane);
     } else if (it.rg.G == 2) {
-      if (*it.irr) sweep_agg_unit<2, true>(A, N, unit, s_pw[warp], lane);
+      if (irregular(it.irr)) sweep_agg_unit<2, true>(A, N, unit, s_pw[warp], lane);
       else sweep_agg_unit<2, false>(A, N, unit, s_pw[warp], lane);
     } else {
-      if (*it.irr) sweep_agg_unit<4, true>(A, N, unit, s_pw[warp], lane);
+      if (irregular(it.irr)) sweep_agg_unit<4, true>(A, N, unit, s_pw[warp], lane);
       else sweep_agg_unit<4, false>(A, N, unit, s_pw[warp], lane);
     }
   });
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kAggThreads, 2) kb_sweep_agg(const BItem* __re
 template <int G, bool SHORT, bool SH>
 static __device__ __forceinline__ void rec_batch_unit(const RecArgs& A, int64_t unit, float2* s_pw,
                                                       int lane) {
-  if (*A.irr) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw, lane);
+  if (irregular(A.irr)) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw, lane);
   else exp_rec_unit<G, SHORT, SH, false>(A, unit, s_pw, lane);
 }
 // MAXG: the most templates per warp of the wave's instances (registers).

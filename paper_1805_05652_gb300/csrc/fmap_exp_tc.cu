@@ -24,7 +24,7 @@
 #include <cudaTypedefs.h>
 #include <math.h>
 
-#include "fmap_device.cuh"
+#include "fmap_front.cuh"
 
 namespace fmap {
 namespace tc {
@@ -161,17 +161,6 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-  uint32_t y;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"(x));
-  return y;
-}
-// Pack (lo_elem -> bits 15:0, hi_elem -> bits 31:16) as bf16x2, round to nearest.
-__device__ __forceinline__ uint32_t pack_bf16(float even, float odd) {
-  uint32_t y;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(y) : "f"(odd), "f"(even));
   return y;
 }
 __device__ __forceinline__ void mul_x2(float& r0, float& r1, float a0, float a1, float b) {
@@ -671,31 +660,6 @@ k_exp_tc(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUte
   }
 }
 
-// Split X into hi + lo operands ([4T][n_pad], zero padded): TF32 (stored as
-// FP32 bit patterns with 13 low zero bits) or BF16.
-template <bool BF16>
-__global__ void k_split_x(const float* __restrict__ fafb, int32_t n_sft, int32_t ncols,
-                          int32_t n_pad, void* __restrict__ hi, void* __restrict__ lo) {
-  const int64_t total = (int64_t)ncols * n_pad;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = i / n_pad;
-    const int32_t a = (int32_t)(i - c * n_pad);
-    const float x = a < n_sft ? fafb[c * n_sft + a] : 0.0f;
-    if constexpr (BF16) {
-      const uint32_t hp = pack_bf16(x, 0.0f);
-      const float hx = __uint_as_float(hp << 16);
-      const uint32_t lp = pack_bf16(x - hx, 0.0f);
-      ((uint16_t*)hi)[i] = (uint16_t)(hp & 0xffffu);
-      ((uint16_t*)lo)[i] = (uint16_t)(lp & 0xffffu);
-    } else {
-      const uint32_t hb = to_tf32(x);
-      ((uint32_t*)hi)[i] = hb;
-      ((uint32_t*)lo)[i] = to_tf32(x - __uint_as_float(hb));
-    }
-  }
-}
-
 }  // namespace tc
 
 // ---------------------------------------------------------------- host -----
@@ -717,6 +681,13 @@ size_t exp_tc_operand_bytes(const fmap_grid&, int32_t n_sft, int32_t n_templates
                             fmap_precision prec) {
   const size_t elem = prec == FMAP_BF16X3 ? 2 : 4;
   return 2 * elem * (size_t)4 * (size_t)std::max(n_templates, 1) * (size_t)n_pad_of(n_sft) + 256;
+}
+
+void exp_tc_operands(const fmap_plan_s* p, void** hi, void** lo, int32_t* n_pad) {
+  const size_t elem = p->precision == FMAP_BF16X3 ? 2 : 4;
+  *n_pad = n_pad_of(p->n_sft);
+  *hi = p->ws.xop;
+  *lo = (uint8_t*)p->ws.xop + (size_t)4 * p->n_templates * *n_pad * elem;
 }
 
 static PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
@@ -756,21 +727,11 @@ cudaError_t launch_exp_tc(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cuda
   if (tiles == 0 || p->n_templates == 0) return cudaSuccess;
   const bool bf16 = p->precision == FMAP_BF16X3;
   const int32_t T = p->n_templates;
-  const int32_t n_pad = n_pad_of(p->n_sft);
   const int32_t ncols = 4 * T;
   const int N = n_cols_of(T);
-  const size_t elem = bf16 ? 2 : 4;
-  uint8_t* hi = (uint8_t*)p->ws.xop;
-  uint8_t* lo = hi + (size_t)ncols * n_pad * elem;
-  {
-    const int64_t total = (int64_t)ncols * n_pad;
-    const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)p->n_sm * 8);
-    if (bf16)
-      tc::k_split_x<true><<<blocks, 256, 0, s>>>(a->fafb, p->n_sft, ncols, n_pad, hi, lo);
-    else
-      tc::k_split_x<false><<<blocks, 256, 0, s>>>(a->fafb, p->n_sft, ncols, n_pad, hi, lo);
-    p->launches += 1;
-  }
+  void *hi, *lo;
+  int32_t n_pad;
+  exp_tc_operands(p, &hi, &lo, &n_pad);   // (filled by the call's first launch)
   if (!p->tmaps_ready) {
     cudaError_t e = encode_map((CUtensorMap*)p->tmap_hi, hi, bf16, n_pad, ncols, N);
     if (e == cudaSuccess) e = encode_map((CUtensorMap*)p->tmap_lo, lo, bf16, n_pad, ncols, N);

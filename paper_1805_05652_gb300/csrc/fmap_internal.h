@@ -159,6 +159,7 @@ __host__ __device__ inline int64_t grid_t0(const fmap_grid& g, const int64_t* ax
 __host__ __device__ inline int64_t grid_tau(const fmap_grid& g, const int64_t* ax, int64_t n) {
   return ax ? ax[g.n_t0 + n] : g.tau_min + n * g.dtau;
 }
+constexpr int kIrrWords = 32;
 // Entries of the exp copy step: two per tau, then one per atom and set.
 // (plan_axes, after the plan struct: the axes to pass kernels, or null.)
 __host__ __device__ inline int64_t exp_copy_entries(int32_t n_sft, int32_t n_ant, int32_t n_x,
@@ -189,7 +190,7 @@ struct Workspace {
   size_t bytes = 0;
   int32_t* rel_t = nullptr;      // [round_up(N, 64) + 64] t - t[0], zero padded
   int64_t* t_base = nullptr;     // [1] t[0]
-  int32_t* irr = nullptr;        // [1] nonzero: a gap is not 1..kPowTab-1 whole SFTs (exp)
+  int32_t* irr = nullptr;        // [kIrrWords] any nonzero: a gap is not 1..kPowTab-1 whole SFTs (exp)
   uint32_t* dev_err = nullptr;   // [1] latched device error bits
   int32_t* i0 = nullptr;         // [n_t0] first atom with t >= t0_m
   int32_t* jend = nullptr;       // [n_t0][n_tau] one past the last atom of each window
@@ -291,8 +292,11 @@ inline const int64_t* plan_axes(const fmap_plan_s* p) { return p->explicit_axes 
 
 // ---- host launchers (each returns cudaGetLastError of its launches and
 // adds the number of kernels it launched to p->launches) -------------------
-cudaError_t launch_prep(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
-cudaError_t launch_index(fmap_plan_s* p, const int64_t* d_t, cudaStream_t s);
+// Input checks, index tables, the cleared marked-entry bitmask and the copies
+// of the atoms that the plan's form reads.
+cudaError_t launch_front(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
+// Split operands of the tensor-core forms in the plan's workspace ([4T][n_pad]).
+void exp_tc_operands(const fmap_plan_s* p, void** hi, void** lo, int32_t* n_pad);
 // Each compute launcher reports how many partial slots per template it wrote.
 // launch_rect records `mark` (if non-null) between its prefix scans and the
 // per-cell kernel.
@@ -302,7 +306,6 @@ cudaError_t launch_exp_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s)
 // Chunk maps of the antenna rows (and, in recurrence plans that start from
 // them, of the data).
 cudaError_t launch_exp_agg(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
-cudaError_t launch_exp_perm(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 cudaError_t launch_table_antenna(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 cudaError_t launch_exp_plain(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaStream_t s,
                              int64_t* tiles_used);

@@ -14,19 +14,11 @@
 #include <math.h>
 
 #include "fmap_batch.cuh"
-#include "fmap_device.cuh"
+#include "fmap_front.cuh"
 
 namespace fmap {
 
-constexpr int kScanThreads = 256;
-constexpr int kScanPer = 4;
-constexpr int kScanTile = kScanThreads * kScanPer;
 constexpr int kCellThreads = 256;
-
-// Antenna prefix entry: (sum a2, sum b2, sum ab, 0) as float pairs.
-struct __align__(32) P4 {
-  float4 hi, lo;
-};
 
 constexpr int kTileRows = 4;    // t0 rows of a warp tile of the cells kernel
 constexpr int kTileCols = 64;   // tau columns of a warp tile
@@ -35,212 +27,6 @@ constexpr int kTileCols = 64;   // tau columns of a warp tile
 int64_t rect_tiles(const fmap_grid& g) {
   return (int64_t)((g.n_t0 + kTileRows - 1) / kTileRows) *
          ((g.n_tau + kTileCols - 1) / kTileCols);
-}
-
-// Prefix sums of NC rows of n atoms by one block: out[2 i], out[2 i + 1] = hi,
-// lo of sum_{a < i} for i = 0..n (columns past NC are 0).  The sums are exact
-// 64-bit integers in units of 2^-S, S the largest with n max|x| 2^S < 2^61 per
-// row, and the pair holds the top 48 bits.  (The same scan in FP64, which GB300
-// runs at 1/64 of the FP32 rate, took eight FP64 operations per atom and row:
-// 423 us for 1024 templates of 5000 atoms, and 24 us for one block alone.)
-// The unit is fixed by the row's maximum, so rows whose level changes by more
-// than 2^35 / n from one stretch of 32 atoms to another (an outlier or a step;
-// the windows before it would lose their sums), rows below 2^-58 and blocks of
-// fewer than 64 atoms are summed in FP64.
-// A tile of kScanTile atoms at a time: each thread sums kScanPer neighbours,
-// the warps scan the threads' sums by shuffles, and the entries leave through
-// shared memory so that the block writes whole lines.
-struct ScanSmem {
-  float tile[4][kScanTile];
-  float4 ent[2 * kScanTile];
-  unsigned long long wsum[4][kScanThreads / 32];
-  float wmax[4][kScanThreads / 32], wmin[4][kScanThreads / 32];
-};
-constexpr int32_t kScanFixMin = 64;   // fewest atoms of an integer scan
-
-// Exponent e of a row with maximum mx (mx < 2^e).
-__host__ __device__ inline int scan_exponent(float mx) {
-  int e = 0;
-  if (mx > 0.0f) frexpf(mx, &e);
-  return e;
-}
-// Place of entry float4 k in the staging buffer: a thread's entries are 2 kScanPer
-// float4 apart, so the low three bits take its number and a warp's stores spread
-// over the banks.
-__device__ __forceinline__ int scan_place(int k) { return k ^ ((k / (2 * kScanPer)) & 7); }
-
-// The two accumulators: integers in units of down = 1 / up (both powers of two;
-// the scaling is exact but for underflow), and FP64.
-template <typename Acc> struct ScanAcc;
-template <> struct ScanAcc<unsigned long long> {
-  static __device__ __forceinline__ unsigned long long in(float x, float up) {
-    return (unsigned long long)__float2ll_rn(x * up);
-  }
-  static __device__ __forceinline__ float2 pair(unsigned long long v, float down) {
-    const float h = __ll2float_rn((long long)v);
-    return make_float2(h * down, __ll2float_rn((long long)v - __float2ll_rn(h)) * down);
-  }
-};
-template <> struct ScanAcc<double> {
-  static __device__ __forceinline__ double in(float x, float) { return (double)x; }
-  static __device__ __forceinline__ float2 pair(double v, float) {
-    const float h = (float)v;
-    return make_float2(h, (float)(v - (double)h));
-  }
-};
-
-template <int NC, typename Acc>
-__device__ __forceinline__ void rect_scan_tiles(const float* __restrict__ x, int32_t n,
-                                                const float (&up)[NC], const float (&down)[NC],
-                                                float4* __restrict__ out, ScanSmem& sm) {
-  constexpr int NW = kScanThreads / 32;
-  using A = ScanAcc<Acc>;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  Acc(*wsum)[NW] = reinterpret_cast<Acc(*)[NW]>(sm.wsum);
-  Acc carry[NC];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) carry[c] = Acc(0);
-  for (int32_t base = 0; base < n; base += kScanTile) {
-    __syncthreads();
-    for (int k = tid; k < kScanTile; k += kScanThreads)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) sm.tile[c][k] = base + k < n ? x[c * (int64_t)n + base + k] : 0.0f;
-    __syncthreads();
-    Acc v[NC][kScanPer], own[NC], inc[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      own[c] = Acc(0);
-      const float4* t4 = reinterpret_cast<const float4*>(&sm.tile[c][tid * kScanPer]);
-#pragma unroll
-      for (int e = 0; e < kScanPer; e += 4) {
-        const float4 t = t4[e / 4];
-        v[c][e] = A::in(t.x, up[c]);
-        v[c][e + 1] = A::in(t.y, up[c]);
-        v[c][e + 2] = A::in(t.z, up[c]);
-        v[c][e + 3] = A::in(t.w, up[c]);
-        own[c] += v[c][e] + v[c][e + 1] + v[c][e + 2] + v[c][e + 3];
-      }
-      inc[c] = own[c];
-    }
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const Acc y = __shfl_up_sync(0xffffffffu, inc[c], d);
-        if (lane >= d) inc[c] += y;
-      }
-    if (lane == 31)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) wsum[c][warp] = inc[c];
-    __syncthreads();
-    Acc run[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      run[c] = carry[c];
-#pragma unroll
-      for (int w = 0; w < NW; ++w) {
-        const Acc t = wsum[c][w];
-        if (w < warp) run[c] += t;
-        carry[c] += t;
-      }
-      const Acc before = __shfl_up_sync(0xffffffffu, inc[c], 1);
-      if (lane > 0) run[c] += before;
-    }
-#pragma unroll
-    for (int e = 0; e < kScanPer; ++e) {
-      float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        run[c] += v[c][e];
-        const float2 p = A::pair(run[c], down[c]);
-        hi[c] = p.x;
-        lo[c] = p.y;
-      }
-      const int k = 2 * (tid * kScanPer + e);
-      sm.ent[scan_place(k)] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-      sm.ent[scan_place(k + 1)] = make_float4(lo[0], lo[1], lo[2], lo[3]);
-    }
-    __syncthreads();
-    const int32_t m = 2 * min(kScanTile, n - base);
-    for (int32_t k = tid; k < m; k += kScanThreads) out[2 * (int64_t)(base + 1) + k] = sm.ent[scan_place(k)];
-  }
-}
-
-// (out of line: the common path's registers and instructions stay its own)
-template <int NC>
-__device__ __noinline__ void rect_scan_fp64(const float* __restrict__ x, int32_t n,
-                                            float4* __restrict__ out, ScanSmem& sm) {
-  const float one[NC] = {};
-  rect_scan_tiles<NC, double>(x, n, one, one, out, sm);
-}
-
-template <int NC>
-__device__ __forceinline__ void rect_scan_body(const float* __restrict__ x, int32_t n,
-                                               float4* __restrict__ out, ScanSmem& sm) {
-  constexpr int NW = kScanThreads / 32;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 2) out[tid] = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool fix = n >= kScanFixMin;
-  float up[NC], down[NC];
-  if (fix) {
-    // each row's maximum, and the smallest maximum of its stretches of 32 atoms
-    // (all-zero stretches do not count)
-    float mx[NC], mn[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      mx[c] = 0.0f;
-      mn[c] = 3.402823466e38f;
-#pragma unroll 4
-      for (int32_t a = tid; a < n + lane - 31; a += kScanThreads) {   // (whole stretches)
-        const float m = __uint_as_float(
-            __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(x[c * (int64_t)n + a]))));
-        mx[c] = fmaxf(mx[c], m);
-        if (m > 0.0f) mn[c] = fminf(mn[c], m);
-      }
-      const int32_t rest = n & ~31;   // the last atoms: part of the maximum only
-      if (warp == 0 && rest + lane < n) mx[c] = fmaxf(mx[c], fabsf(x[c * (int64_t)n + rest + lane]));
-      mx[c] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx[c])));
-      if (lane == 0) {
-        sm.wmax[c][warp] = mx[c];
-        sm.wmin[c][warp] = mn[c];
-      }
-    }
-    __syncthreads();
-    const int bits = 32 - __clz(n);   // n < 2^bits
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-#pragma unroll
-      for (int w = 0; w < NW; ++w) {
-        mx[c] = fmaxf(mx[c], sm.wmax[c][w]);
-        mn[c] = fminf(mn[c], sm.wmin[c][w]);
-      }
-      const int e = scan_exponent(mx[c]), S = 61 - bits - e;
-      fix = fix && (mx[c] == 0.0f || (S <= 119 && S >= -100 && scan_exponent(mn[c]) >= e + bits - 35));
-      const int Sc = max(-100, min(119, S));
-      up[c] = __int_as_float((Sc + 127) << 23);
-      down[c] = __int_as_float((127 - Sc) << 23);
-    }
-  }
-  if (fix) rect_scan_tiles<NC, unsigned long long>(x, n, up, down, out, sm);
-  else rect_scan_fp64<NC>(x, n, out, sm);
-}
-
-// Scans of the antenna sets (blocks [0, n_ant)), then of the templates' data.
-__device__ __forceinline__ void rect_scan_unit(const float* antenna, const float* fafb, int32_t n,
-                                               int32_t n_ant, P4* pa, float4* px, int32_t b,
-                                               ScanSmem& sm) {
-  if (b < n_ant)
-    rect_scan_body<3>(antenna + (int64_t)b * 3 * n, n, (float4*)(pa + (int64_t)b * (n + 1)), sm);
-  else
-    rect_scan_body<4>(fafb + (int64_t)(b - n_ant) * 4 * n, n,
-                      px + (int64_t)(b - n_ant) * 2 * (n + 1), sm);
-}
-
-__global__ void __launch_bounds__(kScanThreads, 2)
-k_rect_scans(const float* __restrict__ antenna, const float* __restrict__ fafb, int32_t n,
-             int32_t n_ant, P4* __restrict__ pa, float4* __restrict__ px) {
-  extern __shared__ __align__(16) unsigned char s_scan[];
-  rect_scan_unit(antenna, fafb, n, n_ant, pa, px, blockIdx.x, *reinterpret_cast<ScanSmem*>(s_scan));
 }
 
 // Per-cell coefficients (shared by the templates of one antenna set) from the
@@ -679,23 +465,11 @@ cudaError_t launch_rect_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s
   if (cells == 0) return cudaSuccess;
   const int n_ant = a->shared_antenna ? 1 : p->n_templates;
   if (n_ant == 0) return cudaSuccess;
-  // the FP32 form takes its data sums from the atoms
-  const int n_x = p->precision == FMAP_FP32 ? 0 : p->n_templates;
-  if (p->n_sft > 0) {
-    cudaError_t e = cudaFuncSetAttribute(k_rect_scans, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(ScanSmem));
-    if (e != cudaSuccess) return e;
-    k_rect_scans<<<(unsigned)(n_ant + n_x), kScanThreads, sizeof(ScanSmem), s>>>(
-        a->antenna, a->fafb, p->n_sft, n_ant, (P4*)p->ws.pa, p->ws.px);
-  } else {
-    cudaMemsetAsync(p->ws.pa, 0, sizeof(P4) * n_ant, s);
-    cudaMemsetAsync(p->ws.px, 0, 2 * sizeof(float4) * p->n_templates, s);
-  }
   const int64_t total = cells * n_ant;
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)p->n_sm * 16);
   k_rect_coef<<<blocks, 256, 0, s>>>(p->ws.i0, p->ws.jend, (const P4*)p->ws.pa, p->n_sft, g.n_t0,
                                      g.n_tau, n_ant, p->ws.coef, p->ws.flag_bits);
-  p->launches += (p->n_sft > 0) ? 2 : 1;
+  p->launches += 1;
   return cudaGetLastError();
 }
 
@@ -716,8 +490,6 @@ cudaError_t launch_rect(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaSt
     p->launches += 1;
     return cudaGetLastError();
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   if (mark) cudaEventRecord(mark, s);
   const int32_t T = p->n_templates, sh = a->shared_antenna ? 1 : 0;
   *tiles_used = rect_partial_slots(g, T, sh);
@@ -727,7 +499,7 @@ cudaError_t launch_rect(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaSt
   if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
   const size_t smem = rect_cells_smem(T, sh);
   const void* kfn = sh ? (const void*)k_rect_cells<true> : (const void*)k_rect_cells<false>;
-  e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (sh)
     k_rect_cells<true><<<(unsigned)blocks, kCellThreads, smem, s>>>(
@@ -748,7 +520,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) kb_rect_scans(const BItem* __
   extern __shared__ __align__(16) unsigned char s_scan[];
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
     rect_scan_unit(it.antenna, it.fafb, it.n_sft, it.n_ant, (P4*)it.pa, it.px, (int32_t)k,
-                   *reinterpret_cast<ScanSmem*>(s_scan));
+                   it.dev_err, *reinterpret_cast<ScanSmem*>(s_scan));
   });
 }
 size_t rect_scan_smem() { return sizeof(ScanSmem); }

@@ -17,17 +17,9 @@
 // tau at a time.  Nothing passes between warps.
 #pragma once
 
-#include "fmap_device.cuh"
+#include "fmap_front.cuh"
 
 namespace fmap {
-
-// Decay after an atom, by its code in the copy step's arrays: 1..kPowTab-1 the
-// gap to the next atom in whole SFTs (the tau's float-float powers of the
-// one-SFT decay), 0 any other gap (FP64 exp), -1 the last atom (no next one).
-__host__ __device__ inline int32_t gap_code(int32_t gap, int32_t t_sft) {
-  const int32_t k = gap / t_sft;
-  return k >= 1 && k < kPowTab && k * t_sft == gap ? k : 0;
-}
 
 // (out of line: the FP64 exp's registers stay out of the sweeps' loops)
 static __device__ __noinline__ float2 slow_decay(int32_t gap, double inv_s) {
