@@ -13,6 +13,8 @@
 //   adds atom after atom to FP32 running sums as tau grows.
 #include <math.h>
 
+#include <type_traits>
+
 #include "fmap_batch.cuh"
 #include "fmap_front.cuh"
 
@@ -121,8 +123,6 @@ constexpr int kMaxRowSpread = 8;
 constexpr int kBlockTemplates = 128;
 constexpr size_t kRawBytes = (size_t)kSlots * kSlotEntries * 32;
 constexpr size_t kQBytes = (size_t)kSlots * kSlotEntries * 16;
-static_assert((size_t)kCellWarps * kLaneCells * 32 * 16 <= kRawBytes,
-              "global-path window sums must fit in the stage buffer");
 
 // Template lanes per warp tile.
 __host__ __device__ __forceinline__ int rect_tlanes(int32_t n_templates) {
@@ -270,133 +270,141 @@ __device__ __forceinline__ void rect_cells_body(const int32_t* __restrict__ i0ta
   // barrier every stage.  The call's outputs are then undefined and the
   // plan's status reports the timeout.
   bool dead = false;
-  if (staged) issue(0);
-  for (int st = 0; st < n_st; ++st) {
-    const uint32_t qs = q_s0 + (uint32_t)((st & 1) * kQBytes);
-    if (staged) {
-      if (!dead && G.y > 0 && t_begin + st * st_t + wi < t_end) {
-        const bool got = mbar_wait_or_abort(&s_bar[warp], (uint32_t)(st & 1), err, wait_ns);
-        if (!__all_sync(0xffffffffu, got)) {
-          mbar_wait_bounded(&s_bar[warp], (uint32_t)(st & 1), kWaitNs);
-          __syncwarp();
-          dead = true;
-        }
-      }
-      if (!dead && G.y > 0 && t_begin + st * st_t + wi < t_end) {
-        const uint32_t rs = raw_s + (uint32_t)(warp * kSlotEntries * 32);
-        const uint32_t qd = qs + (uint32_t)(warp * kSlotEntries * 16);
-        uint64_t hb0, hb1, lb0, lb1;
-        lds_pairs(rs, hb0, hb1);
-        lds_pairs(rs + 16, lb0, lb1);
-        auto rebase = [&](int e) {
-          uint64_t h0, h1, l0, l1;
-          lds_pairs(rs + 32 * e, h0, h1);
-          lds_pairs(rs + 32 * e + 16, l0, l1);
-          const uint64_t q0 = add2(sub2(h0, hb0), sub2(l0, lb0));
-          const uint64_t q1 = add2(sub2(h1, hb1), sub2(l1, lb1));
-          asm volatile("st.shared.v2.b64 [%0], {%1, %2};\n" ::"r"(qd + (uint32_t)(e * 16)),
-                       "l"(q0), "l"(q1) : "memory");
-        };
-        for (int e = lane; e < G.y; e += 32) rebase(e);
-        for (int e = kRowCap + lane; e < kRowCap + G.w; e += 32) rebase(e);
-        fence_proxy_async_smem();   // the reads of raw above vs the next copy into it
-        __syncwarp();
-        if (st + 1 < n_st) issue(st + 1);
-      }
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-    }
-    if (rows == 0 || dead) continue;   // warp below the grid, or given up: barriers only
-    for (int g = tlane; g < st_t; g += tl) {
-      const int32_t tm = t_begin + st * st_t + g;
-      if (tm >= t_end) break;
-      if (!kShared) load_coef(coef + (int64_t)tm * cells);
-      float v[kLaneCells];
-      if (staged) {
-        const uint32_t sq = qs + (uint32_t)((grp * st_t + g) * kSlotEntries * 16);
-#pragma unroll
-        for (int r = 0; r < kTileRows; ++r) {
-          uint64_t ia, ib;
-          lds_pairs(sq + ro[r], ia, ib);
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int i = 2 * r + q;
-            uint64_t ja, jb;
-            lds_pairs(sq + qo[i], ja, jb);
-            v[i] = two_f_pairs(sub2(ja, ia), sub2(jb, ib), nb2[i], k1[i], k2[i], tiny2);
+  // (each path with a loop of its own: its registers do not add to the other's)
+  auto run = [&](auto is_staged) {
+    constexpr bool kStaged = decltype(is_staged)::value;
+    if (kStaged) issue(0);
+    for (int st = 0; st < n_st; ++st) {
+      const uint32_t qs = q_s0 + (uint32_t)((st & 1) * kQBytes);
+      if constexpr (kStaged) {
+        if (!dead && G.y > 0 && t_begin + st * st_t + wi < t_end) {
+          const bool got = mbar_wait_or_abort(&s_bar[warp], (uint32_t)(st & 1), err, wait_ns);
+          if (!__all_sync(0xffffffffu, got)) {
+            mbar_wait_bounded(&s_bar[warp], (uint32_t)(st & 1), kWaitNs);
+            __syncwarp();
+            dead = true;
           }
         }
-      } else {
-        // Window sums from the float pairs in global memory, parked in the
-        // warp's part of the (unused) stage buffer.
-        const float4* pt = px + (int64_t)tm * 2 * np1;
-        const uint32_t wb = raw_s + (uint32_t)(warp * kLaneCells * 32 * 16 + lane * 16);
-        __syncwarp();
-#pragma unroll 1
-        for (int i = 0; i < kLaneCells; ++i) {
-          const int32_t i0 = i0tab[m0 + min(i >> 1, rows - 1)];
-          const int32_t j = in_grid(i) ? jend[cell0 + cell_off(i)] : i0;
-          const float4 hi = pt[2 * (int64_t)i0], li = pt[2 * (int64_t)i0 + 1];
-          const float4 hj = pt[2 * (int64_t)j], lj = pt[2 * (int64_t)j + 1];
-          const uint64_t a = add2(sub2(pk2(hj.x, hj.y), pk2(hi.x, hi.y)), sub2(pk2(lj.x, lj.y), pk2(li.x, li.y)));
-          const uint64_t b = add2(sub2(pk2(hj.z, hj.w), pk2(hi.z, hi.w)), sub2(pk2(lj.z, lj.w), pk2(li.z, li.w)));
-          asm volatile("st.shared.v2.b64 [%0], {%1, %2};\n" ::"r"(wb + (uint32_t)(i * 32 * 16)),
-                       "l"(a), "l"(b) : "memory");
+        if (!dead && G.y > 0 && t_begin + st * st_t + wi < t_end) {
+          const uint32_t rs = raw_s + (uint32_t)(warp * kSlotEntries * 32);
+          const uint32_t qd = qs + (uint32_t)(warp * kSlotEntries * 16);
+          uint64_t hb0, hb1, lb0, lb1;
+          lds_pairs(rs, hb0, hb1);
+          lds_pairs(rs + 16, lb0, lb1);
+          auto rebase = [&](int e) {
+            uint64_t h0, h1, l0, l1;
+            lds_pairs(rs + 32 * e, h0, h1);
+            lds_pairs(rs + 32 * e + 16, l0, l1);
+            const uint64_t q0 = add2(sub2(h0, hb0), sub2(l0, lb0));
+            const uint64_t q1 = add2(sub2(h1, hb1), sub2(l1, lb1));
+            asm volatile("st.shared.v2.b64 [%0], {%1, %2};\n" ::"r"(qd + (uint32_t)(e * 16)),
+                         "l"(q0), "l"(q1) : "memory");
+          };
+          for (int e = lane; e < G.y; e += 32) rebase(e);
+          for (int e = kRowCap + lane; e < kRowCap + G.w; e += 32) rebase(e);
+          fence_proxy_async_smem();   // the reads of raw above vs the next copy into it
+          __syncwarp();
+          if (st + 1 < n_st) issue(st + 1);
         }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < kLaneCells; ++i) {
-          uint64_t a, b;
-          lds_pairs(wb + (uint32_t)(i * 32 * 16), a, b);
-          v[i] = two_f_pairs(a, b, nb2[i], k1[i], k2[i], tiny2);
-        }
+        asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
       }
-      const float mx = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                             fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-      if (map) {
-        float* mr = map + (int64_t)tm * cells + cell0;
-        if (rows == kTileRows && col1) {
+      if (rows == 0 || dead) continue;   // warp below the grid, or given up: barriers only
+      for (int g = tlane; g < st_t; g += tl) {
+        const int32_t tm = t_begin + st * st_t + g;
+        if (tm >= t_end) break;
+        if (!kShared) load_coef(coef + (int64_t)tm * cells);
+        float v[kLaneCells];
+        if constexpr (kStaged) {
+          const uint32_t sq = qs + (uint32_t)((grp * st_t + g) * kSlotEntries * 16);
 #pragma unroll
-          for (int r = 0; r < kTileRows; ++r, mr += n_tau) {
-            st_stream(mr, fmaxf(v[2 * r], 0.0f));
-            st_stream(mr + 32, fmaxf(v[2 * r + 1], 0.0f));
+          for (int r = 0; r < kTileRows; ++r) {
+            uint64_t ia, ib;
+            lds_pairs(sq + ro[r], ia, ib);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const int i = 2 * r + q;
+              uint64_t ja, jb;
+              lds_pairs(sq + qo[i], ja, jb);
+              v[i] = two_f_pairs(sub2(ja, ia), sub2(jb, ib), nb2[i], k1[i], k2[i], tiny2);
+            }
           }
         } else {
+          // Window sums from the float pairs in global memory, a row at a time:
+          // six loads in flight per lane.  (One cell at a time, with its indices
+          // loaded again for every template, the path was a chain of memory
+          // latencies.)
+          const float4* pt = px + (int64_t)tm * 2 * np1;
+          auto entry = [&](int64_t k, uint64_t& h0, uint64_t& h1, uint64_t& l0, uint64_t& l1) {
+            const ulonglong2 h = *reinterpret_cast<const ulonglong2*>(pt + 2 * k);
+            const ulonglong2 l = *reinterpret_cast<const ulonglong2*>(pt + 2 * k + 1);
+            h0 = h.x, h1 = h.y, l0 = l.x, l1 = l.y;
+          };
 #pragma unroll
-          for (int i = 0; i < kLaneCells; ++i)
-            if (in_grid(i)) st_stream(mr + cell_off(i), fmaxf(v[i], 0.0f));
+          for (int r = 0; r < kTileRows; ++r) {
+            uint64_t hi0, hi1, li0, li1, hj0[2], hj1[2], lj0[2], lj1[2];
+            entry(G.x + (int32_t)(ro[r] / 16u), hi0, hi1, li0, li1);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              entry(G.z + (int32_t)(qo[2 * r + q] / 16u) - kRowCap, hj0[q], hj1[q], lj0[q], lj1[q]);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const int i = 2 * r + q;
+              v[i] = two_f_pairs(add2(sub2(hj0[q], hi0), sub2(lj0[q], li0)),
+                                 add2(sub2(hj1[q], hi1), sub2(lj1[q], li1)), nb2[i], k1[i], k2[i],
+                                 tiny2);
+            }
+          }
+        }
+        const float mx = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
+                               fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+        if (map) {
+          float* mr = map + (int64_t)tm * cells + cell0;
+          if (rows == kTileRows && col1) {
+#pragma unroll
+            for (int r = 0; r < kTileRows; ++r, mr += n_tau) {
+              st_stream(mr, fmaxf(v[2 * r], 0.0f));
+              st_stream(mr + 32, fmaxf(v[2 * r + 1], 0.0f));
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < kLaneCells; ++i)
+              if (in_grid(i)) st_stream(mr + cell_off(i), fmaxf(v[i], 0.0f));
+          }
+        }
+        // 2F >= 0, so its bit pattern orders like the value; 0 marks "no valid cell".
+        const unsigned mu = __reduce_max_sync(0xffffffffu, mx >= 0.0f ? __float_as_uint(mx) + 1u : 0u);
+        if (mu == 0u) {
+          if (lane == 0) parts[(int64_t)tm * stride + wt] = partial_empty();
+          continue;
+        }
+        const float M = __uint_as_float(mu - 1u);
+        const float mc = -M * kHalfLog2e;
+        float e[kLaneCells];
+#pragma unroll
+        for (int i = 0; i < kLaneCells; ++i) e[i] = ex2_approx(fmaf(v[i], kHalfLog2e, mc));
+        // The lane's sum is in [0, 8] (every term <= 1); summed over the warp in
+        // 2^-23 fixed point by an integer reduction (absolute error <= 32 x
+        // 2^-24 against a sum >= 1, the maximum cell's own term).
+        const float sl = ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
+        const unsigned sfix = __reduce_add_sync(0xffffffffu, __float2uint_rn(sl * 8388608.0f));
+        // Only lanes holding the maximum look for their first cell at it.
+        unsigned cand = (unsigned)kNoArg;
+        if (mx == M) {
+#pragma unroll
+          for (int i = kLaneCells - 1; i >= 0; --i)
+            if (v[i] == M) cand = (unsigned)(cell0 + cell_off(i));
+        }
+        const int32_t arg = (int32_t)__reduce_min_sync(0xffffffffu, cand);
+        if (lane == 0) {
+          const float4 pv = make_float4(M, __int_as_float(arg), (float)sfix * (1.0f / 8388608.0f),
+                                        __int_as_float(nval));
+          *reinterpret_cast<float4*>(parts + (int64_t)tm * stride + wt) = pv;
         }
       }
-      // 2F >= 0, so its bit pattern orders like the value; 0 marks "no valid cell".
-      const unsigned mu = __reduce_max_sync(0xffffffffu, mx >= 0.0f ? __float_as_uint(mx) + 1u : 0u);
-      if (mu == 0u) {
-        if (lane == 0) parts[(int64_t)tm * stride + wt] = partial_empty();
-        continue;
-      }
-      const float M = __uint_as_float(mu - 1u);
-      const float mc = -M * kHalfLog2e;
-      float e[kLaneCells];
-#pragma unroll
-      for (int i = 0; i < kLaneCells; ++i) e[i] = ex2_approx(fmaf(v[i], kHalfLog2e, mc));
-      // The lane's sum is in [0, 8] (every term <= 1); summed over the warp in
-      // 2^-23 fixed point by an integer reduction (absolute error <= 32 x
-      // 2^-24 against a sum >= 1, the maximum cell's own term).
-      const float sl = ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
-      const unsigned sfix = __reduce_add_sync(0xffffffffu, __float2uint_rn(sl * 8388608.0f));
-      // Only lanes holding the maximum look for their first cell at it.
-      unsigned cand = (unsigned)kNoArg;
-      if (mx == M) {
-#pragma unroll
-        for (int i = kLaneCells - 1; i >= 0; --i)
-          if (v[i] == M) cand = (unsigned)(cell0 + cell_off(i));
-      }
-      const int32_t arg = (int32_t)__reduce_min_sync(0xffffffffu, cand);
-      if (lane == 0) {
-        const float4 pv = make_float4(M, __int_as_float(arg), (float)sfix * (1.0f / 8388608.0f),
-                                      __int_as_float(nval));
-        *reinterpret_cast<float4*>(parts + (int64_t)tm * stride + wt) = pv;
-      }
     }
-  }
+  };
+  if (staged) run(std::true_type{});
+  else run(std::false_type{});
   __syncthreads();   // every wait on the mbarriers is done before they are retired
   if (tid < kSlots) mbar_inval(&s_bar[tid]);
 }
