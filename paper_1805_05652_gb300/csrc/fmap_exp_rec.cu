@@ -707,9 +707,12 @@ static __device__ __forceinline__ void rec_batch_unit(const RecArgs& A, int64_t 
   if (irregular(A.irr)) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw, lane);
   else exp_rec_unit<G, SHORT, SH, false>(A, unit, s_pw, lane);
 }
-// MAXG: the most templates per warp of the wave's instances (registers).
+// MAXG: the most templates per warp of the wave's instances (registers).  Three
+// blocks per SM: the body holds every variant of its unit, and at four (128
+// registers) it spilt 250 bytes in the row loop (the 48-instance batch: 1181 us
+// against 915).
 template <int MAXG>
-__global__ void __launch_bounds__(kRecThreads, MAXG == 1 ? 4 : 3)
+__global__ void __launch_bounds__(kRecThreads, 3)
 kb_exp_rec(const BItem* __restrict__ items, BUnits u) {
   __shared__ float2 s_pw[kRecWarps][kSweepTab];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

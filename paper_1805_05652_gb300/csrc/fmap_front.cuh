@@ -70,13 +70,13 @@ __device__ __forceinline__ void prep_body(const int64_t* __restrict__ t, int32_t
 // front kernel, where the checks run beside their readers).
 struct RelStored {
   const int32_t* r;
-  __device__ __forceinline__ int32_t operator[](int32_t i) const { return r[i]; }
+  __device__ __forceinline__ int32_t operator[](int32_t i) const { return __ldg(r + i); }
 };
 struct RelTimes {
   const int64_t* t;
   int64_t base;
   __device__ __forceinline__ int32_t operator[](int32_t i) const {
-    return (int32_t)((t[i] - base) & 0x7fffffffLL);
+    return (int32_t)((__ldg(t + i) - base) & 0x7fffffffLL);
   }
 };
 
@@ -149,7 +149,7 @@ struct IndexSmem {
 };
 template <typename Rel>
 __device__ __forceinline__ void index_body(const Rel& rel_t, int64_t tb, int32_t n_sft,
-                                           const fmap_grid& g, const int64_t* __restrict__ ax,
+                                           const fmap_grid g, const int64_t* __restrict__ ax,
                                            int32_t* __restrict__ i0tab,
                                            int32_t* __restrict__ jend, int32_t m0, int32_t R,
                                            IndexSmem& sm) {
