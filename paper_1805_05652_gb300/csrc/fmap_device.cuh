@@ -264,6 +264,23 @@ __device__ __forceinline__ double tab_weight64(double u, const float2* tab, int3
   const float2 e = tab[k];
   return (double)e.x + (u - (double)k) * (double)e.y;
 }
+// The same in float-float (~2^-46 relative) for dt = t - t0 in [0, 2^31) and su a
+// float pair: FP64 runs at 1/64 of the FP32 rate.
+__device__ __forceinline__ FF tab_weight_ff(int32_t dt, FF su, const float2* tab, int32_t n) {
+  const float dh = (float)dt;
+  const FF u = ff_mul(FF{dh, (float)((int64_t)dt - (int64_t)dh)}, su);
+  if (u.h >= (float)n) return FF{0.0f, 0.0f};   // (the sentinel)
+  float k = floorf(u.h);
+  FF f = two_sum(u.h - k, u.l);
+  if (f.h < 0.0f) {
+    k -= 1.0f;
+    f = two_sum(u.h - k, u.l);
+  }
+  const float2 e = tab[max((int32_t)k, 0)];
+  const float p = __fmul_rn(f.h, e.y);
+  const FF s = two_sum(e.x, p);
+  return fast_two_sum(s.h, s.l + fmaf(f.l, e.y, fmaf(f.h, e.y, -p)));
+}
 // Sample units per second of (t - t0) for a tau: (n - 1) / (X tau), X = c / 8.
 __host__ __device__ __forceinline__ double tab_scale(int32_t n, int32_t cut8, int64_t tau) {
   return (double)(n - 1) * 8.0 / ((double)cut8 * (double)tau);

@@ -302,62 +302,94 @@ struct ScanArgs {
   int32_t* ref_cand;
 };
 
-// Calls f(cell, owned) for every cell of share `part` (of A.parts) of listed
-// tile k (lanes of one warp): a main tile by its geometry, a fix-up slot by
-// its share of the fix-up list;
-// owned says whether the tile's partial summed the cell (a main tile's
-// cells of Coef.valid 1, a fix-up slot's of 3), so that no cell is taken
-// twice.
+// Calls f(cell, bin, take), all 32 lanes of the warp together, for the cells of
+// share `part` (of A.parts) of listed tile k: a main tile by its geometry, a fix-up
+// slot by its share of the fix-up list.  take: the cell lies in a bin up to `last`
+// and the tile's partial summed it (a main tile's cells of Coef.valid 1, a fix-up
+// slot's of 3), so that no cell is taken twice.  Steps that take none are left
+// out: only the few cells near the maximum cost more than the load of their
+// value, four steps of which are in flight at once.  (With every cell's
+// coefficient loaded, 64-bit divisions and a match over the lanes' bins, a share of
+// 256 cells took eight dependent round trips: 25 us of a 1000 x 1000 band of 16
+// templates.)
 template <typename F>
 __device__ __forceinline__ void ref_tile_cells(const ScanArgs& A, int32_t j, int64_t k,
-                                               int32_t part, int lane, F f) {
+                                               int32_t part, float M, int32_t last, int lane,
+                                               F f) {
+  const float* mp = A.map + (int64_t)j * A.cells;
   if (k < A.n_tiles) {
+    constexpr int U = 4;
     const TileGeom& g = A.geo;
-    const int64_t tr = g.col_major ? k % g.ntr : k / g.ntc;
-    const int64_t tc = g.col_major ? k / g.ntr : k % g.ntc;
-    const int64_t r0 = tr * g.R, c0 = tc * g.C;
-    const int64_t rows = min((int64_t)g.R, (int64_t)A.n_t0 - r0);
-    const int64_t cols = min((int64_t)g.C, (int64_t)A.n_tau - c0);
-    const int64_t n = rows * cols;
-    for (int64_t q = n * part / A.parts + lane; q < n * (part + 1) / A.parts; q += 32) {
-      const int64_t r = q / cols, cc = q - r * cols;
-      const int64_t c = (r0 + r) * A.n_tau + c0 + cc;
-      f(c, ref_valid_of(A.coef, A.shared, A.cells, j, c) == 1.0f);
+    const int32_t kk = (int32_t)k;   // (tiles: fewer than cells, < 2^31)
+    const int32_t tr = g.col_major ? kk % g.ntr : kk / g.ntc;
+    const int32_t tc = g.col_major ? kk / g.ntr : kk % g.ntc;
+    const int32_t r0 = tr * g.R, c0 = tc * g.C;
+    const uint32_t rows = (uint32_t)min(g.R, A.n_t0 - r0), cols = (uint32_t)min(g.C, A.n_tau - c0);
+    const uint32_t n = rows * cols, per = (n + (uint32_t)A.parts - 1u) / (uint32_t)A.parts;
+    const uint32_t lo = (uint32_t)min((uint64_t)part * per, (uint64_t)n), hi = min(n, lo + per);
+    const uint32_t dr = 32u / cols, dc = 32u - dr * cols;   // a step of 32 cells
+    uint32_t r = (lo + lane) / cols, cc = lo + lane - r * cols;
+    for (uint32_t q0 = lo; q0 < hi; q0 += 32u * U) {
+      int32_t c[U];
+      float v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        c[u] = (r0 + (int32_t)r) * A.n_tau + c0 + (int32_t)cc;
+        v[u] = q0 + 32u * u + lane < hi ? mp[c[u]] : -INFINITY;
+        r += dr;
+        cc += dc;
+        if (cc >= cols) {
+          cc -= cols;
+          ++r;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int b = ref_bin_of(v[u], M);
+        bool take = b >= 0 && b <= last;
+        if (!__any_sync(0xffffffffu, take)) continue;
+        take = take && ref_valid_of(A.coef, A.shared, A.cells, j, c[u]) == 1.0f;
+        f(c[u], b, take);
+      }
     }
   } else {
     const int64_t cap = A.shared ? A.cells : A.cells * A.n_templates;
     const int64_t n = min((int64_t)*A.n_flag, cap);
-    const int64_t b = k - A.n_tiles;
     int64_t lo, hi;
-    fix_slot_range(b, n, &lo, &hi);
+    fix_slot_range((int32_t)(k - A.n_tiles), n, &lo, &hi);
     const int64_t m = hi - lo;
-    for (int64_t e = lo + m * part / A.parts + lane; e < lo + m * (part + 1) / A.parts; e += 32) {
-      const int64_t entry = A.flag_list[e];
-      if (!A.shared && entry / A.cells != j) continue;
-      const int64_t c = A.shared ? entry : entry % A.cells;
-      f(c, ref_valid_of(A.coef, A.shared, A.cells, j, c) == 3.0f);
+    const int64_t end = lo + m * (part + 1) / A.parts;
+    for (int64_t e0 = lo + m * part / A.parts; e0 < end; e0 += 32) {
+      bool take = e0 + lane < end;
+      int64_t c = take ? A.flag_list[e0 + lane] : 0;
+      if (!A.shared) c -= (int64_t)j * A.cells;   // (another template's entry: out of range)
+      take = take && c >= 0 && c < A.cells;
+      const int b = take ? ref_bin_of(mp[c], M) : -1;
+      take = b >= 0 && b <= last;
+      if (!__any_sync(0xffffffffu, take)) continue;
+      take = take && ref_valid_of(A.coef, A.shared, A.cells, j, c) == 3.0f;
+      f((int32_t)c, b, take);
     }
   }
 }
 
-// Calls f(cell, its bin or -1) for the cells of the first nt listed tiles, whose
-// shares go to `step` warps.
+// Calls f as above for the cells of the first nt listed tiles, whose shares go to
+// `step` warps.
 template <typename F>
 __device__ __forceinline__ void ref_scan_cells(const ScanArgs& A, int32_t j, int32_t nt, float M,
-                                               int64_t first, int64_t step, int lane, F f) {
-  const float* mp = A.map + (int64_t)j * A.cells;
-  for (int64_t it = first; it < (int64_t)nt * A.parts; it += step) {
-    const int64_t k = it / A.parts;
-    ref_tile_cells(A, j, A.ref_tile[(int64_t)j * kRefMaxTiles + k], (int32_t)(it - k * A.parts),
-                   lane, [&](int64_t c, bool owned) {
-      f((int32_t)c, owned ? ref_bin_of(mp[c], M) : -1);
-    });
+                                               int32_t last, int64_t first, int64_t step, int lane,
+                                               F f) {
+  const uint32_t n = (uint32_t)nt * (uint32_t)A.parts;   // (at most kRefMaxTiles x 1024)
+  for (uint32_t it = (uint32_t)first; it < n; it += (uint32_t)step) {
+    const uint32_t k = it / (uint32_t)A.parts;
+    ref_tile_cells(A, j, A.ref_tile[(int64_t)j * kRefMaxTiles + k],
+                   (int32_t)(it - k * (uint32_t)A.parts), M, last, lane, f);
   }
 }
 
-// Pass 2 over the listed tiles' cells: the histogram, which also keeps the
-// cells in bins up to the tile pass's bound (cut[j]) while they fit
-// kRefCandCap; then, in the template's last block, the cut and the collection of
+// Pass 2 over the listed tiles' cells: the histogram of the bins up to the tile
+// pass's bound (cut[j]; the cut never passes it), which also keeps those cells
+// while they fit kRefCandCap; then, in the template's last block, the cut and the collection of
 // the cells up to it from the kept cells when they fit (the same set: every
 // cell the cut takes lies in a bin <= cut[j]), else a flag (done[0] < 0) that
 // leaves the collection to a second scan of the tiles, k_ref_collect.  Grid (x, T),
@@ -377,22 +409,18 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_scan(const ScanArgs A) {
   const int32_t nt = s.N > 0 ? min(A.ref_ntile[j], kRefMaxTiles) : 0;
   const float* mp = A.map + (int64_t)j * A.cells;
   int32_t* cand = A.ref_cand + (int64_t)j * kRefCandCap;
-  ref_scan_cells(A, j, nt, s.M, blockIdx.x * NW + warp, (int64_t)gridDim.x * NW, lane, [&](int32_t c, int b) {
-    // one shared-memory atomic per distinct bin among the lanes here
-    // (noise maps put most cells of the window in a few bins)
-    const unsigned act = __activemask();
-    const unsigned peers = __match_any_sync(act, b);
-    if (b >= 0 && lane == __ffs(peers) - 1) atomicAdd(&h[b], __popc(peers));
-    // keep the cells of bins <= keep: one global atomic per warp step
-    const bool kept = b >= 0 && b <= keep;
-    const unsigned sel = __ballot_sync(act, kept);
+  ref_scan_cells(A, j, nt, s.M, keep, blockIdx.x * NW + warp, (int64_t)gridDim.x * NW, lane,
+                 [&](int32_t c, int b, bool take) {
+    if (take) atomicAdd(&h[b], 1);
+    // one global atomic per warp step
+    const unsigned sel = __ballot_sync(0xffffffffu, take);
     if (sel) {
       const int leader = __ffs(sel) - 1;
       int32_t base = 0;
       if (lane == leader) base = atomicAdd(A.ref_ncand + j, __popc(sel));
-      base = __shfl_sync(act, base, leader);
+      base = __shfl_sync(0xffffffffu, base, leader);
       const int32_t at = base + __popc(sel & ((1u << lane) - 1u));
-      if (kept && at < kRefCandCap) cand[at] = c;
+      if (take && at < kRefCandCap) cand[at] = c;
     }
   });
   __syncthreads();
@@ -434,8 +462,9 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_collect(const ScanArgs A) {
   constexpr int NW = kRefThreads / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int32_t last = A.cut[j], nt = min(A.ref_ntile[j], kRefMaxTiles);
-  ref_scan_cells(A, j, nt, s.M, blockIdx.x * NW + warp, (int64_t)gridDim.x * NW, lane, [&](int32_t c, int b) {
-    if (b < 0 || b > last) return;
+  ref_scan_cells(A, j, nt, s.M, last, blockIdx.x * NW + warp, (int64_t)gridDim.x * NW, lane,
+                 [&](int32_t c, int, bool take) {
+    if (!take) return;
     const int32_t slot = atomicAdd(A.ref_n + j, 1);
     if (slot < kRefMaxCells) A.ref_cell[(int64_t)j * kRefMaxCells + slot] = c;
   });
@@ -478,7 +507,7 @@ struct RefArgs {
 // exp) and moves on by gaps of k SFTs, each the product of two float pairs held by
 // the lanes: the powers k mod 16 of the one-SFT decay (the tau's table) and 16
 // floor(k / 16) (by squaring); FP64 exp for other gaps.  A table window evaluates w
-// per atom in FP64, a rectangular one has w = 1.  The seven sums meet in a fixed
+// per atom in float-float, a rectangular one has w = 1.  The seven sums meet in a fixed
 // butterfly; D and 2F are formed from them in FP64, by one lane per cell of the
 // block's, which records the fast and refined values and writes the refined value
 // to the map.  (With one contiguous run of atoms per lane, an FP64 exp for every gap
@@ -505,7 +534,7 @@ __device__ __forceinline__ void ref_cell_sums(const RefArgs& A, int32_t j, int32
   const float* ant = A.antenna + (A.shared ? 0 : (int64_t)j * 3 * n);
   const float* x = A.fafb + (int64_t)j * 4 * n;
   const bool ex = g.window == FMAP_EXP, tw = g.window == FMAP_TABLE;
-  const double su = tw ? tab_scale(A.n_tab, exp_cut8_of(g), grid_tau(g, A.ax, nn)) : 0.0;
+  const FF su = ff_of(tw ? tab_scale(A.n_tab, exp_cut8_of(g), grid_tau(g, A.ax, nn)) : 0.0);
 #pragma unroll
   for (int q = 0; q < 7; ++q) s[q] = FF{0.0f, 0.0f};
   if (je > i0) {
@@ -556,7 +585,7 @@ __device__ __forceinline__ void ref_cell_sums(const RefArgs& A, int32_t j, int32
         if ((uint32_t)k >= 512u || k * t_sft != gap) r = ff_of(exp(-(double)gap * inv_tau));
         w = ff_mul(w, r);
       }
-      if (tw) w = ff_of(tab_weight64((double)((int64_t)t - t0rel) * su, A.wtab, A.n_tab));
+      if (tw) w = tab_weight_ff((int32_t)((int64_t)t - t0rel), su, A.wtab, A.n_tab);
       if (on) {
         if (g.window == FMAP_RECT) {
 #pragma unroll
