@@ -39,6 +39,8 @@
 // can hold the FP64 maximum, and the summary says so (ARGMAX_EXACT).
 #include <math.h>
 
+#include <algorithm>
+
 #include "fmap_device.cuh"
 
 namespace fmap {
@@ -57,7 +59,7 @@ static double fast_tol(const fmap_plan_s* p) { return p->precision == FMAP_FP64 
 
 // Coef.valid of cell c for template j: 1 summed by the main kernel, 3
 // recomputed by the fix-up (and summed in a fix-up slot), else invalid.
-__device__ __forceinline__ float ref_valid_of(const Coef* __restrict__ coef, int32_t shared,
+__device__ __forceinline__ float ref_valid_of(const Coef* coef, int32_t shared,
                                               int64_t cells, int32_t j, int64_t c) {
   return coef[shared ? c : (int64_t)j * cells + c].valid;
 }
@@ -402,11 +404,14 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_scan(const ScanArgs A) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int NW = kRefThreads / 32;
   static_assert(kRefThreads == kRefBins, "one bin per thread");
-  h[tid] = 0;
-  __syncthreads();
   const TStat s = A.st[j];
   const int32_t keep = A.cut[j];   // bins the histogram pass keeps
   const int32_t nt = s.N > 0 ? min(A.ref_ntile[j], kRefMaxTiles) : 0;
+  // the blocks that have a share (the first one always takes part)
+  const int32_t n_blk = (int32_t)min(gridDim.x, max(1u, ((uint32_t)nt * (uint32_t)A.parts + NW - 1u) / NW));
+  if ((int32_t)blockIdx.x >= n_blk) return;
+  h[tid] = 0;
+  __syncthreads();
   const float* mp = A.map + (int64_t)j * A.cells;
   int32_t* cand = A.ref_cand + (int64_t)j * kRefCandCap;
   ref_scan_cells(A, j, nt, s.M, keep, blockIdx.x * NW + warp, (int64_t)gridDim.x * NW, lane,
@@ -425,7 +430,7 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_scan(const ScanArgs A) {
   });
   __syncthreads();
   if (h[tid]) atomicAdd(A.hist + (int64_t)j * kRefBins + tid, h[tid]);
-  if (!ref_last_block(&A.st[j].done[0], gridDim.x)) return;
+  if (!ref_last_block(&A.st[j].done[0], n_blk)) return;
   h[tid] = __ldcg(A.hist + (int64_t)j * kRefBins + tid);
   if (tid == 0) s_n = 0;
   __syncthreads();
@@ -478,6 +483,8 @@ struct RefArgs {
   const int64_t* ax;
   const float2* wtab;
   int32_t n_tab;
+  const float4* perm_ant;   // exponential windows: the sweeps' copies of the atoms
+  const float4* perm_x;     // (or null: the caller's rows)
   const int32_t* i0;
   const int32_t* jend;
   const float* antenna;
@@ -489,7 +496,6 @@ struct RefArgs {
   const int32_t* ref_cell;
   float* ref_fast;
   double* ref_val;
-  const TauTab* tauc;      // exponential windows
   // the summaries
   TStat* st;
   const int32_t* cut;
@@ -498,22 +504,15 @@ struct RefArgs {
   fmap_summary* out;
 };
 
-// Pass 3: one warp per collected cell, lane l taking the window's atoms i0 + l +
-// 32 q (coalesced loads, a step ahead), summed in float-float arithmetic (a value
-// is an unevaluated pair h + l; GB300 runs FP64 at 1/64 of the FP32 rate): products
-// with their FMA error, added by TwoSum with the errors collected in l (Ogita, Rump
-// and Oishi's cascaded form, ~n^2 2^-48 relative for a lane's n atoms).  An
-// exponential weight starts from the decay between t0 and the first atom (FP64
-// exp) and moves on by gaps of k SFTs, each the product of two float pairs held by
-// the lanes: the powers k mod 16 of the one-SFT decay (the tau's table) and 16
-// floor(k / 16) (by squaring); FP64 exp for other gaps.  A table window evaluates w
-// per atom in float-float, a rectangular one has w = 1.  The seven sums meet in a fixed
-// butterfly; D and 2F are formed from them in FP64, by one lane per cell of the
-// block's, which records the fast and refined values and writes the refined value
-// to the map.  (With one contiguous run of atoms per lane, an FP64 exp for every gap
-// other than one SFT and the FP64 end of each cell in a warp of its own, the FP64
-// pipe was 66 % busy: 1034 us for 5 x 512 cells of a year's data with 4 % missing
-// SFTs.)
+// Pass 3: one warp per collected cell, its atoms summed in float-float arithmetic (a
+// value is an unevaluated pair h + l, ~2^-44 relative; GB300 runs FP64 at 1/64 of
+// the FP32 rate).  The seven sums meet in a fixed butterfly; D and 2F are formed
+// from them in FP64 by one lane.
+// Exponential windows: ref_exp_sums.  The others: lane l takes the window's atoms
+// i0 + l + 32 q (coalesced loads, a step ahead), added by TwoSum with the errors
+// collected in l (Ogita, Rump and Oishi's cascaded form, ~n^2 2^-48 relative for a
+// lane's n atoms); a table window evaluates w per atom in float-float and multiplies
+// with the products' FMA error, a rectangular one has w = 1.
 __device__ __forceinline__ void ref_acc(FF& s, FF w, float x) {
   const float p = __fmul_rn(w.h, x);
   const float e = fmaf(w.l, x, fmaf(w.h, x, -p));
@@ -522,41 +521,98 @@ __device__ __forceinline__ void ref_acc(FF& s, FF w, float x) {
   s.l += t.l + e;
 }
 
-// The seven sums of collected cell c of template j (every lane gets them).
+// The butterfly over the lanes' seven sums (every lane gets the totals).
+__device__ __forceinline__ void ref_butterfly(FF (&s)[7]) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      const FF o{__shfl_xor_sync(0xffffffffu, s[q].h, d), __shfl_xor_sync(0xffffffffu, s[q].l, d)};
+      s[q] = ff_add(s[q], o);
+    }
+}
+
+// The seven sums of an exponential window: lane l takes the l-th of 32 contiguous
+// runs of its atoms, the first weight from an FP64 exp and the others as products
+// of the gaps' decays.  2F of an exponential window does not change with t0 while
+// the window holds the same atoms, so that at grid steps below one SFT the maximum
+// is often shared by neighbouring cells up to rounding: this order of the
+// operations is part of which of them is reported, and is not to be changed.
+// Lane k holds the decay of k SFTs (the FP64 exp of that gap: with one for every
+// gap of more than one SFT, the FP64 pipe was 66 % busy: 1034 us for 5 x 512
+// cells of a year's data with 4 % missing SFTs, about 350 us so); the atoms come from
+// the sweeps' copies, a step ahead.
+__device__ __forceinline__ void ref_exp_sums(const RefArgs& A, int32_t j, int32_t c, int lane,
+                                             FF (&s)[7]) {
+  const fmap_grid& g = A.g;
+  const int32_t m = c / g.n_tau, nn = c - m * g.n_tau;
+  const int32_t i0 = A.i0[m], len = max(0, A.jend[c] - i0);
+  const int64_t t0rel = grid_t0(g, A.ax, m) - *A.t_base;
+  const double inv_tau = 1.0 / (double)grid_tau(g, A.ax, nn);
+  const int64_t n = A.n_sft;
+  const float4* ant = A.perm_ant + (A.shared ? 0 : (int64_t)j * n);
+  const float4* px = A.perm_x ? A.perm_x + (int64_t)j * n : nullptr;
+  const float* x = A.fafb + (int64_t)j * 4 * n;
+#pragma unroll
+  for (int q = 0; q < 7; ++q) s[q] = FF{0.0f, 0.0f};
+  if (len > 0) {   // (the whole warp)
+    const int32_t a_lo = i0 + (int32_t)((int64_t)len * lane / 32);
+    const int32_t run = i0 + (int32_t)((int64_t)len * (lane + 1) / 32) - a_lo;
+    const int32_t last = i0 + len - 1, most = (len + 31) / 32;
+    const FF rk = ff_of(exp(-(double)((int64_t)lane * g.t_sft) * inv_tau));
+    float4 va, vx;
+    auto load = [&](int32_t a) {   // (past the lane's run: unused)
+      a = min(a, last);
+      va = ant[a];
+      vx = px ? px[a] : make_float4(x[a], x[n + a], x[2 * n + a], x[3 * n + a]);
+    };
+    load(a_lo);
+    FF w = ff_of(exp(-(double)((int64_t)A.rel_t[min(a_lo, last)] - t0rel) * inv_tau));
+    int32_t k = 0;   // SFTs from the atom before (0: not a gap of the copies' codes)
+    for (int32_t i = 0; i < most; ++i) {
+      const float4 ua = va, ux = vx;
+      if (i + 1 < most) load(a_lo + i + 1);
+      FF r{__shfl_sync(0xffffffffu, rk.h, k & 31), __shfl_sync(0xffffffffu, rk.l, k & 31)};
+      if (i < run) {
+        if (i > 0) {
+          if (k <= 0) {
+            const int32_t gap = A.rel_t[a_lo + i] - A.rel_t[a_lo + i - 1];
+            r = ff_of(exp(-(double)gap * inv_tau));
+          }
+          w = ff_mul(w, r);
+        }
+        const FF w2 = ff_mul(w, w);
+        ff_acc(s[0], w2, ua.x);
+        ff_acc(s[1], w2, ua.y);
+        ff_acc(s[2], w2, ua.z);
+        ff_acc(s[3], w, ux.x);
+        ff_acc(s[4], w, ux.y);
+        ff_acc(s[5], w, ux.z);
+        ff_acc(s[6], w, ux.w);
+        k = __float_as_int(ua.w);
+      }
+    }
+  }
+  ref_butterfly(s);
+}
+
+// The seven sums of collected cell c of template j (every lane gets them), other
+// windows.
 __device__ __forceinline__ void ref_cell_sums(const RefArgs& A, int32_t j, int32_t c, int lane,
-                                              uint32_t inv_t, FF (&s)[7]) {
+                                              FF (&s)[7]) {
   const fmap_grid& g = A.g;
   const int32_t m = c / g.n_tau, nn = c - m * g.n_tau;
   const int32_t i0 = A.i0[m], je = A.jend[c];
   const int64_t t0rel = grid_t0(g, A.ax, m) - *A.t_base;
   const int64_t n = A.n_sft;
-  const int32_t t_sft = (int32_t)g.t_sft;
   const float* ant = A.antenna + (A.shared ? 0 : (int64_t)j * 3 * n);
   const float* x = A.fafb + (int64_t)j * 4 * n;
-  const bool ex = g.window == FMAP_EXP, tw = g.window == FMAP_TABLE;
+  const bool tw = g.window == FMAP_TABLE;
   const FF su = ff_of(tw ? tab_scale(A.n_tab, exp_cut8_of(g), grid_tau(g, A.ax, nn)) : 0.0);
 #pragma unroll
   for (int q = 0; q < 7; ++q) s[q] = FF{0.0f, 0.0f};
   if (je > i0) {
-    FF w{1.0f, 0.0f}, lo{1.0f, 0.0f}, hi{1.0f, 0.0f};
-    double inv_tau = 0.0;
-    int32_t t = A.rel_t[i0];
-    if (ex) {
-      const TauTab* tt = A.tauc + nn;
-      inv_tau = tt->inv_tau;
-      const float2 v = tt->pw[0][lane & 15];
-      lo = FF{v.x, v.y};
-      // lane h: the power 16 h, by squaring
-      const float2 v1 = tt->pw[0][1], v15 = tt->pw[0][15];
-      FF p = ff_mul(FF{v15.x, v15.y}, FF{v1.x, v1.y});
-#pragma unroll
-      for (int b = 0; b < 5; ++b) {
-        if (lane & (1 << b)) hi = ff_mul(hi, p);
-        p = ff_mul(p, p);
-      }
-      const int64_t d0 = (int64_t)t - t0rel;
-      if (d0 != 0) w = ff_of(exp(-(double)d0 * inv_tau));
-    }
+    FF w{1.0f, 0.0f};
     float v[7];
     int32_t tn;
     auto load = [&](int32_t b) {   // (lanes past the window: its last atom, unused)
@@ -572,19 +628,9 @@ __device__ __forceinline__ void ref_cell_sums(const RefArgs& A, int32_t j, int32
       float u[7];
 #pragma unroll
       for (int q = 0; q < 7; ++q) u[q] = v[q];
-      const int32_t gap = tn - t;
-      t = tn;
+      const int32_t t = tn;
       const bool on = b + lane < je;
       if (b + 32 < je) load(b + 32);
-      if (ex) {
-        const int32_t k = (int32_t)__umulhi((uint32_t)gap << 1, inv_t);
-        const int kl = k & 15, kh = (k >> 4) & 31;
-        const FF rl{__shfl_sync(0xffffffffu, lo.h, kl), __shfl_sync(0xffffffffu, lo.l, kl)};
-        const FF rh{__shfl_sync(0xffffffffu, hi.h, kh), __shfl_sync(0xffffffffu, hi.l, kh)};
-        FF r = ff_mul(rh, rl);
-        if ((uint32_t)k >= 512u || k * t_sft != gap) r = ff_of(exp(-(double)gap * inv_tau));
-        w = ff_mul(w, r);
-      }
       if (tw) w = tab_weight_ff((int32_t)((int64_t)t - t0rel), su, A.wtab, A.n_tab);
       if (on) {
         if (g.window == FMAP_RECT) {
@@ -606,17 +652,12 @@ __device__ __forceinline__ void ref_cell_sums(const RefArgs& A, int32_t j, int32
   }
 #pragma unroll
   for (int q = 0; q < 7; ++q) s[q] = fast_two_sum(s[q].h, s[q].l);
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1)
-#pragma unroll
-    for (int q = 0; q < 7; ++q) {
-      const FF o{__shfl_xor_sync(0xffffffffu, s[q].h, d), __shfl_xor_sync(0xffffffffu, s[q].l, d)};
-      s[q] = ff_add(s[q], o);
-    }
+  ref_butterfly(s);
 }
 
-// 2F of the cell in slot k of template j from its sums, in FP64 (one lane).
-__device__ __forceinline__ void ref_cell_end(const RefArgs& A, int32_t j, int32_t k, const FF* s) {
+// 2F of the cell in slot k of template j from its sums, in FP64 (one lane; records
+// the fast and the refined value, and writes the latter to the map).
+__device__ __forceinline__ void ref_cell_end(const RefArgs& A, int32_t j, int32_t k, const FF (&s)[7]) {
   const int64_t slot = (int64_t)j * kRefMaxCells + k;
   const int32_t c = A.ref_cell[slot];
   const int32_t len = A.jend[c] - A.i0[c / A.g.n_tau];
@@ -731,8 +772,7 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_cells(const RefArgs A) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int32_t j = blockIdx.y;
   const int32_t n_cand = min(A.ref_n[j], kRefMaxCells);
-  const uint32_t t_sft = (uint32_t)A.g.t_sft;
-  const uint32_t inv_t = (uint32_t)(((1ull << 31) + t_sft - 1) / t_sft);   // (as gap_inverse)
+  const bool ex = A.g.window == FMAP_EXP;
   constexpr int NW = kRefThreads / 32;
   __shared__ FF s_sum[NW][7];
   if (n_cand <= 0) {
@@ -742,11 +782,20 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_cells(const RefArgs A) {
   for (int32_t k0 = blockIdx.x * NW; k0 < n_cand; k0 += gridDim.x * NW) {
     if (k0 + warp < n_cand) {
       FF s[7];
-      ref_cell_sums(A, j, A.ref_cell[(int64_t)j * kRefMaxCells + k0 + warp], lane, inv_t, s);
+      const int32_t c = A.ref_cell[(int64_t)j * kRefMaxCells + k0 + warp];
+      if (ex) {
+        // (from the registers of the cell's own warp: from shared memory the compiler
+        // fuses other products, and other cells of a tie are reported)
+        ref_exp_sums(A, j, c, lane, s);
+        if (lane == 0) ref_cell_end(A, j, k0 + warp, s);
+      } else {
+        ref_cell_sums(A, j, c, lane, s);
 #pragma unroll
-      for (int q = 0; q < 7; ++q)
-        if (lane == q) s_sum[warp][q] = s[q];
+        for (int q = 0; q < 7; ++q)
+          if (lane == q) s_sum[warp][q] = s[q];
+      }
     }
+    if (ex) continue;   // (the whole block)
     __syncthreads();
     if (warp == 0 && lane < NW && k0 + lane < n_cand) ref_cell_end(A, j, k0 + lane, s_sum[lane]);
     __syncthreads();
@@ -802,15 +851,19 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   S.ref_cell = w.ref_cell;
   S.ref_ncand = w.ref_ncand;
   S.ref_cand = w.ref_cand;
-  // a warp per share of about kScanShare cells of a listed tile (about cap
-  // tiles per template), at least a few blocks over the GPU
+  // a warp per share of about kScanShare cells of a listed tile (about cap tiles per
+  // template), between one and 32 blocks per SM over all templates: a block's own
+  // costs (its launch, the histogram, its place in the count) are several shares'.
+  // (128 blocks for each of 1024 templates, 2000 x 2000 cells: 357 us, and 60 us of
+  // the launch that mostly has nothing to collect; 221 us so.)
   const int64_t tile_cells = (int64_t)S.geo.R * S.geo.C;
   S.parts = (int32_t)std::min<int64_t>(std::max<int64_t>((tile_cells + kScanShare - 1) / kScanShare, 1),
                                        1024);
   const int wpb = kRefThreads / 32;
-  const unsigned gx = (unsigned)std::max<int64_t>(
-      (2 * (int64_t)cap * S.parts + wpb - 1) / wpb, ((int64_t)p->n_sm * 4 + T - 1) / T);
-  const dim3 grid(std::min<unsigned>(gx, 4096u), (unsigned)T);
+  const int64_t gx = std::clamp<int64_t>((2 * (int64_t)cap * S.parts + wpb - 1) / wpb,
+                                         ((int64_t)p->n_sm + T - 1) / T,
+                                         ((int64_t)p->n_sm * 32 + T - 1) / T);
+  const dim3 grid((unsigned)gx, (unsigned)T);
   k_ref_scan<<<grid, kRefThreads, 0, s>>>(S);
   k_ref_collect<<<grid, kRefThreads, 0, s>>>(S);
   RefArgs A;
@@ -824,6 +877,8 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   A.i0 = w.i0;
   A.jend = w.jend;
   A.antenna = a->antenna;
+  A.perm_ant = w.perm_ant;
+  A.perm_x = w.perm_x;
   A.fafb = a->fafb;
   A.shared = sh;
   A.map = d_2F;
@@ -832,7 +887,6 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   A.ref_cell = w.ref_cell;
   A.ref_fast = w.ref_fast;
   A.ref_val = w.ref_val;
-  A.tauc = g.window == FMAP_EXP ? w.tauc : nullptr;
   A.st = w.tstat;
   A.cut = w.ref_bin;
   A.ref_ntile = w.ref_ntile;
