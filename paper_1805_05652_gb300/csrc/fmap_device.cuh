@@ -9,6 +9,19 @@
 
 namespace fmap {
 
+// The short kernels that end a call follow one another on its stream with
+// programmatic dependence (launch_after): the next one's blocks are placed as soon
+// as this one's have all started, and wait there for its end, so that a launch
+// costs no drain and refill (331 SFTs, 150 x 177 cells: 110 -> 97 us a call).
+// Each calls stream_order() first, in all of its threads: it returns when
+// everything earlier on the stream is done and visible (each waits for the one
+// before, so the order is complete).  What a kernel of the chain writes, the later
+// ones read by plain loads only: the read-only path (__ldg, or a const __restrict__
+// parameter) may be taken ahead of the wait.
+__device__ __forceinline__ void stream_order() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
 constexpr int32_t kNoArg = 0x7fffffff;
 
 // ---- PTX helpers: shared-memory addresses, the global timer, mbarriers ----

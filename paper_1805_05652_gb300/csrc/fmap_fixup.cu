@@ -100,8 +100,8 @@ k_flag_scan(int32_t* __restrict__ blockcnt, int64_t n_blocks, int32_t* __restric
 // (one per thread) places its set bits after the set bits of the words before
 // it (an exclusive scan of the words' counts over the block).
 // Returns the unit's count (to the last thread of the block).
-__device__ __forceinline__ int32_t flag_write_body(const uint32_t* __restrict__ bits, int64_t n_entries,
-             int64_t base, int64_t* __restrict__ list,
+__device__ __forceinline__ int32_t flag_write_body(const uint32_t* bits, int64_t n_entries,
+             int64_t base, int64_t* list,
     const uint3 bid) {
   __shared__ int32_t warp_cnt[kFlagBlock / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -145,8 +145,8 @@ __device__ __forceinline__ int32_t flag_write_body(const uint32_t* __restrict__ 
 // took 6.5 us and their gaps for 31 or 122 units alike.
 constexpr int64_t kFlagOnce = 128;
 __global__ void __launch_bounds__(kFlagBlock)
-k_flag_list(const uint32_t* __restrict__ bits, int64_t n_entries, int64_t* __restrict__ list,
-            int32_t* __restrict__ n_flag) {
+k_flag_list(const uint32_t* bits, int64_t n_entries, int64_t* list, int32_t* n_flag) {
+  stream_order();
   __shared__ int32_t part[kFlagBlock / 32];
   __shared__ int32_t s_base;
   const int tid = threadIdx.x;
@@ -155,7 +155,7 @@ k_flag_list(const uint32_t* __restrict__ bits, int64_t n_entries, int64_t* __res
   const int32_t n4 = (int32_t)blockIdx.x * (kFlagWords / 4);
 #pragma unroll 4
   for (int32_t i = tid; i < n4; i += kFlagBlock) {
-    const uint4 v = __ldg(w + i);
+    const uint4 v = w[i];
     c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
   }
   c = (int32_t)__reduce_add_sync(0xffffffffu, (unsigned)c);
@@ -201,7 +201,7 @@ __device__ __forceinline__ float fix_two_f(const FF* a, FF D, const FF* s) {
 // per template and a block per entry read a line per lane instead (590 us of the
 // 1024-template exponential workload, 890 us of the rectangular one).
 template <int G>
-__device__ __forceinline__ void fixup_cells_body(const int64_t* __restrict__ list, int64_t n,
+__device__ __forceinline__ void fixup_cells_body(const int64_t* list, int64_t n,
         int32_t shared_antenna,
         const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_base, int32_t n_sft,
         const fmap_grid& g, const int64_t* __restrict__ ax, const float2* __restrict__ wtab, int32_t n_tab, const int32_t* __restrict__ i0tab, const int32_t* __restrict__ jend,
@@ -295,7 +295,7 @@ int64_t fixup_blocks_y(int32_t n_templates, bool shared) {
 
 template <int G>
 __global__ void __launch_bounds__(kFixThreads)
-k_fixup(const int64_t* __restrict__ list, const int32_t* __restrict__ n_flag,
+k_fixup(const int64_t* list, const int32_t* n_flag,
         int32_t shared_antenna, const int32_t* __restrict__ rel_t,
         const int64_t* __restrict__ t_base, int32_t n_sft, const fmap_grid g, const int64_t* __restrict__ ax, const float2* __restrict__ wtab, int32_t n_tab,
         const int32_t* __restrict__ i0tab, const int32_t* __restrict__ jend,
@@ -303,6 +303,7 @@ k_fixup(const int64_t* __restrict__ list, const int32_t* __restrict__ n_flag,
         int32_t n_templates, float* __restrict__ map, Partial* __restrict__ parts,
         int64_t stride, int64_t slot0, Coef* __restrict__ coef,
         const TauTab* __restrict__ tauc) {
+  stream_order();
   const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
   const int64_t n = min((int64_t)*n_flag, shared_antenna ? cells : cells * n_templates);
   const int32_t used = fix_slots_used(n);
@@ -319,8 +320,8 @@ cudaError_t launch_flag_and_fixup(fmap_plan_s* p, const fmap_atoms* a, float* d_
   if (n_entries == 0 || p->n_templates == 0) return cudaSuccess;
   const int64_t n_blocks = (n_entries + kFlagUnit - 1) / kFlagUnit;
   if (n_blocks <= kFlagOnce) {
-    k_flag_list<<<(unsigned)n_blocks, kFlagBlock, 0, s>>>(p->ws.flag_bits, n_entries, p->ws.flag_list,
-                                                          p->ws.n_flag);
+    launch_after(p, k_flag_list, (unsigned)n_blocks, kFlagBlock, s, p->ws.flag_bits, n_entries,
+                 p->ws.flag_list, p->ws.n_flag);
     p->launches += 1;
   } else {
     k_flag_count<<<(unsigned)n_blocks, kFlagBlock, 0, s>>>(p->ws.flag_bits, n_entries, p->ws.flag_blocks);
@@ -334,7 +335,7 @@ cudaError_t launch_flag_and_fixup(fmap_plan_s* p, const fmap_atoms* a, float* d_
   // (few template groups: every slot at once; many: a few slots at a time)
   const dim3 grid((unsigned)(y <= 16 ? kFixSlots : kFixBlocks), (unsigned)y);
   auto run = [&](auto kern) {
-    kern<<<grid, kFixThreads, 0, s>>>(p->ws.flag_list, p->ws.n_flag, a->shared_antenna, p->ws.rel_t,
+    launch_after(p, kern, grid, kFixThreads, s, p->ws.flag_list, p->ws.n_flag, a->shared_antenna, p->ws.rel_t,
                                       p->ws.t_base, p->n_sft, p->grid, plan_axes(p), p->ws.wtab,
                                       p->n_tab, p->ws.i0, p->ws.jend, a->antenna, a->fafb,
                                       p->n_templates, d_2F, p->ws.partials, p->part_stride,

@@ -151,6 +151,7 @@ struct HeadArgs {
 };
 
 __global__ void __launch_bounds__(kTileThreads) k_ref_head(const HeadArgs A) {
+  stream_order();
   constexpr int NW = kTileThreads / 32;
   __shared__ int32_t h[kRefBins];
   __shared__ unsigned s_mu[NW], s_cnt[NW], s_arg[NW];
@@ -398,6 +399,7 @@ __device__ __forceinline__ void ref_scan_cells(const ScanArgs& A, int32_t j, int
 // one warp per share of a tile.  The histogram and the counts were cleared by the
 // first pass.
 __global__ void __launch_bounds__(kRefThreads) k_ref_scan(const ScanArgs A) {
+  stream_order();
   __shared__ int32_t h[kRefBins];
   __shared__ int32_t s_cut, s_n;
   const int32_t j = blockIdx.y;
@@ -461,6 +463,7 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_scan(const ScanArgs A) {
 // (a strong signal's tiles hold many cells near the maximum).  Every block of
 // the others ends at once.
 __global__ void __launch_bounds__(kRefThreads) k_ref_collect(const ScanArgs A) {
+  stream_order();
   const int32_t j = blockIdx.y;
   const TStat s = A.st[j];
   if (s.done[0] >= 0) return;
@@ -769,6 +772,7 @@ __device__ __forceinline__ void ref_summary(const RefArgs& A, int32_t j, int32_t
 }
 
 __global__ void __launch_bounds__(kRefThreads) k_ref_cells(const RefArgs A) {
+  stream_order();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int32_t j = blockIdx.y;
   const int32_t n_cand = min(A.ref_n[j], kRefMaxCells);
@@ -828,7 +832,7 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   H.ref_ntile = w.ref_ntile;
   H.ref_tile = w.ref_tile;
   H.cut = w.ref_bin;
-  k_ref_head<<<T, kTileThreads, 0, s>>>(H);
+  launch_after(p, k_ref_head, T, kTileThreads, s, H);
   ScanArgs S;
   S.map = d_2F;
   S.coef = w.coef;
@@ -864,8 +868,8 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
                                          ((int64_t)p->n_sm + T - 1) / T,
                                          ((int64_t)p->n_sm * 32 + T - 1) / T);
   const dim3 grid((unsigned)gx, (unsigned)T);
-  k_ref_scan<<<grid, kRefThreads, 0, s>>>(S);
-  k_ref_collect<<<grid, kRefThreads, 0, s>>>(S);
+  launch_after(p, k_ref_scan, grid, kRefThreads, s, S);
+  launch_after(p, k_ref_collect, grid, kRefThreads, s, S);
   RefArgs A;
   A.rel_t = w.rel_t;
   A.t_base = w.t_base;
@@ -893,7 +897,7 @@ cudaError_t launch_refine(fmap_plan_s* p, const fmap_atoms* a, float* d_2F,
   A.log_prior = p->log_prior;
   A.tol = fast_tol(p);
   A.out = d_summary;
-  k_ref_cells<<<dim3((unsigned)((cap + wpb - 1) / wpb), (unsigned)T), kRefThreads, 0, s>>>(A);
+  launch_after(p, k_ref_cells, dim3((unsigned)((cap + wpb - 1) / wpb), (unsigned)T), kRefThreads, s, A);
   p->launches += 4;
   return cudaGetLastError();
 }

@@ -199,6 +199,7 @@ static fmap_status launch_request(fmap_server_s* s, Request* r) {
   if (!r->plan) return FMAP_ERR_NOMEM;
   fmap_status st = plan_init(r->plan, &r->grid, r->n_sft, r->T, r->prec, r->pflags, d, r->ws_bytes);
   if (st != FMAP_OK) return st;
+  r->plan->early_launch = false;   // (other requests' streams run beside this one)
   char* q = d + align256(r->ws_bytes);
   const size_t n = (size_t)r->n_sft, T = (size_t)r->T;
   int64_t* d_t = (int64_t*)q;
