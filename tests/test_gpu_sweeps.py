@@ -91,3 +91,34 @@ def test_exp_off_lattice_times(prec, kind):
         t[150:] += 40 * T_SFT
         t[260:] += 16 * T_SFT
     _check(synth.Instance(t, inst.antenna, inst.fafb, grid), prec)
+
+
+@pytest.mark.parametrize("n_t0,n_tau", [(1, 1), (9, 33), (3, 64), (12, 65), (20, 129)])
+@pytest.mark.parametrize("n_templates", [1, 2, 5])
+def test_rect_wide_rows(n_t0, n_tau, n_templates):
+    """Rows that start more atoms apart than a staged group takes, at the edges of
+    the cells' tiles, by one, two and four template lanes per tile."""
+    grid = Grid(-T_SFT, 4 * T_SFT, n_t0, 2 * T_SFT, T_SFT, n_tau, RECT)
+    _check(synth.make_instance(950 + n_tau, n_det=2, presence=0.9, n_merged=500,
+                               n_templates=n_templates, grid=grid), "fp64")
+
+
+@pytest.mark.parametrize("at", [1, 2047, 2300, 4498])
+def test_exp_one_irregular_gap(at):
+    """One gap off the SFT lattice, in any of the parts the atoms are checked in."""
+    grid = Grid(-T_SFT, 60 * T_SFT, 45, 3 * T_SFT, 23 * T_SFT, 40, EXP)
+    inst = synth.make_instance(960, n_det=1, presence=0.9, n_merged=4500, n_templates=2, grid=grid)
+    t = inst.t.copy()
+    t[at:] += 777
+    _check(synth.Instance(t, inst.antenna, inst.fafb, grid), "rec")
+
+
+@pytest.mark.parametrize("n_tau", [1, 32, 33, 64, 65, 257])
+def test_table_antenna_columns(n_tau):
+    """Window tables at the edges of the antenna sums' 64 columns per warp and 256
+    per block, with samples of both signs that end above zero."""
+    x = np.linspace(0.0, 1.0, 37)
+    table = (np.cos(5.0 * x) * np.exp(-x)).astype(np.float32)
+    grid = Grid(-700, 1500, 7, 1200, 900, n_tau, synth.TABLE, T_SFT, 0, None, None, table)
+    _check(synth.make_instance(970, n_det=2, presence=0.9, n_merged=300, n_templates=2, grid=grid),
+           "fp64")
