@@ -68,8 +68,8 @@ typedef enum { FMAP_RECT = 0, FMAP_EXP = 1, FMAP_TABLE = 2 } fmap_window;
  * with error-free FMA products, ~2^-44 relative: GB300 runs FP64 at 1/64 of
  * the FP32 rate), the 2F coefficients FP32 from them (once per cell), and
  * the log-Bayes reduction FP64:
- *   FMAP_FP64   rect: FP64 prefix sums over SFTs (data rows kept as float
- *               pairs), O(1) compensated differences per cell;
+ *   FMAP_FP64   rect: exact prefix sums over SFTs (64-bit integers or FP64,
+ *               kept as float pairs), O(1) compensated differences per cell;
  *               exp:  FP64 contraction on the CUDA cores.
  *   FMAP_FP32   rect: one thread per t0 row with FP32 running sums of Fa, Fb
  *               (the paper's rectangular kernel, Sec. 3);
@@ -421,8 +421,8 @@ fmap_status fmap_server_peak(fmap_server_t* server, int64_t* peak_running);
 /*
  * Uneven batches: many independent F-map instances (each with its own atoms,
  * grid, window and template count; Sec. 3's per-template F-map, batched) run
- * by one captured CUDA graph.  Rectangular instances use the FP64 prefix
- * path, exponential ones the decayed-suffix recurrence (FMAP_FP64 accuracy
+ * by one captured CUDA graph.  Rectangular instances use the prefix
+ * path (FMAP_FP64), exponential ones the decayed-suffix recurrence (FMAP_FP64 accuracy
  * class, n_sft <= 9000).  Each phase of the pipeline is one persistent launch
  * over the work units of all instances (atomic work counter, heaviest
  * instances first); instances are grouped in waves whose workspace fits
@@ -451,13 +451,13 @@ fmap_status fmap_batch_run(fmap_batch_t* batch, fmap_stream stream);
  * any instance. */
 fmap_status fmap_batch_status(fmap_batch_t* batch, fmap_stream stream);
 /* Phases of a batch run, in launch order (FMAP_BATCH_N_PHASES entries):
- * input checks, index tables, exp chunk-major atom copies, rect antenna
- * prefixes, exp antenna sums and coefficients, rect coefficients, rect data
- * prefixes, exp recurrence and cells, rect cells, three steps of the
+ * input checks, index tables, exp atom copies, rect prefixes, exp antenna sums
+ * and coefficients (with the sweeps' chunk maps), rect coefficients, one that is
+ * empty (rect data prefixes: with the antenna's), exp recurrence and cells, rect cells, three steps of the
  * ill-conditioned cell compaction, float-float fix-up, two reduction levels. */
 #define FMAP_BATCH_N_PHASES 15
 /* Waves, kernel launches per run, workspace bytes, chosen occupancy per phase
- * (FMAP_BATCH_N_PHASES entries, nullable) and templates per block of the
+ * (FMAP_BATCH_N_PHASES entries, nullable) and templates per warp of the
  * recurrence. */
 fmap_status fmap_batch_info(fmap_batch_t* batch, int32_t* n_waves, int64_t* launches_per_run,
                             size_t* workspace_bytes, int32_t* occupancy,

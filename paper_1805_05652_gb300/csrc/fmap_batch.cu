@@ -2,7 +2,7 @@
 // window and template count) run by one captured CUDA graph.
 //
 // Every instance gets a plan carved out of one batch workspace: rectangular
-// windows take the FP64 prefix path, exponential windows the decayed-suffix
+// windows take the prefix path (FMAP_FP64), exponential windows the decayed-suffix
 // recurrence (FP64-class accuracy).  The single-plan pipeline -- input
 // checks, index tables, antenna sums and 2F coefficients, data sums and
 // cells, fix-up of ill-conditioned cells, reductions -- runs phase by

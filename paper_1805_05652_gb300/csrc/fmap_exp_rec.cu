@@ -21,10 +21,11 @@
 // into short runs to make enough warps, from the decayed sums of chunks of
 // atoms formed ahead by k_sweep_agg.
 //
-// Bound by instruction issue.  One block per tau with E in shared memory and a
-// scan over the atoms per template (two block barriers, four passes over shared
-// memory) took 73.8 ms for 1024 templates x 5000 SFTs over 2000 x 2000 cells,
-// latency-bound at 44 % issue.
+// Bound by waits for the atoms' loads and by issue: about 350 instructions per row
+// and four templates at 36 % issue, 12 warps per SM (168 registers): 23.2 ms for
+// 1024 templates x 5000 SFTs over 2000 x 2000 cells.  One block per tau with E in
+// shared memory and a scan over the atoms per template (two block barriers, four
+// passes over shared memory) took 73.8 ms there.
 #include <math.h>
 
 #include <algorithm>
