@@ -386,6 +386,8 @@ __global__ void __launch_bounds__(256) kb_exp_perm(const BItem* __restrict__ ite
                   it.irr, it.dev_err, it.g, it.ax, it.tauc, e0 + threadIdx.x, min(total, e0 + kPermPerUnit), 256);
   });
 }
+// (three blocks per SM, with a few spills, against two at 110 registers: 48 uneven
+// instances 707 against 766 us)
 __global__ void __launch_bounds__(kAntThreads, 3) kb_exp_ant(const BItem* __restrict__ items,
                                                              BUnits u) {
   __shared__ float2 s_pw[kAntWarps][kSweepTab];
