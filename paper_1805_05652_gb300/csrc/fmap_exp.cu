@@ -206,13 +206,15 @@ k_exp_antenna(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t_b
 // 32 tau anyway; rows
 // per warp so that about 16 warps per SM run at once, at least 4 (the start
 // costs about as much as eight); in a batch, whose instances fill the GPU
-// together, 64.
+// together, 64, or fewer where a row's step spans many SFTs.
 AntGeom ant_geom(const fmap_grid& g, int32_t n_sft, int64_t n_ant, bool batch, int64_t agg_room) {
   AntGeom q{};
   q.n_grp = std::max(1, (g.n_tau + 31) / 32);
   const int64_t warps = q.n_grp * std::max<int64_t>(n_ant, 1);   // per run of rows
   const int64_t want = ((int64_t)kSms * 16 + warps - 1) / warps;
-  q.rows = batch ? 64 : (int32_t)std::max<int64_t>(4, (g.n_t0 + want - 1) / want);
+  const int64_t step = g.dt0 / std::max<int64_t>(g.t_sft, 1);   // SFTs per row
+  q.rows = batch ? (int32_t)std::clamp<int64_t>(1024 / (step + 3), 8, 64)
+                 : (int32_t)std::max<int64_t>(4, (g.n_t0 + want - 1) / want);
   q.n_seg = std::max(1, (g.n_t0 + q.rows - 1) / q.rows);
   q.chunk = n_sft <= 1024 ? 16 : n_sft <= 4096 ? 32 : 128;
   q.n_chunks = (n_sft + q.chunk - 1) / q.chunk;

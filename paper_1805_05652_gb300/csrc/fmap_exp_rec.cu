@@ -575,6 +575,10 @@ RecGeom rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, bool shared, bool
   const double more = std::min<double>((double)n_sft, std::max(0.0, (double)g.dt0 / (double)g.t_sft - 1.0));
   const int32_t chunk0 = n_sft <= 512 ? 16 : n_sft <= 1024 ? 32 : n_sft <= 4096 ? 64 : 128;
   const double slots = kSms * 4.0;
+  // (a batch's instances run side by side: runs of 48 rows, or of as much work where
+  // a row's step spans several SFTs: 44 instances of up to 456 x 456 cells and 5329
+  // SFTs 1319 -> 951 us)
+  const double batch_rows = std::max(8.0, 48.0 * 360.0 / (360.0 + 110.0 * more));
   for (int G = 1; G <= g_max && (G == 1 || G <= T); G *= 2) {
     const int32_t tgrp = std::max(1, (T + G - 1) / G);
     if (G == 4 && (double)n_grp * tgrp < slots) break;   // (few warps per scheduler: two templates)
@@ -593,7 +597,7 @@ RecGeom rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, bool shared, bool
       for (int32_t seg = 1; seg <= 256; seg = seg < 4 ? seg + 1 : seg + seg / 3) {
         const int32_t rows = (g.n_t0 + seg - 1) / seg;
         if (seg > 1 && rows < 4) break;
-        if (batch && seg > 1 && rows < 48) break;   // (instances run side by side)
+        if (batch && seg > 1 && rows < batch_rows) break;
         const double work = start + rows * (150.0 + 210.0 * G + more * (60.0 + 50.0 * G));
         // a batch has other instances to fill the GPU: total work counts
         const double t = ahead + work * (batch ? (double)n_grp * tgrp * seg / slots + 0.3
