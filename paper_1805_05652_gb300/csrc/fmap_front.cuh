@@ -170,9 +170,16 @@ __device__ __forceinline__ void index_body(const Rel& rel_t, int64_t tb, int32_t
     }
   }
   __syncthreads();
-  // Both ends grow with t0, so the group's rows search within [lo of its
-  // first row, hi of its last), staged once when it fits.
-  const int32_t base = s_lo[0], span = s_hi[R - 1] - base;
+  // The group's rows search within the union of their ranges, staged once when it
+  // fits.  (Both ends grow with t0 where the timestamps increase, which the checks
+  // only report: the union is taken over all of the rows, so that no search
+  // leaves the staged part in any case.)
+  int32_t base = s_lo[0], top = s_hi[0];
+  for (int32_t r = 1; r < R; ++r) {
+    base = min(base, s_lo[r]);
+    top = max(top, s_hi[r]);
+  }
+  const int32_t span = top - base;
   const bool staged = span <= kIdxCap;
   if (staged)
     for (int k = tid; k < span; k += kIdxThreads) s_t[k] = rel_t[base + k];

@@ -1,0 +1,57 @@
+"""Timestamps that do not increase are reported (FMAP_ERR_DATA), and until the
+caller asks for the status every kernel of the call still runs on them: window ends
+that are not ordered stay inside every array, and the same plan or batch then
+computes the ordered data as if nothing had happened."""
+
+import numpy as np
+import pytest
+
+import synth
+from synth import EXP, T_SFT, Grid
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1805_05652_gb300 as fm  # noqa: E402
+
+
+def _blocks(n, block, seed):
+    """Times on the T_SFT lattice, the first in place, the others in blocks of
+    `block` atoms in random order."""
+    rng = np.random.default_rng(seed)
+    t = np.arange(n, dtype=np.int64) * T_SFT
+    q = np.arange(1, n) // block
+    order = rng.permutation(q.max() + 1)
+    t[1:] = t[1:][np.argsort(order[q], kind="stable")]
+    return t
+
+
+def _batch_recovers(inst, bad_t):
+    dev = torch.device("cuda:0")
+    t = torch.from_numpy(bad_t).to(dev)
+    a, x = torch.from_numpy(inst.antenna).to(dev), torch.from_numpy(inst.fafb).to(dev)
+    b = fm.Batch([(inst.grid, t, a, x)], autotune=False)
+    b.run()
+    assert b.status() == fm.FMAP_ERR_DATA
+    t.copy_(torch.from_numpy(inst.t))
+    b.run()
+    assert b.status() == fm.FMAP_OK
+    got = b.maps[0].cpu().numpy()
+    b.close()
+    c = fm.Batch([(inst.grid, t, a, x)], autotune=False)
+    c.run()
+    assert c.status() == fm.FMAP_OK
+    assert np.array_equal(got, c.maps[0].cpu().numpy())
+    c.close()
+
+
+def test_index_group_past_the_last_rows_range():
+    """A group of t0 rows whose first rows' windows reach further than its last
+    row's, with a union of ranges longer than the index step stages (8192)."""
+    n = 9000
+    grid = Grid(0, 100 * T_SFT, 24, 100 * T_SFT, 600 * T_SFT, 5, EXP)
+    inst = synth.make_instance(990, n_slots=n, grid=grid)
+    _batch_recovers(inst, _blocks(n, 300, 21))
