@@ -202,7 +202,7 @@ __device__ __forceinline__ void rect_cells_body(const int32_t* __restrict__ i0ta
   bool staged = true;
   for (int k = 0; k < n_grp; ++k) {
     const int4 e = s_grp[k];
-    if (e.y > 0 && (e.y - 1 > kMaxRowSpread || e.y > kRowCap || e.w > kJCap)) staged = false;
+    if (e.y > 0 && (e.y - 1 > kMaxRowSpread || e.y > kRowCap || e.w > kJCap || e.w < 1)) staged = false;
   }
   const int4 G = s_grp[grp];
 
@@ -212,16 +212,12 @@ __device__ __forceinline__ void rect_cells_body(const int32_t* __restrict__ i0ta
   auto in_grid = [&](int i) { return (i >> 1) < rows && ((i & 1) ? col1 : col0); };
   auto cell_off = [&](int i) { return (int64_t)(i >> 1) * n_tau + 32 * (i & 1); };
 
-  // Byte offsets within a slot's Q of the lane's window ends and row starts.
-  uint32_t qo[kLaneCells], ro[kTileRows];
+  // Prefix entries of the lane's window ends and row starts.
+  int32_t je[kLaneCells], is[kTileRows];
 #pragma unroll
-  for (int i = 0; i < kLaneCells; ++i) {
-    const int32_t j = in_grid(i) ? jend[cell0 + cell_off(i)] : G.z;
-    qo[i] = 16u * (uint32_t)(kRowCap + j - G.z);
-  }
+  for (int i = 0; i < kLaneCells; ++i) je[i] = in_grid(i) ? jend[cell0 + cell_off(i)] : G.z;
 #pragma unroll
-  for (int r = 0; r < kTileRows; ++r)
-    ro[r] = rows > 0 ? 16u * (uint32_t)(i0tab[m0 + min(r, rows - 1)] - G.x) : 0u;
+  for (int r = 0; r < kTileRows; ++r) is[r] = rows > 0 ? i0tab[m0 + min(r, rows - 1)] : G.x;
 
   float k1[kLaneCells], k2[kLaneCells];
   uint64_t nb2[kLaneCells];
@@ -273,6 +269,18 @@ __device__ __forceinline__ void rect_cells_body(const int32_t* __restrict__ i0ta
   // (each path with a loop of its own: its registers do not add to the other's)
   auto run = [&](auto is_staged) {
     constexpr bool kStaged = decltype(is_staged)::value;
+    // Byte offsets of the entries within a slot's Q.  Timestamps that do not increase
+    // (which the checks only report) leave a group's window ends unordered: an
+    // offset outside the slot is clamped to its last entry.
+    uint32_t qo[kLaneCells], ro[kTileRows];
+    if constexpr (kStaged) {
+#pragma unroll
+      for (int i = 0; i < kLaneCells; ++i)
+        qo[i] = 16u * min((uint32_t)(kRowCap + je[i] - G.z), (uint32_t)kSlotEntries - 1u);
+#pragma unroll
+      for (int r = 0; r < kTileRows; ++r)
+        ro[r] = 16u * min((uint32_t)(is[r] - G.x), (uint32_t)kRowCap - 1u);
+    }
     if (kStaged) issue(0);
     for (int st = 0; st < n_st; ++st) {
       const uint32_t qs = q_s0 + (uint32_t)((st & 1) * kQBytes);
@@ -342,10 +350,10 @@ __device__ __forceinline__ void rect_cells_body(const int32_t* __restrict__ i0ta
 #pragma unroll
           for (int r = 0; r < kTileRows; ++r) {
             uint64_t hi0, hi1, li0, li1, hj0[2], hj1[2], lj0[2], lj1[2];
-            entry(G.x + (int32_t)(ro[r] / 16u), hi0, hi1, li0, li1);
+            entry(is[r], hi0, hi1, li0, li1);
 #pragma unroll
             for (int q = 0; q < 2; ++q)
-              entry(G.z + (int32_t)(qo[2 * r + q] / 16u) - kRowCap, hj0[q], hj1[q], lj0[q], lj1[q]);
+              entry(je[2 * r + q], hj0[q], hj1[q], lj0[q], lj1[q]);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               const int i = 2 * r + q;

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import synth
-from synth import EXP, T_SFT, Grid
+from synth import EXP, RECT, T_SFT, Grid
 
 pytestmark = pytest.mark.gpu
 
@@ -48,6 +48,22 @@ def _batch_recovers(inst, bad_t):
     c.close()
 
 
+def _plan_recovers(inst, bad_t, prec, flags=0):
+    dev = torch.device("cuda:0")
+    a, x = torch.from_numpy(inst.antenna).to(dev), torch.from_numpy(inst.fafb).to(dev)
+    good, bad = torch.from_numpy(inst.t).to(dev), torch.from_numpy(bad_t).to(dev)
+    p = fm.Plan(inst.grid, inst.n_sft, inst.n_templates, prec, flags)
+    first, s0 = p.compute(good, a, x)
+    assert p.status() == fm.FMAP_OK
+    first, s0 = first.cpu().numpy(), s0.cpu().numpy()
+    p.compute(bad, a, x)
+    assert p.status() == fm.FMAP_ERR_DATA
+    again, s1 = p.compute(good, a, x)
+    assert p.status() == fm.FMAP_OK
+    assert np.array_equal(again.cpu().numpy(), first) and np.array_equal(s1.cpu().numpy(), s0)
+    p.close()
+
+
 def test_index_group_past_the_last_rows_range():
     """A group of t0 rows whose first rows' windows reach further than its last
     row's, with a union of ranges longer than the index step stages (8192)."""
@@ -55,3 +71,16 @@ def test_index_group_past_the_last_rows_range():
     grid = Grid(0, 100 * T_SFT, 24, 100 * T_SFT, 600 * T_SFT, 5, EXP)
     inst = synth.make_instance(990, n_slots=n, grid=grid)
     _batch_recovers(inst, _blocks(n, 300, 21))
+
+
+@pytest.mark.parametrize("n_templates", [1, 2, 4])
+@pytest.mark.parametrize("step", [1, 30])
+@pytest.mark.parametrize("block", [1, 7, 60, 300])
+def test_rect_window_ends_out_of_order(block, step, n_templates):
+    """Rectangular cells whose group's window ends lie below its first one, over
+    staged prefixes (steps of one SFT) and over global ones (30 SFTs)."""
+    grid = Grid(0, step * T_SFT, 40, 2 * T_SFT, 3 * T_SFT, 70, RECT)
+    inst = synth.make_instance(991, n_slots=1500, n_templates=n_templates, grid=grid)
+    for seed in range(3):
+        _plan_recovers(inst, _blocks(1500, block, seed), "fp64")
+    _batch_recovers(inst, _blocks(1500, block, 3))
