@@ -265,14 +265,17 @@ __device__ __forceinline__ void tau_tab_fill(const fmap_grid& g, int64_t tau, in
 }
 // Generic window w(x) from its table (entries k = 0..n-1: (w_k, w_{k+1} -
 // w_k), then the sentinel (0, 0)): linear between samples, 0 past the last.
-// u = x (n - 1) / X is the position in sample units (u >= 0).
+// u = x (n - 1) / X is the position in sample units.  u >= 0 where the timestamps
+// increase; a window may hold an earlier atom where they do not (which the checks
+// only report): the index stays in the table there too (as unsigned numbers,
+// negative ones lie past the sentinel).
 __device__ __forceinline__ float tab_weight(float u, const float2* tab, int32_t n) {
-  const int32_t k = min(__float2int_rz(u), n);   // u beyond the table: the sentinel
+  const uint32_t k = min((uint32_t)__float2int_rz(u), (uint32_t)n);   // u beyond the table: the sentinel
   const float2 e = tab[k];
   return fmaf(u - (float)k, e.y, e.x);
 }
 __device__ __forceinline__ double tab_weight64(double u, const float2* tab, int32_t n) {
-  const double fk = floor(u);
+  const double fk = fmax(floor(u), 0.0);
   const int32_t k = fk >= (double)n ? n : (int32_t)fk;
   const float2 e = tab[k];
   return (double)e.x + (u - (double)k) * (double)e.y;

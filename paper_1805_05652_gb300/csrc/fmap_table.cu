@@ -51,10 +51,11 @@ __device__ __forceinline__ void ff2_add_prod(FF2& S, uint64_t w, uint64_t nw, ui
   S.l = add2(S.l, add2(se, pe));
   S.h = s;
 }
-// tab_weight for u >= 0: the index floor(min(u, n)) by an addition to 2^23
-// rounded towards zero (n < 2^11).
+// tab_weight by an addition: the index floor(u), clamped to [0, n], is the mantissa
+// of its sum with 2^23 rounded towards zero (n < 2^11; below 0 the sum would leave
+// the binade and the mantissa's low bits mean another place).
 __device__ __forceinline__ float tab_weight_pos(float u, const float2* tab, float n) {
-  const float r = __fadd_rz(fminf(u, n), 8388608.0f);
+  const float r = __fadd_rz(fmaxf(fminf(u, n), 0.0f), 8388608.0f);
   const float2 e = tab[__float_as_uint(r) & 0xfffu];
   return fmaf(u - (r - 8388608.0f), e.y, e.x);
 }

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import synth
-from synth import EXP, RECT, T_SFT, Grid
+from synth import EXP, RECT, TABLE, T_SFT, Grid
 
 pytestmark = pytest.mark.gpu
 
@@ -84,3 +84,34 @@ def test_rect_window_ends_out_of_order(block, step, n_templates):
     for seed in range(3):
         _plan_recovers(inst, _blocks(1500, block, seed), "fp64")
     _batch_recovers(inst, _blocks(1500, block, 3))
+
+
+_X = np.linspace(0.0, 1.0, 257)
+_TABLE = tuple((np.cos(5.0 * _X) * np.exp(-_X)).astype(np.float32).tolist())
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "tf32", "bf16x3"])
+@pytest.mark.parametrize("kind", ["swap", 1, 7, 60])
+def test_table_times_before_t0(kind, prec):
+    """Sampled windows with atoms that start before the window's t0: one swapped
+    neighbouring pair, and blocks out of order."""
+    grid = Grid(0, T_SFT // 2, 60, 2 * T_SFT, T_SFT, 70, TABLE, T_SFT, 0, None, None, _TABLE)
+    inst = synth.make_instance(992, n_slots=300, n_templates=2, grid=grid)
+    if kind == "swap":
+        bad = inst.t.copy()
+        bad[[20, 21]] = bad[[21, 20]]
+    else:
+        bad = _blocks(300, kind, 5)
+    _plan_recovers(inst, bad, prec)
+
+
+@pytest.mark.parametrize("prec,rec", [("fp64", True), ("fp64", False), ("fp32", False),
+                                      ("tf32", False), ("bf16x3", False)])
+@pytest.mark.parametrize("block", [1, 60, 300])
+def test_exp_times_out_of_order(block, prec, rec):
+    grid = Grid(0, 3 * T_SFT, 60, T_SFT, 5 * T_SFT, 70, EXP)
+    inst = synth.make_instance(993, n_slots=1200, n_templates=3, grid=grid)
+    flags = fm.FMAP_PLAN_EXP_RECURRENCE if rec else 0
+    _plan_recovers(inst, _blocks(1200, block, 6), prec, flags)
+    if rec:
+        _batch_recovers(inst, _blocks(1200, block, 7))
