@@ -212,7 +212,8 @@ AntGeom ant_geom(const fmap_grid& g, int32_t n_sft, int64_t n_ant, bool batch, i
   q.n_grp = std::max(1, (g.n_tau + 31) / 32);
   const int64_t warps = q.n_grp * std::max<int64_t>(n_ant, 1);   // per run of rows
   const int64_t want = ((int64_t)kSms * 16 + warps - 1) / warps;
-  const int64_t step = g.dt0 / std::max<int64_t>(g.t_sft, 1);   // SFTs per row
+  // SFTs per row (a single row's dt0 is not restricted, nor used)
+  const int64_t step = g.n_t0 > 1 ? g.dt0 / std::max<int64_t>(g.t_sft, 1) : 1;
   q.rows = batch ? (int32_t)std::clamp<int64_t>(1024 / (step + 3), 8, 64)
                  : (int32_t)std::max<int64_t>(4, (g.n_t0 + want - 1) / want);
   q.n_seg = std::max(1, (g.n_t0 + q.rows - 1) / q.rows);

@@ -572,7 +572,8 @@ RecGeom rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, bool shared, bool
     const int64_t tau = g.tau_min + (int64_t)std::max(0, g.n_tau - 1) * k / 15 * g.dtau;
     win += std::min<double>(n_sft, (double)window_len(g, tau) / (double)g.t_sft) / 16.0;
   }
-  const double more = std::min<double>((double)n_sft, std::max(0.0, (double)g.dt0 / (double)g.t_sft - 1.0));
+  const double more = g.n_t0 > 1 ? std::min<double>((double)n_sft, std::max(0.0, (double)g.dt0 / (double)g.t_sft - 1.0))
+                                 : 0.0;
   const int32_t chunk0 = n_sft <= 512 ? 16 : n_sft <= 1024 ? 32 : n_sft <= 4096 ? 64 : 128;
   const double slots = kSms * 4.0;
   // (a batch's instances run side by side: runs of 48 rows, or of as much work where
