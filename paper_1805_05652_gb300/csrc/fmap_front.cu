@@ -159,7 +159,7 @@ cudaError_t launch_front(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
       x_checked = true;
     }
   }
-  F.n_ant_vals = ant_checked ? 0 : 3 * n * std::max(F.n_ant, 1);
+  F.n_ant_vals = ant_checked ? 0 : 3 * n * F.n_ant;
   F.n_x_vals = x_checked ? 0 : 4 * n * F.T;
   // enough threads for the timestamps and the bitmask, and for the value checks at
   // a few values per thread
