@@ -187,7 +187,7 @@ static Layout layout_of(const fmap_grid* g, int32_t n_sft, int32_t T, fmap_preci
   L.rel_t = take(sizeof(int32_t) * (size_t)rel_t_entries(n_sft));
   L.t_base = take(sizeof(int64_t) + sizeof(int32_t) * kIrrWords);
   L.irr = L.t_base + sizeof(int64_t);
-  L.dev_err = take(sizeof(uint32_t));
+  L.dev_err = take(sizeof(uint32_t) * (1 + kLevelWords));
   L.i0 = take(sizeof(int32_t) * std::max<int32_t>(g->n_t0, 1));
   L.jend = take(sizeof(int32_t) * std::max<int64_t>(cells, 1));
   L.ax = take(sizeof(int64_t) * std::max<int64_t>((int64_t)g->n_t0 + g->n_tau, 1));
@@ -342,6 +342,7 @@ fmap_status plan_init(fmap_plan_s* p, const fmap_grid* grid, int32_t n_sft, int3
   w.t_base = (int64_t*)(b + L.t_base);
   w.irr = (int32_t*)(b + L.irr);
   w.dev_err = (uint32_t*)(b + L.dev_err);
+  w.level = w.dev_err + 1;
   w.i0 = (int32_t*)(b + L.i0);
   w.jend = (int32_t*)(b + L.jend);
   w.ax = (int64_t*)(b + L.ax);
@@ -516,7 +517,7 @@ static fmap_status compute(fmap_plan_t* p, const fmap_atoms* a, float* d_2F,
   // summaries can be refined
   if (!d_2F && p->ws.own_map) d_2F = p->ws.own_map;
   if (p->needs_err_reset) {   // (outside any graph: an unread error is kept)
-    FMAP_CUDA(cudaMemsetAsync(p->ws.dev_err, 0, sizeof(uint32_t), s));
+    FMAP_CUDA(cudaMemsetAsync(p->ws.dev_err, 0, sizeof(uint32_t) * (1 + kLevelWords), s));
     p->needs_err_reset = false;
   }
   if ((p->flags & FMAP_PLAN_GRAPH) && !p->timing) {
@@ -651,7 +652,7 @@ fmap_status fmap_marginalise(fmap_plan_t* p, const float* d_2F, const uint8_t* d
   if (st != FMAP_OK) return st;
   p->last_stream = (cudaStream_t)stream;
   if (p->needs_err_reset) {
-    FMAP_CUDA(cudaMemsetAsync(p->ws.dev_err, 0, sizeof(uint32_t), (cudaStream_t)stream));
+    FMAP_CUDA(cudaMemsetAsync(p->ws.dev_err, 0, sizeof(uint32_t) * (1 + kLevelWords), (cudaStream_t)stream));
     p->needs_err_reset = false;
   }
   FMAP_CUDA(launch_marginalise(p, d_2F, d_valid, d_summary, (cudaStream_t)stream));

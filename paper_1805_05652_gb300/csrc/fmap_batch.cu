@@ -217,6 +217,7 @@ static BItem make_bitem(const fmap_plan_s* p, const fmap_batch_item& it, uint32_
   b.perm_x = w.perm_x;
   b.agg = w.agg;
   b.irr = w.irr;
+  b.level = w.level;
   b.tauc = w.tauc;
   b.ax = nullptr;   // batches take uniform grids
   b.px = w.px;

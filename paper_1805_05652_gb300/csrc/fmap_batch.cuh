@@ -41,6 +41,7 @@ struct BItem {
   float4* perm_x;
   float* agg;
   int32_t* irr;
+  uint32_t* level;
   TauTab* tauc;
   int64_t* ax;
   float4* px;

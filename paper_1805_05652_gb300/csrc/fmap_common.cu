@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(256) kb_prep(const BItem* __restrict__ items, 
     const int64_t ru = it.n_sft > 0 ? (it.n_alloc + 255) / 256 : 0;
     if (k < ru) {
       prep_body(it.t, it.n_sft, it.n_alloc, it.rel_t, it.t_base, it.dev_err, it.antenna,
-                (int64_t)3 * it.n_sft * it.n_ant, it.fafb, (int64_t)4 * it.n_sft * it.T, it.irr,
+                (int64_t)3 * it.n_sft * it.n_ant, it.fafb, (int64_t)4 * it.n_sft * it.T, it.irr, it.level,
                 make_uint3((unsigned)k, 0, 0), dim3((unsigned)ru));
     } else {
       const int64_t w0 = (k - ru) * kBitsPerUnit;

@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(256) kb_exp_perm(const BItem* __restrict__ ite
     const int64_t total = exp_copy_entries(it.n_sft, it.n_ant, n_x, it.g.n_tau);
     const int64_t e0 = k * kPermPerUnit;
     exp_perm_body(RelStored{it.rel_t}, it.n_sft, it.antenna, it.n_ant, it.fafb, n_x, it.perm_ant, it.perm_x,
-                  it.irr, it.dev_err, it.g, it.ax, it.tauc, e0 + threadIdx.x, min(total, e0 + kPermPerUnit), 256);
+                  it.irr, it.level, it.dev_err, it.g, it.ax, it.tauc, e0 + threadIdx.x, min(total, e0 + kPermPerUnit), 256);
   });
 }
 // (three blocks per SM, with a few spills, against two at 110 registers: 48 uneven

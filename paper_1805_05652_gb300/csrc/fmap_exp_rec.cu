@@ -13,8 +13,22 @@
 // the data set.  E at j enters through
 // the tail factor e^{-(t_j - t_{i0})/tau} <= e^{-3}..e^{-2} for the 3 tau cut:
 // there a plain FP32 recurrence with float-pair decays (no systematic decay
-// error; its random rounding error is scaled by the tail) is enough.  Windows
-// cut before 3 tau, whose tail is near 1, carry E at j like E at i0.
+// error; its random rounding error, up to 4e-6 of E for tau of thousands of SFTs, is
+// scaled by the tail) is enough, as long as E at j is of the window sum's size.
+// Windows cut before 3 tau, whose tail is near 1, carry E at j like E at i0.
+//
+// Where E at j can be much larger than the window's sum, the sweep takes care
+// (CARE): E at j is carried like E at i0, the tail's exponent is a float pair, and where
+// a window holds a small part of the atoms that its E covers, E starts anew from the
+// window alone.  That is for warps whose windows may start in a long outage (they hold
+// its last atoms only, and the tail is near 1), by the data's longest gap, and for data
+// whose level varies more than kLevelRange-fold (a glitch behind the windows).  2F
+// against the FP64 oracle at worst: in an outage of 3500 SFTs, tau of 1000-1750,
+// 2.8e-5 without and 1.3e-6 with; an atom 4000 times the noise up to 1350 SFTs behind the
+// windows 4.0e-5 and 9.8e-6.  Four templates per warp take it as two pairs (the second
+// E's registers); 1024 templates of 5000 SFTs, 2000 x 2000 cells: 22.2 ms, with an
+// outage of 1500 SFTs 37 ms (38 without the care: other gaps than the tabulated ones
+// take an FP64 exp).
 //
 // A warp starts from zero at its last row's window ends and sums those windows
 // first (long runs of rows, many templates), or, where the rows must be split
@@ -42,8 +56,10 @@ constexpr int kRecMaxSft = 9000;    // the recurrence's declared range
 // FP32 sums of a run are the largest rounding error of short windows (measured
 // against 64 bits, 400-630 SFTs: 1.2e-7 of the map's norm with runs of 3, 3e-7
 // with 24), while a renormalisation costs 26 instructions per template.
+// (A row run's first sums: kRecRun for any N.)
+constexpr int32_t kRecRun = 21;
 __host__ __device__ __forceinline__ int32_t rec_run(int32_t n) {
-  return min(21, max(3, ((n + 255) / 256) | 1));
+  return min(kRecRun, max(3, ((n + 255) / 256) | 1));
 }
 constexpr int kRecThreads = 32 * kRecWarps;
 constexpr int kAggThreads = 32 * kSweepWarps;
@@ -147,6 +163,7 @@ struct RecArgs {
   const int32_t* rel_t;
   const int64_t* t_base;
   const int32_t* irr;   // any word nonzero: some gap has code 0
+  const uint32_t* level;   // the data's range of levels (level_note)
   int32_t n, T;
   fmap_grid g;
   RecGeom q;
@@ -235,20 +252,18 @@ __device__ __forceinline__ void rec_agg_unit(const RecArgs& A, int64_t unit, flo
 }
 
 // SHORT: windows cut before 3 tau.  SH: coefficients shared by the templates.
-// IRR: some gap is not 1..15 whole SFTs.
-template <int G, bool SHORT, bool SH, bool IRR>
-__device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, float2* s_pw,
-                                             int lane) {
+// IRR: some gap is not 1..15 whole SFTs.  CARE: see the top.  The unit's templates
+// from tg0 on; u1: its rows and tau.
+template <int G, bool SHORT, bool SH, bool IRR, bool CARE>
+__device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int64_t u1,
+                                             float2* s_pw, int lane) {
   const fmap_grid& g = A.g;
   const RecGeom& q = A.q;
   constexpr int NC = SH ? 1 : G;   // coefficient sets
   // each cursor's next atom is loaded a step ahead, where registers allow
   constexpr bool PF = G < 4;
-  static_assert(PF || !SHORT, "four templates: the 3 tau cut only");
-  // unit: template groups fastest (they share the rows' indices and
-  // coefficients), then row runs, then tau from the longest windows down
-  const int32_t tg0 = (int32_t)(unit % q.n_tgrp) * G;
-  const int64_t u1 = unit / q.n_tgrp;
+  constexpr bool END = SHORT || CARE;   // E at j is carried like E at i0
+  static_assert(PF || !END, "four templates: the 3 tau cut, level data");
   const int32_t seg = (int32_t)(u1 % q.n_seg);
   const int32_t grp = q.n_grp - 1 - (int32_t)(u1 / q.n_seg);
   const int32_t n = A.n, n_tau = g.n_tau, run = rec_run(n);
@@ -259,6 +274,9 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, flo
   const TauTab* tt = A.tauc + nn;
   sweep_tab_load<1>(s_pw, tt, lane);
   const float c2 = tt->c2[0];
+  const float c2l = CARE ? (float)(-1.4426950408889634 * tt->inv_tau - (double)c2) : 0.0f;
+  const float half_tau = -0.72134752f / (c2 * (float)g.t_sft);   // tau / (2 T_sft)
+  int32_t jz = A.n;   // CARE: where E at j starts from zero, at the latest
   const int64_t cells = (int64_t)g.n_t0 * n_tau;
   const int64_t tb = n > 0 ? *A.t_base : 0;
   const float4* x = A.x + (int64_t)tg0 * n;
@@ -268,8 +286,9 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, flo
   int32_t i0 = A.i0tab[m_hi - 1], j = A.jend[(int64_t)(m_hi - 1) * n_tau + nn];
   Cursor<G> Ei;
   Ei.zero();
-  typename std::conditional<SHORT, Cursor<G>, PlainCursor<G>>::type Ej;
+  typename std::conditional<END, Cursor<G>, PlainCursor<G>>::type Ej;
   Ej.zero();
+  int32_t run_j = 0;   // END: the most atoms a lane's Ej took since its renormalisation
   int32_t ic, jc;
   if (q.n_chunks > 0) {
     // E at the first atoms of the chunks after those holding j and i0
@@ -328,27 +347,25 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, flo
     jc = min(n, bj * q.chunk);
   } else {
     // E starts from zero at each lane's window end of the last row
-    jc = j;
+    jc = jz = j;
     ic = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)j);
     const int32_t j_all = (int32_t)__reduce_min_sync(0xffffffffu, (unsigned)j);
     int32_t tn = n > 0 ? atom_time(A, ic) : 0;
-    int32_t since = 0;   // atoms since a renormalisation (lanes not yet at their ends: E is 0)
-    while (ic > max(i0, j_all)) {   // atoms past some lanes' ends
-      --ic;
-      Atom<G> at;
-      at.load(x, xs, ic);
-      const int32_t t = __ldg(A.rel_t + ic);
-      const FF r = sweep_gap_decay<1, IRR>(s_pw, tn - t, inv, t_sft, lane, tt);
-      tn = t;
-      if (ic < j) Ei.step(r, at);
-      // (without it the FP32 sums span up to 31 tau steps: 2F of the first rows off by
-      // 3.4e-7 rms at steps of 30 SFTs, against 1.3e-7)
-      if (++since >= run) {
-        Ei.renorm();
-        since = 0;
+    for (const int32_t end = max(i0, j_all); ic > end;) {   // atoms past some lanes' ends
+      // (without a renormalisation the FP32 sums span up to 31 tau steps: 2F of the
+      // first rows off by 3.4e-7 rms at steps of 30 SFTs, against 1.3e-7)
+      const int32_t stop = max(end, ic - kRecRun);
+      while (ic > stop) {
+        --ic;
+        Atom<G> at;
+        at.load(x, xs, ic);
+        const int32_t t = __ldg(A.rel_t + ic);
+        const FF r = sweep_gap_decay<1, IRR>(s_pw, tn - t, inv, t_sft, lane, tt);
+        tn = t;
+        if (ic < j) Ei.step(r, at);
       }
+      Ei.renorm();   // (the lanes' runs differ: from here they are equal)
     }
-    Ei.renorm();   // (the lanes' runs differ: from here they are equal)
   }
   // times of the cursors' atoms, and of the next ones (loaded a step ahead)
   int32_t ti = n > 0 ? atom_time(A, ic) : 0, tj = n > 0 ? atom_time(A, jc) : 0;
@@ -423,16 +440,22 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, flo
         ti = t;
         if (Ei.run >= run) Ei.renorm();
       }
-      while (jc > j) {
-        --jc;
-        const Atom<G> cur = aj;
-        const int32_t t = ej;
-        ej = __ldg(A.rel_t + max(jc - 1, 0));
-        aj.load(x, xs, jc - 1);
-        Ej.step(sweep_gap_decay<1, IRR>(s_pw, tj - t, inv, t_sft, lane, tt), cur);
-        tj = t;
-        if constexpr (SHORT)
-          if (Ej.run >= run) Ej.renorm();
+      // (END: the lanes step together, so that they renormalise together)
+      while (END ? __any_sync(0xffffffffu, jc > j) : jc > j) {
+        if (!END || jc > j) {
+          --jc;
+          const Atom<G> cur = aj;
+          const int32_t t = ej;
+          ej = __ldg(A.rel_t + max(jc - 1, 0));
+          aj.load(x, xs, jc - 1);
+          Ej.step(sweep_gap_decay<1, IRR>(s_pw, tj - t, inv, t_sft, lane, tt), cur);
+          tj = t;
+        }
+        if constexpr (END)
+          if (++run_j >= run) {
+            Ej.renorm();
+            run_j = 0;
+          }
       }
     } else {
       const FF ri = sweep_gap_decay<1, IRR>(s_pw, ti - ei, inv, t_sft, lane, tt);
@@ -471,9 +494,47 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, flo
     // for the default 3 tau cut.  Windows cut before 3 tau make it large, where
     // the difference E[i0] - tail E[j] loses 1 / (1 - tail): there a tail
     // above 1/2 comes from the correctly rounded-to-1-ulp exp2f.
-    const float dj = (float)(tj - ti);
-    float tail = rec_ex2(c2 * dj);
-    if (SHORT && tail > 0.5f) tail = exp2f(c2 * dj);
+    const float dj = (float)(tj - ti), xj = c2 * dj;
+    float tail = rec_ex2(xj);
+    if (END && tail > 0.5f) tail = exp2f(xj);
+    // (what the rounded slope and exponent leave: up to 4e-7)
+    if (CARE) tail = fmaf(tail, 0.69314718f * fmaf(c2l, dj, fmaf(c2, dj, -xj)), tail);
+    if constexpr (CARE) {
+      // E at j against the window's sum, in noise: tail times the root of the atoms
+      // that E sums (up to tau / 2 SFTs, none past jz) against the root of the
+      // window's.  Where it is larger, E at i0 is summed anew from the window alone.
+      const float part = tail * tail * fminf(half_tau, (float)(jz - j)), own = (float)(j - i0);
+      if (__any_sync(0xffffffffu, j > i0 + 1 && part > 4.0f * own)) {
+        const bool anew = j > i0 && part > own;   // (others that soon will)
+        const int32_t top = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)(anew ? j : i0));
+        if (anew) {
+          Ei.zero();
+          Ej.zero();
+          jz = j;
+        }
+        int32_t tn = atom_time(A, top);
+        constexpr int B = 4;   // atoms loaded ahead of the serial chain
+        for (int32_t a1 = top; a1 > i0; a1 -= B) {
+          Atom<G> at[B];
+          int32_t t[B];
+#pragma unroll
+          for (int u = 0; u < B; ++u) {
+            at[u].load(x, xs, a1 - 1 - u);
+            t[u] = __ldg(A.rel_t + max(a1 - 1 - u, 0));
+          }
+#pragma unroll
+          for (int u = 0; u < B; ++u) {
+            const int32_t a = a1 - 1 - u;
+            if (a < i0) break;
+            const FF r = sweep_gap_decay<1, IRR>(s_pw, tn - t[u], inv, t_sft, lane, tt);
+            tn = t[u];
+            if (anew && a < j) Ei.step(r, at[u]);
+          }
+          if ((top - a1) / B % 5 == 4) Ei.renorm();   // (every 20 atoms)
+        }
+        Ei.renorm();
+      }
+    }
     float pre2 = 1.0f;
     const int32_t d0 = (int32_t)(ti - t0r);
     if (d0 != 0) {
@@ -520,6 +581,43 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int64_t unit, flo
   }
 }
 
+// unit: template groups fastest (they share the rows' indices and coefficients),
+// then row runs, then tau from the longest windows down.
+// Sweeps of data that is not regular, out of line: their registers and instructions
+// stay out of the others' (in a plan's kernel the careful one only: one gap of 20 SFTs
+// in 1024 templates' data 27.7 ms, 34.4 with both; in a batch's both: 48 uneven
+// instances 2808 us, 2878 with one).  G templates from tg0 on, up to tg1.
+template <int G, bool SHORT, bool SH, bool CARE>
+__device__ __noinline__ void rec_unit_apart(const RecArgs& A, int32_t tg0, int32_t tg1, int64_t u1,
+                                            float2* s_pw, int lane) {
+  for (int32_t t0 = tg0; t0 < tg1; t0 += G)
+    exp_rec_unit<G, SHORT, SH, true, CARE>(A, t0, u1, s_pw, lane);
+}
+// A window whose tail is above 1/4 ends within 1.4 tau of its first atom: its t0 lies
+// in a gap of more than the rest of its length.
+template <int G, bool SHORT, bool SH, bool BATCH>
+__device__ __forceinline__ void rec_unit(const RecArgs& A, int64_t unit, float2* s_pw, int lane) {
+  const int32_t tg0 = (int32_t)(unit % A.q.n_tgrp) * G;
+  const int64_t u1 = unit / A.q.n_tgrp;
+  const int32_t gap = longest_gap(A.irr);
+  const bool varies = !SHORT && level_varies(A.level);
+  if (!gap && !varies) return exp_rec_unit<G, SHORT, SH, false, false>(A, tg0, u1, s_pw, lane);
+  if constexpr (!SHORT) {
+    const int32_t grp = A.q.n_grp - 1 - (int32_t)(u1 / A.q.n_seg);
+    const float rest = (float)exp_cut8_of(A.g) / 8.0f - 1.4f;   // (of the group's shortest windows)
+    if (varies || (float)gap > rest * (float)grid_tau(A.g, A.ax, grp * 32)) {
+      const RecArgs B = A;   // (its address is taken)
+      return rec_unit_apart<G < 4 ? G : 2, false, SH, true>(B, tg0, min(tg0 + G, A.T), u1, s_pw, lane);
+    }
+  }
+  if constexpr (BATCH) {
+    const RecArgs B = A;
+    rec_unit_apart<G, SHORT, SH, false>(B, tg0, min(tg0 + G, A.T), u1, s_pw, lane);
+  } else {
+    exp_rec_unit<G, SHORT, SH, true, false>(A, tg0, u1, s_pw, lane);
+  }
+}
+
 // (registers: the state of four templates takes about 160, of one about 100)
 template <int G, bool SHORT, bool SH>
 __global__ void __launch_bounds__(kRecThreads, G == 4 ? 3 : G == 2 ? 4 : 5)
@@ -528,8 +626,7 @@ k_exp_rec(const RecArgs A, int64_t units) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t unit = (int64_t)blockIdx.x * kRecWarps + warp;
   if (unit >= units) return;
-  if (irregular(A.irr)) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw[warp], lane);
-  else exp_rec_unit<G, SHORT, SH, false>(A, unit, s_pw[warp], lane);
+  rec_unit<G, SHORT, SH, false>(A, unit, s_pw[warp], lane);
 }
 // Chunk maps of the antenna rows (units [0, ant_units)), then of the data.
 struct AntAgg {
@@ -632,7 +729,7 @@ RecGeom rec_geom(const fmap_grid& g, int32_t n_sft, int32_t T, bool shared, bool
 // (the data's chunk maps follow the antenna rows')
 static RecArgs rec_args(const fmap_plan_s* p, const RecGeom& q, const AntGeom& a, int64_t n_ant,
                         float* d_2F) {
-  return RecArgs{p->ws.rel_t, p->ws.t_base, p->ws.irr, p->n_sft, p->n_templates, p->grid, q,
+  return RecArgs{p->ws.rel_t, p->ws.t_base, p->ws.irr, p->ws.level, p->n_sft, p->n_templates, p->grid, q,
                  p->ws.i0, p->ws.jend, p->ws.coef, p->ws.perm_x, p->ws.tauc,
                  plan_axes(p), p->ws.agg + ant_agg_floats(a, n_ant), d_2F, p->ws.partials, p->part_stride};
 }
@@ -689,7 +786,7 @@ cudaError_t launch_exp_rec(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cud
 
 // ---- persistent multi-instance dispatchers (uneven batches) ----
 static __device__ __forceinline__ RecArgs rec_args(const BItem& it) {
-  return RecArgs{it.rel_t, it.t_base, it.irr, it.n_sft, it.T, it.g, it.rg, it.i0, it.jend, it.coef,
+  return RecArgs{it.rel_t, it.t_base, it.irr, it.level, it.n_sft, it.T, it.g, it.rg, it.i0, it.jend, it.coef,
                  it.perm_x, it.tauc, it.ax, it.agg + ant_agg_floats(it.ag, it.n_ant), it.map,
                  it.partials, it.part_stride};
 }
@@ -714,12 +811,6 @@ __global__ void __launch_bounds__(kAggThreads, 2) kb_sweep_agg(const BItem* __re
     }
   });
 }
-template <int G, bool SHORT, bool SH>
-static __device__ __forceinline__ void rec_batch_unit(const RecArgs& A, int64_t unit, float2* s_pw,
-                                                      int lane) {
-  if (irregular(A.irr)) exp_rec_unit<G, SHORT, SH, true>(A, unit, s_pw, lane);
-  else exp_rec_unit<G, SHORT, SH, false>(A, unit, s_pw, lane);
-}
 // MAXG: the most templates per warp of the wave's instances (registers).  Three
 // blocks per SM: the body holds every variant of its unit, and at four (128
 // registers) it spilt 250 bytes in the row loop (the 48-instance batch: 1181 us
@@ -735,24 +826,24 @@ kb_exp_rec(const BItem* __restrict__ items, BUnits u) {
     const RecArgs A = rec_args(it);
     const bool brief = exp_cut8_of(it.g) < 24;
     if constexpr (MAXG >= 4)
-      if (it.rg.G == 4) return rec_batch_unit<4, false, true>(A, unit, s_pw[warp], lane);
+      if (it.rg.G == 4) return rec_unit<4, false, true, true>(A, unit, s_pw[warp], lane);
     if constexpr (MAXG >= 2)
       if (it.rg.G == 2) {
         if (it.shared) {
-          if (brief) rec_batch_unit<2, true, true>(A, unit, s_pw[warp], lane);
-          else rec_batch_unit<2, false, true>(A, unit, s_pw[warp], lane);
+          if (brief) rec_unit<2, true, true, true>(A, unit, s_pw[warp], lane);
+          else rec_unit<2, false, true, true>(A, unit, s_pw[warp], lane);
         } else {
-          if (brief) rec_batch_unit<2, true, false>(A, unit, s_pw[warp], lane);
-          else rec_batch_unit<2, false, false>(A, unit, s_pw[warp], lane);
+          if (brief) rec_unit<2, true, false, true>(A, unit, s_pw[warp], lane);
+          else rec_unit<2, false, false, true>(A, unit, s_pw[warp], lane);
         }
         return;
       }
     if (it.shared) {
-      if (brief) rec_batch_unit<1, true, true>(A, unit, s_pw[warp], lane);
-      else rec_batch_unit<1, false, true>(A, unit, s_pw[warp], lane);
+      if (brief) rec_unit<1, true, true, true>(A, unit, s_pw[warp], lane);
+      else rec_unit<1, false, true, true>(A, unit, s_pw[warp], lane);
     } else {
-      if (brief) rec_batch_unit<1, true, false>(A, unit, s_pw[warp], lane);
-      else rec_batch_unit<1, false, false>(A, unit, s_pw[warp], lane);
+      if (brief) rec_unit<1, true, false, true>(A, unit, s_pw[warp], lane);
+      else rec_unit<1, false, false, true>(A, unit, s_pw[warp], lane);
     }
   });
 }

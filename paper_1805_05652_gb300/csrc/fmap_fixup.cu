@@ -302,8 +302,10 @@ k_fixup(const int64_t* list, const int32_t* n_flag,
         const float* __restrict__ antenna, const float* __restrict__ fafb,
         int32_t n_templates, float* __restrict__ map, Partial* __restrict__ parts,
         int64_t stride, int64_t slot0, Coef* __restrict__ coef,
-        const TauTab* __restrict__ tauc) {
+        const TauTab* __restrict__ tauc, uint32_t* level) {
   stream_order();
+  // (the data's range of levels, read by the sweeps of this call, starts anew)
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kLevelWords) level[threadIdx.x] = 0u;
   const int64_t cells = (int64_t)g.n_t0 * g.n_tau;
   const int64_t n = min((int64_t)*n_flag, shared_antenna ? cells : cells * n_templates);
   const int32_t used = fix_slots_used(n);
@@ -340,7 +342,7 @@ cudaError_t launch_flag_and_fixup(fmap_plan_s* p, const fmap_atoms* a, float* d_
                                       p->n_tab, p->ws.i0, p->ws.jend, a->antenna, a->fafb,
                                       p->n_templates, d_2F, p->ws.partials, p->part_stride,
                                       p->n_tiles, p->ws.coef,
-                                      p->grid.window == FMAP_EXP ? p->ws.tauc : nullptr);
+                                      p->grid.window == FMAP_EXP ? p->ws.tauc : nullptr, p->ws.level);
   };
   fixup_group(p->n_templates, sh) == 4 ? run(k_fixup<4>) : run(k_fixup<1>);
   p->launches += 1;

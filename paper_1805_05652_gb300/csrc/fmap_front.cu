@@ -20,6 +20,7 @@ struct FrontArgs {
   int32_t* rel_t;
   int64_t* t_base;
   int32_t* irr;
+  uint32_t* level;
   uint4* bits;                  // marked-entry bitmask, cleared here
   int64_t n_bits;               // uint4s
   int32_t* i0;
@@ -72,7 +73,7 @@ __global__ void __launch_bounds__(kFrontThreads) k_front(const FrontArgs F) {
   }
   b -= F.b_irr;
   if (b < F.b_copy) {
-    exp_perm_body(rel, F.n, F.antenna, F.n_ant, F.fafb, F.n_x, F.perm_ant, F.perm_x, nullptr, F.err, F.g,
+    exp_perm_body(rel, F.n, F.antenna, F.n_ant, F.fafb, F.n_x, F.perm_ant, F.perm_x, nullptr, F.level, F.err, F.g,
                   F.ax, F.tauc, (int64_t)b * kFrontThreads + threadIdx.x,
                   exp_copy_entries(F.n, F.n_ant, F.n_x, F.g.n_tau),
                   (int64_t)F.b_copy * kFrontThreads);
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(kFrontThreads) k_front(const FrontArgs F) {
        i += (int64_t)F.b_prep * kFrontThreads)
     F.bits[i] = make_uint4(0u, 0u, 0u, 0u);
   prep_body(F.t, F.n, F.n_alloc, F.rel_t, F.t_base, F.err, F.n_ant_vals ? F.antenna : nullptr,
-            F.n_ant_vals, F.n_x_vals ? F.fafb : nullptr, F.n_x_vals, nullptr,
+            F.n_ant_vals, F.n_x_vals ? F.fafb : nullptr, F.n_x_vals, nullptr, nullptr,
             make_uint3((unsigned)b, 0, 0), dim3((unsigned)F.b_prep));
 }
 
@@ -116,6 +117,7 @@ cudaError_t launch_front(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s) {
   F.rel_t = p->ws.rel_t;
   F.t_base = p->ws.t_base;
   F.irr = p->ws.irr;
+  F.level = p->ws.level;
   F.bits = (uint4*)p->ws.flag_bits;
   F.i0 = p->ws.i0;
   F.jend = p->ws.jend;

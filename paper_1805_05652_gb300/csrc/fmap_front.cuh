@@ -40,8 +40,9 @@ __device__ __forceinline__ void prep_body(const int64_t* __restrict__ t, int32_t
                        int32_t* __restrict__ rel_t, int64_t* __restrict__ t_base,
                        uint32_t* __restrict__ err, const float* __restrict__ ant, int64_t n_ant_vals,
                        const float* __restrict__ x, int64_t n_x_vals, int32_t* __restrict__ irr,
-    const uint3 bid, const dim3 gdim) {
+                       uint32_t* __restrict__ level, const uint3 bid, const dim3 gdim) {
   if (irr && bid.x == 0 && threadIdx.x < kIrrWords) irr[threadIdx.x] = 0;   // (set by the copies)
+  if (level && bid.x == 0 && threadIdx.x < kLevelWords) level[threadIdx.x] = 0u;
   {
     const int64_t g0 = bid.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t step = (int64_t)gdim.x * blockDim.x;
@@ -80,23 +81,37 @@ struct RelTimes {
   }
 };
 
-// irr: kIrrWords words, any of them nonzero if a gap has no code (whole warps).
+// irr: kIrrWords words, the longest gaps without a code (s) of parts of the atoms, 0
+// where every gap has one (whole warps).
+static_assert(kIrrWords == 32, "one word per lane");
+__device__ __forceinline__ int32_t longest_gap(const int32_t* __restrict__ irr) {
+  return __reduce_max_sync(0xffffffffu, irr[threadIdx.x & 31]);
+}
 __device__ __forceinline__ bool irregular(const int32_t* __restrict__ irr) {
-  return __any_sync(0xffffffffu, irr[threadIdx.x & 31] != 0);
+  return longest_gap(irr) != 0;
+}
+// (1 where the times do not increase)
+__device__ __forceinline__ int32_t uncoded_gap(int32_t gap, int32_t t_sft) {
+  return gap_code(gap, t_sft) == 0 ? max(gap, 1) : 0;
 }
 
-// Word b of irr: whether any gap of the b-th of nb parts of the atoms is not
+// Word b of irr: the longest gap of the b-th of nb parts of the atoms that is not
 // 1..kPowTab-1 whole SFTs; the words past nb are cleared.
 template <typename Rel>
 __device__ __forceinline__ void irregular_body(const Rel& t, int32_t n, int32_t t_sft,
                                                int32_t* __restrict__ irr, int32_t b, int32_t nb) {
-  int bad = 0;
+  __shared__ int32_t s_gap;
+  if (threadIdx.x == 0) s_gap = 0;
+  __syncthreads();
+  int32_t gap = 0;
   const int32_t per = (n + nb - 1) / nb, i0 = b * per, i1 = min(n - 1, i0 + per);
 #pragma unroll 4
   for (int32_t i = i0 + threadIdx.x; i < i1; i += blockDim.x)
-    bad |= gap_code(t[i + 1] - t[i], t_sft) == 0;
-  bad = __syncthreads_or(bad);
-  if (threadIdx.x == 0) irr[b] = bad;
+    gap = max(gap, uncoded_gap(t[i + 1] - t[i], t_sft));
+  gap = __reduce_max_sync(0xffffffffu, gap);
+  if ((threadIdx.x & 31) == 0 && gap) atomicMax(&s_gap, gap);
+  __syncthreads();
+  if (threadIdx.x == 0) irr[b] = s_gap;
   if (b == 0 && threadIdx.x >= nb && threadIdx.x < kIrrWords) irr[threadIdx.x] = 0;
 }
 
@@ -197,28 +212,44 @@ __device__ __forceinline__ void index_body(const Rel& rel_t, int64_t tb, int32_t
   __syncthreads();   // s_t, s_lo and s_hi are reused by the block's next group
 }
 
+// The data's range of levels, noted by the copies for the sweeps: level[0] the bits
+// of the largest absolute value, level[1] the complement of the bits of the smallest
+// maximum of 32 neighbouring atoms (all-zero ones do not count; 0: there are none).
+// Both only grow; zero before the copies.
+constexpr float kLevelRange = 128.0f;
+__device__ __forceinline__ void level_note(uint32_t* level, unsigned hi, unsigned lo, int lane) {
+  if (lane != 0) return;   // (most warps have nothing new: no atomic)
+  if (hi > __ldcg(level)) atomicMax(level, hi);
+  if (lo != 0xffffffffu && ~lo > __ldcg(level + 1)) atomicMax(level + 1, ~lo);
+}
+__device__ __forceinline__ bool level_varies(const uint32_t* level) {
+  const uint32_t hi = level[0], lo = level[1];
+  return lo != 0u && __uint_as_float(hi) > kLevelRange * __uint_as_float(~lo);
+}
+
 // Copies of one instance's atoms for the sweeps, one 16-byte entry per atom:
 // sets 0..n_ant-1 the antenna rows with the code of the gap to the next atom
 // (gap_code), sets n_ant.. the data rows of each template (recurrence plans);
 // before them the per-tau constants (two entries per tau).  The values are checked
-// on the way; irr, if given, is set where a gap has no code.
+// on the way; irr, if given, takes the gaps without a code.  By whole warps of
+// consecutive entries.
 template <typename Rel>
 __device__ __forceinline__ void exp_perm_body(const Rel& rel_t, int32_t n,
                                               const float* __restrict__ antenna, int32_t n_ant,
                                               const float* __restrict__ fafb, int32_t n_x,
                                               float4* __restrict__ perm_ant,
                                               float4* __restrict__ perm_x,
-                                              int32_t* __restrict__ irr,
+                                              int32_t* __restrict__ irr, uint32_t* level,
                                               uint32_t* __restrict__ err, const fmap_grid& g,
                                               const int64_t* __restrict__ ax,
                                               TauTab* __restrict__ tauc, int64_t e_begin,
                                               int64_t e_end, int64_t e_step) {
   const int64_t n_tau2 = 2 * (int64_t)g.n_tau;
   bool bad = false;
-  for (int64_t e0 = e_begin; e0 < e_end; e0 += e_step) {
+  auto copy = [&](int64_t e0) -> float {   // a data entry's largest absolute value, else -1
     if (e0 < n_tau2) {   // the longest entries first
       tau_tab_fill(g, grid_tau(g, ax, e0 >> 1), (int)(e0 & 1), tauc + (e0 >> 1));
-      continue;
+      return -1.0f;
     }
     const int64_t e = e0 - n_tau2;
     const int64_t set = e / n, i = e - set * n;
@@ -229,15 +260,27 @@ __device__ __forceinline__ void exp_perm_body(const Rel& rel_t, int32_t n,
       const float4 v = make_float4(a[i], a[n + i], a[2 * (int64_t)n + i], __int_as_float(code));
       bad |= not_finite(v.x) || not_finite(v.y) || not_finite(v.z);
       perm_ant[e] = v;
-      if (irr && set == 0 && code == 0) *irr = 1;   // (a batch; cleared by the input checks)
-    } else {
-      const int64_t tq = set - n_ant;
-      const float* x = fafb + tq * 4 * (int64_t)n;
-      const float4 v = make_float4(x[i], x[n + i], x[2 * (int64_t)n + i], x[3 * (int64_t)n + i]);
-      bad |= not_finite(v.x) || not_finite(v.y) || not_finite(v.z) || not_finite(v.w);
-      perm_x[tq * n + i] = v;
+      if (irr && set == 0 && code == 0)   // (a batch; cleared by the input checks)
+        atomicMax(irr + (i & (kIrrWords - 1)), uncoded_gap(rel_t[i + 1] - t, (int32_t)g.t_sft));
+      return -1.0f;
     }
+    const int64_t tq = set - n_ant;
+    const float* x = fafb + tq * 4 * (int64_t)n;
+    const float4 v = make_float4(x[i], x[n + i], x[2 * (int64_t)n + i], x[3 * (int64_t)n + i]);
+    bad |= not_finite(v.x) || not_finite(v.y) || not_finite(v.z) || not_finite(v.w);
+    perm_x[tq * n + i] = v;
+    return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+  };
+  unsigned hi = 0u, lo = 0xffffffffu;
+  for (int64_t e0 = e_begin; __any_sync(0xffffffffu, e0 < e_end); e0 += e_step) {
+    const float top = e0 < e_end ? copy(e0) : -1.0f;
+    if (n_x == 0) continue;
+    const bool whole = __all_sync(0xffffffffu, top >= 0.0f);
+    const unsigned m = __reduce_max_sync(0xffffffffu, top > 0.0f ? __float_as_uint(top) : 0u);
+    hi = max(hi, m);
+    if (whole && m) lo = min(lo, m);
   }
+  if (n_x > 0) level_note(level, hi, lo, threadIdx.x & 31);
   finite_latch(bad, err);
 }
 

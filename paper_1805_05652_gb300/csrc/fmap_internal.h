@@ -161,6 +161,7 @@ __host__ __device__ inline int64_t grid_tau(const fmap_grid& g, const int64_t* a
   return ax ? ax[g.n_t0 + n] : g.tau_min + n * g.dtau;
 }
 constexpr int kIrrWords = 32;
+constexpr int kLevelWords = 2;
 // Entries of the exp copy step: two per tau, then one per atom and set.
 // (plan_axes, after the plan struct: the axes to pass kernels, or null.)
 __host__ __device__ inline int64_t exp_copy_entries(int32_t n_sft, int32_t n_ant, int32_t n_x,
@@ -191,8 +192,10 @@ struct Workspace {
   size_t bytes = 0;
   int32_t* rel_t = nullptr;      // [round_up(N, 64) + 64] t - t[0], zero padded
   int64_t* t_base = nullptr;     // [1] t[0]
-  int32_t* irr = nullptr;        // [kIrrWords] any nonzero: a gap is not 1..kPowTab-1 whole SFTs (exp)
+  int32_t* irr = nullptr;        // [kIrrWords] longest gaps (s) that are not 1..kPowTab-1 whole SFTs (exp; 0: none)
   uint32_t* dev_err = nullptr;   // [1] latched device error bits
+  uint32_t* level = nullptr;     // [kLevelWords] after it: the data's range of levels (exp; level_note), cleared
+                                 // by the fix-up for the plan's next call
   int32_t* i0 = nullptr;         // [n_t0] first atom with t >= t0_m
   int32_t* jend = nullptr;       // [n_t0][n_tau] one past the last atom of each window
   Coef* coef = nullptr;          // [T_ant][n_t0][n_tau]
