@@ -51,12 +51,13 @@ __device__ __forceinline__ void ff2_add_prod(FF2& S, uint64_t w, uint64_t nw, ui
   S.l = add2(S.l, add2(se, pe));
   S.h = s;
 }
-// tab_weight by an addition: the index floor(u), clamped to [0, n], is the mantissa
-// of its sum with 2^23 rounded towards zero (n < 2^11; below 0 the sum would leave
-// the binade and the mantissa's low bits mean another place).
-__device__ __forceinline__ float tab_weight_pos(float u, const float2* tab, float n) {
-  const float r = __fadd_rz(fmaxf(fminf(u, n), 0.0f), 8388608.0f);
-  const float2 e = tab[__float_as_uint(r) & 0xfffu];
+// tab_weight by an addition: for 0 <= u < 2^12 the index floor(u) is the mantissa of
+// the sum of u and 2^23 rounded towards zero.  Any other u (an atom past the cell's
+// window, whose weight the caller drops, or one before t0, where the timestamps do not
+// increase) gives some index of the table (n < 2^11 entries and the sentinel).
+__device__ __forceinline__ float tab_weight_pos(float u, const float2* tab, uint32_t n) {
+  const float r = __fadd_rz(u, 8388608.0f);
+  const float2 e = tab[min(__float_as_uint(r) & 0xfffu, n)];
   return fmaf(u - (r - 8388608.0f), e.y, e.x);
 }
 __device__ __forceinline__ FF ff_fold(FF S) { return fast_two_sum(S.h, S.l); }
@@ -92,7 +93,7 @@ k_table_antenna(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t
   const int64_t tb = n > 0 ? *t_base : 0;
   const int64_t t0rel = grid_t0(g, ax, m) - tb;
   const float* ant = antenna + (int64_t)ta * 3 * n;
-  const float nf = (float)n_tab;
+  const uint32_t nt = (uint32_t)n_tab;
   const uint64_t su2 = pk2(su[0], su[1]);
   FF2 S[3] = {{0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}};
   for (int32_t k0 = i0 + w * kTabKC; k0 < jmax; k0 += kTabWarps * kTabKC) {
@@ -116,7 +117,7 @@ k_table_antenna(const int32_t* __restrict__ rel_t, const int64_t* __restrict__ t
       const ulonglong2 ct = *reinterpret_cast<const ulonglong2*>(&s_at[w][kk][1]);
       float u0, u1;
       up2(mul2(ct.y, su2), u0, u1);
-      float w0 = tab_weight_pos(u0, s_tab, nf), w1 = tab_weight_pos(u1, s_tab, nf);
+      float w0 = tab_weight_pos(u0, s_tab, nt), w1 = tab_weight_pos(u1, s_tab, nt);
       w0 = kk < ke0 ? w0 * w0 : 0.0f;
       w1 = kk < ke1 ? w1 * w1 : 0.0f;
       const uint64_t w2 = pk2(w0, w1), nw2 = pk2(-w0, -w1);
