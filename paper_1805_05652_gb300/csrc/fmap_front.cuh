@@ -295,14 +295,17 @@ struct __align__(32) P4 {
 
 // Prefix sums of NC rows of n atoms by one block: out[2 i], out[2 i + 1] = hi,
 // lo of sum_{a < i} for i = 0..n (columns past NC are 0).  The sums are exact
-// 64-bit integers in units of 2^-S, S the largest with n max|x| 2^S < 2^61 per
+// 64-bit integers in units of 2^-S, S the largest with sum|x| 2^S < 2^62 per
 // row, and the pair holds the top 48 bits.  (The same scan in FP64, which GB300
 // runs at 1/64 of the FP32 rate, took eight FP64 operations per atom and row:
 // 423 us for 1024 templates of 5000 atoms, and 24 us for one block alone.)
-// The unit is fixed by the row's maximum, so rows whose level changes by more
-// than 2^35 / n from one stretch of 32 atoms to another (an outlier or a step;
-// the windows before it would lose their sums), rows below 2^-58 and blocks of
-// fewer than 64 atoms are summed in FP64.
+// The unit is fixed by the row's sum, so rows with an atom (other than 0) below 2^-37
+// of it, which the unit holds to less than 25 bits (before an outlier or a step the
+// windows would lose their sums), rows below 2^-57 and blocks of fewer than 64 atoms
+// are summed in FP64: of noise of 5000 atoms one template in a thousand.  (By the
+// maxima of stretches of 32 atoms, and n max|x| for the sum, none was, but a glitch in
+// every stretch hid the small atoms before the first of them, whose windows lost up to
+// all of their sums; by every atom and n max|x| two templates in a hundred were.)
 // A tile of kScanTile atoms at a time: each thread sums kScanPer neighbours,
 // the warps scan the threads' sums by shuffles, and the entries leave through
 // shared memory so that the block writes whole lines.
@@ -310,14 +313,14 @@ struct ScanSmem {
   float tile[4][kScanTile];
   float4 ent[2 * kScanTile];
   unsigned long long wsum[4][kScanThreads / 32];
-  float wmax[4][kScanThreads / 32], wmin[4][kScanThreads / 32];
+  float wabs[4][kScanThreads / 32], wmin[4][kScanThreads / 32];
 };
 constexpr int32_t kScanFixMin = 64;   // fewest atoms of an integer scan
 
-// Exponent e of a row with maximum mx (mx < 2^e).
-__host__ __device__ inline int scan_exponent(float mx) {
+// Exponent e of v >= 0 (v < 2^e; 0 of 0).
+__host__ __device__ inline int scan_exponent(float v) {
   int e = 0;
-  if (mx > 0.0f) frexpf(mx, &e);
+  if (v > 0.0f) frexpf(v, &e);
   return e;
 }
 // Place of entry float4 k in the staging buffer: a thread's entries are 2 kScanPer
@@ -440,46 +443,42 @@ __device__ __forceinline__ void rect_scan_body(const float* __restrict__ x, int3
   bool fix = n >= kScanFixMin;
   float up[NC], down[NC];
   if (fix) {
-    // each row's maximum, and the smallest maximum of its stretches of 32 atoms
-    // (all-zero stretches do not count)
-    float mx[NC], mn[NC];
+    // each row's sum of absolute values and the smallest of them (zeros do not count)
+    float sum[NC], mn[NC];
     bool bad = false;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      mx[c] = 0.0f;
+      sum[c] = 0.0f;
       mn[c] = 3.402823466e38f;
 #pragma unroll 4
-      for (int32_t a = tid; a < n + lane - 31; a += kScanThreads) {   // (whole stretches)
-        const float m = __uint_as_float(
-            __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(x[c * (int64_t)n + a]))));
+      for (int32_t a = tid; a < n; a += kScanThreads) {
+        const float m = fabsf(x[c * (int64_t)n + a]);
         bad |= not_finite(m);
-        mx[c] = fmaxf(mx[c], m);
+        sum[c] += m;
         if (m > 0.0f) mn[c] = fminf(mn[c], m);
       }
-      const int32_t rest = n & ~31;   // the last atoms: part of the maximum only
-      if (warp == 0 && rest + lane < n) {
-        const float m = fabsf(x[c * (int64_t)n + rest + lane]);
-        bad |= not_finite(m);
-        mx[c] = fmaxf(mx[c], m);
-      }
-      mx[c] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx[c])));
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) sum[c] += __shfl_xor_sync(0xffffffffu, sum[c], d);
+      mn[c] = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(mn[c])));
       if (lane == 0) {
-        sm.wmax[c][warp] = mx[c];
+        sm.wabs[c][warp] = sum[c];
         sm.wmin[c][warp] = mn[c];
       }
     }
     finite_latch(bad, err);
     __syncthreads();
-    const int bits = 32 - __clz(n);   // n < 2^bits
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
+      sum[c] = 0.0f;
 #pragma unroll
       for (int w = 0; w < NW; ++w) {
-        mx[c] = fmaxf(mx[c], sm.wmax[c][w]);
+        sum[c] += sm.wabs[c][w];
         mn[c] = fminf(mn[c], sm.wmin[c][w]);
       }
-      const int e = scan_exponent(mx[c]), S = 61 - bits - e;
-      fix = fix && (mx[c] == 0.0f || (S <= 119 && S >= -100 && scan_exponent(mn[c]) >= e + bits - 35));
+      // (a thread adds n / 256 values: up to 2^24 atoms the FP32 sum is within 2^-8)
+      const int e = scan_exponent(sum[c] * 1.00390625f), S = 62 - e;
+      fix = fix && n <= 1 << 24 && !not_finite(sum[c] * 1.00390625f) &&
+            (sum[c] == 0.0f || (S <= 119 && S >= -100 && scan_exponent(mn[c]) >= e - 36));
       const int Sc = max(-100, min(119, S));
       up[c] = __int_as_float((Sc + 127) << 23);
       down[c] = __int_as_float((127 - Sc) << 23);

@@ -3,7 +3,10 @@
 import numpy as np
 import pytest
 
+import oracle
+import synth
 from synth import EXP, RECT, T_SFT, Grid
+from tests.parity_util import TOL, check_map
 
 pytestmark = pytest.mark.gpu
 
@@ -30,3 +33,28 @@ def test_no_templates_no_antenna_rows(window):
     call(p.handle, a, None, out, None)
     assert p.status() == fm.FMAP_OK
     p.close()
+
+
+@pytest.mark.parametrize("n", [80, 1200, 9000])
+@pytest.mark.parametrize("level", [1e9, 1e12, 1e15])
+def test_prefix_sums_before_periodic_outliers(n, level):
+    """One outlier in every 32 atoms: the windows before the first of them keep their
+    sums, as they do before a single one.  The last atoms of the data alike, behind
+    zeros."""
+    grid = Grid(0, T_SFT, 20, 2 * T_SFT, T_SFT, 8, RECT)
+    head = synth.make_instance(1301, n_det=2, n_slots=n, n_templates=2, grid=grid)
+    head.fafb[:, :, 31::32] *= np.float32(level)
+    last = (n - 1) // 32 * 32 - 32            # the last whole 32 atoms and the rest
+    tail_grid = Grid(last * T_SFT, T_SFT, 20, 2 * T_SFT, T_SFT, 8, RECT)
+    tail = synth.make_instance(1302, n_det=2, n_slots=n, n_templates=2, grid=tail_grid)
+    tail.fafb[:, :, :last] = 0.0
+    tail.fafb[:, :, last + 31:] *= np.float32(level)
+    for inst in (head, tail):
+        t, a, x = (torch.from_numpy(v).cuda() for v in (inst.t, inst.antenna, inst.fafb))
+        p = fm.Plan(inst.grid, n, 2, "fp64")
+        p.set_refine(0)
+        m, _ = p.compute(t, a, x)
+        assert p.status() == fm.FMAP_OK
+        p.close()
+        ref, val, _ = oracle.fmap(inst.t, inst.antenna, inst.fafb, inst.grid.as_tuple(), mode="direct")
+        check_map(m.cpu().numpy().astype(np.float64), ref, val, TOL["fp64"])
