@@ -44,6 +44,7 @@ struct Tuning {
 
 std::mutex g_tune_mu;
 std::map<std::string, Tuning> g_tune_cache;
+constexpr size_t kTuneCacheMax = 1024;   // size classes kept
 
 // max_g: the most templates per warp of the wave's recurrences.
 const void* phase_kernel(int ph, int max_g) {
@@ -307,19 +308,24 @@ static fmap_status place_wave(fmap_batch_s* B, int w) {
   return FMAP_OK;
 }
 
+static int log2_of(double v) { return (int)std::log2(1.0 + std::max(0.0, v)); }
+
+// Size class: the device and counts of instances per window, log2 of N_SFT, N_t0,
+// N_tau and T, and what else decides how their work splits (antenna rows shared or
+// not, windows cut before 3 tau, log2 of the SFTs per t0 row).
 static std::string signature(const fmap_batch_s* B) {
-  // size class: counts of instances per (window, log2 N_SFT, log2 cells, log2 T)
   std::map<std::string, int> h;
-  for (size_t i = 0; i < B->items.size(); ++i) {
-    const fmap_batch_item& it = B->items[i];
-    const int64_t cells = (int64_t)it.grid.n_t0 * it.grid.n_tau;
-    const std::string k = std::to_string(it.grid.window) + "/" +
-                          std::to_string((int)std::log2(1.0 + it.atoms.n_sft)) + "/" +
-                          std::to_string((int)std::log2(1.0 + cells)) + "/" +
-                          std::to_string((int)std::log2(1.0 + it.atoms.n_templates));
+  for (const fmap_batch_item& it : B->items) {
+    const fmap_grid& g = it.grid;
+    const double step = g.n_t0 > 1 ? (double)g.dt0 / (double)g.t_sft : 1.0;
+    std::string k;
+    for (const int v : {(int)g.window, log2_of(it.atoms.n_sft), log2_of(g.n_t0), log2_of(g.n_tau),
+                        log2_of(it.atoms.n_templates), it.atoms.shared_antenna ? 1 : 0,
+                        g.window == FMAP_EXP && exp_cut8_of(g) < 24 ? 1 : 0, log2_of(step)})
+      k += std::to_string(v) + "/";
     h[k] += 1;
   }
-  std::string s;
+  std::string s = std::to_string(B->device) + ":";
   for (auto& kv : h) s += kv.first + ":" + std::to_string(kv.second) + ";";
   return s;
 }
@@ -399,6 +405,7 @@ static fmap_status autotune(fmap_batch_s* B) {
   if (st != FMAP_OK) return st;
   B->tune = best;
   std::lock_guard<std::mutex> lk(g_tune_mu);
+  if (g_tune_cache.size() >= kTuneCacheMax) g_tune_cache.clear();
   g_tune_cache[sig] = best;
   return FMAP_OK;
 }
