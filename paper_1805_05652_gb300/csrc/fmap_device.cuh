@@ -136,12 +136,12 @@ __device__ __forceinline__ FF fast_two_sum(float a, float b) {
   return {s, b - (s - a)};
 }
 __device__ __forceinline__ FF ff_mul(FF a, FF b) {
-  const float p = a.h * b.h;
+  const float p = __fmul_rn(a.h, b.h);
   const float e = fmaf(a.h, b.h, -p);
   return fast_two_sum(p, e + fmaf(a.h, b.l, a.l * b.h));
 }
 __device__ __forceinline__ FF ff_mul_f(FF a, float b) {
-  const float p = a.h * b;
+  const float p = __fmul_rn(a.h, b);
   const float e = fmaf(a.h, b, -p);
   return fast_two_sum(p, fmaf(a.l, b, e));
 }
@@ -159,7 +159,7 @@ __device__ __forceinline__ void ff_acc(FF& s, FF w, float x) {
 // normalisation of r e): TwoProd of the high parts, TwoSum with s, one
 // final renormalisation; ~2^-46 relative, as ff_add(s, ff_mul(r, e)).
 __device__ __forceinline__ FF ff_fma_sum(FF s, FF r, FF e) {
-  const float p = r.h * e.h;
+  const float p = __fmul_rn(r.h, e.h);
   const float pe = fmaf(r.h, e.h, -p);
   const float t = s.h + p;
   const float bb = t - s.h;
@@ -309,7 +309,7 @@ __host__ __device__ __forceinline__ double tab_scale(int32_t n, int32_t cut8, in
 // and the low part r.l of the decay).  The pair is left unnormalised between
 // calls; ch_norm folds c back into h.
 __device__ __forceinline__ void ch_step(FF r, float x, float& h, float& c) {
-  const float p = r.h * h;
+  const float p = __fmul_rn(r.h, h);
   const float pe = fmaf(r.h, h, -p);
   const float s = p + x;
   const float bb = s - p;
@@ -319,7 +319,7 @@ __device__ __forceinline__ void ch_step(FF r, float x, float& h, float& c) {
 }
 // R <- r R for the compensated running product of the decays.
 __device__ __forceinline__ void ch_mul(FF r, float& h, float& c) {
-  const float p = r.h * h;
+  const float p = __fmul_rn(r.h, h);
   const float pe = fmaf(r.h, h, -p);
   c = fmaf(r.h, c, fmaf(r.l, h, pe));
   h = p;

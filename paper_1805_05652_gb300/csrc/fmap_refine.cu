@@ -658,8 +658,14 @@ __device__ __forceinline__ void ref_cell_sums(const RefArgs& A, int32_t j, int32
   ref_butterfly(s);
 }
 
+// a b + c d with the second product rounded and the first fused into the sum.
+__device__ __forceinline__ double ref_sum2(double a, double b, double c, double d) {
+  return __fma_rn(a, b, __dmul_rn(c, d));
+}
 // 2F of the cell in slot k of template j from its sums, in FP64 (one lane; records
-// the fast and the refined value, and writes the latter to the map).
+// the fast and the refined value, and writes the latter to the map).  Which products
+// are fused is part of which cell of a tie is reported, so the code says it rather
+// than the compiler.
 __device__ __forceinline__ void ref_cell_end(const RefArgs& A, int32_t j, int32_t k, const FF (&s)[7]) {
   const int64_t slot = (int64_t)j * kRefMaxCells + k;
   const int32_t c = A.ref_cell[slot];
@@ -668,12 +674,15 @@ __device__ __forceinline__ void ref_cell_end(const RefArgs& A, int32_t j, int32_
 #pragma unroll
   for (int q = 0; q < 7; ++q) v7[q] = (double)s[q].h + (double)s[q].l;
   const double Aa = v7[0], Bb = v7[1], Cc = v7[2];
-  const double D = Aa * Bb - Cc * Cc;
+  const double D = __fma_rn(Aa, Bb, -__dmul_rn(Cc, Cc));
   const bool ok = len >= 2 && D > 0.0;
   double v = 0.0;
-  if (ok)
-    v = 2.0 * (Bb * (v7[3] * v7[3] + v7[4] * v7[4]) + Aa * (v7[5] * v7[5] + v7[6] * v7[6]) -
-               2.0 * Cc * (v7[3] * v7[5] + v7[4] * v7[6])) / D;
+  if (ok) {
+    const double fa2 = ref_sum2(v7[3], v7[3], v7[4], v7[4]);
+    const double fb2 = ref_sum2(v7[5], v7[5], v7[6], v7[6]);
+    const double fab = ref_sum2(v7[3], v7[5], v7[4], v7[6]);
+    v = 2.0 * __fma_rn(-2.0 * Cc, fab, ref_sum2(Bb, fa2, Aa, fb2)) / D;
+  }
   float* mp = A.map + (int64_t)j * A.cells + c;
   A.ref_fast[slot] = *mp;
   A.ref_val[slot] = ok ? v : -1.0;
@@ -788,8 +797,6 @@ __global__ void __launch_bounds__(kRefThreads) k_ref_cells(const RefArgs A) {
       FF s[7];
       const int32_t c = A.ref_cell[(int64_t)j * kRefMaxCells + k0 + warp];
       if (ex) {
-        // (from the registers of the cell's own warp: from shared memory the compiler
-        // fuses other products, and other cells of a tie are reported)
         ref_exp_sums(A, j, c, lane, s);
         if (lane == 0) ref_cell_end(A, j, k0 + warp, s);
       } else {
