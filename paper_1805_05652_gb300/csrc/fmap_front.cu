@@ -47,7 +47,9 @@ struct FrontArgs {
 constexpr int kFrontThreads = 256;
 static_assert(kFrontThreads == kIdxThreads && kFrontThreads == kScanThreads, "roles share blocks");
 
-__global__ void __launch_bounds__(kFrontThreads) k_front(const FrontArgs F) {
+// (three blocks per SM: at two, by registers, 329 scans of 4606 atoms took a second wave
+// and the call 399 us for 363)
+__global__ void __launch_bounds__(kFrontThreads, 3) k_front(const FrontArgs F) {
   extern __shared__ __align__(16) unsigned char s_front[];
   int32_t b = blockIdx.x;
   if (b < F.b_scan) {

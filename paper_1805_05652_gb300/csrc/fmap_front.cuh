@@ -299,13 +299,13 @@ struct __align__(32) P4 {
 // row, and the pair holds the top 48 bits.  (The same scan in FP64, which GB300
 // runs at 1/64 of the FP32 rate, took eight FP64 operations per atom and row:
 // 423 us for 1024 templates of 5000 atoms, and 24 us for one block alone.)
-// The unit is fixed by the row's sum, so rows with an atom (other than 0) below 2^-37
-// of it, which the unit holds to less than 25 bits (before an outlier or a step the
-// windows would lose their sums), rows below 2^-57 and blocks of fewer than 64 atoms
-// are summed in FP64: of noise of 5000 atoms one template in a thousand.  (By the
-// maxima of stretches of 32 atoms, and n max|x| for the sum, none was, but a glitch in
-// every stretch hid the small atoms before the first of them, whose windows lost up to
-// all of their sums; by every atom and n max|x| two templates in a hundred were.)
+// The unit is fixed by the row's sum, so rows with two neighbouring atoms (not both 0)
+// below 2^-37 of it, which the unit holds to less than 25 bits (before an outlier or a
+// step the windows, of two atoms at least, would lose their sums), rows below 2^-57
+// and blocks of fewer than 64 atoms are summed in FP64.  (By the maxima of stretches of
+// 32 atoms a glitch in every stretch hid the small atoms before the first of them,
+// whose windows lost up to all of their sums; by every atom for itself a zero crossing
+// of the antenna pattern put a year's b^2, and 18 us more, on the FP64 path.)
 // A tile of kScanTile atoms at a time: each thread sums kScanPer neighbours,
 // the warps scan the threads' sums by shuffles, and the entries leave through
 // shared memory so that the block writes whole lines.
@@ -443,20 +443,36 @@ __device__ __forceinline__ void rect_scan_body(const float* __restrict__ x, int3
   bool fix = n >= kScanFixMin;
   float up[NC], down[NC];
   if (fix) {
-    // each row's sum of absolute values and the smallest of them (zeros do not count)
+    // each row's sum of absolute values, and the smallest maximum of two neighbours
+    // (two zeros do not count)
     float sum[NC], mn[NC];
     bool bad = false;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       sum[c] = 0.0f;
       mn[c] = 3.402823466e38f;
-#pragma unroll 4
-      for (int32_t a = tid; a < n; a += kScanThreads) {
-        const float m = fabsf(x[c * (int64_t)n + a]);
-        bad |= not_finite(m);
-        sum[c] += m;
-        if (m > 0.0f) mn[c] = fminf(mn[c], m);
+    }
+#pragma unroll 2
+    for (int32_t a0 = 32 * warp; a0 < n; a0 += kScanThreads) {   // (the rows' loads together)
+      const int32_t a = a0 + lane;
+      float m[NC], next[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const float* r = x + c * (int64_t)n + a;
+        m[c] = a < n ? fabsf(r[0]) : 0.0f;
+        next[c] = lane == 31 && a + 1 < n ? fabsf(r[1]) : 0.0f;
       }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        bad |= not_finite(m[c]);
+        sum[c] += m[c];
+        const float y = __shfl_down_sync(0xffffffffu, m[c], 1);
+        const float top = fmaxf(m[c], lane < 31 ? y : next[c]);
+        if (a + 1 < n && top > 0.0f) mn[c] = fminf(mn[c], top);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
 #pragma unroll
       for (int d = 16; d > 0; d >>= 1) sum[c] += __shfl_xor_sync(0xffffffffu, sum[c], d);
       mn[c] = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(mn[c])));
