@@ -129,10 +129,4 @@ __device__ __forceinline__ void batch_loop(const BItem* __restrict__ items, cons
   }
 }
 
-// Host launchers of the per-phase dispatchers (one per file holding the body).
-cudaError_t launch_batch_phase(int phase, const BItem* d_items, const BUnits& u, int grid,
-                               size_t dyn_smem, cudaStream_t s);
-int batch_phase_threads(int phase);
-const void* batch_phase_kernel(int phase);
-
 }  // namespace fmap

@@ -127,29 +127,12 @@ k_reduce_groups(const Partial* __restrict__ parts, int64_t n_tiles, int64_t fix0
   reduce_groups_body(parts, n_tiles, fix0, n_flag, entries, stride, n_groups, groups, blockIdx, gridDim);
 }
 
-// Level 2: one block per template over its groups; writes the summary and,
-// when tstat is given, the statistics the refinement starts from (and clears
-// that template's refinement histogram and candidate count).
+// Level 2: one block per template over its groups; writes the summary.
 __device__ __forceinline__ void reduce_final_body(const Partial64* __restrict__ groups, int64_t n_groups, int32_t n_tau,
-               double log_prior, fmap_summary* __restrict__ out, TStat* __restrict__ tstat,
-    const uint3 bid, const dim3 gdim, int32_t* __restrict__ ref_hist = nullptr,
-    int32_t* __restrict__ ref_n = nullptr) {
-  if (ref_hist) {
-    for (int b = threadIdx.x; b < kRefBins; b += blockDim.x) ref_hist[(int64_t)bid.x * kRefBins + b] = 0;
-    if (threadIdx.x == 0) ref_n[bid.x] = 0;
-  }
+               double log_prior, fmap_summary* __restrict__ out, const uint3 bid, const dim3 gdim) {
   const Partial64* gp = groups + (int64_t)bid.x * n_groups;
   const Partial64 r = block_merge(n_groups, [&](int64_t b) { return gp[b]; });
   if (threadIdx.x == 0) {
-    if (tstat) {
-      TStat t;
-      t.S = r.sum;
-      t.M = r.max2F;
-      t.arg = r.arg;
-      t.N = r.nvalid;
-      t.done[0] = t.done[1] = 0;
-      tstat[bid.x] = t;
-    }
     fmap_summary o;
     o.flags = 0;
     o.n_valid = r.nvalid;
@@ -170,24 +153,20 @@ __device__ __forceinline__ void reduce_final_body(const Partial64* __restrict__ 
 
 __global__ void __launch_bounds__(kRedThreads)
 k_reduce_final(const Partial64* __restrict__ groups, int64_t n_groups, int32_t n_tau,
-               double log_prior, fmap_summary* __restrict__ out, TStat* __restrict__ tstat,
-               int32_t* __restrict__ ref_hist, int32_t* __restrict__ ref_n) {
-  reduce_final_body(groups, n_groups, n_tau, log_prior, out, tstat, blockIdx, gridDim, ref_hist,
-                    ref_n);
+               double log_prior, fmap_summary* __restrict__ out) {
+  reduce_final_body(groups, n_groups, n_tau, log_prior, out, blockIdx, gridDim);
 }
 
 int64_t reduce_groups_of(int64_t slots) { return std::max<int64_t>(1, (slots + kRedGroup - 1) / kRedGroup); }
 
 static cudaError_t reduce_into(const Partial* parts, int64_t n_tiles, int64_t fix0,
                                const int32_t* n_flag, int64_t entries, int64_t stride, int32_t T, int32_t n_tau, double log_prior,
-                               Partial64* groups, fmap_summary* d_summary, cudaStream_t s,
-                               TStat* tstat = nullptr, int32_t* ref_hist = nullptr,
-                               int32_t* ref_n = nullptr) {
+                               Partial64* groups, fmap_summary* d_summary, cudaStream_t s) {
   const int64_t n_groups = reduce_groups_of(n_tiles + (n_flag ? kFixSlots : 0));
   k_reduce_groups<<<dim3((unsigned)n_groups, (unsigned)T), kRedThreads, 0, s>>>(
       parts, n_tiles, fix0, n_flag, entries, stride, n_groups, groups);
   k_reduce_final<<<T, kRedThreads, 0, s>>>(groups, n_groups, n_tau > 0 ? n_tau : 1, log_prior,
-                                           d_summary, tstat, ref_hist, ref_n);
+                                           d_summary);
   return cudaGetLastError();
 }
 
@@ -200,8 +179,7 @@ cudaError_t launch_final_reduce(fmap_plan_s* p, int64_t n_tiles, const fmap_atom
   p->launches += 2;
   return reduce_into(p->ws.partials, n_tiles, p->n_tiles, fix ? p->ws.n_flag : nullptr, entries,
                      p->part_stride, p->n_templates, p->grid.n_tau, p->log_prior,
-                     (Partial64*)p->ws.groups, d_summary, s, p->ws.tstat, p->ws.ref_hist,
-                     p->ws.ref_n);
+                     (Partial64*)p->ws.groups, d_summary, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -311,7 +289,7 @@ __global__ void __launch_bounds__(kRedThreads) kb_red_final(const BItem* __restr
                                                             BUnits u) {
   batch_loop(items, u, [&](const BItem& it, int64_t k) {
     reduce_final_body((const Partial64*)it.red_buf, it.red_groups, it.g.n_tau > 0 ? it.g.n_tau : 1,
-                      it.log_prior, it.summary, nullptr, make_uint3((unsigned)k, 0, 0),
+                      it.log_prior, it.summary, make_uint3((unsigned)k, 0, 0),
                       dim3((unsigned)it.T));
   });
 }

@@ -421,26 +421,6 @@ __device__ __forceinline__ Partial partial_block_reduce(Partial p, Partial* scra
   return r;
 }
 
-// The same over consecutive calls of one loop with a single barrier:
-// scratch holds 2 x NWARPS entries, used alternately by parity, so a call's
-// warp partials never overwrite those warp 0 may still read from the call
-// before (the barrier of the call in between orders them).
-template <int NWARPS>
-__device__ __forceinline__ Partial partial_block_reduce_alt(Partial p, Partial* scratch,
-                                                            int parity) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  Partial* sc = scratch + (parity & 1) * NWARPS;
-  p = partial_warp_reduce(p);
-  if (lane == 0) sc[warp] = p;
-  __syncthreads();
-  Partial r = partial_empty();
-  if (warp == 0) {
-    r = lane < NWARPS ? sc[lane] : partial_empty();
-    r = partial_warp_reduce(r);
-  }
-  return r;
-}
-
 // 2F from the sums of one template and the cell's coefficients.
 __device__ __forceinline__ float two_f(const Coef& c, float fa_re, float fa_im, float fb_re,
                                        float fb_im) {
@@ -484,26 +464,6 @@ __device__ __forceinline__ Coef make_coef_ff(FF A, FF B, FF C, int32_t count) {
   const FF gap = ff_sub(d100, ab);
   c.valid = (df > 0.0f && gap.h + gap.l >= 0.0f) ? 1.0f : 2.0f;
   return c;
-}
-
-// First index with t[i] > x (x as int64), over n entries of int64 times.
-__device__ __forceinline__ int32_t upper_bound_i64(const int64_t* t, int32_t n, int64_t x) {
-  int32_t lo = 0, hi = n;
-  while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    if (t[mid] <= x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// First index with t[i] >= x.
-__device__ __forceinline__ int32_t lower_bound_i64(const int64_t* t, int32_t n, int64_t x) {
-  int32_t lo = 0, hi = n;
-  while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    if (t[mid] < x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
 }
 
 }  // namespace fmap
