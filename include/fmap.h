@@ -149,13 +149,13 @@ enum {
   /* exponential windows only, with FMAP_FP64: the data sums by the decayed
    * suffix recurrence E[i] = x_i + e^{-(t_{i+1} - t_i)/tau} E[i+1] (an exact
    * rearrangement of Eq. winexp's window sums: window [i0, j) =
-   * e^{-(t_i0 - t0)/tau} (E[i0] - e^{-(t_j - t_i0)/tau} E[j])), one scan per
-   * (tau, data column) in compensated FP32 instead of a sum per cell:
-   * O(N_tau N_SFT + cells) per template.  Needs n_sft <= 9000 (one
-   * template's suffix sums in shared memory; FMAP_ERR_UNSUPPORTED otherwise);
-   * with two or more templates the workspace also holds the per-cell window
-   * records and per-atom decays of every tau (32 B per cell, 4 B per atom
-   * and tau), formed by a block's first template and re-read by the rest. */
+   * e^{-(t_i0 - t0)/tau} (E[i0] - e^{-(t_j - t_i0)/tau} E[j])), by sweeps over
+   * the t0 rows that carry E at both window ends in compensated FP32, instead
+   * of a sum per cell: O(N_tau N_SFT + cells) per template.  n_sft <= 9000 (the
+   * range its accuracy is stated and checked over; FMAP_ERR_UNSUPPORTED
+   * otherwise).  The workspace also holds a copy of the atoms, and, where the
+   * rows are split into short runs, decayed sums of chunks of atoms (with two
+   * or more templates up to 4 B per atom and tau and 16 B per cell more). */
   FMAP_PLAN_EXP_RECURRENCE = 2u,
   /* the plan holds a [T][n_t0][n_tau] float map of its own (the workspace
    * grows by 4 T n_t0 n_tau bytes), used by summary-only compute calls
@@ -332,9 +332,10 @@ fmap_status fmap_compute_host(fmap_plan_t* plan, const fmap_atoms* host_atoms, f
 
 /* Per-phase device timing of a plan's compute calls, taken with CUDA events
  * recorded on each call's stream.  Phases (FMAP_N_PHASES):
- *   0 input checks and window index tables,
- *   1 antenna sums / prefix sums (rect: FP64 scans; exp: float-float suffix
- *     sums and the per-cell 2F coefficients),
+ *   0 input checks, window index tables, the copies of the atoms and (rect) the
+ *     prefix sums of antenna and data rows: the call's first launch,
+ *   1 antenna sums (exp and table: float-float) and the per-cell 2F coefficients
+ *     (with the sweeps' chunk sums),
  *   2 the windowed contraction with the fused 2F epilogue (the dominant
  *     kernel),
  *   3 the recomputation of ill-conditioned cells, the final per-template
@@ -427,7 +428,7 @@ fmap_status fmap_server_peak(fmap_server_t* server, int64_t* peak_running);
  * over the work units of all instances (atomic work counter, heaviest
  * instances first); instances are grouped in waves whose workspace fits
  * workspace_budget (0: 8 GiB).  FMAP_BATCH_AUTOTUNE times the candidate
- * occupancies of each phase and the templates per block of the recurrence on
+ * occupancies of each phase and the templates per warp of the recurrence on
  * the batch itself (cached per batch shape) before the graph is captured.
  * The items' device pointers are baked into the graph: keep them valid, and
  * rerun fmap_batch_run after changing the atoms' values in place.

@@ -14,7 +14,7 @@
 // launches are captured once into a CUDA graph that fmap_batch_run replays.
 //
 // Autotuning (FMAP_BATCH_AUTOTUNE): the occupancy of each phase's persistent
-// launch and the templates per block of the recurrence are chosen by timing
+// launch and the templates per warp of the recurrence are chosen by timing
 // the candidates on the batch itself, per size class of the batch (a
 // signature of its shape); choices are cached in memory for later batches of
 // the same class.
@@ -39,7 +39,7 @@ constexpr int kOccCandidates[] = {1, 2, 4, 8};
 
 struct Tuning {
   int occ[BP_ALL];
-  int rec_tpb;   // templates per block of the recurrence phase
+  int rec_tpb;   // templates per warp of the recurrence phase, at most
 };
 
 std::mutex g_tune_mu;

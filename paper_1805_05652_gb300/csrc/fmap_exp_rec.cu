@@ -35,9 +35,10 @@
 // into short runs to make enough warps, from the decayed sums of chunks of
 // atoms formed ahead by k_sweep_agg.
 //
-// Bound by waits for the atoms' loads and by issue: about 350 instructions per row
-// and four templates at 36 % issue, 12 warps per SM (168 registers): 23.2 ms for
-// 1024 templates x 5000 SFTs over 2000 x 2000 cells.  One block per tau with E in
+// Bound by waits for the atoms' loads and by issue: about 340 instructions per row
+// and four templates, starts included, at 43 % issue, 12 warps per SM (168 registers):
+// 21.1 ms for 1024 templates x 5000 SFTs over 2000 x 2000 cells (23.2 with the careful
+// sweep's registers in the same kernel).  One block per tau with E in
 // shared memory and a scan over the atoms per template (two block barriers, four
 // passes over shared memory) took 73.8 ms there.
 #include <math.h>

@@ -293,6 +293,8 @@ int64_t fixup_blocks_y(int32_t n_templates, bool shared) {
   return (n_templates + g - 1) / g;
 }
 
+// (The read-only inputs, i0tab, jend, rel_t, t_base, tauc and the atoms, are written
+// ahead of the ordinary launch that the chain follows: see stream_order.)
 template <int G>
 __global__ void __launch_bounds__(kFixThreads)
 k_fixup(const int64_t* list, const int32_t* n_flag,

@@ -206,7 +206,7 @@ struct Workspace {
   int32_t* n_flag = nullptr;       // [1] number of ill-conditioned entries
   int64_t* flag_list = nullptr;    // [T_ant cells] their indices, ascending
   // rect
-  float4* pa = nullptr;          // [T_ant][N+1][2] FP64 antenna prefix (a2, b2, ab, 0) as hi4, lo4
+  float4* pa = nullptr;          // [T_ant][N+1][2] float-pair antenna prefix (a2, b2, ab, 0) as hi4, lo4
   float4* px = nullptr;          // [T][N+1][2] float-float data prefix (hi4, lo4)
   // refinement: per-template fast statistics, histogram, chosen cut, the
   // candidates (cell, fast 2F, FP64 2F) and the plan's own map (if any)
@@ -322,8 +322,7 @@ cudaError_t launch_front(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);
 // Split operands of the tensor-core forms in the plan's workspace ([4T][n_pad]).
 void exp_tc_operands(const fmap_plan_s* p, void** hi, void** lo, int32_t* n_pad);
 // Each compute launcher reports how many partial slots per template it wrote.
-// launch_rect records `mark` (if non-null) between its prefix scans and the
-// per-cell kernel.
+// launch_rect records `mark` (if non-null) ahead of the per-cell kernel.
 cudaError_t launch_rect(fmap_plan_s* p, const fmap_atoms* a, float* d_2F, cudaStream_t s,
                         int64_t* tiles_used, cudaEvent_t mark);
 cudaError_t launch_exp_coef(fmap_plan_s* p, const fmap_atoms* a, cudaStream_t s);

@@ -140,8 +140,10 @@ static size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 // model (per template: a term in the atoms scanned, one in the windowed
 // sums N_sums and one in the cells N_t0 N_tau, plus a constant), with the
 // constants fitted on GB300 to the serving mix (summaries refined; median
-// error ~20 %).  Used only to choose between the exponential forms and the
-// stream priority: a poor estimate costs speed, never accuracy.
+// error ~20 %) when the recurrence was a block scan per tau: by sweeps it takes a
+// third of the estimate on large requests, so that some requests of 0.4 to 1 ms do
+// not get the high-priority stream.  Used only to choose between the exponential
+// forms and the stream priority: a poor estimate costs speed, never accuracy.
 struct CostModel {
   // N_sums of an exponential / rectangular grid, from a 64 x 64 sample of
   // its cells: a window holds min(L, data end - max(t0, first atom)) of the
@@ -430,7 +432,7 @@ fmap_status fmap_submit(fmap_server_t* s, const fmap_grid* grid, const fmap_atom
     r->prec = s->cfg.rect_precision;
     est = CostModel::rect_ms(*grid, r->n_sft, r->T);
   } else {
-    // (data sets past the recurrence's shared-memory limit take exp_precision)
+    // (data sets past the recurrence's range take exp_precision)
     const bool rec_ok = exp_rec_supported(r->n_sft, grid->n_t0);
     const double rec = CostModel::exp_rec_ms(*grid, r->n_sft, r->T);
     bool use_rec = rec_ok && s->cfg.exp_mode == FMAP_SERVER_EXP_RECURRENCE;
