@@ -19,16 +19,16 @@
 //
 // Where E at j can be much larger than the window's sum, the sweep takes care
 // (CARE): E at j is carried like E at i0, the tail's exponent is a float pair, and where
-// a window holds a small part of the atoms that its E covers, E starts anew from the
-// window alone.  That is for warps whose windows may start in a long outage (they hold
-// its last atoms only, and the tail is near 1), by the data's longest gap, and for data
-// whose level varies more than kLevelRange-fold (a glitch behind the windows).  2F
+// tail E[j] is much larger than the window's sum, E starts anew from the window alone.
+// That is for warps whose windows may start in a long outage (they hold their last atoms
+// only, and the tail is near 1), by the data's longest gap, and for data whose level
+// varies more than kLevelRange-fold (a glitch behind the windows).  2F
 // against the FP64 oracle at worst: in an outage of 3500 SFTs, tau of 1000-1750,
 // 2.8e-5 without and 1.3e-6 with; an atom 4000 times the noise up to 1350 SFTs behind the
-// windows 4.0e-5 and 9.8e-6.  Four templates per warp take it as two pairs (the second
-// E's registers); 1024 templates of 5000 SFTs, 2000 x 2000 cells: 22.2 ms, with an
-// outage of 1500 SFTs 37 ms (38 without the care: other gaps than the tabulated ones
-// take an FP64 exp).
+// windows 4.0e-5 and 1.5e-6; both on small coarse grids up to 2.7e-3 and 5.2e-6.  Four
+// templates per warp take it as two pairs (the second E's registers); 1024 templates of
+// 5000 SFTs, 2000 x 2000 cells: 22.3 ms, with an outage of 400 / 1500 SFTs 33.6 / 38.8 ms
+// (31.9 / 38.0 without the care: gaps off the table take an FP64 exp).
 //
 // A warp starts from zero at its last row's window ends and sums those windows
 // first (long runs of rows, many templates), or, where the rows must be split
@@ -276,8 +276,6 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
   sweep_tab_load<1>(s_pw, tt, lane);
   const float c2 = tt->c2[0];
   const float c2l = CARE ? (float)(-1.4426950408889634 * tt->inv_tau - (double)c2) : 0.0f;
-  const float half_tau = -0.72134752f / (c2 * (float)g.t_sft);   // tau / (2 T_sft)
-  int32_t jz = A.n;   // CARE: where E at j starts from zero, at the latest
   const int64_t cells = (int64_t)g.n_t0 * n_tau;
   const int64_t tb = n > 0 ? *A.t_base : 0;
   const float4* x = A.x + (int64_t)tg0 * n;
@@ -348,7 +346,7 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
     jc = min(n, bj * q.chunk);
   } else {
     // E starts from zero at each lane's window end of the last row
-    jc = jz = j;
+    jc = j;
     ic = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)j);
     const int32_t j_all = (int32_t)__reduce_min_sync(0xffffffffu, (unsigned)j);
     int32_t tn = n > 0 ? atom_time(A, ic) : 0;
@@ -500,18 +498,41 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
     if (END && tail > 0.5f) tail = exp2f(xj);
     // (what the rounded slope and exponent leave: up to 4e-7)
     if (CARE) tail = fmaf(tail, 0.69314718f * fmaf(c2l, dj, fmaf(c2, dj, -xj)), tail);
+    float pre2 = 1.0f;
+    const int32_t d0 = (int32_t)(ti - t0r);
+    if (d0 != 0) {
+      const float pre = rec_ex2(c2 * (float)d0);
+      pre2 = pre * pre;
+    }
     if constexpr (CARE) {
-      // E at j against the window's sum, in noise: tail times the root of the atoms
-      // that E sums (up to tau / 2 SFTs, none past jz) against the root of the
-      // window's.  Where it is larger, E at i0 is summed anew from the window alone.
-      const float part = tail * tail * fminf(half_tau, (float)(jz - j)), own = (float)(j - i0);
-      if (__any_sync(0xffffffffu, j > i0 + 1 && part > 4.0f * own)) {
-        const bool anew = j > i0 && part > own;   // (others that soon will)
-        const int32_t top = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)(anew ? j : i0));
+      // 2F's error is about 2 eps sqrt(S max(2F, 1)), with eps that of E read in FP32 and
+      // S what 2F would be of tail E[j] at its worst direction.  Where S is more than 16
+      // max(2F, 1) for any template, E at i0 is summed anew from the window alone, and E
+      // at j starts from zero at its end.  (Its atoms outnumber the window's by as much
+      // then, or it holds a glitch that the rows to come never see again: the sums stay
+      // few.)
+      bool much = false, soon = false;
+      const uint64_t qi = Ei.scale(), qj = Ej.scale(), pt = pk2(tail, tail);
+#pragma unroll
+      for (int k = 0; k < G; ++k) {
+        const float4 c = cf[SH ? 0 : k];
+        const uint64_t e0 = mul2(pt, Ej.get(k, 0, qj)), e1 = mul2(pt, Ej.get(k, 1, qj));
+        const float k1 = c.x * pre2, k2 = c.z * pre2;
+        const float v = two_f_pairs(sub2(Ei.get(k, 0, qi), e0), sub2(Ei.get(k, 1, qi), e1),
+                                    pk2(-c.y, -c.y), k1, k2, tiny2);
+        float x0, y0, x1, y1;
+        up2(mul2(e0, e0), x0, y0);
+        up2(mul2(e1, e1), x1, y1);
+        const float S = fmaf(fmaf(k2 * c.y, c.y, k1), x0 + y0, k2 * (x1 + y1)), scale = fmaxf(v, 1.0f);
+        much |= c.w == 1.0f && S > 16.0f * scale;
+        soon |= c.w == 1.0f && S > scale;
+      }
+      if (__any_sync(0xffffffffu, much)) {
+        const int32_t top = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)(much ? j : i0));
+        const bool anew = soon && j <= top;   // (those on the way there at no cost)
         if (anew) {
           Ei.zero();
           Ej.zero();
-          jz = j;
         }
         int32_t tn = atom_time(A, top);
         constexpr int B = 4;   // atoms loaded ahead of the serial chain
@@ -535,12 +556,6 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
         }
         Ei.renorm();
       }
-    }
-    float pre2 = 1.0f;
-    const int32_t d0 = (int32_t)(ti - t0r);
-    if (d0 != 0) {
-      const float pre = rec_ex2(c2 * (float)d0);
-      pre2 = pre * pre;
     }
     const uint64_t qi = Ei.scale(), qj = Ej.scale(), nt = pk2(-tail, -tail);
 #pragma unroll
@@ -595,21 +610,19 @@ __device__ __noinline__ void rec_unit_apart(const RecArgs& A, int32_t tg0, int32
     exp_rec_unit<G, SHORT, SH, true, CARE>(A, t0, u1, s_pw, lane);
 }
 // A window whose tail is above 1/4 ends within 1.4 tau of its first atom: its t0 lies
-// in a gap of more than the rest of its length.
+// in a gap of more than the rest of its length (of shorter ones, more than half of it).
 template <int G, bool SHORT, bool SH, bool BATCH>
 __device__ __forceinline__ void rec_unit(const RecArgs& A, int64_t unit, float2* s_pw, int lane) {
   const int32_t tg0 = (int32_t)(unit % A.q.n_tgrp) * G;
   const int64_t u1 = unit / A.q.n_tgrp;
   const int32_t gap = longest_gap(A.irr);
-  const bool varies = !SHORT && level_varies(A.level);
+  const bool varies = level_varies(A.level);
   if (!gap && !varies) return exp_rec_unit<G, SHORT, SH, false, false>(A, tg0, u1, s_pw, lane);
-  if constexpr (!SHORT) {
-    const int32_t grp = A.q.n_grp - 1 - (int32_t)(u1 / A.q.n_seg);
-    const float rest = (float)exp_cut8_of(A.g) / 8.0f - 1.4f;   // (of the group's shortest windows)
-    if (varies || (float)gap > rest * (float)grid_tau(A.g, A.ax, grp * 32)) {
-      const RecArgs B = A;   // (its address is taken)
-      return rec_unit_apart<G < 4 ? G : 2, false, SH, true>(B, tg0, min(tg0 + G, A.T), u1, s_pw, lane);
-    }
+  const int32_t grp = A.q.n_grp - 1 - (int32_t)(u1 / A.q.n_seg);
+  const float cut = (float)exp_cut8_of(A.g) / 8.0f, rest = fmaxf(cut - 1.4f, 0.5f * cut);
+  if (varies || (float)gap > rest * (float)grid_tau(A.g, A.ax, grp * 32)) {   // (the group's shortest windows)
+    const RecArgs B = A;   // (its address is taken)
+    return rec_unit_apart<G < 4 ? G : 2, SHORT, SH, true>(B, tg0, min(tg0 + G, A.T), u1, s_pw, lane);
   }
   if constexpr (BATCH) {
     const RecArgs B = A;

@@ -98,6 +98,32 @@ def test_outage_and_glitch_in_a_batch(n_templates):
         check_map(got, ref, val, TOL["rec"])
 
 
+@pytest.mark.parametrize("cut8", [0, 4, 12])
+@pytest.mark.parametrize("n_templates,own", [(1, False), (3, True), (6, False)])
+def test_glitch_behind_an_outage(n_templates, own, cut8):
+    """Windows whose t0 lies in an outage and whose end lies before a glitch, on a coarse
+    grid: E at their ends is a thousand times their sums.  Windows of 3 tau and
+    shorter ones, plans and batches."""
+    n, first = 240, 90
+    grid = Grid(0, 40 * T_SFT // 3, 50, 15 * T_SFT, 11 * T_SFT, 60, EXP, T_SFT, cut8)
+    inst = synth.make_instance(1206, n_det=2, presence=0.9, n_merged=n, n_templates=n_templates, grid=grid,
+                               shared_antenna=not own)
+    t, x = inst.t.copy(), inst.fafb.copy()
+    t[first:] += 300 * T_SFT
+    x[:, :, first + 40] *= np.float32(1e3)
+    inst = synth.Instance(t, inst.antenna, x, grid, not own)
+    ref, val, _ = oracle.fmap(t, inst.antenna, x, grid.as_tuple(), mode="fast")
+    d = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (t, inst.antenna, x)]
+    p = fm.Plan(grid, n, n_templates, "fp64",
+                fm.FMAP_PLAN_EXP_RECURRENCE | (fm.FMAP_PLAN_PER_TEMPLATE_ANTENNA if own else 0))
+    p.set_refine(0)
+    m, _ = p.compute(*d)
+    assert p.status() == fm.FMAP_OK
+    p.close()
+    for got in (m.cpu().numpy().astype(np.float64), _batch_maps([inst])[0]):
+        check_map(got, ref, val, TOL["rec"])
+
+
 def test_level_of_one_call_is_not_the_next_ones():
     """A call on data with a glitch, and the same plan on data without: the second's map
     is bit for bit that of a plan that never saw the first."""
