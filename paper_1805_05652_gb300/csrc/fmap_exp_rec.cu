@@ -17,18 +17,19 @@
 // scaled by the tail) is enough, as long as E at j is of the window sum's size.
 // Windows cut before 3 tau, whose tail is near 1, carry E at j like E at i0.
 //
-// Where E at j can be much larger than the window's sum, the sweep takes care
-// (CARE): E at j is carried like E at i0, the tail's exponent is a float pair, and where
-// tail E[j] is much larger than the window's sum, E starts anew from the window alone.
-// That is for warps whose windows may start in a long outage (they hold their last atoms
-// only, and the tail is near 1), by the data's longest gap, and for data whose level
-// varies more than kLevelRange-fold (a glitch behind the windows).  2F
-// against the FP64 oracle at worst: in an outage of 3500 SFTs, tau of 1000-1750,
-// 2.8e-5 without and 1.3e-6 with; an atom 4000 times the noise up to 1350 SFTs behind the
-// windows 4.0e-5 and 1.5e-6; both on small coarse grids up to 2.7e-3 and 5.2e-6.  Four
-// templates per warp take it as two pairs (the second E's registers); 1024 templates of
-// 5000 SFTs, 2000 x 2000 cells: 22.3 ms, with an outage of 400 / 1500 SFTs 33.6 / 38.8 ms
-// (31.9 / 38.0 without the care: gaps off the table take an FP64 exp).
+// Where E at j can be much larger than the window's sum, the sweep takes care (CARE):
+// both E, the tail and the difference in float-float, as in the antenna sums.  That is
+// for warps whose windows may start in a long outage (they hold their last atoms only,
+// and the tail is near 1), by the data's longest gap, and for data whose level varies
+// more than kLevelRange-fold (a glitch behind the windows).  2F against the FP64 oracle
+// at worst: in an outage of 3500 SFTs, tau of 1000-1750, 2.8e-5 without and 5e-7 with; an
+// atom 4000 times the noise up to 1350 SFTs behind the windows 4.0e-5 and 3e-7; both on
+// small coarse grids up to 2.7e-3 and 3e-6.  Four templates per warp take it as two pairs
+// (registers); 1024 templates of 5000 SFTs, 2000 x 2000 cells: 22.9 ms, with an outage
+// of 400 / 1500 SFTs 33.7 / 38.2 ms (31.9 / 38.0 without the care: gaps off the table take
+// an FP64 exp), with a glitch 56 ms.  (Plain sums that start anew from the window where
+// little is left of it: the same accuracy within a factor of ten, a glitch 110 ms, a band of 16
+// templates 4.4 ms instead of 0.48.)
 //
 // A warp starts from zero at its last row's window ends and sums those windows
 // first (long runs of rows, many templates), or, where the rows must be split
@@ -36,9 +37,8 @@
 // atoms formed ahead by k_sweep_agg.
 //
 // Bound by waits for the atoms' loads and by issue: about 340 instructions per row
-// and four templates, starts included, at 43 % issue, 12 warps per SM (168 registers):
-// 21.1 ms for 1024 templates x 5000 SFTs over 2000 x 2000 cells (23.2 with the careful
-// sweep's registers in the same kernel).  One block per tau with E in
+// and four templates, starts included, at 42 % issue, 12 warps per SM (168 registers):
+// 22.1 ms for 1024 templates x 5000 SFTs over 2000 x 2000 cells.  One block per tau with E in
 // shared memory and a scan over the atoms per template (two block barriers, four
 // passes over shared memory) took 73.8 ms there.
 #include <math.h>
@@ -160,6 +160,43 @@ struct PlainCursor {
   __device__ __forceinline__ uint64_t get(int g, int c, uint64_t) const { return E[g][c]; }
 };
 
+// E of G templates in float-float, an atom at a time (the careful sweep).
+template <int G>
+struct CareCursor {
+  uint64_t Kh[G][2], Kl[G][2];
+  static constexpr int32_t run = 0;
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) Kh[g][c] = Kl[g][c] = 0ull;
+  }
+  __device__ __forceinline__ void renorm() {}
+  __device__ __forceinline__ void step(FF r, const Atom<G>& a) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      set(g, 0, ff2_fma_sum(a.x[g].x, r, FF2{Kh[g][0], Kl[g][0]}));
+      set(g, 1, ff2_fma_sum(a.x[g].y, r, FF2{Kh[g][1], Kl[g][1]}));
+    }
+  }
+  __device__ __forceinline__ void set(int g, int c, const FF2& v) {
+    Kh[g][c] = v.h;
+    Kl[g][c] = v.l;
+  }
+};
+// E at i0 - tail E at j
+template <int G>
+__device__ __forceinline__ uint64_t care_diff(const CareCursor<G>& i, const CareCursor<G>& j, int g,
+                                              int c, FF tail) {
+  const FF2 d = ff2_fma_sum(i.Kh[g][c], FF{-tail.h, -tail.l}, FF2{j.Kh[g][c], j.Kl[g][c]});
+  return add2(d.h, add2(d.l, i.Kl[g][c]));
+}
+// 1 / r for a decay r in (0, 1] that is not tiny
+__device__ __forceinline__ FF ff_rcp(FF r) {
+  const float y = __frcp_rn(r.h);
+  return fast_two_sum(y, y * fmaf(-r.l, y, fmaf(-r.h, y, 1.0f)));
+}
+
 struct RecArgs {
   const int32_t* rel_t;
   const int64_t* t_base;
@@ -191,6 +228,14 @@ __device__ __forceinline__ int32_t atom_time(const RecArgs& A, int32_t a) {
   return a < A.n ? __ldg(A.rel_t + a) : __ldg(A.rel_t + A.n - 1) + (int32_t)A.g.t_sft;
 }
 
+// Whether the sweep of a group of 32 tau takes care (see the top).  A window whose tail is
+// above 1/4 ends within 1.4 tau of its first atom: its t0 lies in a gap of more than the
+// rest of its length (of shorter ones, more than half of it); gap: the data's longest.
+__device__ __forceinline__ bool rec_careful(const RecArgs& A, int32_t grp, int32_t gap) {
+  const float cut = (float)exp_cut8_of(A.g) / 8.0f, rest = fmaxf(cut - 1.4f, 0.5f * cut);
+  return (gap > 0 && (float)gap > rest * (float)grid_tau(A.g, A.ax, grp * 32)) || level_varies(A.level);
+}
+
 // Chunk maps of one (template group, 32 tau, chunk): E[first] = S + R E[next].
 template <int G, bool IRR>
 __device__ __forceinline__ void rec_agg_unit(const RecArgs& A, int64_t unit, float2* s_pw,
@@ -207,6 +252,7 @@ __device__ __forceinline__ void rec_agg_unit(const RecArgs& A, int64_t unit, flo
   const uint2 xs = make_uint2((uint32_t)A.n, (uint32_t)(n_t - 1));
   const int32_t lo = ch * q.chunk, hi = min(A.n, lo + q.chunk);
   const int32_t run = rec_run(A.n);
+  const bool care = rec_careful(A, grp, longest_gap(A.irr));   // every atom in float-float
   Cursor<G> E;
   E.zero();
   FF R{1.0f, 0.0f};
@@ -227,6 +273,10 @@ __device__ __forceinline__ void rec_agg_unit(const RecArgs& A, int64_t unit, flo
       if (a1 - 1 - u < lo) break;
       E.step(sweep_gap_decay<1, IRR>(s_pw, tn - t[u], inv, t_sft, lane, tt), at[u]);
       tn = t[u];
+      if (care) {
+        R = ff_mul(R, FF{E.Qh, E.Qc});
+        E.renorm();
+      }
     }
     if (E.run >= run) {
       R = ff_mul(R, FF{E.Qh, E.Qc});
@@ -263,8 +313,8 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
   constexpr int NC = SH ? 1 : G;   // coefficient sets
   // each cursor's next atom is loaded a step ahead, where registers allow
   constexpr bool PF = G < 4;
-  constexpr bool END = SHORT || CARE;   // E at j is carried like E at i0
-  static_assert(PF || !END, "four templates: the 3 tau cut, level data");
+  constexpr bool END = SHORT && !CARE;   // E at j is carried like E at i0
+  static_assert(PF || !(SHORT || CARE), "four templates: the 3 tau cut, level data");
   const int32_t seg = (int32_t)(u1 % q.n_seg);
   const int32_t grp = q.n_grp - 1 - (int32_t)(u1 / q.n_seg);
   const int32_t n = A.n, n_tau = g.n_tau, run = rec_run(n);
@@ -275,7 +325,6 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
   const TauTab* tt = A.tauc + nn;
   sweep_tab_load<1>(s_pw, tt, lane);
   const float c2 = tt->c2[0];
-  const float c2l = CARE ? (float)(-1.4426950408889634 * tt->inv_tau - (double)c2) : 0.0f;
   const int64_t cells = (int64_t)g.n_t0 * n_tau;
   const int64_t tb = n > 0 ? *A.t_base : 0;
   const float4* x = A.x + (int64_t)tg0 * n;
@@ -283,10 +332,16 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
   const int32_t t_sft = (int32_t)g.t_sft;
   const uint32_t inv = gap_inverse(t_sft);
   int32_t i0 = A.i0tab[m_hi - 1], j = A.jend[(int64_t)(m_hi - 1) * n_tau + nn];
-  Cursor<G> Ei;
+  typename std::conditional<CARE, CareCursor<G>, Cursor<G>>::type Ei;
   Ei.zero();
-  typename std::conditional<END, Cursor<G>, PlainCursor<G>>::type Ej;
+  typename std::conditional<CARE, CareCursor<G>,
+                            typename std::conditional<END, Cursor<G>, PlainCursor<G>>::type>::type Ej;
   Ej.zero();
+  // CARE: the tail factor in float-float, by the decays that the cursors pass; lost: too
+  // small a decay or tail to go on from (formed anew by an FP64 exp when it counts again)
+  constexpr float kTailLost = 1e-18f, kDecayLost = 1e-6f;
+  FF tail_ff{0.0f, 0.0f};
+  bool lost = true;
   int32_t run_j = 0;   // END: the most atoms a lane's Ej took since its renormalisation
   int32_t ic, jc;
   if (q.n_chunks > 0) {
@@ -435,7 +490,12 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
         const int32_t t = ei;
         ei = __ldg(A.rel_t + max(ic - 1, 0));
         ai.load(x, xs, ic - 1);
-        Ei.step(sweep_gap_decay<1, IRR>(s_pw, ti - t, inv, t_sft, lane, tt), cur);
+        const FF r = sweep_gap_decay<1, IRR>(s_pw, ti - t, inv, t_sft, lane, tt);
+        Ei.step(r, cur);
+        if constexpr (CARE) {
+          tail_ff = ff_mul(tail_ff, r);
+          lost |= r.h < kDecayLost || tail_ff.h < kTailLost;
+        }
         ti = t;
         if (Ei.run >= run) Ei.renorm();
       }
@@ -447,7 +507,12 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
           const int32_t t = ej;
           ej = __ldg(A.rel_t + max(jc - 1, 0));
           aj.load(x, xs, jc - 1);
-          Ej.step(sweep_gap_decay<1, IRR>(s_pw, tj - t, inv, t_sft, lane, tt), cur);
+          const FF r = sweep_gap_decay<1, IRR>(s_pw, tj - t, inv, t_sft, lane, tt);
+          Ej.step(r, cur);
+          if constexpr (CARE) {
+            tail_ff = ff_mul(tail_ff, ff_rcp(r));
+            lost |= r.h < kDecayLost;
+          }
           tj = t;
         }
         if constexpr (END)
@@ -496,68 +561,29 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
     const float dj = (float)(tj - ti), xj = c2 * dj;
     float tail = rec_ex2(xj);
     if (END && tail > 0.5f) tail = exp2f(xj);
-    // (what the rounded slope and exponent leave: up to 4e-7)
-    if (CARE) tail = fmaf(tail, 0.69314718f * fmaf(c2l, dj, fmaf(c2, dj, -xj)), tail);
+    if constexpr (CARE) {
+      lost |= tail < kTailLost;
+      if (lost) {
+        tail_ff = FF{tail, 0.0f};
+        if (tail >= kTailLost) {
+          const float2 v = slow_decay(tj - ti, tt->inv_tau);
+          tail_ff = FF{v.x, v.y};
+          lost = false;
+        }
+      }
+    }
     float pre2 = 1.0f;
     const int32_t d0 = (int32_t)(ti - t0r);
     if (d0 != 0) {
       const float pre = rec_ex2(c2 * (float)d0);
       pre2 = pre * pre;
     }
-    if constexpr (CARE) {
-      // 2F's error is about 2 eps sqrt(S max(2F, 1)), with eps that of E read in FP32 and
-      // S what 2F would be of tail E[j] at its worst direction.  Where S is more than 16
-      // max(2F, 1) for any template, E at i0 is summed anew from the window alone, and E
-      // at j starts from zero at its end.  (Its atoms outnumber the window's by as much
-      // then, or it holds a glitch that the rows to come never see again: the sums stay
-      // few.)
-      bool much = false, soon = false;
-      const uint64_t qi = Ei.scale(), qj = Ej.scale(), pt = pk2(tail, tail);
-#pragma unroll
-      for (int k = 0; k < G; ++k) {
-        const float4 c = cf[SH ? 0 : k];
-        const uint64_t e0 = mul2(pt, Ej.get(k, 0, qj)), e1 = mul2(pt, Ej.get(k, 1, qj));
-        const float k1 = c.x * pre2, k2 = c.z * pre2;
-        const float v = two_f_pairs(sub2(Ei.get(k, 0, qi), e0), sub2(Ei.get(k, 1, qi), e1),
-                                    pk2(-c.y, -c.y), k1, k2, tiny2);
-        float x0, y0, x1, y1;
-        up2(mul2(e0, e0), x0, y0);
-        up2(mul2(e1, e1), x1, y1);
-        const float S = fmaf(fmaf(k2 * c.y, c.y, k1), x0 + y0, k2 * (x1 + y1)), scale = fmaxf(v, 1.0f);
-        much |= c.w == 1.0f && S > 16.0f * scale;
-        soon |= c.w == 1.0f && S > scale;
-      }
-      if (__any_sync(0xffffffffu, much)) {
-        const int32_t top = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)(much ? j : i0));
-        const bool anew = soon && j <= top;   // (those on the way there at no cost)
-        if (anew) {
-          Ei.zero();
-          Ej.zero();
-        }
-        int32_t tn = atom_time(A, top);
-        constexpr int B = 4;   // atoms loaded ahead of the serial chain
-        for (int32_t a1 = top; a1 > i0; a1 -= B) {
-          Atom<G> at[B];
-          int32_t t[B];
-#pragma unroll
-          for (int u = 0; u < B; ++u) {
-            at[u].load(x, xs, a1 - 1 - u);
-            t[u] = __ldg(A.rel_t + max(a1 - 1 - u, 0));
-          }
-#pragma unroll
-          for (int u = 0; u < B; ++u) {
-            const int32_t a = a1 - 1 - u;
-            if (a < i0) break;
-            const FF r = sweep_gap_decay<1, IRR>(s_pw, tn - t[u], inv, t_sft, lane, tt);
-            tn = t[u];
-            if (anew && a < j) Ei.step(r, at[u]);
-          }
-          if ((top - a1) / B % 5 == 4) Ei.renorm();   // (every 20 atoms)
-        }
-        Ei.renorm();
-      }
+    uint64_t qi = 0ull, qj = 0ull;
+    const uint64_t nt = pk2(-tail, -tail);
+    if constexpr (!CARE) {
+      qi = Ei.scale();
+      qj = Ej.scale();
     }
-    const uint64_t qi = Ei.scale(), qj = Ej.scale(), nt = pk2(-tail, -tail);
 #pragma unroll
     for (int k = 0; k < G; ++k) {
       const float4 c = cf[SH ? 0 : k];
@@ -566,8 +592,14 @@ __device__ __forceinline__ void exp_rec_unit(const RecArgs& A, int32_t tg0, int6
       const bool ok = c.w == 1.0f && in_grid;
       const float k1 = ok ? c.x * pre2 : -INFINITY, k2 = ok ? c.z * pre2 : 0.0f;
       if (SH ? k == 0 : true) nv[SH ? 0 : k] += ok ? 1 : 0;
-      const uint64_t f0 = fma2(nt, Ej.get(k, 0, qj), Ei.get(k, 0, qi));
-      const uint64_t f1 = fma2(nt, Ej.get(k, 1, qj), Ei.get(k, 1, qi));
+      uint64_t f0, f1;
+      if constexpr (CARE) {
+        f0 = care_diff(Ei, Ej, k, 0, tail_ff);
+        f1 = care_diff(Ei, Ej, k, 1, tail_ff);
+      } else {
+        f0 = fma2(nt, Ej.get(k, 0, qj), Ei.get(k, 0, qi));
+        f1 = fma2(nt, Ej.get(k, 1, qj), Ei.get(k, 1, qi));
+      }
       const float v = two_f_pairs(f0, f1, pk2(-c.y, -c.y), k1, k2, tiny2);
       if (store && k < n_t) (mp + k * cells)[cell] = fmaxf(v, 0.0f);
       // rows come in descending order: the later one wins a tie
@@ -609,18 +641,14 @@ __device__ __noinline__ void rec_unit_apart(const RecArgs& A, int32_t tg0, int32
   for (int32_t t0 = tg0; t0 < tg1; t0 += G)
     exp_rec_unit<G, SHORT, SH, true, CARE>(A, t0, u1, s_pw, lane);
 }
-// A window whose tail is above 1/4 ends within 1.4 tau of its first atom: its t0 lies
-// in a gap of more than the rest of its length (of shorter ones, more than half of it).
 template <int G, bool SHORT, bool SH, bool BATCH>
 __device__ __forceinline__ void rec_unit(const RecArgs& A, int64_t unit, float2* s_pw, int lane) {
   const int32_t tg0 = (int32_t)(unit % A.q.n_tgrp) * G;
   const int64_t u1 = unit / A.q.n_tgrp;
   const int32_t gap = longest_gap(A.irr);
-  const bool varies = level_varies(A.level);
-  if (!gap && !varies) return exp_rec_unit<G, SHORT, SH, false, false>(A, tg0, u1, s_pw, lane);
-  const int32_t grp = A.q.n_grp - 1 - (int32_t)(u1 / A.q.n_seg);
-  const float cut = (float)exp_cut8_of(A.g) / 8.0f, rest = fmaxf(cut - 1.4f, 0.5f * cut);
-  if (varies || (float)gap > rest * (float)grid_tau(A.g, A.ax, grp * 32)) {   // (the group's shortest windows)
+  if (!gap && !level_varies(A.level))
+    return exp_rec_unit<G, SHORT, SH, false, false>(A, tg0, u1, s_pw, lane);
+  if (rec_careful(A, A.q.n_grp - 1 - (int32_t)(u1 / A.q.n_seg), gap)) {
     const RecArgs B = A;   // (its address is taken)
     return rec_unit_apart<G < 4 ? G : 2, SHORT, SH, true>(B, tg0, min(tg0 + G, A.T), u1, s_pw, lane);
   }

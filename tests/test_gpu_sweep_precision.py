@@ -124,6 +124,27 @@ def test_glitch_behind_an_outage(n_templates, own, cut8):
         check_map(got, ref, val, TOL["rec"])
 
 
+@pytest.mark.parametrize("n_templates", [1, 2, 7])
+def test_care_over_steps_of_many_tau(n_templates):
+    """Rows 150 SFTs apart and tau from one SFT: between two rows the decays of a cursor's
+    atoms pass below the FP32 range and back."""
+    grid = Grid(0, 150 * T_SFT, 12, T_SFT, 3 * T_SFT, 70, EXP)
+    inst = synth.make_instance(1207, n_det=2, presence=0.9, n_merged=1900, n_templates=n_templates, grid=grid)
+    t, x = inst.t.copy(), inst.fafb.copy()
+    t[700:] += 60 * T_SFT
+    x[:, :, 300::400] *= np.float32(1e3)
+    inst = synth.Instance(t, inst.antenna, x, grid)
+    ref, val, _ = oracle.fmap(t, inst.antenna, x, grid.as_tuple(), mode="fast")
+    d = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (t, inst.antenna, x)]
+    p = fm.Plan(grid, 1900, n_templates, "fp64", fm.FMAP_PLAN_EXP_RECURRENCE)
+    p.set_refine(0)
+    m, _ = p.compute(*d)
+    assert p.status() == fm.FMAP_OK
+    p.close()
+    for got in (m.cpu().numpy().astype(np.float64), _batch_maps([inst])[0]):
+        check_map(got, ref, val, TOL["rec"])
+
+
 def test_level_of_one_call_is_not_the_next_ones():
     """A call on data with a glitch, and the same plan on data without: the second's map
     is bit for bit that of a plan that never saw the first."""
